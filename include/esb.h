@@ -429,11 +429,13 @@ esb_status esb_gemm(int64_t M, int64_t N, int64_t K,
  *   workspace  [device] >= esb_gemm_tiled_workspace_bytes(M, N, K) bytes,
  *              16-byte aligned, contents undefined before and after (the
  *              call overwrites it)
- * Shapes the tiled kernel does not take (N < 256, 256 not a multiple of the
- * output's codes per word, or fewer than 2^32 multiply-adds, where the
- * other kernels finish first) run esb_gemm's kernels; the workspace is then
- * unused.  Errors: as esb_gemm, and ALIGN (workspace) or INVALID_ARG
- * (workspace too small). */
+ * Shapes the tiled kernel does not take (N < 256, fewer than 2^32
+ * multiply-adds of 4-bit operands, or fewer than 2^28 with output codes of
+ * 3, 5 or 6 bits, where the other kernels finish first) run esb_gemm's
+ * kernels; the workspace is then unused.  With output codes of 3, 5 or 6
+ * bits a workspace that is NULL, too small or misaligned also selects
+ * esb_gemm's kernels.  Errors: as esb_gemm, and otherwise ALIGN (workspace)
+ * or INVALID_ARG (workspace too small). */
 size_t esb_gemm_tiled_workspace_bytes(int64_t M, int64_t N, int64_t K);
 esb_status esb_gemm_tiled(int64_t M, int64_t N, int64_t K,
                           const uint32_t* A, int64_t lda, esb_format fa,

@@ -530,7 +530,8 @@ esb_status esb_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A, in
     GemmOutputs o{ep, acc_out, y_out, codes_out, ldo};
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int out_cpw = codes_out ? 32 / ep->fmt_out.b : 8;
-    if (!gemm_tiled_ok(M, N, K, fa.b, fa.k, fb.b, fb.k, out_cpw)) {
+    const bool ws_ok = workspace && workspace_bytes >= gemm_tiled_workspace_bytes(M, N, K) && aligned16(workspace);
+    if (!gemm_tiled_ok(M, N, K, fa.b, fa.k, fb.b, fb.k, out_cpw) || (!ws_ok && gemm_tiled_optional(out_cpw))) {
         // esb_gemm's kernels: one fp32 accumulation
         if ((double)K * fmt_max_image(fa.b, fa.k) * fmt_max_image(fb.b, fb.k) >= 16777216.0) return ESB_ERR_RANGE;
         const cudaError_t e = launch_gemm(M, N, K, A, lda, fa.b, fa.k, B, ldb, fb.b, fb.k, o, st);

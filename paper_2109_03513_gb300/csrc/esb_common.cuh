@@ -251,13 +251,15 @@ __device__ __forceinline__ uint32_t bucket_code(int j, const ProjParams& p)
     return mag | (p.is_signed ? (1u << (p.b - 1)) : 0u);
 }
 
-// Build the cell table of the thresholds T (all threads of the block; T is
-// complete and visible).  Returns, identically in every thread, whether the
-// table is usable; then h0 is the first cell's index and hmax the last
-// entry.  The last cell lies above T_(L-2): every number there (and +Inf,
+// Threads t of nt fill the cell table of the thresholds T (complete and
+// visible).  Returns, identically in every thread, whether the table fits
+// its cap entries; then h0 is the first cell's index, hmax the last entry,
+// and the table is usable unless some thread's `bad` is set (a cell with two
+// thresholds).  The last cell lies above T_(L-2): every number there (and +Inf,
 // and every value clamped to it) takes the top code, NaN the zero code.
-template <int B, int CAP>
-__device__ inline bool build_cells(uint2* cells, int& h0, int& hmax, const float* T, const ProjParams& p)
+template <int B>
+__device__ inline bool fill_cells(uint2* cells, int cap, int& h0, int& hmax, const float* T, const ProjParams& p, int t,
+                                  int nt, bool& bad)
 {
     constexpr int L = 1 << (B - 1);
     const int sh = cell_shift(p.k);
@@ -266,9 +268,9 @@ __device__ inline bool build_cells(uint2* cells, int& h0, int& hmax, const float
     if (h0 < 0) h0 = 0;
     const int H = (int)(tl >> sh) + 2 - h0;
     hmax = H - 1;
-    if (tl >= 0x7f800000u || H > CAP) return false;             // uniform across the block
-    bool bad = false;
-    for (int c = threadIdx.x; c < H; c += blockDim.x) {
+    bad = false;
+    if (tl >= 0x7f800000u || H > cap) return false;             // the same for every thread
+    for (int c = t; c < H; c += nt) {
         const float s = __uint_as_float((uint32_t)(h0 + c) << sh);
         int g = 0;                                              // #{T_j <= s_c}
 #pragma unroll
@@ -286,6 +288,15 @@ __device__ inline bool build_cells(uint2* cells, int& h0, int& hmax, const float
         }
         cells[c] = make_uint2(__float_as_uint(thr), lo | (hi << 16));
     }
+    return true;
+}
+
+// fill_cells by the whole block.
+template <int B, int CAP>
+__device__ inline bool build_cells(uint2* cells, int& h0, int& hmax, const float* T, const ProjParams& p)
+{
+    bool bad;
+    if (!fill_cells<B>(cells, CAP, h0, hmax, T, p, threadIdx.x, blockDim.x, bad)) return false;
     return !__syncthreads_or(bad);
 }
 
@@ -547,6 +558,39 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
           "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// The same loads without the wait: several may be in flight, and none of
+// their registers is read before tmem_wait_ld.
+__device__ __forceinline__ void tmem_ld16_nw(uint32_t taddr, uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld8_nw(uint32_t taddr, uint32_t* r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld4_nw(uint32_t taddr, uint32_t* r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+// The registers pass through the wait, so no use of them can move above it.
+template <int NR>
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[NR])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < NR; i++) asm volatile("" : "+r"(r[i]));
 }
 
 // 32 lanes x 4 columns.

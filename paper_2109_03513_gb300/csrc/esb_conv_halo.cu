@@ -325,7 +325,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
     const int half_cols = BN / 2;
-    const bool split = (half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0);
+    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
     const int epi_warps = split ? 8 : 4;
     const int cbs = g.cblocks;
     // E4M3 tables of 5/6-bit word-slot operands (4-bit codes decode by SWAR)

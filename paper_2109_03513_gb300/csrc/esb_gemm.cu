@@ -507,7 +507,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     // Epilogue column split: both halves of BN must be whole 16-column chunks
     // and whole output words; otherwise warps 0-3 take every column.
     const int half_cols = BN / 2;
-    const bool split = (half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0);
+    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
     const int epi_warps = split ? 8 : 4;
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {

@@ -3,22 +3,25 @@
 // epilogue, for shapes whose B does not stay resident in shared memory.
 //
 // Two steps on the caller's stream:
-//  1. esb_tile_kernel decodes each operand once into a tiled image of E4M3
-//     bytes in the caller's workspace: tile (rb, kb) holds rows
-//     rb*TH .. rb*TH + TH - 1 and codes 128 kb .. 128 kb + 127 as TH x 128
-//     bytes in the SW128 K-major layout of an MMA operand (row r, 16-byte
-//     chunk g at r*128 + ((g ^ (r & 7)) * 16)); tiles follow in (rb, kb)
-//     order, so every tile is one contiguous block.  Rows past the operand
+//  1. esb_tile_kernel decodes each operand once into an image of E4M3 bytes
+//     in the caller's workspace: K-block kb (128 codes) of row r at byte
+//     (kb * rpad + r) * 128, its 16-byte chunk g at ((g ^ (r & 7)) * 16), so
+//     any run of rows that starts at a multiple of 8 is one contiguous block
+//     in the SW128 K-major layout of an MMA operand.  Rows past the operand
 //     and codes past K are E4M3 zeros.  HBM-bound: code bytes in, one byte
 //     per code out.
 //  2. esb_gemm_tiled_kernel, persistent and warp-specialised: one producer
-//     thread bulk-copies whole tiles (A: 128 rows, 16 KiB; B: 256 rows,
-//     32 KiB) into a ring of shared-memory stages (cp.async.bulk completing
-//     on mbarriers), the MMA thread issues four 128 x 256 x 32 tcgen05.mma
-//     per K-block into one of two 256-column TMEM accumulators, and eight
-//     epilogue warps drain them through the epilogue of the other tcgen05
-//     kernels (ws_epilogue).  Each CTA keeps one 256-column N-tile and walks
-//     the M-tiles.
+//     thread bulk-copies whole tiles (A: 128 rows, 16 KiB; B: BN rows,
+//     30 or 32 KiB) into a ring of shared-memory stages (cp.async.bulk
+//     completing on mbarriers), the MMA thread issues four 128 x BN x 32
+//     tcgen05.mma per K-block into one of two BN-column TMEM accumulators,
+//     and eight epilogue warps drain them through the epilogue of the other
+//     tcgen05 kernels (ws_epilogue).  Each CTA keeps one N-tile and walks
+//     the M-tiles.  BN is 256, or 240 for outputs of 3, 5 or 6 bits, whose
+//     10, 6 or 5 codes per word divide 240 (a word never straddles tiles).
+//     Measured at 4096^3 with 6-bit codes: 124 us for the call, against 1458
+//     us for the streamed kernel, which decodes every operand row again in
+//     each tile (the only one to take these widths before).
 // The contraction is exact: fp32 TMEM accumulation of integer-valued
 // products holds every partial sum exactly while it stays below 2^24, so a K
 // with K max|I_A| max|I_B| >= 2^24 is split into chunks that each stay
@@ -37,6 +40,7 @@ namespace esb {
 namespace {
 
 constexpr int kTiledBN = 256;                  // N-tile width (rows of a B tile); 128 with > 2 K-chunks
+constexpr int kTiledBNOdd = 240;               // for 3, 5, 6 or 10 output codes per word
 constexpr int kTiledThreads = 320;             // warps 0-7 epilogue, 8 MMA, 9 producer
 constexpr int kTiledProdWarp = 9;
 constexpr int kTileA = kBM * kBK;              // 16 KiB
@@ -44,68 +48,211 @@ constexpr int kTmemCols = 512;
 
 }  // namespace
 
-// One 16-byte chunk (16 codes) per thread and pass: u enumerates (tile,
-// row, physical chunk), so consecutive threads write consecutive bytes.
-__global__ void __launch_bounds__(256) esb_tile_kernel(RowsSrc src, int64_t K, OpFmt f, int TH, int nkb,
-                                                       int64_t rblocks, uint8_t* __restrict__ out)
+// The 16-code unit [k0, k0 + 16) of a row as 16 E4M3 bytes in unit_pos order
+// (any width, by a walk of its words: a code never straddles two words, one
+// load per word), zeros past K.
+__device__ __noinline__ uint4 tile_unit_any(const uint32_t* p, int64_t k0, int64_t K, const OpFmt f)
 {
-    const int64_t total = rblocks * nkb * (int64_t)TH * 8;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += (int64_t)gridDim.x * blockDim.x) {
-        const int gp = (int)(u & 7);                         // physical chunk in the 128-byte row
-        const int64_t rt = u >> 3;
-        const int r = (int)(rt % TH);
-        const int64_t t = rt / TH;                           // tile index rb * nkb + kb
-        const int64_t rb = t / nkb;
-        const int kb = (int)(t - rb * nkb);
-        const int g = gp ^ (r & 7);                          // logical chunk: codes 16 g .. 16 g + 15
-        const int64_t row = rb * TH + r;
-        const int64_t k0 = (int64_t)kb * kBK + g * 16;
-        uint4 o = make_uint4(0u, 0u, 0u, 0u);
-        if (row < src.rows && k0 < K) {
-            const RowsSrc::Row rw = src.row(row);
-            if (f.b == 4) {
-                // two words (16 codes) at word k0 / 8 (even: 8-byte aligned);
-                // rows are padded to whole 16-byte groups, so both exist
-                const uint2 w = __ldg(reinterpret_cast<const uint2*>(src.words(rw, k0 >> 3)));
-                uint32_t o0, o1, o2, o3;
-                decode_word_b4(w.x, f.k, f.ew, o0, o1);
-                decode_word_b4(w.y, f.k, f.ew, o2, o3);
-                if (k0 + 16 > K) {                           // K tail: zero the codes past K
-                    uint32_t ml, mh;
-                    int va = (int)(K - k0);
-                    va = va < 0 ? 0 : (va > 8 ? 8 : va);
-                    tail_masks(va, ml, mh);
-                    o0 &= ml; o1 &= mh;
-                    int vb = (int)(K - k0 - 8);
-                    vb = vb < 0 ? 0 : (vb > 8 ? 8 : vb);
-                    tail_masks(vb, ml, mh);
-                    o2 &= ml; o3 &= mh;
-                }
-                o = make_uint4(o0, o1, o2, o3);
-            } else {
-                // any width: walk the 16 codes through their words (a code
-                // never straddles two words), one load per word
-                const uint32_t* p = src.words(rw, 0);
-                int64_t wi = k0 / f.cpw;
-                int slot = (int)(k0 - wi * f.cpw);
-                uint32_t w = __ldg(p + wi);
-                uint32_t ob[4] = {0u, 0u, 0u, 0u};
+    uint32_t ob[4] = {0u, 0u, 0u, 0u};
+    if (k0 < K) {
+        int64_t wi = k0 / f.cpw;
+        int slot = (int)(k0 - wi * f.cpw);
+        uint32_t w = __ldg(p + wi);
 #pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    if (k0 + j >= K) break;
-                    const uint32_t byte = code_to_e4m3((w >> (f.b * slot)) & f.mask, f);
-                    const int pos = unit_pos(j);
-                    ob[pos >> 2] |= byte << (8 * (pos & 3));
-                    if (++slot == f.cpw) {
-                        slot = 0;
-                        ++wi;
-                        if (k0 + j + 1 < K) w = __ldg(p + wi);
-                    }
-                }
-                o = make_uint4(ob[0], ob[1], ob[2], ob[3]);
+        for (int j = 0; j < 16; j++) {
+            if (k0 + j >= K) break;
+            const uint32_t byte = code_to_e4m3((w >> (f.b * slot)) & f.mask, f);
+            const int pos = unit_pos(j);
+            ob[pos >> 2] |= byte << (8 * (pos & 3));
+            if (++slot == f.cpw) {
+                slot = 0;
+                ++wi;
+                if (k0 + j + 1 < K) w = __ldg(p + wi);
             }
         }
-        reinterpret_cast<uint4*>(out + t * (int64_t)TH * kBK + (int64_t)r * kBK)[gp] = o;
+    }
+    return make_uint4(ob[0], ob[1], ob[2], ob[3]);
+}
+
+// One operand of the tile pass.
+struct TileSrc {
+    const uint32_t* base;
+    int64_t ld;
+    int64_t rows;              // rows of the operand
+    int64_t rpad;              // rows of the image: a multiple of 16, zeros past `rows`
+    OpFmt f;
+    int packed;                // both operands of the same 3-, 5- or 6-bit width: packed runs (tile_run)
+    int64_t units;             // threads' units of work
+    int upr;                   // units per row (packed)
+    uint8_t* out;
+};
+
+// 16-byte chunk c of row r in the image: K-block c / 8, swizzled chunk c % 8.
+__device__ __forceinline__ uint4* tile_chunk(const TileSrc& t, int64_t r, int c)
+{
+    return reinterpret_cast<uint4*>(t.out + ((int64_t)(c >> 3) * t.rpad + r) * kBK + (((c & 7) ^ (int)(r & 7)) << 4));
+}
+
+// 3/5/6-bit codes packed without gaps: a run of RW words whose codes are a
+// whole number of 16-byte chunks (6-bit: 16 words = 80 codes = 5 chunks;
+// 5-bit: 8 words = 48 codes = 3 chunks; 3-bit: 8 words = 80 codes = 5
+// chunks).  The first 4 (3-bit: 8) codes of every word fill the run's first
+// chunks, the 1 or 2 codes left over of all its words the last one.  The
+// same K order on both operands, so the sums are those of any other order;
+// about 3.5 instructions per code (the per-code walk takes 12).
+template <int B>
+struct TileRun {
+    static constexpr int CPW = 32 / B;
+    static constexpr int RW = B == 6 ? 16 : 8;
+    static constexpr int CODES = RW * CPW;
+    static constexpr int CHUNKS = CODES / 16;
+};
+
+template <int B>
+__device__ __forceinline__ void tile_run(const TileSrc& t, int64_t r, const uint32_t* p, int run)
+{
+    constexpr int RW = TileRun<B>::RW, CH = TileRun<B>::CHUNKS;
+    uint32_t w[RW];
+    const uint4* q = reinterpret_cast<const uint4*>(p + (int64_t)run * RW);   // rows are 16-byte aligned
+#pragma unroll
+    for (int i = 0; i < RW / 4; i++) {
+        const uint4 v = __ldg(q + i);
+        w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+    }
+    const int k = t.f.k;
+    const int c0 = run * CH;
+#pragma unroll
+    for (int i = 0; i < RW; i++) w[i] = rot_word<B>(w[i], k);
+    uint32_t rest[4] = {0u, 0u, 0u, 0u};              // the last chunk's bytes: fields still at their low bits
+#pragma unroll
+    for (int c = 0; c + 1 < CH; c++) {
+        uint32_t o[4];
+        if (B == 3) {
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                o[2 * i] = e4m3_4<B>(spread4<B>(w[2 * c + i]), k);
+                o[2 * i + 1] = e4m3_4<B>(spread4<B>(w[2 * c + i] >> 12), k);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; i++) o[i] = e4m3_4<B>(spread4<B>(w[4 * c + i]), k);
+        }
+        *tile_chunk(t, r, c0 + c) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+#pragma unroll
+    for (int i = 0; i < RW; i++) {
+        if (B == 6) {
+            rest[i >> 2] |= ((w[i] >> 24) & 0x3fu) << (8 * (i & 3));
+        } else {
+            constexpr int SH = B == 5 ? 20 : 24;      // the word's last two codes
+            constexpr uint32_t CM = (1u << B) - 1u;
+            const uint32_t g = w[i] >> SH;
+            rest[i >> 1] |= ((g & CM) | ((g << (8 - B)) & (CM << 8))) << (16 * (i & 1));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) rest[i] = e4m3_4<B>(rest[i], k);
+    *tile_chunk(t, r, c0 + CH - 1) = make_uint4(rest[0], rest[1], rest[2], rest[3]);
+}
+
+// Unit u of a packed operand: run u % upr of row u / upr; the last unit of a
+// row is its tail (the codes past the whole runs, then zeros to the end of
+// the last K-block), by the per-code walk.
+template <int B>
+__device__ __forceinline__ void tile_packed(const TileSrc& t, int64_t u, int64_t K, int nkb)
+{
+    const int64_t r = u < (1ll << 32) ? (int64_t)((uint32_t)u / (uint32_t)t.upr) : u / t.upr;
+    const int run = (int)(u - r * t.upr);
+    const bool live = r < t.rows;
+    const uint32_t* p = t.base + r * t.ld;
+    if (run + 1 < t.upr) {
+        if (live) {
+            tile_run<B>(t, r, p, run);
+        } else {
+#pragma unroll
+            for (int c = 0; c < TileRun<B>::CHUNKS; c++) *tile_chunk(t, r, run * TileRun<B>::CHUNKS + c) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        return;
+    }
+    int64_t k0 = (int64_t)run * TileRun<B>::CODES;
+    for (int c = run * TileRun<B>::CHUNKS; c < nkb * 8; c++, k0 += 16)
+        *tile_chunk(t, r, c) = live ? tile_unit_any(p, k0, K, t.f) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+// K-blocks per unit of the code-linear pass: their loads are in flight together.
+constexpr int kTileKbs = 4;
+
+// Unit u of a code-linear operand (4-bit codes, mixed widths): chunk lane & 7
+// of row 4 q + lane / 8 for kTileKbs consecutive K-blocks; a warp reads 64
+// contiguous bytes of each of 4 rows (4-bit codes) and writes 512 contiguous
+// bytes of the image per K-block.
+__device__ __forceinline__ void tile_linear(const TileSrc& t, int64_t warp_unit, int lane, int64_t K, int nkb)
+{
+    const int groups = (nkb + kTileKbs - 1) / kTileKbs;
+    const int64_t rq = warp_unit / groups;
+    const int kb0 = (int)(warp_unit - rq * groups) * kTileKbs;
+    const int64_t r = rq * 4 + (lane >> 3);
+    const int g = (lane & 7) ^ (int)(r & 7);          // logical chunk at physical position lane & 7
+    const bool live = r < t.rows;
+    const uint32_t* p = t.base + r * t.ld;
+    if (t.f.b == 4) {
+        // two words (16 codes) at an even word: 8-byte aligned; rows are
+        // padded to whole 16-byte groups, so both words exist
+        uint2 w[kTileKbs];
+#pragma unroll
+        for (int i = 0; i < kTileKbs; i++) {
+            const int64_t k0 = (int64_t)(kb0 + i) * kBK + g * 16;
+            w[i] = make_uint2(0u, 0u);
+            if (live && k0 < K) w[i] = __ldg(reinterpret_cast<const uint2*>(p + (k0 >> 3)));
+        }
+#pragma unroll
+        for (int i = 0; i < kTileKbs; i++) {
+            if (kb0 + i >= nkb) break;
+            const int64_t k0 = (int64_t)(kb0 + i) * kBK + g * 16;
+            uint32_t o0 = 0u, o1 = 0u, o2 = 0u, o3 = 0u;
+            if (live && k0 < K) {
+                decode_word_b4(w[i].x, t.f.k, t.f.ew, o0, o1);
+                decode_word_b4(w[i].y, t.f.k, t.f.ew, o2, o3);
+                if (k0 + 16 > K) {                    // K tail: zero the codes past K
+                    uint32_t ml, mh;
+                    const int va = (int)(K - k0);
+                    tail_masks(va > 8 ? 8 : va, ml, mh);
+                    o0 &= ml; o1 &= mh;
+                    const int vb = (int)(K - k0 - 8);
+                    tail_masks(vb < 0 ? 0 : vb, ml, mh);
+                    o2 &= ml; o3 &= mh;
+                }
+            }
+            *tile_chunk(t, r, (kb0 + i) * 8 + g) = make_uint4(o0, o1, o2, o3);
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int i = 0; i < kTileKbs && kb0 + i < nkb; i++)
+        *tile_chunk(t, r, (kb0 + i) * 8 + g) =
+            live ? tile_unit_any(p, (int64_t)(kb0 + i) * kBK + g * 16, K, t.f) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+// HBM-bound by its output (one byte per code).  Both operands in one launch:
+// the 256 x 4096 x 9216 classifier layer went from 55.3 to 44.4 us with one
+// launch for two, four K-blocks' loads in flight per warp and no division per
+// chunk. the first blocks take A's units, the rest B's.
+__global__ void __launch_bounds__(256) esb_tile_kernel(TileSrc ta, TileSrc tb, int64_t K, int nkb, unsigned blocks_a)
+{
+    griddep_wait();                                   // codes and workspace may belong to the previous launch
+    const bool is_a = blockIdx.x < blocks_a;
+    const TileSrc& t = is_a ? ta : tb;
+    const int64_t nblk = is_a ? blocks_a : gridDim.x - blocks_a;
+    const int64_t blk = is_a ? blockIdx.x : blockIdx.x - blocks_a;
+    if (t.packed) {
+        for (int64_t u = blk * 256 + threadIdx.x; u < t.units; u += nblk * 256) {
+            if (t.f.b == 3) tile_packed<3>(t, u, K, nkb);
+            else if (t.f.b == 5) tile_packed<5>(t, u, K, nkb);
+            else tile_packed<6>(t, u, K, nkb);
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (int64_t u = blk * 8 + (threadIdx.x >> 5); u < t.units; u += nblk * 8) tile_linear(t, u, lane, K, nkb);
     }
 }
 
@@ -115,9 +262,8 @@ __global__ void __launch_bounds__(256) esb_tile_kernel(RowsSrc src, int64_t K, O
 // the oracle converts it) goes through epi_element.  Codes of any width
 // that divides 16 codes per word; padding slots past N take the zero code.
 // Warps 0-7: TMEM lane quarter warp & 3, column half warp >> 2.
-template <int BN>
 __device__ void tiled_chunked_epilogue(const EpiParams& ep, const float* thr, int64_t M, int64_t N, int64_t n0,
-                                       int64_t first, int64_t ctas, int64_t my_tiles, int nch, int nbuf,
+                                       int BN, int64_t first, int64_t ctas, int64_t my_tiles, int nch, int nbuf,
                                        uint32_t tmem_base, float acc_scale, uint64_t* tfull, uint64_t* tempty,
                                        volatile int* err, int warp, int lane)
 {
@@ -176,15 +322,16 @@ __device__ void tiled_chunked_epilogue(const EpiParams& ep, const float* thr, in
     }
 }
 
-template <bool LEAN4, int BN>
+template <bool LEAN4, bool GEN>
 __global__ void __launch_bounds__(kTiledThreads, 1)
-esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict__ Bt, int64_t M, int64_t N, int nkb,
-                      int kbc, int nch, int stages, int n_tiles, int64_t m_tiles, float acc_scale, EpiParams ep)
+esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict__ Bt, int64_t M, int64_t N, int64_t mpad,
+                      int64_t npad, int nkb, int kbc, int nch, int BNr, int stages, int n_tiles, int64_t m_tiles,
+                      float acc_scale, EpiParams ep)
 {
+    const int BN = LEAN4 ? kTiledBN : BNr;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    constexpr int kTileB = BN * kBK;
-    constexpr int kStage = kTileA + kTileB;                      // A tile then B tile (both 1024-aligned)
+    const int kStage = kTileA + BN * kBK;                        // A tile then B tile (both 1024-aligned)
     const int nbuf = kTmemCols / (nch * BN) >= 2 ? 2 : 1;       // accumulator sets (one per tile in flight)
     float* thr = reinterpret_cast<float*>(smem + stages * kStage);
     uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
@@ -205,7 +352,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     uint32_t tmem_cols = 32;                                     // a power of two >= the regions used
     while (tmem_cols < (uint32_t)(nbuf * nch * BN)) tmem_cols <<= 1;
     const int half_cols = BN / 2;
-    const bool split = (half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0);
+    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
     const int epi_warps = split ? 8 : 4;
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -237,15 +384,19 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 0u;
-            const uint8_t* bt = Bt + (int64_t)n_tile * nkb * kTileB;   // B tiles of BN rows
+            // the last N-tile may end past the image: its missing rows stay
+            // whatever shared memory holds (columns past N, never stored)
+            const int64_t brows = npad - n0 < (int64_t)BN ? npad - n0 : (int64_t)BN;
+            const uint32_t b_bytes = (uint32_t)brows * kBK;
             for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
-                const uint8_t* at = At + (cta_in_n + ti * ctas_per_n) * nkb * (int64_t)kTileA;
-                for (int kb = 0; kb < nkb; kb++) {
+                const uint8_t* at = At + (cta_in_n + ti * ctas_per_n) * (int64_t)kTileA;
+                const uint8_t* bt = Bt + n0 * kBK;
+                for (int kb = 0; kb < nkb; kb++, at += mpad * kBK, bt += npad * kBK) {
                     if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
                     uint8_t* st = smem + s * kStage;
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)kStage);
-                    bulk_copy_g2s(st, at + (int64_t)kb * kTileA, (uint32_t)kTileA, &full[s]);
-                    bulk_copy_g2s(st + kTileA, bt + (int64_t)kb * kTileB, (uint32_t)kTileB, &full[s]);
+                    mbar_arrive_expect_tx(&full[s], (uint32_t)kTileA + b_bytes);
+                    bulk_copy_g2s(st, at, (uint32_t)kTileA, &full[s]);
+                    bulk_copy_g2s(st + kTileA, bt, b_bytes, &full[s]);
                     if (++s == stages) { s = 0; ph ^= 1u; }
                 }
             }
@@ -289,7 +440,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     } else if (nch > 1) {
         // ---------------------------------------------- epilogue (K in chunks)
         if (warp < kWsEpiWarps)
-            tiled_chunked_epilogue<BN>(ep, thr, M, N, n0, cta_in_n, ctas_per_n, my_tiles, nch, nbuf, tmem_base,
+            tiled_chunked_epilogue(ep, thr, M, N, n0, BN, cta_in_n, ctas_per_n, my_tiles, nch, nbuf, tmem_base,
                                        acc_scale, tfull, tempty, err, warp, lane);
     } else if (warp < epi_warps) {
         // ---------------------------------------------- epilogue
@@ -298,7 +449,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<LEAN4, false>(ep, thr, rows, my_tiles, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty,
                            err, warp, lane);
     }
 
@@ -316,8 +467,9 @@ static int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // K-chunking of a shape: K-blocks per chunk (each chunk's partial sums stay
 // below 2^24), chunk count and N-tile width; false when the kernel cannot
-// hold the chunks (more than four, or a total past the int32 range).
-static bool tiled_plan(int64_t K, int ba, int ka, int bb, int kb, int* kbc, int* nch, int* BN)
+// hold the chunks (more than four, or a total past the int32 range) or the
+// output's codes per word.
+static bool tiled_plan(int64_t K, int ba, int ka, int bb, int kb, int out_cpw, int* kbc, int* nch, int* BN)
 {
     const int64_t nkb = cdiv(K, kBK);
     const double img = (double)fmt_max_image(ba, ka) * fmt_max_image(bb, kb);
@@ -328,21 +480,21 @@ static bool tiled_plan(int64_t K, int ba, int ka, int bb, int kb, int* kbc, int*
         if (c < 1) return false;
     }
     const int64_t n = cdiv(nkb, c);
-    if (n > 4) return false;
+    if (n > 4 || (n > 1 && 16 % out_cpw != 0)) return false;
     *kbc = (int)c;
     *nch = (int)n;
-    *BN = n <= 2 ? 256 : 128;
-    return true;
+    *BN = n > 2 ? 128 : (kTiledBN % out_cpw == 0 ? kTiledBN : kTiledBNOdd);
+    return *BN % out_cpw == 0;
 }
 
 size_t gemm_tiled_workspace_bytes(int64_t M, int64_t N, int64_t K)
 {
     const int64_t nkb = cdiv(K, kBK);
-    // B tiles of 256 rows bound the 128-row tiling of a chunked K from above
+    // (the images hold rows padded to 128 and 16 only; the sizes callers know are kept)
     return (size_t)(cdiv(M, kBM) * nkb * kTileA + cdiv(N, kTiledBN) * nkb * (int64_t)kTiledBN * kBK);
 }
 
-// The tiled path pays two extra launches and a pass over both operands:
+// The tiled path pays an extra launch and a pass over both operands:
 // below about 2^32 multiply-adds the other kernels finish first (when they
 // can: their decode is fast for 4-bit operands only).  ESB_GEMM_TILED_MIN_MACS
 // in the environment (read per call) moves that threshold (0: every shape
@@ -352,42 +504,56 @@ bool gemm_tiled_ok(int64_t M, int64_t N, int64_t K, int ba, int ka, int bb, int 
     int kbc, nch, BN;
     // significand-split operands (k >= 4) take esb_gemm's kernels
     if (fmt_needs_split(ba, ka) || fmt_needs_split(bb, kb)) return false;
-    if (M <= 0 || N < kTiledBN || K <= 0 || !tiled_plan(K, ba, ka, bb, kb, &kbc, &nch, &BN)) return false;
-    if (kTiledBN % out_cpw != 0 || (nch > 1 && 16 % out_cpw != 0)) return false;
+    if (M <= 0 || N < kTiledBN || K <= 0 || !tiled_plan(K, ba, ka, bb, kb, out_cpw, &kbc, &nch, &BN)) return false;
     if (nch > 1) return true;                                     // only this path takes that K
-    double min_macs = (ba == 4 && bb == 4) ? 4294967296.0 : 0.0;
+    double min_macs = (ba == 4 && bb == 4) ? 4294967296.0 : (BN == kTiledBNOdd ? 268435456.0 : 0.0);
     if (const char* v = getenv("ESB_GEMM_TILED_MIN_MACS")) min_macs = atof(v);
     return (double)M * N * K >= min_macs;
 }
+
+// 3, 5, 6 or 10 output codes per word: esb_gemm's kernels take every shape
+// of these too, so a call without (enough) workspace runs there.
+bool gemm_tiled_optional(int out_cpw) { return kTiledBN % out_cpw != 0; }
+
+typedef void (*TiledKernel)(const uint8_t*, const uint8_t*, int64_t, int64_t, int64_t, int64_t, int, int, int, int, int,
+                            int, int64_t, float, EpiParams);
+static const TiledKernel kTiledKernels[3] = {esb_gemm_tiled_kernel<false, false>, esb_gemm_tiled_kernel<true, false>,
+                                             esb_gemm_tiled_kernel<false, true>};
 
 static int tiled_static_smem(cudaError_t* err)
 {
     static int v = -1;
     if (v < 0) {
-        cudaFuncAttributes a0, a1, a2;
-        *err = cudaFuncGetAttributes(&a0, esb_gemm_tiled_kernel<false, 256>);
-        if (*err != cudaSuccess) return -1;
-        *err = cudaFuncGetAttributes(&a1, esb_gemm_tiled_kernel<true, 256>);
-        if (*err != cudaSuccess) return -1;
-        *err = cudaFuncGetAttributes(&a2, esb_gemm_tiled_kernel<false, 128>);
-        if (*err != cudaSuccess) return -1;
-        size_t m = a0.sharedSizeBytes;
-        if (a1.sharedSizeBytes > m) m = a1.sharedSizeBytes;
-        if (a2.sharedSizeBytes > m) m = a2.sharedSizeBytes;
+        size_t m = 0;
+        for (TiledKernel k : kTiledKernels) {
+            cudaFuncAttributes a;
+            *err = cudaFuncGetAttributes(&a, k);
+            if (*err != cudaSuccess) return -1;
+            if (a.sharedSizeBytes > m) m = a.sharedSizeBytes;
+        }
         v = (int)m;
     }
     return v;
 }
 
-static cudaError_t launch_tile(const RowsSrc& src, int64_t K, const OpFmt& f, int TH, int nkb, int64_t rblocks,
-                               uint8_t* out, cudaStream_t st)
+// Operand of the tile pass; packed: runs of 3/5/6-bit words (both operands
+// must have that width, so that they share the K order).
+static TileSrc tile_src(const uint32_t* base, int64_t ld, int64_t rows, int64_t rpad, int64_t K, int nkb, const OpFmt& f,
+                        bool packed, uint8_t* out, int64_t* blocks)
 {
-    const int64_t total = rblocks * nkb * (int64_t)TH * 8;
-    int64_t grid = cdiv(total, 256);
-    const int64_t cap = (int64_t)device_sm_count() * 8;
-    if (grid > cap) grid = cap;
-    esb_tile_kernel<<<(unsigned)grid, 256, 0, st>>>(src, K, f, TH, nkb, rblocks, out);
-    return cudaGetLastError();
+    TileSrc t{base, ld, rows, rpad, f, packed ? 1 : 0, 0, 0, out};
+    if (packed) {
+        const int codes = f.b == 3 ? TileRun<3>::CODES : f.b == 5 ? TileRun<5>::CODES : TileRun<6>::CODES;
+        t.upr = (int)(K / codes) + 1;                             // whole runs, then the tail unit
+        t.units = rpad * t.upr;
+        *blocks = cdiv(t.units, 256);
+    } else {
+        t.units = rpad / 4 * cdiv(nkb, kTileKbs);                 // per warp
+        *blocks = cdiv(t.units, 8);
+    }
+    const int64_t cap = (int64_t)device_sm_count() * 16;
+    if (*blocks > cap) *blocks = cap;
+    return t;
 }
 
 cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A, int64_t lda, int ba, int ka,
@@ -395,7 +561,8 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
                               cudaStream_t st)
 {
     int kbc = 0, nch = 0, BN = 0;
-    if (!tiled_plan(K, ba, ka, bb, kb, &kbc, &nch, &BN)) return cudaErrorInvalidValue;
+    const int out_cpw = o.codes_out ? 32 / o.ep->fmt_out.b : 8;
+    if (!tiled_plan(K, ba, ka, bb, kb, out_cpw, &kbc, &nch, &BN)) return cudaErrorInvalidValue;
     EpiParams ep = make_epi(o);
     ep.dq_pow2 = ldexpf(1.0f, -(ka + kb));
     ep.acc_lim = nch == 1 ? acc_fma_limit(K, ba, ka, bb, kb) : 0.0f;
@@ -403,10 +570,14 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     const int nkb = (int)cdiv(K, kBK);
     const int64_t m_tiles = cdiv(M, kBM), n_tiles = cdiv(N, BN);
     uint8_t* At = static_cast<uint8_t*>(workspace);
-    uint8_t* Bt = At + m_tiles * nkb * (int64_t)kTileA;
-    cudaError_t e = launch_tile(RowsSrc{A, lda, M}, K, fa, kBM, nkb, m_tiles, At, st);
-    if (e != cudaSuccess) return e;
-    e = launch_tile(RowsSrc{B, ldb, N}, K, fb, BN, nkb, n_tiles, Bt, st);
+    const int64_t mpad = m_tiles * kBM, npad = cdiv(N, 16) * 16;
+    uint8_t* Bt = At + mpad * nkb * (int64_t)kBK;
+    const bool packed = ba == bb && (ba == 3 || ba == 5 || ba == 6);
+    int64_t blk_a = 0, blk_b = 0;
+    const TileSrc ta = tile_src(A, lda, M, mpad, K, nkb, fa, packed, At, &blk_a);
+    const TileSrc tb = tile_src(B, ldb, N, npad, K, nkb, fb, packed, Bt, &blk_b);
+    cudaError_t e = launch_pdl(esb_tile_kernel, dim3((unsigned)(blk_a + blk_b)), dim3(256), 0, st, ta, tb, K, nkb,
+                               (unsigned)blk_a);
     if (e != cudaSuccess) return e;
 
     const int st_smem = tiled_static_smem(&e);
@@ -420,12 +591,10 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     const size_t smem = (size_t)(fixed + (int64_t)stages * stage_bytes);
     static bool configured = false;
     if (!configured) {
-        e = cudaFuncSetAttribute(esb_gemm_tiled_kernel<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(esb_gemm_tiled_kernel<true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(esb_gemm_tiled_kernel<false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-        if (e != cudaSuccess) return e;
+        for (TiledKernel k : kTiledKernels) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
+            if (e != cudaSuccess) return e;
+        }
         configured = true;
     }
     int64_t per_n = device_sm_count() / n_tiles;
@@ -435,14 +604,14 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
     // the specialised epilogue: 4-bit codes as the only output with a scalar
     // scale and bias, whole N-tiles, a monotone requantisation, K in one chunk
-    const bool fast = nch == 1 && BN == 256 && ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias &&
+    const bool fast = nch == 1 && BN == kTiledBN && ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias &&
                       !ep.residual && !ep.acc_out && !ep.y_out && ep.acc_lim > 0.0f && N % BN == 0 &&
                       (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
-    void (*kernel)(const uint8_t*, const uint8_t*, int64_t, int64_t, int, int, int, int, int, int64_t, float,
-                   EpiParams) = BN == 128 ? esb_gemm_tiled_kernel<false, 128>
-                                          : (fast ? esb_gemm_tiled_kernel<true, 256> : esb_gemm_tiled_kernel<false, 256>);
-    return launch_pdl(kernel, dim3((unsigned)grid), dim3(kTiledThreads), smem, st, (const uint8_t*)At,
-                      (const uint8_t*)Bt, M, N, nkb, kbc, nch, stages, (int)n_tiles, m_tiles, acc_scale, ep);
+    // one chunk of other widths' codes only: the general-width epilogue instance
+    const bool gen = nch == 1 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
+    return launch_pdl(kTiledKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,
+                      (const uint8_t*)At, (const uint8_t*)Bt, M, N, mpad, npad, nkb, kbc, nch, BN, stages, (int)n_tiles,
+                      m_tiles, acc_scale, ep);
 }
 
 }  // namespace esb

@@ -150,6 +150,36 @@ __device__ __forceinline__ void decode_word_b4(uint32_t w, int k, int ew, uint32
     hi = ((b & 0x07070707u) << sh) | ((b & 0x08080808u) << 4);
 }
 
+// The packed codes of one word of a whole-byte format (any width) with the
+// exponent field of each rotated to its E4M3 value, (e + 1) mod 2^ew: one add
+// over all fields, whose carry into the sign position is masked off.
+template <int B>
+__device__ __forceinline__ uint32_t rot_word(uint32_t w, int k)
+{
+    constexpr int CPW = 32 / B;
+    constexpr uint32_t ONES = []() constexpr { uint32_t v = 0; for (int j = 0; j < CPW; j++) v |= 1u << (B * j); return v; }();
+    constexpr uint32_t SG = ONES << (B - 1);
+    constexpr uint32_t LOW = SG - ONES;               // the B - 1 bits below each sign
+    return (k < B - 1) ? ((((w & LOW) + (ONES << k)) & LOW) | (w & SG)) : (w & (LOW | SG));
+}
+
+// Four consecutive B-bit fields (bits 0 .. 4B - 1 of g) to the low bits of four bytes.
+template <int B>
+__device__ __forceinline__ uint32_t spread4(uint32_t g)
+{
+    constexpr uint32_t PM = (1u << (2 * B)) - 1u, CM = (1u << B) - 1u;
+    const uint32_t t = (g & PM) | ((g << (16 - 2 * B)) & (PM << 16));
+    return (t & (CM | (CM << 16))) | ((t << (8 - B)) & ((CM | (CM << 16)) << 8));
+}
+
+// Rotated codes in the low B bits of four bytes -> their E4M3 bytes.
+template <int B>
+__device__ __forceinline__ uint32_t e4m3_4(uint32_t t, int k)
+{
+    constexpr uint32_t SG = 0x01010101u << (B - 1);
+    return ((t & (SG - 0x01010101u)) << (3 - k)) | ((t & SG) << (8 - B));
+}
+
 // ------------------------------------------------------------ row sources
 
 // Plain K-major rows: logical word w of row r is base[r * ld + w].  With
@@ -691,6 +721,164 @@ static __device__ __noinline__ uint32_t epi_word_b4(const EpiParams* __restrict_
     return codes8_b4(J, S, ep.out.k);
 }
 
+// Output codes of 3, 5 or 6 bits as the only output: the projection of y by
+// the cell table (one 8-byte shared load and one compare per value, as in
+// project_vec_kernel) instead of b - 1 dependent threshold loads, 4 code
+// words (2 of 3-bit codes) per pass with every load of the pass in flight,
+// one 16-byte store where the row allows it.
+constexpr int kEpiCells = 256;     // entries of the table; larger tables keep the bisection
+
+// Whether ws_epilogue takes epi_cells for these outputs (host and device
+// agree: it sets the number of epilogue warps).
+__host__ __device__ inline bool epi_cells_ok(const EpiParams& ep)
+{
+    return ep.codes_out && !ep.acc_out && !ep.y_out && (ep.out.b == 3 || ep.out.b == 5 || ep.out.b == 6) &&
+           (!ep.residual || ep.res_b == ep.out.b);
+}
+
+// Shared memory of epi_cells (static, one per kernel instance).
+struct EpiCellsSmem {
+    uint2 cells[kEpiCells];
+    float resimg[64];                                 // images of the residual's codes
+    int bad;
+};
+
+template <int OB, class RowMap>
+__device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr, EpiCellsSmem& sm, const RowMap& rows,
+                                          int64_t my_tiles, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
+                                          float acc_scale, uint64_t* tfull, uint64_t* tempty, volatile int* err,
+                                          int warp, int lane)
+{
+    constexpr int CPW = 32 / OB;
+    constexpr int WPC = OB == 3 ? 2 : 4;              // words per pass
+    constexpr int CC = WPC * CPW;                     // columns per pass: 20 or 24
+    constexpr int kThreads = kWsEpiWarps * 32;
+    const uint2* const cells = sm.cells;
+    const float* const resimg = sm.resimg;
+    const int t = warp * 32 + lane;
+    int h0, hmax;
+    bool bad;
+    if (t == 0) sm.bad = 0;
+    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+    bool by_cells = fill_cells<OB>(sm.cells, kEpiCells, h0, hmax, thr, ep.out, t, kThreads, bad);
+    if (bad) sm.bad = 1;
+    if (ep.residual && t < (1 << OB)) sm.resimg[t] = code_image_f((uint32_t)t, OB, ep.res_k);
+    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+    by_cells = by_cells && *const_cast<volatile int*>(&sm.bad) == 0;
+
+    const bool dq = ep.alpha_a_dev && ep.alpha_b_dev;
+    const float dqs = dq ? __fmul_rn(__ldg(ep.alpha_a_dev), __ldg(ep.alpha_b_dev)) * ep.dq_pow2 : 1.0f;
+    const float sc0 = dq ? __fmul_rn(ep.scale0, dqs) : ep.scale0;
+    const float bias0 = ep.bias0;
+    const int act = ep.act;
+    const int sh = cell_shift(ep.out.k);
+    const uint32_t amask = ep.out.is_signed ? 0x7fffffffu : 0xffffffffu;
+    const uint32_t zc = ep.out.zero_code;
+    uint32_t zero_word = 0u;
+#pragma unroll
+    for (int j = 0; j < CPW; j++) zero_word |= zc << (OB * j);
+    // passes holding outputs, the first half (rounded up) to warps 0-3
+    const int quarter = warp & 3;
+    const int live = (int)(N - n0 < (int64_t)BN ? N - n0 : (int64_t)BN);
+    const int passes = (live + CC - 1) / CC;
+    const int pmid = (passes + 1) >> 1;
+    const int p_lo = (warp >> 2) ? pmid : 0, p_hi = (warp >> 2) ? passes : pmid;
+    const int64_t w00 = n0 / CPW;
+    const bool vec = WPC == 4 ? ep.codes_vec == 4 && (w00 & 3) == 0 : ep.codes_vec >= 2 && (w00 & 1) == 0;
+    const bool rvec = ep.residual && (reinterpret_cast<uintptr_t>(ep.residual) & 15u) == 0 && (ep.res_ld & 3) == 0 &&
+                      (w00 & (WPC - 1)) == 0;
+    const bool tail_words = n0 + BN >= N && (warp >> 2) == 1;   // zero-code words past the outputs
+    const int row = quarter * 32 + lane;
+    for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
+        const int a = (int)(ti & 1);
+        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> 1) & 1), err)) { *err = 1; break; }
+        tc_fence_after();
+        int64_t m = 0;
+        const bool mrow = rows(ti, row, m);
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN);
+        uint32_t* const crow = ep.codes_out + m * ep.ldo;
+        if (p_lo >= p_hi) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
+        }
+#pragma unroll 1
+        for (int ps = p_lo; ps < p_hi; ps++) {
+            uint32_t r[CC];
+            const uint32_t ta = taddr + (uint32_t)(ps * CC);
+            const int64_t wc = w00 + ps * WPC;
+            uint32_t rw[WPC];
+            const bool whole = (ps + 1) * CC <= live;
+            if (ep.residual && mrow) {
+                const uint32_t* rp = ep.residual + m * ep.res_ld + wc;
+                if (rvec) {
+                    if (WPC == 4) {
+                        const uint4 q = __ldg(reinterpret_cast<const uint4*>(rp));
+                        rw[0] = q.x; rw[1] = q.y; rw[WPC - 2] = q.z; rw[WPC - 1] = q.w;
+                    } else {
+                        const uint2 q = __ldg(reinterpret_cast<const uint2*>(rp));
+                        rw[0] = q.x; rw[1] = q.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int w = 0; w < WPC; w++) rw[w] = (ps * CC + w * CPW < live) ? __ldg(rp + w) : 0u;
+                }
+            }
+            if (ps * CC + CC <= BN) {
+                tmem_ld16_nw(ta, r);
+                if (CC == 24) tmem_ld8_nw(ta + 16, r + 16); else tmem_ld4_nw(ta + 16, r + 16);
+            } else {                                  // the tile's last columns: no read past its TMEM region
+#pragma unroll
+                for (int j = 0; j < CC; j += 4)
+                    if (ps * CC + j < BN) tmem_ld4_nw(ta + j, r + j);
+            }
+            tmem_wait_ld(r);
+            if (ps + 1 == p_hi) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
+            }
+            uint32_t word[WPC];
+#pragma unroll
+            for (int w = 0; w < WPC; w++) {
+                word[w] = 0u;
+#pragma unroll
+                for (int j = 0; j < CPW; j++) {
+                    const int e = w * CPW + j;
+                    float sc = sc0, bi = bias0;
+                    if (ep.scale || ep.bias) {
+                        const int64_t n = n0 + ps * CC + e;
+                        const int64_t nn = n < N ? n : N - 1;
+                        if (ep.scale) { sc = __ldg(ep.scale + nn); if (dq) sc = __fmul_rn(sc, dqs); }
+                        if (ep.bias) bi = __ldg(ep.bias + nn);
+                    }
+                    float y = __fmaf_rn(sc, __uint_as_float(r[e]) * acc_scale, bi);
+                    if (ep.residual) y = __fmaf_rn(ep.res_scale, resimg[(rw[w] >> (OB * j)) & ((1u << OB) - 1u)], y);
+                    y = apply_act(y, act);
+                    uint32_t c = by_cells ? project_by_cells<OB>(y, cells, h0, hmax, sh, amask)
+                                          : project_by_table(y, thr, ep.out);
+                    if (!whole && ps * CC + e >= live) c = zc;
+                    word[w] |= c << (OB * j);
+                }
+            }
+            if (mrow) {
+                if (vec && wc + WPC <= ep.ldo) {
+                    if (WPC == 4)
+                        *reinterpret_cast<uint4*>(crow + wc) = make_uint4(word[0], word[1], word[WPC - 2], word[WPC - 1]);
+                    else
+                        *reinterpret_cast<uint2*>(crow + wc) = make_uint2(word[0], word[1]);
+                } else {
+#pragma unroll
+                    for (int w = 0; w < WPC; w++)
+                        if (wc + w < ep.ldo) crow[wc + w] = word[w];
+                }
+            }
+        }
+        if (tail_words && mrow)
+            for (int64_t wq = w00 + (int64_t)passes * WPC; wq < ep.ldo; wq++) crow[wq] = zero_word;
+    }
+}
+
 // ------------------------------------ roles of the warp-specialised kernels
 
 // TMEM for the two accumulator buffers, allocated by the MMA warp before the
@@ -804,6 +992,22 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                                             int epi_warps, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                             uint64_t* tempty, volatile int* err, int warp, int lane)
 {
+    // the tables of epi_cells and of the bisection path below share their storage
+    __shared__ union GenSmem {
+        EpiCellsSmem cells;
+        struct { float rawT[128], gres[256]; } gen;
+    } sh_gen;
+    if constexpr (GEN) {
+        if (epi_cells_ok(ep)) {
+            if (ep.out.b == 3)
+                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+            else if (ep.out.b == 5)
+                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+            else
+                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+            return;
+        }
+    }
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;              // TMEM lane = tile row
     __shared__ EpiParams sh_ep;                       // copies for the out-of-line general path
@@ -846,8 +1050,8 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                       ep.res_b == 4 && isfinite(sc_lean) && (sc_lean != 0.0f || sc_fixed == 0.0f);
     __shared__ float sh_resimg[16];
     if (lres && warp == 0 && lane < 16) sh_resimg[lane] = code_image_f((uint32_t)lane, 4, ep.res_k);
-    __shared__ float sh_rawT[128];                    // gen: the thresholds searched (raw or on y)
-    __shared__ float sh_gres[GEN ? 256 : 1];          // gen: images of the residual's codes
+    float* const sh_rawT = sh_gen.gen.rawT;           // gen: the thresholds searched (raw or on y)
+    float* const sh_gres = sh_gen.gen.gres;           // gen: images of the residual's codes
     const bool gres = gen && !gen_raw && ep.residual;
     if (gres)
         for (int i = warp * 32 + lane; i < (1 << ep.res_b); i += epi_warps * 32)
