@@ -404,6 +404,18 @@ __device__ __forceinline__ float code_image_f(uint32_t c, int b, int k)
     return s ? -m : m;
 }
 
+// ------------------------------------------------------ fp32 pair sums
+
+// (hi, lo) += x, Knuth's TwoSum with the rounding error kept in lo.
+__device__ __forceinline__ void df_add(float& hi, float& lo, float x)
+{
+    const float s = hi + x;
+    const float bp = s - hi;
+    const float e = (hi - (s - bp)) + (x - bp);
+    hi = s;
+    lo += e;
+}
+
 // ------------------------------------------------------------- PTX helpers
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -655,6 +667,27 @@ __host__ __device__ inline uint32_t idesc_e4m3_f32(int n)
     d |= (uint32_t)(n >> 3) << 17;      // N >> 3
     d |= (uint32_t)(128 >> 4) << 24;    // M >> 4
     return d;
+}
+
+// ------------------------------------------------------------- host side
+
+// Launch with programmatic stream serialisation: the grid may start while
+// the previous kernel of the stream finishes; the kernel's griddep_wait
+// orders its dependent reads and writes after it.
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 }  // namespace esb

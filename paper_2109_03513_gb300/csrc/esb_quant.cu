@@ -369,16 +369,6 @@ constexpr int kCalMaxBlocks = 1023;   // + one 32-byte ticket record = 32 KiB of
 constexpr int kCalChunksPerThread = 1;
 constexpr int kCalStashMax = 13;      // granules per warp kept in shared memory (4 x 8 x 13 x 512 B = 208 KiB per SM)
 
-// (hi, lo) += x, Knuth's TwoSum with the rounding error kept in lo.
-__device__ __forceinline__ void df_add(float& hi, float& lo, float x)
-{
-    const float s = hi + x;
-    const float bp = s - hi;
-    const float e = (hi - (s - bp)) + (x - bp);
-    hi = s;
-    lo += e;
-}
-
 // (hi, lo) += (h2, l2)
 __device__ __forceinline__ void df_add2(float& hi, float& lo, float h2, float l2)
 {

@@ -1338,25 +1338,6 @@ __device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err)
 
 // ------------------------------------------------------------- host side
 
-// Launch with programmatic stream serialisation: the grid may start while
-// the previous kernel of the stream finishes; the kernel's griddep_wait
-// orders its dependent reads and writes after it.
-template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 int pick_bn(int64_t N, int out_cpw);          // N-tile width (esb_gemm.cu)
 int max_dyn_smem();                           // opt-in shared memory per block
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call

@@ -1,0 +1,71 @@
+"""The training kernels at the edges of their paths: every width of
+dn_project (flat 4-bit granules, words packed through shared memory, a sigma
+no threshold can stand for), and dn_backward where fp32 pairs cannot carry
+the values (infinities, underflow, constant inputs) or pointers are not
+16-byte aligned."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as o
+from paper_2109_03513_gb300 import esb, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 8), (37, 24), (5, 136), (3, 1), (2, 331)])
+@pytest.mark.parametrize("fmt", [(2, 0, True), (3, 1, True), (4, 2, True), (4, 1, False), (5, 2, True), (6, 5, True),
+                                 (7, 3, True), (8, 4, False)])
+@pytest.mark.parametrize("sigma", [1.7, 0.0, float("inf"), float("nan")])
+def test_dn_project_widths(rows, cols, fmt, sigma):
+    x = synth.normal((rows, cols), seed=rows + cols, mean=0.3, std=2.0)
+    x[0, 0] = float("inf")
+    if cols > 2:
+        x[-1, 1], x[-1, 2] = float("nan"), -float("inf")
+    st = torch.tensor([0.3, sigma], dtype=torch.float64, device="cuda")
+    codes, xq = esb.esb_dn_project(x.cuda(), st, esb.Fmt(*fmt), rounding=rows & 1)
+    a = float(np.float32(esb.esb_alpha_star(fmt[0], fmt[1])[0]))
+    with np.errstate(all="ignore"):
+        co, xqo = o.dn_project(x.numpy(), 0.3, sigma, a, *fmt, rounding=rows & 1)
+    assert np.array_equal(codes.cpu().numpy().view(np.uint32), o.pack(co.reshape(rows, cols), fmt[0], fmt[1], ld_words=codes.shape[1]))
+    assert np.array_equal(xq.cpu().numpy().ravel(), xqo)
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (3, 0), (4097, 0), (70001, 1)])
+@pytest.mark.parametrize("kind", ["ordinary", "tiny", "huge", "inf", "zero", "mean"])
+def test_dn_backward_ranges(n, shift, kind):
+    """Against fp64: one rounding to fp32 (2^-24 relative), plus the pairs'
+    2^-44 of the larger of the two terms that are subtracted."""
+    x = synth.normal((n + shift,), seed=n, mean=0.4, std=1.3)
+    g = synth.normal((n + shift,), seed=n + 1)
+    if kind == "tiny":
+        g = g * 1e-36
+    elif kind == "huge":
+        g, x = g * 1e30, x * 1e25
+    elif kind == "inf":
+        g[n // 2 + shift] = float("inf")
+    elif kind == "zero":
+        g.zero_()
+    elif kind == "mean":
+        x = x + 1e4
+    xd, gd = x.cuda()[shift:], g.cuda()[shift:]
+    xc, gc = x[shift:].double(), g[shift:].double()
+    mu, sg = float(xc.mean()), float((xc - xc.mean()).square().mean().sqrt())
+    st = torch.tensor([mu, sg], dtype=torch.float64, device="cuda")
+    got = esb.esb_dn_backward(gd, xd, st).cpu().double()
+    s = sg + 1e-7
+    t1, c = (gc - gc.mean()) / s, xc - mu
+    t2 = c * ((gc * c).sum() / (n * sg * s * s)) if sg > 0 else torch.zeros_like(c)
+    exp = t1 - t2
+    if kind == "inf":
+        assert torch.equal(torch.isfinite(got), torch.isfinite(exp)) and torch.equal(torch.isnan(got), torch.isnan(exp))
+        return
+    mean_err = 2.0 ** -40 * float(gc.abs().mean()) / s
+    tol = 2.0 ** -24 * exp.abs() + 2.0 ** -40 * (t1.abs() + t2.abs()) + mean_err + 2.0 ** -149
+    assert bool(((got - exp).abs() <= tol).all())
