@@ -75,111 +75,81 @@ __device__ __forceinline__ void halo_mma_fixed(uint32_t d, uint32_t a_st, uint32
     }
 }
 
-// One packed word of a 5- or 6-bit format in the word-slot layout (8 K
-// slots per word, see plan_slots): code j to byte j through the E4M3 table,
-// the slots past the word's codes zero.
-__device__ __forceinline__ void decode_word_slot8(uint32_t w, const uint8_t* lut, int b, uint32_t& lo, uint32_t& hi)
-{
-    const int cpw = 32 / b;
-    const uint32_t mask = (1u << b) - 1u;
-    uint32_t o[2] = {0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-        if (j < cpw) o[j >> 2] |= (uint32_t)lut[(w >> (b * j)) & mask] << (8 * (j & 3));
-    lo = o[0];
-    hi = o[1];
-}
-
-// One packed word of a 2- or 3-bit format in the word-slot layout (16 K
-// slots per word): a whole 16-byte plane entry.
-__device__ __forceinline__ uint4 decode_word_slot16(uint32_t w, const uint8_t* lut, int b)
-{
-    const int cpw = 32 / b;
-    const uint32_t mask = (1u << b) - 1u;
-    uint32_t o[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 16; j++)
-        if (j < cpw) o[j >> 2] |= (uint32_t)lut[(w >> (b * j)) & mask] << (8 * (j & 3));
-    return make_uint4(o[0], o[1], o[2], o[3]);
-}
-
-// Decode modes of the halo fill: 4-bit codes (SWAR), 5/6-bit word slots
-// (8 per word), 2/3-bit word slots (16 per word).
-enum { kHaloB4 = 0, kHaloSlot8 = 1, kHaloSlot16 = 2 };
-
 // One 4-word piece (piece pc of the pixel in slot `slot`) into its planes:
 // 2 planes (pc * 2 ..) for 8-slot words, 4 planes (pc * 4 ..) for 16-slot
-// words; ok = false writes the E4M3 zero (outside the image).
-template <int MODE>
-__device__ __forceinline__ void halo_store_piece(uint8_t* st, int pb, int slot, int pc, bool ok, const uint4 v, int k,
-                                                 int ew, const uint8_t* lut, int b)
+// words.  Pieces outside the image are zero codes.
+template <int B>
+__device__ __forceinline__ void halo_store_piece(uint8_t* st, int pb, int slot, int pc, const uint4& v, int k, int ew)
 {
-    if (MODE == kHaloSlot16) {
-        uint8_t* dst = st + (4 * pc) * pb + slot * 16;
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    constexpr int RW = SlotFmt<B>::SPW / 4;           // registers per word; planes per piece
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint8_t* dst = st + (RW * pc) * pb + slot * 16;
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-            *reinterpret_cast<uint4*>(dst + i * pb) = ok ? decode_word_slot16(w[i], lut, b) : make_uint4(0u, 0u, 0u, 0u);
-        return;
+    for (int c = 0; c < RW; c++) {
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4 / RW; i++) decode_slots<B>(w[c * (4 / RW) + i], k, ew, o + i * RW);
+        *reinterpret_cast<uint4*>(dst + c * pb) = make_uint4(o[0], o[1], o[2], o[3]);
     }
-    uint4 c0 = make_uint4(0u, 0u, 0u, 0u), c1 = c0;
-    if (ok) {
-        if (MODE == kHaloSlot8) {
-            decode_word_slot8(v.x, lut, b, c0.x, c0.y);
-            decode_word_slot8(v.y, lut, b, c0.z, c0.w);
-            decode_word_slot8(v.z, lut, b, c1.x, c1.y);
-            decode_word_slot8(v.w, lut, b, c1.z, c1.w);
-        } else {
-            decode_word_b4(v.x, k, ew, c0.x, c0.y);
-            decode_word_b4(v.y, k, ew, c0.z, c0.w);
-            decode_word_b4(v.z, k, ew, c1.x, c1.y);
-            decode_word_b4(v.w, k, ew, c1.z, c1.w);
-        }
-    }
-    uint8_t* dst = st + (2 * pc) * pb + slot * 16;
-    *reinterpret_cast<uint4*>(dst) = c0;
-    *reinterpret_cast<uint4*>(dst + pb) = c1;
 }
 
-// Producer: decode one channel block of one tile's halo into stage st.
-// Lane l owns slots l, l + 32, ...; each slot takes NPC 16-byte pieces
-// (4 words = two 16-code chunks each) of its pixel.  The pieces of up to
-// 16 / NPC slot groups are loaded before any decode, so a fill makes at
-// most a few round trips to memory.
-template <int NPC, int MODE>
-__device__ __forceinline__ void halo_fill_t(const HaloGeom& g, int p0, const uint32_t* xi, uint8_t* st, int lane,
-                                            int k, int ew, const uint8_t* lut, int b)
+// Item i of a stage fill is piece i % npc of slot i / npc (1 <= npc <= 4; i
+// below 2^14: exact with a 16-bit reciprocal).
+__device__ __forceinline__ int halo_slot(int i, int npc, uint32_t recip)
 {
-    constexpr int GB = 16 / NPC;                                   // slot groups per batch
-    const int groups = (g.ns + 31) >> 5;
-    const int nb = (groups + GB - 1) / GB;
-    const int per = (groups + nb - 1) / nb;                        // balanced batches
+    return npc == 4 ? i >> 2 : (int)(((uint32_t)i * recip) >> 16);
+}
+
+// Register fills (several channel blocks): every producer thread takes
+// kFillLoads pieces of a batch, so a batch is kWsProdWarps * 32 * kFillLoads
+// items and a stage a few batches.  Filling each stage with all producer
+// warps, rather than a stage per warp, keeps them all busy when only two
+// stages fit beside the filters, and the next batch's loads are in flight
+// while the current one is decoded.
+constexpr int kFillLoads = 4;
+constexpr int kFillBatch = kWsProdWarps * 32 * kFillLoads;
+
+struct HaloCursor {                                   // a batch: tile, channel block, first item
+    int64_t ti;
+    int cb, i0;
+};
+
+// Geometry of a batch's stage: items, pieces per slot.
+__device__ __forceinline__ int halo_npc(const HaloGeom& g, int cb) { return min(16, g.ldx - cb * 16) >> 2; }
+
+__device__ __forceinline__ void halo_load(const HaloGeom& g, int T, int cb, int i0, int t, uint32_t zw, uint4 (&v)[kFillLoads])
+{
+    const int nimg = T / g.tpi;
+    const int p0 = (T - nimg * g.tpi) * g.rows_out;
+    const int npc = halo_npc(g, cb);
+    const uint32_t recip = 65536u / (uint32_t)npc + 1u;
     const int wsm = (1 << g.lws) - 1;
-#pragma unroll 1
-    for (int g0 = 0; g0 < groups; g0 += per) {
-        uint4 v[GB][NPC];
-        uint32_t okm = 0u;
+    const uint32_t* xi = g.X + (int64_t)nimg * g.H * g.W * g.ldx + cb * 16;
 #pragma unroll
-        for (int u = 0; u < GB; u++) {
-            const int slot = (g0 + u) * 32 + lane;
-            const int rel = slot - g.pad;
-            const int hi = rel >> g.lws;                           // halo row (-1: left guard)
-            const int j = rel & wsm;
-            const int h = p0 - g.pad + hi;
-            const bool ok = u < per && slot < g.ns && rel >= 0 && hi < g.hr && j < g.W && (unsigned)h < (unsigned)g.H;
-            const uint4* px = reinterpret_cast<const uint4*>(xi + ((int64_t)h * g.W + j) * g.ldx);
+    for (int u = 0; u < kFillLoads; u++) {
+        const int i = i0 + u * kWsProdWarps * 32 + t;
+        const int slot = halo_slot(i, npc, recip), pc = i - slot * npc;
+        const int rel = slot - g.pad;
+        const int hi = rel >> g.lws;                               // halo row (-1: left guard)
+        const int j = rel & wsm;
+        const int h = p0 - g.pad + hi;
+        const bool ok = slot < g.ns && rel >= 0 && hi < g.hr && j < g.W && (unsigned)h < (unsigned)g.H;
+        v[u] = make_uint4(zw, zw, zw, zw);
+        if (ok) v[u] = __ldg(reinterpret_cast<const uint4*>(xi + ((int64_t)h * g.W + j) * g.ldx) + pc);
+    }
+}
+
+template <int B>
+__device__ __forceinline__ void halo_store(const HaloGeom& g, int cb, int i0, int t, uint8_t* st, const uint4 (&v)[kFillLoads],
+                                           int k, int ew)
+{
+    const int npc = halo_npc(g, cb);
+    const uint32_t recip = 65536u / (uint32_t)npc + 1u;
 #pragma unroll
-            for (int pc = 0; pc < NPC; pc++) v[u][pc] = ok ? __ldg(px + pc) : make_uint4(0u, 0u, 0u, 0u);
-            okm |= (ok ? 1u : 0u) << u;
-        }
-#pragma unroll
-        for (int u = 0; u < GB; u++) {
-            const int slot = (g0 + u) * 32 + lane;
-            if (u >= per || slot >= g.ns) break;
-            const bool ok = (okm >> u) & 1u;
-#pragma unroll
-            for (int pc = 0; pc < NPC; pc++) halo_store_piece<MODE>(st, g.pb, slot, pc, ok, v[u][pc], k, ew, lut, b);
-        }
+    for (int u = 0; u < kFillLoads; u++) {
+        const int i = i0 + u * kWsProdWarps * 32 + t;
+        const int slot = halo_slot(i, npc, recip);
+        if (slot < g.ns) halo_store_piece<B>(st, g.pb, slot, i - slot * npc, v[u], k, ew);
     }
 }
 
@@ -207,92 +177,29 @@ __device__ __forceinline__ void halo_issue_rows(const HaloGeom& g, int64_t T, ui
     }
 }
 
-// The decoders' share of one bulk-filled tile: slots first, first + stride,
-// ... (zeros for padding slots and rows outside the image).
-template <int NPC, int MODE>
-__device__ __forceinline__ void halo_decode_t(const HaloGeom& g, int64_t T, uint8_t* st, int first, int stride, int k,
-                                              int ew, const uint8_t* lut, int b)
+// The decoders' share of one bulk-filled tile: items first, first + stride,
+// ... (zero codes for padding slots and rows outside the image).
+template <int B>
+__device__ __noinline__ void halo_decode(const HaloGeom g, int T, uint8_t* st, int first, int stride, int k, int ew)
 {
-    const int nimg = (int)(T / g.tpi);
-    const int p0 = (int)(T - (int64_t)nimg * g.tpi) * g.rows_out;
+    const int nimg = T / g.tpi;
+    const int p0 = (T - nimg * g.tpi) * g.rows_out;
     const uint8_t* raw = st + g.planes_bytes;
     const int wsm = (1 << g.lws) - 1;
+    const int npc = g.ldx >> 2;
+    const uint32_t recip = 65536u / (uint32_t)npc + 1u;
+    const uint32_t zw = fmt_zero_word(B, k);
+    const int items = g.ns * npc;
 #pragma unroll 1                                      // compact: it shares the SM's instruction cache
-    for (int slot = first; slot < g.ns; slot += stride) {
+    for (int i = first; i < items; i += stride) {
+        const int slot = halo_slot(i, npc, recip), pc = i - slot * npc;
         const int rel = slot - g.pad;
         const int hi = rel >> g.lws;
         const int j = rel & wsm;
         const int h = p0 - g.pad + hi;
         const bool ok = rel >= 0 && hi < g.hr && j < g.W && (unsigned)h < (unsigned)g.H;
         const uint4* src = reinterpret_cast<const uint4*>(raw + ((size_t)hi * g.W + j) * g.ldx * 4);
-#pragma unroll 1                                      // one piece at a time: a small loop body
-        for (int pc = 0; pc < NPC; pc++)
-            halo_store_piece<MODE>(st, g.pb, slot, pc, ok, ok ? src[pc] : make_uint4(0u, 0u, 0u, 0u), k, ew, lut, b);
-    }
-}
-
-// lut: the E4M3 table of a 5/6-bit word-slot input (nullptr: 4-bit codes).
-__device__ __noinline__ void halo_decode(const HaloGeom g, int64_t T, uint8_t* st, int first, int stride, int k, int ew,
-                                         const uint8_t* lut, int b)
-{
-    if (lut && g.spw == 16) {
-        switch (g.ldx >> 2) {
-        case 1: halo_decode_t<1, kHaloSlot16>(g, T, st, first, stride, k, ew, lut, b); break;
-        case 2: halo_decode_t<2, kHaloSlot16>(g, T, st, first, stride, k, ew, lut, b); break;
-        case 3: halo_decode_t<3, kHaloSlot16>(g, T, st, first, stride, k, ew, lut, b); break;
-        default: halo_decode_t<4, kHaloSlot16>(g, T, st, first, stride, k, ew, lut, b); break;
-        }
-        return;
-    }
-    if (lut) {
-        switch (g.ldx >> 2) {
-        case 1: halo_decode_t<1, kHaloSlot8>(g, T, st, first, stride, k, ew, lut, b); break;
-        case 2: halo_decode_t<2, kHaloSlot8>(g, T, st, first, stride, k, ew, lut, b); break;
-        case 3: halo_decode_t<3, kHaloSlot8>(g, T, st, first, stride, k, ew, lut, b); break;
-        default: halo_decode_t<4, kHaloSlot8>(g, T, st, first, stride, k, ew, lut, b); break;
-        }
-        return;
-    }
-    switch (g.ldx >> 2) {
-    case 1: halo_decode_t<1, kHaloB4>(g, T, st, first, stride, k, ew, lut, b); break;
-    case 2: halo_decode_t<2, kHaloB4>(g, T, st, first, stride, k, ew, lut, b); break;
-    case 3: halo_decode_t<3, kHaloB4>(g, T, st, first, stride, k, ew, lut, b); break;
-    default: halo_decode_t<4, kHaloB4>(g, T, st, first, stride, k, ew, lut, b); break;
-    }
-}
-
-// Channel block cb (words 16 cb .. of each pixel) of tile T's halo.
-__device__ __noinline__ void halo_fill(const HaloGeom g, int64_t T, int cb, uint8_t* st, int lane, int k, int ew,
-                                       const uint8_t* lut, int b)
-{
-    const int nimg = (int)(T / g.tpi);
-    const int p0 = (int)(T - (int64_t)nimg * g.tpi) * g.rows_out;
-    const int w0 = cb * 16;
-    const int npc = min(16, g.ldx - w0) >> 2;                      // pieces per slot (1..4)
-    const uint32_t* xi = g.X + (int64_t)nimg * g.H * g.W * g.ldx + w0;
-    if (lut && g.spw == 16) {
-        switch (npc) {
-        case 1: halo_fill_t<1, kHaloSlot16>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        case 2: halo_fill_t<2, kHaloSlot16>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        case 3: halo_fill_t<3, kHaloSlot16>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        default: halo_fill_t<4, kHaloSlot16>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        }
-        return;
-    }
-    if (lut) {
-        switch (npc) {
-        case 1: halo_fill_t<1, kHaloSlot8>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        case 2: halo_fill_t<2, kHaloSlot8>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        case 3: halo_fill_t<3, kHaloSlot8>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        default: halo_fill_t<4, kHaloSlot8>(g, p0, xi, st, lane, k, ew, lut, b); break;
-        }
-        return;
-    }
-    switch (npc) {
-    case 1: halo_fill_t<1, kHaloB4>(g, p0, xi, st, lane, k, ew, lut, b); break;
-    case 2: halo_fill_t<2, kHaloB4>(g, p0, xi, st, lane, k, ew, lut, b); break;
-    case 3: halo_fill_t<3, kHaloB4>(g, p0, xi, st, lane, k, ew, lut, b); break;
-    default: halo_fill_t<4, kHaloB4>(g, p0, xi, st, lane, k, ew, lut, b); break;
+        halo_store_piece<B>(st, g.pb, slot, pc, ok ? src[pc] : make_uint4(zw, zw, zw, zw), k, ew);
     }
 }
 
@@ -328,11 +235,6 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
     const int epi_warps = split ? 8 : 4;
     const int cbs = g.cblocks;
-    // E4M3 tables of 5/6-bit word-slot operands (4-bit codes decode by SWAR)
-    __shared__ uint8_t lut_a[64], lut_b[64];
-    const bool slot_a = fa.spw != 0;
-    if (slot_a) build_e4m3_lut(lut_a, fa, tid, kWsThreads);
-    if (fb.spw != 0) build_e4m3_lut(lut_b, fb, tid, kWsThreads);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -349,8 +251,8 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     }
     if (tid == 0) {
         for (int s = 0; s < stages; s++) {
-            // bulk path: the kKHaloDecoders decoder warps fill a stage together
-            mbar_init(&full[s], g.raw_bytes > 0 ? kHaloDecoders : 1);
+            // the decoder warps (register path: every producer warp) fill a stage together
+            mbar_init(&full[s], g.raw_bytes > 0 ? kHaloDecoders : kWsProdWarps);
             mbar_init(&empty[s], 1);
             mbar_init(&rawb[s], 1);                   // the issuer's arrive.expect_tx, then the copies' bytes
         }
@@ -377,7 +279,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     if (!(bulk && warp == kWsProdWarp0)) {
         const int nbdec = bulk ? kWsThreads - 32 : kWsThreads;
         const int t = (bulk && warp > kWsProdWarp0) ? tid - 32 : tid;
-        ws_decode_b<FAST>(srcB, n0, K, fb, BN, nkb, sB, t, nbdec, fb.spw ? lut_b : nullptr);
+        ws_decode_b<FAST>(srcB, n0, K, fb, BN, nkb, sB, t, nbdec);
         fence_proxy_async_smem();
         if (warp == kWsMmaWarp) asm volatile("bar.sync 1, %0;" ::"r"(nbdec) : "memory");
         else asm volatile("bar.arrive 1, %0;" ::"r"(nbdec) : "memory");
@@ -406,39 +308,56 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
                 }
             } else {
                 const int d = p - 1;                  // decoder index 0 .. kHaloDecoders - 1
-                for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
-                    if (!wait_or_abort(&rawb[s], ph, err)) { *err = 1; break; }
-                    halo_decode(g, cta_in_n + ti * ctas_per_n, sA + s * g.stage_bytes, d * 32 + lane,
-                                kHaloDecoders * 32, fa.k, fa.ew, slot_a ? lut_a : nullptr, fa.b);
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&full[s]);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
-                }
+                auto decode_tiles = [&](auto width) {
+                    for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
+                        if (!wait_or_abort(&rawb[s], ph, err)) { *err = 1; break; }
+                        halo_decode<decltype(width)::value>(g, (int)(cta_in_n + ti * ctas_per_n), sA + s * g.stage_bytes,
+                                                            d * 32 + lane, kHaloDecoders * 32, fa.k, fa.ew);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&full[s]);
+                        if (++s == stages) { s = 0; ph ^= 1u; }
+                    }
+                };
+                if (FAST) decode_tiles(IntC<4>());
+                else with_width(fa.b, decode_tiles);
             }
-        } else {
-        // Register path (several channel blocks): warp p fills iterations p,
-        // p + nprod, ... of this CTA's (tile, channel block) sequence; at most
-        // `stages` producers are active (an mbarrier's parity tells apart
-        // only adjacent phases).
-        const int nprod = stages < kWsProdWarps ? stages : kWsProdWarps;
-        const int64_t total_it = (p < nprod) ? my_tiles * cbs : 0;
-        // stage s and its phase ph follow it incrementally (no division in
-        // the loop): it advances by nprod <= stages, so s wraps at most once
-        int s = p;
-        uint32_t ph = 0u;
-        for (int64_t it = p; it < total_it && !*err; it += nprod) {
-            const int64_t ti = (cbs == 1) ? it : it / cbs;
-            const int cb = (int)(it - ti * cbs);
-            if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
-            halo_fill(g, cta_in_n + ti * ctas_per_n, cb, sA + s * g.stage_bytes, lane, fa.k, fa.ew,
-                      slot_a ? lut_a : nullptr, fa.b);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&full[s]);
-            s += nprod;
-            if (s >= stages) { s -= stages; ph ^= 1u; }
-        }
+        } else if constexpr (!FAST) {
+            // Register path (several channel blocks): the (tile, channel
+            // block) stages in order, each filled by every producer warp.
+            const int t = p * 32 + lane;
+            with_width(fa.b, [&](auto width) {
+                constexpr int B = decltype(width)::value;
+                const uint32_t zw = fmt_zero_word(B, fa.k);
+                uint4 v[kFillLoads];
+                HaloCursor c{0, 0, 0};
+                int s = 0;
+                uint32_t ph = 0u;
+                if (my_tiles > 0) halo_load(g, (int)cta_in_n, 0, 0, t, zw, v);
+                while (c.ti < my_tiles && !*err) {
+                    if (c.i0 == 0 && !wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
+                    // the next batch: the same stage's rest, else the next stage's start
+                    HaloCursor nx = c;
+                    nx.i0 += kFillBatch;
+                    const bool last = nx.i0 >= g.ns * halo_npc(g, c.cb);
+                    if (last) {
+                        nx.i0 = 0;
+                        if (++nx.cb == cbs) { nx.cb = 0; nx.ti++; }
+                    }
+                    uint4 vn[kFillLoads];
+                    if (nx.ti < my_tiles) halo_load(g, (int)(cta_in_n + nx.ti * ctas_per_n), nx.cb, nx.i0, t, zw, vn);
+                    halo_store<B>(g, c.cb, c.i0, t, sA + s * g.stage_bytes, v, fa.k, fa.ew);
+                    if (last) {
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&full[s]);
+                        if (++s == stages) { s = 0; ph ^= 1u; }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kFillLoads; u++) v[u] = vn[u];
+                    c = nx;
+                }
+            });
         }
     } else if (warp == kWsMmaWarp) {
         // ---------------------------------------------- MMA issue
@@ -473,15 +392,21 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
                     } else if (r3 && ws == 16 && units_tap == 8 && pairs == 4 && BN == 64) {   // 14 x 14 x 256
                         halo_mma_fixed<16, 3, 3, 8, 4, 64>(d, a_st, b_blk, idesc, acc);
                     } else {
+                        // offsets in the descriptors' low words (16-byte units; the
+                        // address fields cannot carry out of them)
+                        const uint64_t ad0 = smem_desc_noswz(a_st, (uint32_t)g.pb, 128u), bd0 = smem_desc_sw128(b_base);
+                        const uint32_t alo = (uint32_t)ad0, blo = (uint32_t)bd0;
+                        const uint64_t ahi = ad0 & ~0xffffffffull, bhi = bd0 & ~0xffffffffull;
+                        const uint32_t pstep = (uint32_t)(2 * g.pb) >> 4, bstep = (uint32_t)(BN * kBK) >> 4;
+                        int kq0 = cb * (g.spw >> 1);
                         for (int r = 0; r < g.R; r++) {
-                            for (int sx = 0; sx < g.S; sx++) {
-                                const uint32_t at = a_st + (uint32_t)((r * ws + sx) * 16);
-                                const int kq0 = (r * g.S + sx) * units_tap + cb * (g.spw >> 1);
-                                for (int j = 0; j < pairs; j++) {
-                                    const int kq = kq0 + j;
-                                    const uint32_t bb = b_base + (uint32_t)((kq >> 2) * BN * kBK + (kq & 3) * 32);
-                                    mma_f8f6f4(d, smem_desc_noswz(at + (uint32_t)(2 * j * g.pb), (uint32_t)g.pb, 128u),
-                                               smem_desc_sw128(bb), idesc, acc);
+                            for (int sx = 0; sx < g.S; sx++, kq0 += units_tap) {
+                                uint32_t at = alo + (uint32_t)(r * ws + sx);
+#pragma unroll 4
+                                for (int j = 0; j < pairs; j++, at += pstep) {
+                                    const uint32_t kq = (uint32_t)(kq0 + j);
+                                    const uint32_t bt = blo + (kq >> 2) * bstep + (kq & 3u) * 2u;
+                                    mma_f8f6f4(d, ahi | at, bhi | bt, idesc, acc);
                                     acc = 1u;
                                 }
                             }

@@ -55,7 +55,7 @@ struct ConvSrc {
     const uint32_t* X;
     int ldx;
     int rows;                     // n * P * Q
-    int H, W, P, Q, S, stride, pad;
+    int H, W, P, Q, R, S, stride, pad;
     // Words of each pixel in the logical K (<= ldx): the words that hold
     // channels, so a pixel row's padding words (e.g. the 3 of a first
     // layer's 4-word rows) take no K.  The logical word w is word w % kw of
@@ -123,6 +123,13 @@ struct ConvSrc {
             }
         }
     }
+    // The in-image tap ranges in one word, for a filter of at most 255 x 255
+    // taps (a count past 255 is as good as 255).
+    __device__ __forceinline__ uint32_t bounds(const Row& x) const
+    {
+        return (uint32_t)min(x.rlo, 255) | (uint32_t)min(x.rn, 255) << 8 | (uint32_t)min(x.slo, 255) << 16 |
+               (uint32_t)min(x.sn, 255) << 24;
+    }
     // 16-byte pieces (4 logical words) are contiguous in memory
     __host__ __device__ __forceinline__ bool vec4() const { return (kw & 3) == 0; }
     __device__ __forceinline__ const uint32_t* at(const Row& x, const Cursor& c) const
@@ -182,7 +189,7 @@ __device__ __forceinline__ void walk_b4_tab(const ConvSrc& src, const ConvSrc::R
 // Word-slot codes (see plan_slots): the K-block's NW words, CH at a time.
 template <int B>
 __device__ __forceinline__ void walk_slots_tab(const ConvSrc& src, const ConvSrc::Row& row, const int4* tab,
-                                               int64_t k0, const OpFmt& f, const uint8_t* lut, uint8_t* stage, int r)
+                                               int64_t k0, const OpFmt& f, uint8_t* stage, int r)
 {
     constexpr int CPW = 32 / B;
     constexpr int SPW = CPW > 8 ? 16 : (CPW > 4 ? 8 : 4);
@@ -202,22 +209,21 @@ __device__ __forceinline__ void walk_slots_tab(const ConvSrc& src, const ConvSrc
             wv[i] = in ? __ldg(src.X + (row.base + e.z)) : 0u;
             ok |= (in ? 1u : 0u) << i;
         }
-        store_slot_words<B, CH>(wv, ok, lim, lut, stage, r, c0 * SPW / 16);
+        store_slot_words<B, CH>(wv, ok, lim, f, stage, r, c0 * SPW / 16);
     }
 }
 
 __device__ __forceinline__ void walk_row_tab(const ConvSrc& src, const ConvSrc::Row& row, const int4* tab,
-                                             int64_t k0, int64_t K, const OpFmt& f, const uint8_t* lut, uint8_t* stage,
-                                             int r)
+                                             int64_t k0, int64_t K, const OpFmt& f, uint8_t* stage, int r)
 {
     if (f.b == 4) { walk_b4_tab(src, row, tab, k0, K, f, stage, r); return; }
     switch (f.b) {
-    case 2: walk_slots_tab<2>(src, row, tab, k0, f, lut, stage, r); return;
-    case 3: walk_slots_tab<3>(src, row, tab, k0, f, lut, stage, r); return;
-    case 5: walk_slots_tab<5>(src, row, tab, k0, f, lut, stage, r); return;
-    case 6: walk_slots_tab<6>(src, row, tab, k0, f, lut, stage, r); return;
-    case 7: walk_slots_tab<7>(src, row, tab, k0, f, lut, stage, r); return;
-    default: walk_slots_tab<8>(src, row, tab, k0, f, lut, stage, r); return;
+    case 2: walk_slots_tab<2>(src, row, tab, k0, f, stage, r); return;
+    case 3: walk_slots_tab<3>(src, row, tab, k0, f, stage, r); return;
+    case 5: walk_slots_tab<5>(src, row, tab, k0, f, stage, r); return;
+    case 6: walk_slots_tab<6>(src, row, tab, k0, f, stage, r); return;
+    case 7: walk_slots_tab<7>(src, row, tab, k0, f, stage, r); return;
+    default: walk_slots_tab<8>(src, row, tab, k0, f, stage, r); return;
     }
 }
 
@@ -550,9 +556,11 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
         const int nprod = stages < kWsProdWarps ? stages : kWsProdWarps;
         const int64_t total_it = (p < nprod) ? my_tiles * nkb : 0;
         griddep_wait();                               // A may come from the previous launch
-        const uint32_t zwa = fmt_zero_code(4, fa.k) * 0x11111111u;
-        const uint32_t zwb = fmt_zero_code(4, fb.k) * 0x11111111u;
-        const bool b_vec = fb.b == 4 && fb.planes == 1 && srcB.linear() && srcB.vec4();
+        bool a_pieces = by_pieces(srcA, fa);
+        if constexpr (kIsConv<SrcA>) a_pieces = a_pieces && srcA.R <= 255 && srcA.S <= 255;
+        const bool b_pieces = by_pieces(srcB, fb);
+        int64_t rbase[4] = {0, 0, 0, 0};              // im2col rows by pieces: base and packed tap ranges
+        uint32_t rbnd[4] = {0u, 0u, 0u, 0u};
         int64_t cur_tile = -1;
         typename SrcA::Row rows[4];
         // stage s and its phase ph follow it incrementally (no division in
@@ -566,24 +574,47 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                 cur_tile = ti;
                 const int64_t m0 = (cta_in_n + ti * ctas_per_n) * kBM;
 #pragma unroll
-                for (int q = 0; q < 4; q++) rows[q] = srcA.row(m0 + lane + 32 * q);
+                for (int q = 0; q < 4; q++) {
+                    rows[q] = srcA.row(m0 + lane + 32 * q);
+                    if constexpr (kIsConv<SrcA>) { rbase[q] = rows[q].base; rbnd[q] = srcA.bounds(rows[q]); }
+                }
             }
             if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
             uint8_t* st = sA + s * stage_bytes;
-            if (fa.b == 4 && fa.planes == 1 && srcA.linear() && srcA.vec4()) {
-                const int64_t kw0 = (int64_t)kb * 16;
-                typename SrcA::Cursor cur[4];
-#pragma unroll
-                for (int pc = 0; pc < 4; pc++) cur[pc] = srcA.cursor(kw0 + 4 * pc);
-                // one row at a time: a rolled loop keeps the producers' code
-                // small (the SM's instruction caches hold every role's loop;
-                // measured faster than four rows' loads in flight unrolled)
+            if (a_pieces) {
+                with_width(fa.b, [&](auto width) {
+                    constexpr int B = decltype(width)::value;
+                    using S = SlotFmt<B>;
+                    if constexpr (kIsConv<SrcA>) {
+                        // the rows' bases and tap ranges come from the lanes
+                        // that hold them (rows[q] of lane l is row 32 q + l);
+                        // the four sets rotate through one rolled loop body
+                        const int64_t w0 = (int64_t)kb * S::NW + 4 * (lane % S::LPR);
+                        const int64_t left = (B == 4 ? K : fa.korig) - w0 * S::CPW;
+                        const typename SrcA::Cursor c = srcA.cursor(w0);
 #pragma unroll 1
-                for (int q = 0; q < 4; q++) {
-                    uint4 v[4];
-                    load_row_b4(srcA, rows[q], cur, kw0, K, zwa, v);
-                    store_row_b4(st, lane + 32 * q, v, kw0, K, fa);
-                }
+                        for (int q = 0; q < 4; q++) {
+                            fill_q<B>(st, q, kBM, left, fa.k, fa.ew, lane, [&](int u) -> const uint32_t* {
+                                const int sl = u * S::RPI + lane / S::LPR;
+                                const int64_t base = __shfl_sync(0xffffffffu, (long long)rbase[0], sl);
+                                const uint32_t bd = __shfl_sync(0xffffffffu, rbnd[0], sl);
+                                const bool in = (unsigned)(c.r - (int)(bd & 255u)) < ((bd >> 8) & 255u) &&
+                                                (unsigned)(c.s - (int)((bd >> 16) & 255u)) < (bd >> 24);
+                                return in ? srcA.X + base + c.off : nullptr;
+                            });
+                            const int64_t b0 = rbase[0];
+                            const uint32_t d0 = rbnd[0];
+#pragma unroll
+                            for (int i = 0; i < 3; i++) { rbase[i] = rbase[i + 1]; rbnd[i] = rbnd[i + 1]; }
+                            rbase[3] = b0;
+                            rbnd[3] = d0;
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int q = 0; q < 4; q++)
+                            fill_rows_q<B>(srcA, (cta_in_n + ti * ctas_per_n) * kBM, kBM, kb, q, K, fa, st, lane);
+                    }
+                });
             } else if (fa.planes == 1 && srcA.linear()) {
                 bool done = false;
                 if constexpr (kIsConv<SrcA>) {
@@ -594,7 +625,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                         conv_tap_table(srcA, (int64_t)kb * nw, nw, tab, lane);
 #pragma unroll 1
                         for (int q = 0; q < 4; q++)
-                            walk_row_tab(srcA, rows[q], tab, (int64_t)kb * kBK, K, fa, luta, st, lane + 32 * q);
+                            walk_row_tab(srcA, rows[q], tab, (int64_t)kb * kBK, K, fa, st, lane + 32 * q);
                         done = true;
                     }
                 }
@@ -608,23 +639,15 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                 fill_stage_any(srcA, (cta_in_n + ti * ctas_per_n) * kBM, st, lane, (int64_t)kb * kBK, K, fa);
             }
             if (bstream) {
-                // this K-block of the CTA's B rows n0 .. n0 + BN, two rows per lane in flight
+                // this K-block of the CTA's B rows n0 .. n0 + BN
                 uint8_t* sb = st + kBM * kBK;
                 const int64_t k0 = (int64_t)kb * kBK;
-                if (b_vec) {
-                    const int64_t kw0 = (int64_t)kb * 16;
-                    RowsSrc::Cursor cur[4];
-#pragma unroll
-                    for (int pc = 0; pc < 4; pc++) cur[pc] = srcB.cursor(kw0 + 4 * pc);
+                if (b_pieces) {
+                    with_width(fb.b, [&](auto width) {
 #pragma unroll 1
-                    for (int r = lane; r < BN; r += 64) {
-                        const bool two = r + 32 < BN;
-                        uint4 v0[4], v1[4];
-                        load_row_b4(srcB, srcB.row(n0 + r), cur, kw0, K, zwb, v0);
-                        if (two) load_row_b4(srcB, srcB.row(n0 + r + 32), cur, kw0, K, zwb, v1);
-                        store_row_b4(sb, r, v0, kw0, K, fb);
-                        if (two) store_row_b4(sb, r + 32, v1, kw0, K, fb);
-                    }
+                        for (int q = 0; q < (BN + 31) >> 5; q++)
+                            fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sb, lane);
+                    });
                 } else if (fb.planes == 1 && srcB.linear()) {
 #pragma unroll 1
                     for (int r = lane; r < BN; r += 32) walk_row_kblock(srcB, srcB.row(n0 + r), k0, K, fb, lutb, sb, r);
@@ -976,7 +999,7 @@ cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t*
     const int64_t K = (int64_t)d.r * d.s * kwx * (32 / bx);
     const int BN = pick_bn(N, ep.out_cpw);
     ConvSrc a;
-    a.X = X; a.ldx = (int)ldx; a.rows = (int)M; a.H = d.h; a.W = d.w; a.P = P; a.Q = Q; a.S = d.s;
+    a.X = X; a.ldx = (int)ldx; a.rows = (int)M; a.H = d.h; a.W = d.w; a.P = P; a.Q = Q; a.R = d.r; a.S = d.s;
     a.stride = d.stride; a.pad = d.pad; a.kw = kwx;
     RowsSrc b = conv_filter_rows(d, W, ldx, bx, ldw, bw, kwx);
     OpFmt fa = make_opfmt(bx, kx), fb = make_opfmt(bw, kw);

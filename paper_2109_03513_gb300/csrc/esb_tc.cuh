@@ -319,36 +319,118 @@ __device__ __forceinline__ void build_e4m3_lut(uint8_t* lut, const OpFmt& f, int
     for (int c = t; c < (1 << f.b); c += nt) lut[c] = (uint8_t)code_to_e4m3((uint32_t)c, f);
 }
 
+// The K-block geometry of B-bit codes in the word-slot layout (4-bit codes:
+// 8 codes a word, no gaps, the same as 8 slots): SPW K slots per packed word,
+// NW words per K-block, and a warp's split of a row: LPR lanes take one
+// 16-byte piece (4 words) each, RPI rows per pass of 32 lanes.
+template <int B>
+struct SlotFmt {
+    static constexpr int CPW = 32 / B;
+    static constexpr int SPW = CPW > 8 ? 16 : (CPW > 4 ? 8 : 4);
+    static constexpr int NW = kBK / SPW;
+    static constexpr int LPR = NW / 4;
+    static constexpr int RPI = 32 / LPR;
+};
+
+// One packed word -> its SPW E4M3 bytes (slots past the word's codes zero),
+// about 3.5 instructions per code (a byte-table walk takes 7, two of them
+// shared-memory loads with bank conflicts).
+template <int B>
+__device__ __forceinline__ void decode_slots(uint32_t w, int k, int ew, uint32_t* o)
+{
+    if (B == 4) {
+        decode_word_b4(w, k, ew, o[0], o[1]);
+        return;
+    }
+    const uint32_t u = rot_word<B>(w, k);
+#pragma unroll
+    for (int q = 0; q < SlotFmt<B>::SPW / 4; q++) {
+        constexpr int step = (4 * B) & 31;            // 8-bit codes: one group, no shift
+        o[q] = 4 * q < SlotFmt<B>::CPW ? e4m3_4<B>(spread4<B>(q ? u >> (step * q) : u), k) : 0u;
+    }
+}
+
+// The word's first v codes (any v), zero codes after them.
+template <int B>
+__device__ __forceinline__ uint32_t keep_codes(uint32_t w, int v, uint32_t zero_word)
+{
+    if (v >= SlotFmt<B>::CPW) return w;
+    const uint32_t keep = v > 0 ? (1u << (B * v)) - 1u : 0u;
+    return (w & keep) | (zero_word & ~keep);
+}
+
+__device__ __forceinline__ uint32_t fmt_zero_word(int b, int k)
+{
+    uint32_t z = 0u;
+    for (int j = 0; j < 32 / b; j++) z |= fmt_zero_code(b, k) << (b * j);
+    return z;
+}
+
+// Piece pc (4 words, of which the first `left` codes are inside K) of stage
+// row r, decoded and stored.
+template <int B>
+__device__ __forceinline__ void store_piece(uint8_t* stage, int r, int pc, const uint4& v, int64_t left, int k, int ew,
+                                            uint32_t zero_word)
+{
+    using S = SlotFmt<B>;
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    if (left < 4 * S::CPW) {
+#pragma unroll
+        for (int i = 0; i < 4; i++) w[i] = keep_codes<B>(w[i], (int)left - i * S::CPW, zero_word);
+    }
+    constexpr int RW = S::SPW / 4;                    // registers per word
+#pragma unroll
+    for (int c = 0; c < RW; c++) {                    // RW chunks of 16 bytes, 4 / RW words each
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4 / RW; i++) decode_slots<B>(w[c * (4 / RW) + i], k, ew, o + i * RW);
+        *reinterpret_cast<uint4*>(stage + swz(r, RW * pc + c)) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
+// Rows 32 q .. 32 q + 31 of a stage block of nrows rows, a piece per lane:
+// ptr(u) gives the lane's piece of row 32 q + u RPI + lane / LPR (nullptr:
+// zeros).  LPR consecutive lanes read 16 LPR contiguous bytes of a row (one
+// lane per row read 16 bytes of 32 rows at a time, and the L1 took a pass per
+// row), and all LPR loads are in flight together.
+template <int B, class F>
+__device__ __forceinline__ void fill_q(uint8_t* stage, int q, int nrows, int64_t left, int k, int ew, int lane, const F& ptr)
+{
+    using S = SlotFmt<B>;
+    const uint32_t zw = fmt_zero_word(B, k);
+    const int pc = lane % S::LPR, r0 = q * 32 + lane / S::LPR;
+    uint4 v[S::LPR];
+#pragma unroll
+    for (int u = 0; u < S::LPR; u++) {
+        const uint32_t* p = ptr(u);
+        v[u] = (p && left > 0) ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(zw, zw, zw, zw);
+    }
+#pragma unroll
+    for (int u = 0; u < S::LPR; u++)
+        if (r0 + u * S::RPI < nrows) store_piece<B>(stage, r0 + u * S::RPI, pc, v[u], left, k, ew, zw);
+}
+
 // CH loaded words of B-bit codes in the word-slot layout (ok: word i
 // exists; lim: codes of the chunk inside K) -> their E4M3 slots, stored as
 // 16-byte units from unit g0 of stage row r.
 template <int B, int CH>
-__device__ __forceinline__ void store_slot_words(const uint32_t (&wv)[CH], uint32_t ok, int lim, const uint8_t* lut,
+__device__ __forceinline__ void store_slot_words(const uint32_t (&wv)[CH], uint32_t ok, int lim, const OpFmt& f,
                                                  uint8_t* stage, int r, int g0)
 {
-    constexpr int CPW = 32 / B;
-    constexpr int SPW = CPW > 8 ? 16 : (CPW > 4 ? 8 : 4);
-    constexpr uint32_t MASK = (1u << B) - 1u;
-    uint32_t o[CH * SPW / 4];
+    constexpr int CPW = SlotFmt<B>::CPW, RW = SlotFmt<B>::SPW / 4;
+    const uint32_t zw = fmt_zero_word(B, f.k);
 #pragma unroll
-    for (int i = 0; i < CH; i++) {
+    for (int g = 0; g < CH * RW / 4; g++) {
+        uint32_t o[4];
 #pragma unroll
-        for (int q = 0; q < SPW / 4; q++) {
-            uint32_t v = 0u;
-#pragma unroll
-            for (int t = 0; t < 4; t++) {
-                const int j = q * 4 + t;
-                if (j < CPW) {
-                    const uint32_t byte = lut[(wv[i] >> (B * j)) & MASK];
-                    v |= ((i * CPW + j < lim) ? byte : 0u) << (8 * t);
-                }
-            }
-            o[i * (SPW / 4) + q] = ((ok >> i) & 1u) ? v : 0u;
+        for (int i = 0; i < 4 / RW; i++) {
+            const int wi = g * (4 / RW) + i;
+            uint32_t w = ((ok >> wi) & 1u) ? wv[wi] : zw;
+            if (lim < CH * CPW) w = keep_codes<B>(w, lim - wi * CPW, zw);
+            decode_slots<B>(w, f.k, f.ew, o + i * RW);
         }
+        *reinterpret_cast<uint4*>(stage + swz(r, g0 + g)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
-#pragma unroll
-    for (int g = 0; g < CH * SPW / 16; g++)
-        *reinterpret_cast<uint4*>(stage + swz(r, g0 + g)) = make_uint4(o[4 * g], o[4 * g + 1], o[4 * g + 2], o[4 * g + 3]);
 }
 
 // NW loaded words of a 4-bit K-block from code k0 (ok: word i exists)
@@ -380,13 +462,12 @@ __device__ __forceinline__ void store_b4_words(const uint32_t (&wv)[NW], uint32_
 }
 
 // One K-block of a row in the word-slot layout (see plan_slots) for B-bit
-// codes: the block's words are loaded 16 at a time (independent loads in
-// flight), then each word's codes go through the E4M3 table to their fixed
-// bytes.  Words past the row's K words, outside the operand or outside the
+// codes: the block's words are loaded 8 at a time (independent loads in
+// flight), then each word decodes to its fixed bytes.  Words past the row's K words, outside the operand or outside the
 // image, and codes past korig, give the E4M3 zero.
 template <int B, class Src>
 __device__ __forceinline__ void walk_row_slots(const Src& src, const typename Src::Row& row, int64_t k0,
-                                               const OpFmt& f, const uint8_t* lut, uint8_t* stage, int r)
+                                               const OpFmt& f, uint8_t* stage, int r)
 {
     constexpr int CPW = 32 / B;
     constexpr int SPW = CPW > 8 ? 16 : (CPW > 4 ? 8 : 4);
@@ -407,7 +488,7 @@ __device__ __forceinline__ void walk_row_slots(const Src& src, const typename Sr
             ok |= (p ? 1u : 0u) << i;
             src.advance(cur, 1);
         }
-        store_slot_words<B, CH>(wv, ok, lim, lut, stage, r, c0 * SPW / 16);
+        store_slot_words<B, CH>(wv, ok, lim, f, stage, r, c0 * SPW / 16);
     }
 }
 
@@ -423,12 +504,12 @@ __device__ __forceinline__ void walk_row_kblock(const Src& src, const typename S
 {
     if (f.spw) {
         switch (f.b) {
-        case 2: walk_row_slots<2>(src, row, k0, f, lut, stage, r); return;
-        case 3: walk_row_slots<3>(src, row, k0, f, lut, stage, r); return;
-        case 5: walk_row_slots<5>(src, row, k0, f, lut, stage, r); return;
-        case 6: walk_row_slots<6>(src, row, k0, f, lut, stage, r); return;
-        case 7: walk_row_slots<7>(src, row, k0, f, lut, stage, r); return;
-        default: walk_row_slots<8>(src, row, k0, f, lut, stage, r); return;
+        case 2: walk_row_slots<2>(src, row, k0, f, stage, r); return;
+        case 3: walk_row_slots<3>(src, row, k0, f, stage, r); return;
+        case 5: walk_row_slots<5>(src, row, k0, f, stage, r); return;
+        case 6: walk_row_slots<6>(src, row, k0, f, stage, r); return;
+        case 7: walk_row_slots<7>(src, row, k0, f, stage, r); return;
+        default: walk_row_slots<8>(src, row, k0, f, stage, r); return;
         }
     }
     if (f.b == 4) {
@@ -600,52 +681,45 @@ constexpr int kWsThreads = (kWsProdWarp0 + kWsProdWarps) * 32;   // 512: 4 warps
 constexpr int kWsMaxStages = 8;
 
 
-// Decode one 128-code K-block slice (16 words, four 16-byte pieces) of a
-// b = 4 row and store its 8 units to a swizzled stage row.  The loads of
-// all four pieces are issued before any decode.
-// Pieces outside the operand (rows past M or N, out-of-image taps, words
-// past K) are filled with the zero code -- the all-zero bit pattern is not
-// zero in this format (it is the value 1).
-template <class Src>
-__device__ __forceinline__ void load_row_b4(const Src& src, const typename Src::Row& row,
-                                            const typename Src::Cursor (&cur)[4], int64_t kw0, int64_t K,
-                                            uint32_t zero_word, uint4 (&v)[4])
+// Calls fn with the width b as a compile-time constant.
+template <int V> struct IntC { static constexpr int value = V; };
+template <class F>
+__device__ __forceinline__ void with_width(int b, const F& fn)
 {
-#pragma unroll
-    for (int pc = 0; pc < 4; pc++) {
-        const int64_t kk0 = (kw0 + 4 * pc) * 8;       // first code of the piece
-        const uint32_t* p = (kk0 < K) ? src.at(row, cur[pc]) : nullptr;
-        v[pc] = p ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(zero_word, zero_word, zero_word, zero_word);
+    switch (b) {
+    case 2: fn(IntC<2>()); break;
+    case 3: fn(IntC<3>()); break;
+    case 4: fn(IntC<4>()); break;
+    case 5: fn(IntC<5>()); break;
+    case 6: fn(IntC<6>()); break;
+    case 7: fn(IntC<7>()); break;
+    default: fn(IntC<8>()); break;
     }
 }
 
-__device__ __forceinline__ void store_row_b4(uint8_t* stage, int r, const uint4 (&v)[4], int64_t kw0, int64_t K,
-                                             const OpFmt& f)
+// Rows of 16-byte pieces: whole-byte 4-bit codes, or word slots, of a source
+// whose pieces are contiguous.
+template <class Src>
+__device__ __forceinline__ bool by_pieces(const Src& src, const OpFmt& f)
 {
-    const bool tail = (kw0 + 16) * 8 > K;             // only the last K-block can reach past K
-#pragma unroll
-    for (int pc = 0; pc < 4; pc++) {
-        const uint32_t w[4] = {v[pc].x, v[pc].y, v[pc].z, v[pc].w};
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            uint32_t o0, o1, o2, o3;
-            decode_word_b4(w[2 * h], f.k, f.ew, o0, o1);
-            decode_word_b4(w[2 * h + 1], f.k, f.ew, o2, o3);
-            const int64_t wi = kw0 + 4 * pc + 2 * h;  // word index of w[2h]
-            if (tail && (wi + 2) * 8 > K) {           // K tail: zero the codes past K
-                uint32_t ml, mh;
-                int va = (int)(K - wi * 8);
-                va = va < 0 ? 0 : (va > 8 ? 8 : va);
-                tail_masks(va, ml, mh);
-                o0 &= ml; o1 &= mh;
-                int vb = (int)(K - (wi + 1) * 8);
-                vb = vb < 0 ? 0 : (vb > 8 ? 8 : vb);
-                tail_masks(vb, ml, mh);
-                o2 &= ml; o3 &= mh;
-            }
-            *reinterpret_cast<uint4*>(stage + swz(r, 2 * pc + h)) = make_uint4(o0, o1, o2, o3);
-        }
-    }
+    return f.planes == 1 && src.linear() && src.vec4() && (f.b == 4 || f.spw);
+}
+
+// Rows 32 q .. of K-block kb of plain (or filter) rows from row n0, by one
+// warp.  K: the kernel's K (4-bit codes); word slots count codes to korig.
+template <int B>
+__device__ __noinline__ void fill_rows_q(const RowsSrc src, int64_t n0, int nrows, int kb, int q, int64_t K, const OpFmt f,
+                                         uint8_t* stage, int lane)
+{
+    using S = SlotFmt<B>;
+    const int64_t w0 = (int64_t)kb * S::NW + 4 * (lane % S::LPR);
+    const int64_t left = (B == 4 ? K : f.korig) - w0 * S::CPW;
+    const int64_t r0 = n0 + q * 32 + lane / S::LPR;
+    const RowsSrc::Cursor c = src.cursor(w0);
+    const uint32_t* p = src.base + r0 * src.ld + c.w;
+    fill_q<B>(stage, q, nrows, left, f.k, f.ew, lane, [&](int u) -> const uint32_t* {
+        return r0 + u * S::RPI < src.rows ? p + (int64_t)(u * S::RPI) * src.ld : nullptr;
+    });
 }
 
 // Epilogue of one 16-column chunk for outputs other than the lean 4-bit
@@ -743,34 +817,29 @@ struct EpiCellsSmem {
     int bad;
 };
 
-template <int OB, class RowMap>
-__device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr, EpiCellsSmem& sm, const RowMap& rows,
-                                          int64_t my_tiles, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
-                                          float acc_scale, uint64_t* tfull, uint64_t* tempty, volatile int* err,
-                                          int warp, int lane)
+// The tiles of epi_cells once the table is known.  RES: a residual; CH:
+// per-channel scale and/or bias; CELLS: the cell table is usable (else the
+// bisection over thr).  All three are fixed outside the loop, so a pass has no
+// branch and its columns' chains of loads and compares interleave: the
+// epilogue warps are two to a scheduler and bound by latency, not by issue
+// (4096^3, 6-bit: 111 us for the GEMM kernel with these tests per column,
+// 57 us without).
+template <int OB, bool RES, bool CH, bool CELLS, class RowMap>
+__device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float* thr, const EpiCellsSmem& sm, int h0,
+                                                int hmax, const RowMap& rows, int64_t my_tiles, int64_t n0, int64_t N,
+                                                int BN, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
+                                                uint64_t* tempty, volatile int* err, int warp, int lane)
 {
     constexpr int CPW = 32 / OB;
     constexpr int WPC = OB == 3 ? 2 : 4;              // words per pass
     constexpr int CC = WPC * CPW;                     // columns per pass: 20 or 24
-    constexpr int kThreads = kWsEpiWarps * 32;
-    const uint2* const cells = sm.cells;
-    const float* const resimg = sm.resimg;
-    const int t = warp * 32 + lane;
-    int h0, hmax;
-    bool bad;
-    if (t == 0) sm.bad = 0;
-    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-    bool by_cells = fill_cells<OB>(sm.cells, kEpiCells, h0, hmax, thr, ep.out, t, kThreads, bad);
-    if (bad) sm.bad = 1;
-    if (ep.residual && t < (1 << OB)) sm.resimg[t] = code_image_f((uint32_t)t, OB, ep.res_k);
-    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-    by_cells = by_cells && *const_cast<volatile int*>(&sm.bad) == 0;
-
+    constexpr uint32_t CMASK = (1u << OB) - 1u;
     const bool dq = ep.alpha_a_dev && ep.alpha_b_dev;
     const float dqs = dq ? __fmul_rn(__ldg(ep.alpha_a_dev), __ldg(ep.alpha_b_dev)) * ep.dq_pow2 : 1.0f;
     const float sc0 = dq ? __fmul_rn(ep.scale0, dqs) : ep.scale0;
-    const float bias0 = ep.bias0;
-    const int act = ep.act;
+    const float bias0 = ep.bias0, res_scale = ep.res_scale;
+    const bool acted = ep.act != ESB_ACT_NONE;
+    const float act_hi = ep.act == ESB_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
     const int sh = cell_shift(ep.out.k);
     const uint32_t amask = ep.out.is_signed ? 0x7fffffffu : 0xffffffffu;
     const uint32_t zc = ep.out.zero_code;
@@ -785,7 +854,7 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
     const int p_lo = (warp >> 2) ? pmid : 0, p_hi = (warp >> 2) ? passes : pmid;
     const int64_t w00 = n0 / CPW;
     const bool vec = WPC == 4 ? ep.codes_vec == 4 && (w00 & 3) == 0 : ep.codes_vec >= 2 && (w00 & 1) == 0;
-    const bool rvec = ep.residual && (reinterpret_cast<uintptr_t>(ep.residual) & 15u) == 0 && (ep.res_ld & 3) == 0 &&
+    const bool rvec = RES && (reinterpret_cast<uintptr_t>(ep.residual) & 15u) == 0 && (ep.res_ld & 3) == 0 &&
                       (w00 & (WPC - 1)) == 0;
     const bool tail_words = n0 + BN >= N && (warp >> 2) == 1;   // zero-code words past the outputs
     const int row = quarter * 32 + lane;
@@ -808,20 +877,22 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
             const uint32_t ta = taddr + (uint32_t)(ps * CC);
             const int64_t wc = w00 + ps * WPC;
             uint32_t rw[WPC];
-            const bool whole = (ps + 1) * CC <= live;
-            if (ep.residual && mrow) {
+            if (RES) {
                 const uint32_t* rp = ep.residual + m * ep.res_ld + wc;
-                if (rvec) {
-                    if (WPC == 4) {
+#pragma unroll
+                for (int w = 0; w < WPC; w++) rw[w] = 0u;
+                if (mrow) {
+                    if (rvec && WPC == 4) {
                         const uint4 q = __ldg(reinterpret_cast<const uint4*>(rp));
                         rw[0] = q.x; rw[1] = q.y; rw[WPC - 2] = q.z; rw[WPC - 1] = q.w;
-                    } else {
+                    } else if (rvec) {
                         const uint2 q = __ldg(reinterpret_cast<const uint2*>(rp));
                         rw[0] = q.x; rw[1] = q.y;
-                    }
-                } else {
+                    } else {
 #pragma unroll
-                    for (int w = 0; w < WPC; w++) rw[w] = (ps * CC + w * CPW < live) ? __ldg(rp + w) : 0u;
+                        for (int w = 0; w < WPC; w++)
+                            if (ps * CC + w * CPW < live) rw[w] = __ldg(rp + w);
+                    }
                 }
             }
             if (ps * CC + CC <= BN) {
@@ -846,19 +917,29 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
                 for (int j = 0; j < CPW; j++) {
                     const int e = w * CPW + j;
                     float sc = sc0, bi = bias0;
-                    if (ep.scale || ep.bias) {
+                    if (CH) {
                         const int64_t n = n0 + ps * CC + e;
                         const int64_t nn = n < N ? n : N - 1;
                         if (ep.scale) { sc = __ldg(ep.scale + nn); if (dq) sc = __fmul_rn(sc, dqs); }
                         if (ep.bias) bi = __ldg(ep.bias + nn);
                     }
                     float y = __fmaf_rn(sc, __uint_as_float(r[e]) * acc_scale, bi);
-                    if (ep.residual) y = __fmaf_rn(ep.res_scale, resimg[(rw[w] >> (OB * j)) & ((1u << OB) - 1u)], y);
-                    y = apply_act(y, act);
-                    uint32_t c = by_cells ? project_by_cells<OB>(y, cells, h0, hmax, sh, amask)
-                                          : project_by_table(y, thr, ep.out);
-                    if (!whole && ps * CC + e >= live) c = zc;
+                    if (RES) y = __fmaf_rn(res_scale, sm.resimg[(rw[w] >> (OB * j)) & CMASK], y);
+                    const float ya = fminf(fmaxf(y, 0.0f), act_hi);   // NaN -> 0, as apply_act
+                    y = acted ? ya : y;
+                    const uint32_t c = CELLS ? project_by_cells<OB>(y, sm.cells, h0, hmax, sh, amask)
+                                             : project_by_table(y, thr, ep.out);
                     word[w] |= c << (OB * j);
+                }
+            }
+            if ((ps + 1) * CC > live) {               // columns past N: the zero code
+#pragma unroll
+                for (int w = 0; w < WPC; w++) {
+                    const int lw = live - ps * CC - w * CPW;          // live codes of this word
+                    if (lw < CPW) {
+                        const uint32_t keep = lw > 0 ? (1u << (OB * lw)) - 1u : 0u;
+                        word[w] = (word[w] & keep) | (zero_word & ~keep);
+                    }
                 }
             }
             if (mrow) {
@@ -876,6 +957,35 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
         }
         if (tail_words && mrow)
             for (int64_t wq = w00 + (int64_t)passes * WPC; wq < ep.ldo; wq++) crow[wq] = zero_word;
+    }
+}
+
+template <int OB, class RowMap>
+__device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr, EpiCellsSmem& sm, const RowMap& rows,
+                                          int64_t my_tiles, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
+                                          float acc_scale, uint64_t* tfull, uint64_t* tempty, volatile int* err,
+                                          int warp, int lane)
+{
+    constexpr int kThreads = kWsEpiWarps * 32;
+    const int t = warp * 32 + lane;
+    int h0, hmax;
+    bool bad;
+    if (t == 0) sm.bad = 0;
+    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+    const bool fits = fill_cells<OB>(sm.cells, kEpiCells, h0, hmax, thr, ep.out, t, kThreads, bad);
+    if (bad) sm.bad = 1;
+    if (ep.residual && t < (1 << OB)) sm.resimg[t] = code_image_f((uint32_t)t, OB, ep.res_k);
+    asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+    const bool ch = ep.scale || ep.bias, res = ep.residual != nullptr;
+    if (!fits || *const_cast<volatile int*>(&sm.bad) != 0) {
+        if (res) epi_cells_tiles<OB, true, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+    } else if (ch) {
+        if (res) epi_cells_tiles<OB, true, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+    } else {
+        if (res) epi_cells_tiles<OB, true, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     }
 }
 
@@ -900,23 +1010,19 @@ template <bool B4>
 __device__ __forceinline__ void ws_decode_b(const RowsSrc& srcB, int64_t n0, int64_t K, const OpFmt& fb, int BN,
                                             int nkb, uint8_t* sB, int t, int nthreads, const uint8_t* lutb = nullptr)
 {
-    if (B4 || (fb.b == 4 && fb.planes == 1 && srcB.linear() && srcB.vec4())) {
-        // one row chunk per thread and pass (compact: this code runs cold,
-        // once per CTA, on the path to the first MMA)
-        const uint32_t zw = fmt_zero_code(4, fb.k) * 0x11111111u;
-        const int rows_total = nkb * BN;
+    if (B4 || by_pieces(srcB, fb)) {
+        // 32 rows of one K-block per warp and step
+        const int qn = (BN + 31) >> 5;
+        const int nwarp = nthreads >> 5, lane = t & 31;
+        auto go = [&](auto width) {
 #pragma unroll 1
-        for (int pr = t; pr < rows_total; pr += nthreads) {
-            const int kb = pr / BN, r = pr - kb * BN;
-            const RowsSrc::Row row = srcB.row(n0 + r);
-            const int64_t kw0 = (int64_t)kb * 16;
-            RowsSrc::Cursor cur[4];
-#pragma unroll
-            for (int pc = 0; pc < 4; pc++) cur[pc] = srcB.cursor(kw0 + 4 * pc);
-            uint4 v[4];
-            load_row_b4(srcB, row, cur, kw0, K, zw, v);
-            store_row_b4(sB + kb * BN * kBK, r, v, kw0, K, fb);
-        }
+            for (int u = t >> 5; u < nkb * qn; u += nwarp) {
+                const int kb = u / qn, q = u - kb * qn;
+                fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sB + kb * BN * kBK, lane);
+            }
+        };
+        if (B4) go(IntC<4>());
+        else with_width(fb.b, go);
     } else if (lutb && fb.planes == 1 && srcB.linear()) {
         // other widths: one word walk per (K-block, row)
 #pragma unroll 1
