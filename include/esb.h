@@ -502,7 +502,9 @@ enum {
                                       each filter tap a shifted view (tcgen05) */
     ESB_CONV_KERNEL_IM2COL = 2,    /* implicit im2col, filters resident in shared memory */
     ESB_CONV_KERNEL_STREAMED = 3,  /* implicit im2col, filters streamed per K-block */
-    ESB_CONV_KERNEL_DEPTHWISE = 4  /* groups == c, CUDA cores */
+    ESB_CONV_KERNEL_DEPTHWISE = 4, /* groups == c, CUDA cores */
+    ESB_CONV_KERNEL_STEM = 5       /* stride 2 or 4, up to 4 channels: decoded input
+                                      rows, taps are shifted views (tcgen05) */
 };
 
 /* Which of the kernels above esb_conv2d_nhwc launches for geometry d, X
@@ -512,7 +514,7 @@ enum {
  * needs 4-bit codes of the same layout on both sides.  The choice depends only on these and on
  * the device's shared memory (queried on the current device); results are
  * identical whichever kernel runs.  Setting ESB_CONV_IM2COL=1 in the
- * environment before the first call disables the halo kernel.
+ * environment before the first call disables the halo and stem kernels.
  *   kernel [host] receives one ESB_CONV_KERNEL_* value
  * Errors: INVALID_ARG (bad geometry, or the call would be rejected),
  * CUDA (no device). */

@@ -1,0 +1,381 @@
+// esb_conv_stem.cu -- strided ESB convolution of images with up to 4
+// channels (the first layer of a network: 7x7/2, 3x3/2, 11x11/4; Sec. IV-B).
+//
+// A pixel's codes decode to 4 E4M3 bytes, so the taps of one filter row are
+// 4 S contiguous bytes of a decoded input row, and im2col is only a matter of
+// where a row of the MMA operand starts: output q reads from byte 4 (stride q
+// - pad).  That is 16-byte aligned, as the K-major no-swizzle layout needs,
+// for every q = phi i + f of one residue f modulo phi = 4 / stride.  So each
+// input row is decoded once into phi copies, copy f shifted by stride f
+// pixels, U 16-byte units apart; tile row f U + i is output phi i + f of one
+// output row, its K chunk g (4 taps) unit f U + i + g, and the whole operand of
+// filter row r is that decoded row seen through a descriptor with SBO = 128
+// and LBO = 16 bytes (the chunks overlap).  K = R rows x G chunks, G even; the
+// filter's bytes past S taps or past the channels are zero.  Tile rows with i
+// past the segment's outputs compute on neighbouring units and are not stored.
+//
+// A CTA walks consecutive output rows, and decoded rows live in a ring of NR
+// slots: the next output row of the same image needs only `stride` new input
+// rows.  Each row has its own full and empty barrier; the MMA warp's commits
+// free the rows that the next tile does not use.
+//
+// 224 x 224 x 3, 7x7/2 -> 64, batch 64, 4-bit: 372 us on the im2col kernel
+// (49 single words gathered and decoded per output pixel, 5 of the 8 K slots
+// of each word padding), 109 us here, 2.3 us per tile in the issuing thread.
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "esb_tc.cuh"
+
+namespace esb {
+
+namespace {
+
+constexpr int kStemMaxRing = 24;
+
+struct StemGeom {
+    const uint32_t* X;
+    int ldx, H, W, P, Q, R, S, C, stride, pad;
+    int phi;             // output residues per 16-byte step: 4 / stride
+    int G;               // 16-byte chunks (4 taps) per filter row, even
+    int Ui;              // outputs of one residue per segment
+    int U;               // units of one copy: Ui + G - 1
+    int nseg;            // column segments per output row
+    int pitch;           // bytes of a ring slot: 128 + G - 1 units
+    int NR;              // ring slots
+};
+
+// Input pixel word -> its (up to 4) codes as E4M3 bytes, channel order.
+template <int B>
+__device__ __forceinline__ uint32_t stem_pixel(uint32_t w, int k)
+{
+    return e4m3_4<B>(spread4<B>(rot_word<B>(w, k)), k);
+}
+
+// One input row into a ring slot, by one warp: lane l takes pixel positions
+// l, l + 32, ... (every load in flight before the first store), each stored
+// to its place in every copy.
+template <int B>
+__device__ __forceinline__ void stem_row(const StemGeom& g, int n, int h, int x0, uint8_t* slot, int lane, int k,
+                                         uint32_t cmask)
+{
+    constexpr int UN = 8;
+    const int npos = 4 * g.U + g.stride * (g.phi - 1);
+    const bool hin = (unsigned)h < (unsigned)g.H;
+    const uint32_t* xr = g.X + ((int64_t)n * g.H + (hin ? h : 0)) * g.W * g.ldx;
+#pragma unroll 1
+    for (int j0 = 0; j0 < npos; j0 += 32 * UN) {
+        uint32_t w[UN];
+        uint32_t ok = 0u;
+#pragma unroll
+        for (int u = 0; u < UN; u++) {
+            const int x = x0 + j0 + 32 * u + lane;
+            const bool in = hin && (unsigned)x < (unsigned)g.W;
+            w[u] = in ? __ldg(xr + (int64_t)x * g.ldx) : 0u;
+            ok |= (in ? 1u : 0u) << u;
+        }
+#pragma unroll
+        for (int u = 0; u < UN; u++) {
+            const int j = j0 + 32 * u + lane;
+            const uint32_t v = ((ok >> u) & 1u) ? stem_pixel<B>(w[u], k) & cmask : 0u;
+            for (int f = 0; f < g.phi; f++) {
+                const int jf = j - g.stride * f;
+                if ((unsigned)jf < (unsigned)(4 * g.U))
+                    *reinterpret_cast<uint32_t*>(slot + f * g.U * 16 + jf * 4) = v;
+            }
+        }
+    }
+}
+
+// Filter chunk c (row r = c / G, taps 4 (c % G) ..) of output channel row n.
+template <int B>
+__device__ __forceinline__ void stem_filter(const StemGeom& g, const uint32_t* W, int64_t ldw, int64_t n, int64_t N, int c, int k,
+                                            uint32_t cmask, uint8_t* sB, int BN, int row)
+{
+    uint32_t o[4] = {0u, 0u, 0u, 0u};
+    const int r = c / g.G, s0 = (c - r * g.G) * 4;
+    if (n < N && r < g.R) {
+        const uint32_t* p = W + ((n * g.R + r) * g.S + s0) * ldw;
+#pragma unroll
+        for (int t = 0; t < 4; t++)
+            if (s0 + t < g.S) o[t] = stem_pixel<B>(__ldg(p + t * ldw), k) & cmask;
+    }
+    *reinterpret_cast<uint4*>(sB + (c >> 3) * BN * kBK + swz(row, c & 7)) = make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+}  // namespace
+
+template <bool FAST, bool GEN>
+__global__ void __launch_bounds__(kWsThreads, 1)
+esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpFmt fa, OpFmt fb, int BN, int nkb, int n_tiles,
+                     int m_tiles, float acc_scale, EpiParams ep)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* sB = smem;                                        // nkb blocks of BN x 128 bytes (SW128)
+    uint8_t* sA = sB + nkb * BN * kBK;                         // NR decoded rows
+    float* thr = reinterpret_cast<float*>(sA + g.NR * g.pitch);
+    uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
+    uint64_t* empty = full + kStemMaxRing;
+    uint64_t* tfull = empty + kStemMaxRing;
+    uint64_t* tempty = tfull + 2;
+    uint64_t* drain = tempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int tid = threadIdx.x;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int n_tile = (int)(blockIdx.x % n_tiles);
+    const int cta = blockIdx.x / n_tiles, ctas = gridDim.x / n_tiles;
+    const int64_t n0 = (int64_t)n_tile * BN;
+    // consecutive tiles: (image, segment, output row), the row fastest
+    const int t_lo = (int)((int64_t)m_tiles * cta / ctas), t_hi = (int)((int64_t)m_tiles * (cta + 1) / ctas);
+    uint32_t tmem_cols = 32;
+    while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
+    const int half_cols = BN / 2;
+    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
+    const int epi_warps = split ? 8 : 4;
+    // the layout above must fit the dynamic allocation (uniform for the CTA)
+    if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
+        if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
+        return;
+    }
+    if (tid == 0) {
+        for (int s = 0; s < g.NR; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int a = 0; a < 2; a++) {
+            mbar_init(&tfull[a], 1);
+            mbar_init(&tempty[a], epi_warps);
+        }
+        mbar_init(drain, 1);
+        *err = 0;
+        fence_mbar_init();
+    }
+    ws_alloc(warp, tmem_slot, tmem_cols);
+    __syncthreads();                                  // barriers initialised, TMEM allocated
+    griddep_wait();                                   // X, W and the alphas may come from the previous launch
+
+    // padding slots of a pixel's word must not count even if they are not zero codes
+    const uint32_t cmask = g.C >= 4 ? 0xffffffffu : (1u << (8 * g.C)) - 1u;
+    const int nnew = g.stride < g.R ? g.stride : g.R; // rows a following output row adds
+    constexpr int kSetup = kWsProdWarp0 * 32;
+    if (warp < kWsProdWarp0) {
+        // filters: one 16-byte chunk per thread and pass
+        with_width(fb.b, [&](auto width) {
+            for (int i = tid; i < nkb * 8 * BN; i += kSetup) {
+                const int row = i >> 3, c = i & 7;
+                const int kb = row / BN;
+                stem_filter<decltype(width)::value>(g, Wt, ldw, n0 + (row - kb * BN), N, kb * 8 + c, fb.k, cmask, sB, BN,
+                                                    row - kb * BN);
+            }
+        });
+        fence_proxy_async_smem();
+        if (warp == kWsMmaWarp) {
+            asm volatile("bar.sync 1, %0;" ::"n"(kSetup) : "memory");
+        } else {
+            asm volatile("bar.arrive 1, %0;" ::"n"(kSetup) : "memory");
+            ws_thresholds(thr, ep, warp, lane);
+        }
+    }
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp >= kWsProdWarp0) {
+        // ---------------------------------------------- row decoders: row rho by warp rho % 7
+        const int pw = warp - kWsProdWarp0;
+        with_width(fa.b, [&](auto width) {
+            int turn = 0, s = 0;                      // rho % kWsProdWarps, rho % NR
+            uint32_t ph = 0u;
+            for (int T = t_lo; T < t_hi && !*err; T++) {
+                const int strip = T / g.P, p = T - strip * g.P;
+                const int n = strip / g.nseg, seg = strip - n * g.nseg;
+                const int x0 = g.stride * g.phi * seg * g.Ui - g.pad;
+                const int r0 = (T == t_lo || p == 0) ? 0 : g.R - nnew;
+                for (int r = r0; r < g.R; r++) {
+                    if (turn == pw) {
+                        if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
+                        stem_row<decltype(width)::value>(g, n, p * g.stride - g.pad + r, x0, sA + s * g.pitch, lane, fa.k, cmask);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&full[s]);
+                    }
+                    if (++turn == kWsProdWarps) turn = 0;
+                    if (++s == g.NR) { s = 0; ph ^= 1u; }
+                }
+            }
+        });
+    } else if (warp == kWsMmaWarp) {
+        // ---------------------------------------------- MMA issue
+        if (lane == 0) {
+            const uint32_t idesc = idesc_e4m3_f32(BN);
+            const uint64_t bd0 = smem_desc_sw128(smem_u32(sB));
+            const uint32_t a_base = smem_u32(sA);
+            int s = 0, base = 0;                      // next row to arrive; the tile's first row (ring slots)
+            uint32_t ph = 0u;
+            for (int T = t_lo; T < t_hi && !*err; T++) {
+                const int i = T - t_lo, a = i & 1;
+                const int p = T % g.P;
+                if (!wait_or_abort(&tempty[a], (uint32_t)((i >> 1) & 1) ^ 1u, err)) { *err = 1; break; }
+                const int add = (i == 0 || p == 0) ? g.R : nnew;
+                if (add == g.R) base = s;
+                bool ok = true;
+                for (int j = 0; j < add && ok; j++) {
+                    ok = wait_or_abort(&full[s], ph, err);
+                    if (++s == g.NR) { s = 0; ph ^= 1u; }
+                }
+                if (!ok) { *err = 1; break; }
+                tc_fence_after();
+                const uint32_t d = tmem_base + (uint32_t)(a * BN);
+                uint32_t acc = 0u;
+                int slot = base, kq = 0;
+                for (int r = 0; r < g.R; r++) {
+                    const uint64_t ad = smem_desc_noswz(a_base + (uint32_t)(slot * g.pitch), 16u, 128u);
+                    for (int j = 0; j < g.G >> 1; j++, kq++) {
+                        mma_f8f6f4(d, ad + (uint64_t)(2 * j),
+                                   bd0 + (uint64_t)((kq >> 2) * ((BN * kBK) >> 4) + (kq & 3) * 2), idesc, acc);
+                        acc = 1u;
+                    }
+                    if (++slot == g.NR) slot = 0;
+                }
+                // rows the next tile does not use (all of them at the end of an image's segment)
+                const int rel = (T + 1 == t_hi || p + 1 == g.P) ? g.R : nnew;
+                for (int j = 0; j < rel; j++) {
+                    mma_commit(&empty[base]);
+                    if (++base == g.NR) base = 0;
+                }
+                mma_commit(&tfull[a]);
+            }
+            ws_drain(drain, err);
+        }
+    } else if (warp < epi_warps) {
+        // ---------------------------------------------- epilogue
+        const int row = (warp & 3) * 32 + lane;
+        const int f = row / g.U, i = row - f * g.U;
+        const bool live = f < g.phi && i < g.Ui;
+        const int q0 = g.phi * i + f, P = g.P, Q = g.Q, nseg = g.nseg, qstep = g.phi * g.Ui;
+        auto rows = [=](int64_t ti, int, int64_t& m) -> bool {
+            const int T = t_lo + (int)ti;
+            const int strip = T / P, p = T - strip * P;
+            const int n = strip / nseg, q = (strip - n * nseg) * qstep + q0;
+            m = ((int64_t)n * P + p) * Q + q;
+            return live && q < Q;
+        };
+        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty,
+                               err, warp, lane);
+    }
+
+    __syncthreads();
+    if (*err && tid == 0) record_status(ep.status, ESB_ERR_TIMEOUT);
+    if (warp == kWsMmaWarp) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, tmem_cols);
+    }
+}
+
+// ------------------------------------------------------------- host side
+
+typedef void (*StemKernel)(StemGeom, const uint32_t*, int64_t, int64_t, OpFmt, OpFmt, int, int, int, int, float, EpiParams);
+static const StemKernel kStemKernels[3] = {esb_conv_stem_kernel<false, false>, esb_conv_stem_kernel<true, false>,
+                                           esb_conv_stem_kernel<false, true>};
+
+static int stem_static_smem(cudaError_t* err)
+{
+    static int v = -1;
+    if (v < 0) {
+        size_t m = 0;
+        for (StemKernel k : kStemKernels) {
+            cudaFuncAttributes a;
+            *err = cudaFuncGetAttributes(&a, k);
+            if (*err != cudaSuccess) return -1;
+            if (a.sharedSizeBytes > m) m = a.sharedSizeBytes;
+        }
+        v = (int)m;
+    }
+    return v;
+}
+
+struct StemPlan {
+    StemGeom g;
+    int BN, nkb;
+    int64_t smem;
+};
+
+// Up to 4 channels, stride 2 or 4 (stride 1 has the halo kernel), whole-byte
+// formats, and output rows that fill enough of the 128 tile rows: a tile here
+// takes about an eighth of an im2col tile's time, so a fifth of its rows pays.
+static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int bn0, StemPlan* sp,
+                      cudaError_t* err)
+{
+    *err = cudaSuccess;
+    if (d.c > 4 || (d.stride != 2 && d.stride != 4) || fmt_needs_split(bx, kx) || fmt_needs_split(bw, kw) || d.r > 16 || d.s > 16 ||
+        ldx > (1 << 20) || bn0 <= 0)
+        return false;
+    StemGeom& g = sp->g;
+    g.X = nullptr;
+    g.ldx = (int)ldx; g.H = d.h; g.W = d.w; g.P = P; g.Q = Q; g.R = d.r; g.S = d.s; g.C = d.c; g.stride = d.stride; g.pad = d.pad;
+    g.phi = 4 / d.stride;
+    g.G = 2 * ((d.s + 7) / 8);
+    const int per = (Q + g.phi - 1) / g.phi;                       // outputs of one residue in a row
+    const int umax = kBM / g.phi;
+    g.nseg = (per + umax - g.G) / (umax - g.G + 1);
+    g.Ui = (per + g.nseg - 1) / g.nseg;
+    g.U = g.Ui + g.G - 1;
+    if ((double)Q / ((double)g.nseg * kBM) < 0.2 || (int64_t)d.n * P * g.nseg >= (1ll << 30)) return false;
+    g.pitch = (kBM + g.G - 1) * 16;
+    const int st = stem_static_smem(err);
+    if (st < 0) return false;
+    const int64_t maxs = max_dyn_smem() - st;
+    sp->BN = bn0;
+    sp->nkb = (d.r * g.G * 16 + kBK - 1) / kBK;
+    const int64_t fixed = 1024 + (int64_t)sp->nkb * bn0 * kBK + 4 * 128 + (2 * kStemMaxRing + 5) * 8 + 64;
+    int64_t nr = (maxs - fixed) / g.pitch;
+    if (nr > kStemMaxRing) nr = kStemMaxRing;
+    if (nr < d.r + 2 * d.stride) return false;                     // a tile's rows and two more output rows' worth
+    g.NR = (int)nr;
+    sp->smem = fixed + nr * g.pitch;
+    return true;
+}
+
+bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int out_cpw)
+{
+    StemPlan sp;
+    cudaError_t e;
+    return stem_plan(d, P, Q, ldx, bx, kx, bw, kw, pick_bn(d.cout, out_cpw), &sp, &e);
+}
+
+bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa, const uint32_t* W,
+                      int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st, cudaError_t* err)
+{
+    StemPlan sp;
+    if (!stem_plan(d, P, Q, ldx, fa.b, fa.k, fb.b, fb.k, BN, &sp, err)) return *err != cudaSuccess;
+    sp.g.X = X;
+    static bool configured = false;
+    if (!configured) {
+        for (StemKernel k : kStemKernels) {
+            *err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_smem() - stem_static_smem(err));
+            if (*err != cudaSuccess) return true;
+        }
+        configured = true;
+    }
+    const int64_t N = d.cout;
+    const int n_tiles = (int)((N + BN - 1) / BN);
+    const int m_tiles = d.n * P * sp.g.nseg;
+    int64_t per_n = device_sm_count() / n_tiles;
+    if (per_n < 1) per_n = 1;
+    if (per_n > m_tiles) per_n = m_tiles;
+    const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
+    // the specialised epilogue, as in the halo convolution
+    const int half = BN / 2;
+    const bool split = (half % 16 == 0) && (half % ep.out_cpw == 0);
+    const bool fast = ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
+                      ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE) &&
+                      (split ? half : BN) % 32 == 0;
+    const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
+    *err = launch_pdl(kStemKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
+                      (size_t)sp.smem, st, sp.g, W, ldw, N, fa, fb, BN, sp.nkb, n_tiles, m_tiles, acc_scale, ep);
+    return true;
+}
+
+}  // namespace esb

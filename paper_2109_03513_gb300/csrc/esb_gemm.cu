@@ -17,7 +17,7 @@
 // scales it back to the exact int32 sum.
 //
 // Two kernels here share the decode and the epilogue (esb_tc.cuh) with the
-// halo convolution of esb_conv_halo.cu:
+// convolutions of esb_conv_halo.cu and esb_conv_stem.cu:
 //  * esb_gemm_ws_kernel: persistent, warp-specialised.  The CTA decodes
 //    its N-tile of B once into shared memory when it fits beside three A
 //    stages (B resident), else each stage carries the B block of its
@@ -1009,6 +1009,8 @@ cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t*
         if (const int64_t Ks = plan_slots(fa, fb, words * fa.cpw, words)) Kx = Ks;
     }
     cudaError_t e = cudaSuccess;
+    if (!conv_force_im2col() && launch_conv_stem(d, P, Q, X, ldx, make_opfmt(bx, kx), W, ldw, make_opfmt(bw, kw), BN, ep, st, &e))
+        return e;
     if (Kx > 0 && !conv_force_im2col() && fa.planes == 1 && b.kp == 0 &&
         launch_conv_halo(d, P, Q, X, ldx, fa, W, ldw, fb, BN, ep, st, &e))
         return e;
@@ -1030,6 +1032,7 @@ int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx
         const int64_t words = (int64_t)d.r * d.s * kwd;
         if (const int64_t Ks = plan_slots(fa, fb, words * fa.cpw, words)) Kx = Ks;
     }
+    if (!conv_force_im2col() && conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, cpw)) return ESB_CONV_KERNEL_STEM;
     if (Kx > 0 && !conv_force_im2col() && same_layout && conv_halo_ok(d, P, Q, ldx, bx, kx, cpw))
         return ESB_CONV_KERNEL_HALO;
     cudaError_t e = cudaSuccess;

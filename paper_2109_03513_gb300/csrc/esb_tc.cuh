@@ -1449,6 +1449,12 @@ int max_dyn_smem();                           // opt-in shared memory per block
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
 float acc_fma_limit(int64_t K, int ba, int ka, int bb, int kb);   // FMA-pipe requantisation bound (esb_gemm.cu)
 
+// Strided convolution of up to 4 channels (esb_conv_stem.cu); the same
+// contract: false when the shape does not suit it.
+bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int out_cpw);
+bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa, const uint32_t* W,
+                      int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st, cudaError_t* err);
+
 // Stride-1 convolution from a decoded input halo (esb_conv_halo.cu).  Returns
 // false, launching nothing, when the shape does not suit it (stride != 1,
 // A not 4-bit, rows wider than 128 - pad, too little of the tile used, or

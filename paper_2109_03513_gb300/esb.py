@@ -529,6 +529,7 @@ def esb_conv2d_nhwc(X: torch.Tensor, fx: Fmt, W: torch.Tensor, fw: Fmt, n: int, 
 
 
 ESB_CONV_KERNEL_HALO, ESB_CONV_KERNEL_IM2COL, ESB_CONV_KERNEL_STREAMED, ESB_CONV_KERNEL_DEPTHWISE = 1, 2, 3, 4
+ESB_CONV_KERNEL_STEM = 5
 
 
 def esb_conv2d_kernel(n: int, h: int, w: int, c: int, cout: int, r: int, s: int, stride: int, pad: int,
