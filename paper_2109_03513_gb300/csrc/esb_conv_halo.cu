@@ -55,13 +55,11 @@ struct HaloGeom {
 // of which this block holds PAIRS, N-tile BN.  Straight-line issue, nothing
 // but the tcgen05.mma between two MMAs.
 template <int WS, int R, int S, int UT, int PAIRS, int BN>
-__device__ __forceinline__ void halo_mma_fixed(uint32_t d, uint32_t a_st, uint32_t b_blk, uint32_t idesc,
-                                               uint32_t& acc)
+__device__ __forceinline__ void halo_mma_fixed(uint32_t d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                               uint32_t& acc, uint32_t leader)
 {
     constexpr int NS = 128 + (R - 1) * WS + S - 1;
     constexpr uint32_t PB = NS * 16;
-    const uint64_t a_desc = smem_desc_noswz(a_st, PB, 128u);
-    const uint64_t b_desc = smem_desc_sw128(b_blk);
 #pragma unroll
     for (int t = 0; t < R * S; t++) {
 #pragma unroll
@@ -69,7 +67,7 @@ __device__ __forceinline__ void halo_mma_fixed(uint32_t d, uint32_t a_st, uint32
             const uint32_t ao = (uint32_t)((((t / S) * WS + (t % S)) * 16 + 2 * j * (int)PB) >> 4);
             const int kq = t * UT + j;
             const uint32_t bo = (uint32_t)(((kq >> 2) * BN * 128 + (kq & 3) * 32) >> 4);
-            mma_f8f6f4(d, a_desc + ao, b_desc + bo, idesc, acc);
+            mma_f8f6f4(d, a_desc + ao, b_desc + bo, idesc, acc, leader);
             acc = 1u;
         }
     }
@@ -223,7 +221,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = warp_index(), lane = tid & 31;
     const int n_tile = (int)(blockIdx.x % n_tiles);
     const int64_t cta_in_n = blockIdx.x / n_tiles;
     const int64_t ctas_per_n = gridDim.x / n_tiles;
@@ -231,9 +229,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
-    const int half_cols = BN / 2;
-    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
-    const int epi_warps = split ? 8 : 4;
+    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     const int cbs = g.cblocks;
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -258,7 +254,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
         }
         for (int a = 0; a < 2; a++) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], epi_warps);
+            mbar_init(&tempty[a], sp.tempty_count());
         }
         mbar_init(drain, 1);
         *err = 0;
@@ -365,62 +361,61 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
         // (halo_mma_fixed); others compute the offsets in the loop.
         // Descriptors never come from shared memory: the tensor core's own
         // operand reads keep it close to saturated.
-        if (lane == 0) {
-            const uint32_t idesc = idesc_e4m3_f32(BN);
-            const uint32_t b_base = smem_u32(sB), a_base = smem_u32(sA);
-            const int ws = 1 << g.lws;
-            const int units_tap = (g.ldx * g.spw) >> 5;        // 32-slot K steps per tap
-            const bool r3 = g.R == 3 && g.S == 3;
-            int s = 0;                                         // stage and phase of the next K-block
-            uint32_t ph = 0u;
-            for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
-                const int a = (int)(ti & 1);
-                if (!wait_or_abort(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err)) { *err = 1; break; }
+        const uint32_t idesc = idesc_e4m3_f32(BN);
+        const uint32_t leader = elect_one();
+        const int ws = 1 << g.lws;
+        const int units_tap = (g.ldx * g.spw) >> 5;            // 32-slot K steps per tap
+        const bool r3 = g.R == 3 && g.S == 3;
+        const uint64_t a_desc = smem_desc_noswz(smem_u32(sA), (uint32_t)g.pb, 128u);
+        const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
+        // in the descriptors' 16-byte units
+        const uint64_t a_step = (uint64_t)(g.stage_bytes >> 4), p_step = (uint64_t)((2 * g.pb) >> 4);
+        const uint32_t b_step = (uint32_t)(BN * kBK) >> 4;
+        int s = 0;                                             // stage and phase of the next K-block
+        uint32_t ph = 0u;
+        bool ok = true;
+        for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
+            const int a = (int)(ti & 1);
+            ok = warp_wait(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem_base + (uint32_t)(a * BN);
+            uint32_t acc = 0u;
+            for (int cb = 0; cb < cbs; cb++) {
+                ok = warp_wait(&full[s], ph, err);
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t d = tmem_base + (uint32_t)(a * BN);
-                uint32_t acc = 0u;
-                for (int cb = 0; cb < cbs; cb++) {
-                    if (!wait_or_abort(&full[s], ph, err)) { *err = 1; break; }
-                    tc_fence_after();
-                    const uint32_t a_st = a_base + (uint32_t)(s * g.stage_bytes);
-                    const uint32_t b_blk = b_base + (uint32_t)(cb * BN * kBK);   // block cb: 4 K steps on
-                    const int pairs = (min(16, g.ldx - cb * 16) * g.spw) >> 5;   // K steps (plane pairs) of the block
-                    if (r3 && ws == 64 && units_tap == 2 && BN == 64) {           // 56 x 56 x 64
-                        halo_mma_fixed<64, 3, 3, 2, 2, 64>(d, a_st, b_blk, idesc, acc);
-                    } else if (r3 && ws == 32 && units_tap == 4 && BN == 128) {   // 28 x 28 x 128
-                        halo_mma_fixed<32, 3, 3, 4, 4, 128>(d, a_st, b_blk, idesc, acc);
-                    } else if (r3 && ws == 16 && units_tap == 8 && pairs == 4 && BN == 64) {   // 14 x 14 x 256
-                        halo_mma_fixed<16, 3, 3, 8, 4, 64>(d, a_st, b_blk, idesc, acc);
-                    } else {
-                        // offsets in the descriptors' low words (16-byte units; the
-                        // address fields cannot carry out of them)
-                        const uint64_t ad0 = smem_desc_noswz(a_st, (uint32_t)g.pb, 128u), bd0 = smem_desc_sw128(b_base);
-                        const uint32_t alo = (uint32_t)ad0, blo = (uint32_t)bd0;
-                        const uint64_t ahi = ad0 & ~0xffffffffull, bhi = bd0 & ~0xffffffffull;
-                        const uint32_t pstep = (uint32_t)(2 * g.pb) >> 4, bstep = (uint32_t)(BN * kBK) >> 4;
-                        int kq0 = cb * (g.spw >> 1);
-                        for (int r = 0; r < g.R; r++) {
-                            for (int sx = 0; sx < g.S; sx++, kq0 += units_tap) {
-                                uint32_t at = alo + (uint32_t)(r * ws + sx);
+                const uint64_t a_st = a_desc + (uint64_t)s * a_step;
+                const uint64_t b_blk = b_desc + (uint64_t)cb * b_step;               // block cb: 4 K steps on
+                const int pairs = (min(16, g.ldx - cb * 16) * g.spw) >> 5;   // K steps (plane pairs) of the block
+                if (r3 && ws == 64 && units_tap == 2 && BN == 64) {           // 56 x 56 x 64
+                    halo_mma_fixed<64, 3, 3, 2, 2, 64>(d, a_st, b_blk, idesc, acc, leader);
+                } else if (r3 && ws == 32 && units_tap == 4 && BN == 128) {   // 28 x 28 x 128
+                    halo_mma_fixed<32, 3, 3, 4, 4, 128>(d, a_st, b_blk, idesc, acc, leader);
+                } else if (r3 && ws == 16 && units_tap == 8 && pairs == 4 && BN == 64) {   // 14 x 14 x 256
+                    halo_mma_fixed<16, 3, 3, 8, 4, 64>(d, a_st, b_blk, idesc, acc, leader);
+                } else {
+                    uint32_t kq0 = (uint32_t)(cb * (g.spw >> 1));
+                    for (int r = 0; r < g.R; r++) {
+                        for (int sx = 0; sx < g.S; sx++, kq0 += (uint32_t)units_tap) {
+                            uint64_t at = a_st + (uint64_t)(r * ws + sx);
 #pragma unroll 4
-                                for (int j = 0; j < pairs; j++, at += pstep) {
-                                    const uint32_t kq = (uint32_t)(kq0 + j);
-                                    const uint32_t bt = blo + (kq >> 2) * bstep + (kq & 3u) * 2u;
-                                    mma_f8f6f4(d, ahi | at, bhi | bt, idesc, acc);
-                                    acc = 1u;
-                                }
+                            for (int j = 0; j < pairs; j++, at += p_step) {
+                                const uint32_t kq = kq0 + (uint32_t)j;
+                                mma_f8f6f4(d, at, b_desc + (uint64_t)((kq >> 2) * b_step + (kq & 3u) * 2u), idesc, acc, leader);
+                                acc = 1u;
                             }
                         }
                     }
-                    mma_commit(&empty[s]);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
-                if (*err) break;
-                mma_commit(&tfull[a]);
+                mma_commit(&empty[s], leader);
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
-            ws_drain(drain, err);
+            if (ok) mma_commit(&tfull[a], leader);
         }
-    } else if (warp < epi_warps) {
+        if (!ok) *err = 1;
+        ws_drain(drain, err, leader);
+    } else if (warp < sp.warps) {
         // ---------------------------------------------- epilogue
         const int ctas = (int)ctas_per_n, first = (int)cta_in_n;   // tile counts fit in 32 bits (host check)
         const int tpi = g.tpi, rows_out = g.rows_out, lws = g.lws, P = g.P, Q = g.Q;
@@ -432,7 +427,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
             m = ((int64_t)nimg * P + p) * Q + q;
             return q < Q && p < P;
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 
@@ -575,11 +570,9 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     // The specialised instance: 4-bit B, bulk-copied input rows and 4-bit
     // codes as the only output, with a scalar scale and bias, in whole N-tiles
     // and with a monotone requantisation (unsigned codes or an activation).
-    const int half = hp.BN / 2;
-    const bool split = (half % 16 == 0) && (half % ep.out_cpw == 0);
     const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias &&
                       !ep.residual && !ep.acc_out && !ep.y_out && ep.acc_lim > 0.0f && N % hp.BN == 0 &&
-                      (!ep.out.is_signed || ep.act != ESB_ACT_NONE) && (split ? half : hp.BN) % 32 == 0;
+                      (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(fast ? esb_conv_halo_kernel<true, false>
                            : (gen ? esb_conv_halo_kernel<false, true> : esb_conv_halo_kernel<false, false>),

@@ -21,7 +21,7 @@
 //
 // 224 x 224 x 3, 7x7/2 -> 64, batch 64, 4-bit: 372 us on the im2col kernel
 // (49 single words gathered and decoded per output pixel, 5 of the 8 K slots
-// of each word padding), 109 us here, 2.3 us per tile in the issuing thread.
+// of each word padding), 89 us here.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -124,7 +124,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = warp_index(), lane = tid & 31;
     const int n_tile = (int)(blockIdx.x % n_tiles);
     const int cta = blockIdx.x / n_tiles, ctas = gridDim.x / n_tiles;
     const int64_t n0 = (int64_t)n_tile * BN;
@@ -132,9 +132,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
     const int t_lo = (int)((int64_t)m_tiles * cta / ctas), t_hi = (int)((int64_t)m_tiles * (cta + 1) / ctas);
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
-    const int half_cols = BN / 2;
-    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
-    const int epi_warps = split ? 8 : 4;
+    const EpiSplit sp = epi_split<GEN>(ep, BN, t_hi - t_lo);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -147,7 +145,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
         }
         for (int a = 0; a < 2; a++) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], epi_warps);
+            mbar_init(&tempty[a], sp.tempty_count());
         }
         mbar_init(drain, 1);
         *err = 0;
@@ -208,48 +206,51 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
         });
     } else if (warp == kWsMmaWarp) {
         // ---------------------------------------------- MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = idesc_e4m3_f32(BN);
-            const uint64_t bd0 = smem_desc_sw128(smem_u32(sB));
-            const uint32_t a_base = smem_u32(sA);
-            int s = 0, base = 0;                      // next row to arrive; the tile's first row (ring slots)
-            uint32_t ph = 0u;
-            for (int T = t_lo; T < t_hi && !*err; T++) {
-                const int i = T - t_lo, a = i & 1;
-                const int p = T % g.P;
-                if (!wait_or_abort(&tempty[a], (uint32_t)((i >> 1) & 1) ^ 1u, err)) { *err = 1; break; }
-                const int add = (i == 0 || p == 0) ? g.R : nnew;
-                if (add == g.R) base = s;
-                bool ok = true;
-                for (int j = 0; j < add && ok; j++) {
-                    ok = wait_or_abort(&full[s], ph, err);
-                    if (++s == g.NR) { s = 0; ph ^= 1u; }
-                }
-                if (!ok) { *err = 1; break; }
-                tc_fence_after();
-                const uint32_t d = tmem_base + (uint32_t)(a * BN);
-                uint32_t acc = 0u;
-                int slot = base, kq = 0;
-                for (int r = 0; r < g.R; r++) {
-                    const uint64_t ad = smem_desc_noswz(a_base + (uint32_t)(slot * g.pitch), 16u, 128u);
-                    for (int j = 0; j < g.G >> 1; j++, kq++) {
-                        mma_f8f6f4(d, ad + (uint64_t)(2 * j),
-                                   bd0 + (uint64_t)((kq >> 2) * ((BN * kBK) >> 4) + (kq & 3) * 2), idesc, acc);
-                        acc = 1u;
-                    }
-                    if (++slot == g.NR) slot = 0;
-                }
-                // rows the next tile does not use (all of them at the end of an image's segment)
-                const int rel = (T + 1 == t_hi || p + 1 == g.P) ? g.R : nnew;
-                for (int j = 0; j < rel; j++) {
-                    mma_commit(&empty[base]);
-                    if (++base == g.NR) base = 0;
-                }
-                mma_commit(&tfull[a]);
+        const uint32_t idesc = idesc_e4m3_f32(BN);
+        const uint32_t leader = elect_one();
+        const uint64_t a_desc = smem_desc_noswz(smem_u32(sA), 16u, 128u), b_desc = smem_desc_sw128(smem_u32(sB));
+        const uint32_t a_step = (uint32_t)g.pitch >> 4, b_step = (uint32_t)(BN * kBK) >> 4;
+        const int steps = g.G >> 1;
+        int s = 0, base = 0;                          // next row to arrive; the tile's first row (ring slots)
+        uint32_t ph = 0u;
+        int p = t_lo % g.P;
+        bool ok = true;
+        for (int T = t_lo; T < t_hi && ok; T++) {
+            const int i = T - t_lo, a = i & 1;
+            ok = warp_wait(&tempty[a], (uint32_t)((i >> 1) & 1) ^ 1u, err);
+            if (!ok) break;
+            const int add = (i == 0 || p == 0) ? g.R : nnew;
+            if (add == g.R) base = s;
+            for (int j = 0; j < add && ok; j++) {
+                ok = warp_wait(&full[s], ph, err);
+                if (++s == g.NR) { s = 0; ph ^= 1u; }
             }
-            ws_drain(drain, err);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem_base + (uint32_t)(a * BN);
+            uint32_t acc = 0u, kq = 0u;
+            int slot = base;
+            for (int r = 0; r < g.R; r++) {
+                const uint64_t ad = a_desc + (uint64_t)((uint32_t)slot * a_step);
+                for (int j = 0; j < steps; j++, kq++) {
+                    mma_f8f6f4(d, ad + (uint64_t)(2 * j), b_desc + (uint64_t)((kq >> 2) * b_step + (kq & 3u) * 2u), idesc, acc,
+                               leader);
+                    acc = 1u;
+                }
+                if (++slot == g.NR) slot = 0;
+            }
+            mma_commit(&tfull[a], leader);
+            // rows the next tile does not use (all of them at the end of an image's segment)
+            if (++p == g.P) p = 0;
+            const int rel = (T + 1 == t_hi || p == 0) ? g.R : nnew;
+            for (int j = 0; j < rel; j++) {
+                mma_commit(&empty[base], leader);
+                if (++base == g.NR) base = 0;
+            }
         }
-    } else if (warp < epi_warps) {
+        if (!ok) *err = 1;
+        ws_drain(drain, err, leader);
+    } else if (warp < sp.warps) {
         // ---------------------------------------------- epilogue
         const int row = (warp & 3) * 32 + lane;
         const int f = row / g.U, i = row - f * g.U;
@@ -262,7 +263,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
             m = ((int64_t)n * P + p) * Q + q;
             return live && q < Q;
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty,
                                err, warp, lane);
     }
 
@@ -367,11 +368,8 @@ bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     if (per_n > m_tiles) per_n = m_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
     // the specialised epilogue, as in the halo convolution
-    const int half = BN / 2;
-    const bool split = (half % 16 == 0) && (half % ep.out_cpw == 0);
     const bool fast = ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
-                      ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE) &&
-                      (split ? half : BN) % 32 == 0;
+                      ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(kStemKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
                       (size_t)sp.smem, st, sp.g, W, ldw, N, fa, fb, BN, sp.nkb, n_tiles, m_tiles, acc_scale, ep);

@@ -346,9 +346,9 @@ esb_gemm_tc_kernel(SrcA srcA, SrcB srcB, int64_t M, int64_t N, int64_t K, OpFmt 
 #pragma unroll
             for (int j = 0; j < kBK / 32; j++) {
                 mma_f8f6f4(tmem_d, smem_desc_sw128(a0 + j * 32), smem_desc_sw128(b0 + j * 32), idesc,
-                           (kb > 0 || j > 0) ? 1u : 0u);
+                           (kb > 0 || j > 0) ? 1u : 0u, 1u);
             }
-            mma_commit(&mma_bar[s]);
+            mma_commit(&mma_bar[s], 1u);
         }
     }
 
@@ -497,7 +497,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = warp_index(), lane = tid & 31;
     const int n_tile = (int)(blockIdx.x % n_tiles);
     const int64_t cta_in_n = blockIdx.x / n_tiles;
     const int64_t ctas_per_n = gridDim.x / n_tiles;
@@ -510,11 +510,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     __shared__ int4 ptab[kWsProdWarps][32];          // producers' per-stage tap tables (im2col rows)
     if (fa.planes == 1) build_e4m3_lut(luta, fa, tid, kWsThreads);
     if (fb.planes == 1 && fb.b != 4) build_e4m3_lut(lutb, fb, tid, kWsThreads);
-    // Epilogue column split: both halves of BN must be whole 16-column chunks
-    // and whole output words; otherwise warps 0-3 take every column.
-    const int half_cols = BN / 2;
-    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
-    const int epi_warps = split ? 8 : 4;
+    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -528,7 +524,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
         }
         for (int a = 0; a < 2; a++) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], epi_warps);
+            mbar_init(&tempty[a], sp.tempty_count());
         }
         mbar_init(drain, 1);
         *err = 0;
@@ -667,41 +663,47 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
         }
     } else if (warp == kWsMmaWarp) {
         // ---------------------------------------------- MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = idesc_e4m3_f32(BN);
-            const uint32_t b_base = smem_u32(sB), a_base = smem_u32(sA);
-            int s = 0;                                         // stage and phase of the next K-block
-            uint32_t ph = 0u;
-            for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
-                const int a = (int)(ti & 1);
-                if (!wait_or_abort(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err)) { *err = 1; break; }
+        const uint32_t idesc = idesc_e4m3_f32(BN);
+        const uint32_t leader = elect_one();
+        const uint64_t a_desc = smem_desc_sw128(smem_u32(sA)), b_desc = smem_desc_sw128(smem_u32(sB));
+        const uint64_t a_step = (uint64_t)(stage_bytes >> 4), b_step = (uint64_t)((BN * kBK) >> 4);
+        int s = 0;                                             // stage and phase of the next K-block
+        uint32_t ph = 0u;
+        bool ok = true;
+        for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
+            const int a = (int)(ti & 1);
+            ok = warp_wait(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem_base + (uint32_t)(a * BN);
+            uint32_t acc = 0u;
+            for (int kb = 0; kb < nkb; kb++) {
+                ok = warp_wait(&full[s], ph, err);
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t d = tmem_base + (uint32_t)(a * BN);
-                for (int kb = 0; kb < nkb; kb++) {
-                    if (!wait_or_abort(&full[s], ph, err)) { *err = 1; break; }
-                    tc_fence_after();
-                    const uint32_t a0 = a_base + (uint32_t)(s * stage_bytes);
-                    const uint32_t b0 = bstream ? a0 + (uint32_t)(kBM * kBK) : b_base + (uint32_t)(kb * BN * kBK);
+                const uint64_t ad = a_desc + (uint64_t)s * a_step;
+                const uint64_t bd = bstream ? ad + (uint64_t)((kBM * kBK) >> 4) : b_desc + (uint64_t)kb * b_step;
+                // four K steps of 32 codes: 32 bytes along the swizzled row
 #pragma unroll
-                    for (int j = 0; j < kBK / 32; j++)
-                        mma_f8f6f4(d, smem_desc_sw128(a0 + j * 32), smem_desc_sw128(b0 + j * 32), idesc,
-                                   (kb > 0 || j > 0) ? 1u : 0u);
-                    mma_commit(&empty[s]);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
+                for (int j = 0; j < kBK / 32; j++) {
+                    mma_f8f6f4(d, ad + 2 * j, bd + 2 * j, idesc, acc, leader);
+                    acc = 1u;
                 }
-                if (*err) break;
-                mma_commit(&tfull[a]);
+                mma_commit(&empty[s], leader);
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
-            ws_drain(drain, err);
+            if (ok) mma_commit(&tfull[a], leader);
         }
-    } else if (warp < epi_warps) {
+        if (!ok) *err = 1;
+        ws_drain(drain, err, leader);
+    } else if (warp < sp.warps) {
         // ---------------------------------------------- epilogue
         const int64_t ctas = ctas_per_n, first = cta_in_n;
         auto rows = [=](int64_t ti, int row, int64_t& m) -> bool {
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<false, GEN>(ep, thr, rows, my_tiles, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<false, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 

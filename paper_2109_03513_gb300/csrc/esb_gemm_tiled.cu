@@ -343,7 +343,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = warp_index(), lane = tid & 31;
     const int n_tile = (int)(blockIdx.x % n_tiles);
     const int64_t cta_in_n = blockIdx.x / n_tiles;
     const int64_t ctas_per_n = gridDim.x / n_tiles;
@@ -351,9 +351,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
     uint32_t tmem_cols = 32;                                     // a power of two >= the regions used
     while (tmem_cols < (uint32_t)(nbuf * nch * BN)) tmem_cols <<= 1;
-    const int half_cols = BN / 2;
-    const bool split = (GEN && epi_cells_ok(ep)) || ((half_cols % 16 == 0) && (half_cols % ep.out_cpw == 0));
-    const int epi_warps = split ? 8 : 4;
+    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -366,7 +364,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
         }
         for (int a = 0; a < 2; a++) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], nch > 1 ? kWsEpiWarps : epi_warps);
+            mbar_init(&tempty[a], nch > 1 ? kWsEpiWarps : sp.tempty_count());
         }
         mbar_init(drain, 1);
         *err = 0;
@@ -403,53 +401,56 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
         }
     } else if (warp == kWsMmaWarp) {
         // ---------------------------------------------- MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = idesc_e4m3_f32(BN);
-            const uint32_t base = smem_u32(smem);
-            int s = 0;
-            uint32_t ph = 0u;
-            for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
-                const int a = (int)(ti % nbuf);
-                if (!wait_or_abort(&tempty[a], (uint32_t)((ti / nbuf) & 1) ^ 1u, err)) { *err = 1; break; }
-                tc_fence_after();
-                uint32_t d = tmem_base + (uint32_t)(a * nch * BN);
-                uint32_t acc = 0u;
-                for (int kb = 0; kb < nkb; kb++) {
-                    if (kb > 0 && kb % kbc == 0) {       // next K-chunk: its own accumulator
-                        d += (uint32_t)BN;
-                        acc = 0u;
-                    }
-                    if (!wait_or_abort(&full[s], ph, err)) { *err = 1; break; }
-                    tc_fence_after();
-                    const uint32_t st = base + (uint32_t)(s * kStage);
-                    const uint64_t ad = smem_desc_sw128(st), bd = smem_desc_sw128(st + kTileA);
-                    // four K steps of 32 codes: 32 bytes along the swizzled row
-                    mma_f8f6f4(d, ad, bd, idesc, acc);
-                    mma_f8f6f4(d, ad + 2, bd + 2, idesc, 1u);
-                    mma_f8f6f4(d, ad + 4, bd + 4, idesc, 1u);
-                    mma_f8f6f4(d, ad + 6, bd + 6, idesc, 1u);
-                    acc = 1u;
-                    mma_commit(&empty[s]);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
+        const uint32_t idesc = idesc_e4m3_f32(BN);
+        const uint32_t leader = elect_one();
+        const uint64_t a_desc = smem_desc_sw128(smem_u32(smem));
+        int s = 0;
+        uint32_t ph = 0u;
+        bool ok = true;
+        for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
+            const int a = nbuf == 2 ? (int)(ti & 1) : 0;
+            ok = warp_wait(&tempty[a], (uint32_t)((nbuf == 2 ? ti >> 1 : ti) & 1) ^ 1u, err);
+            if (!ok) break;
+            tc_fence_after();
+            uint32_t d = tmem_base + (uint32_t)(a * nch * BN);
+            uint32_t acc = 0u;
+            int left = kbc;                              // K-blocks left of the chunk
+            for (int kb = 0; kb < nkb; kb++, left--) {
+                if (left == 0) {                         // next K-chunk: its own accumulator
+                    left = kbc;
+                    d += (uint32_t)BN;
+                    acc = 0u;
                 }
-                if (*err) break;
-                mma_commit(&tfull[a]);
+                ok = warp_wait(&full[s], ph, err);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t ad = a_desc + (uint64_t)s * (uint64_t)(kStage >> 4), bd = ad + (uint64_t)(kTileA >> 4);
+                // four K steps of 32 codes: 32 bytes along the swizzled row
+#pragma unroll
+                for (int j = 0; j < kBK / 32; j++) {
+                    mma_f8f6f4(d, ad + 2 * j, bd + 2 * j, idesc, acc, leader);
+                    acc = 1u;
+                }
+                mma_commit(&empty[s], leader);
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
-            ws_drain(drain, err);
+            if (ok) mma_commit(&tfull[a], leader);
         }
+        if (!ok) *err = 1;
+        ws_drain(drain, err, leader);
     } else if (nch > 1) {
         // ---------------------------------------------- epilogue (K in chunks)
         if (warp < kWsEpiWarps)
             tiled_chunked_epilogue(ep, thr, M, N, n0, BN, cta_in_n, ctas_per_n, my_tiles, nch, nbuf, tmem_base,
                                        acc_scale, tfull, tempty, err, warp, lane);
-    } else if (warp < epi_warps) {
+    } else if (warp < sp.warps) {
         // ---------------------------------------------- epilogue
         const int64_t first = cta_in_n, ctas = ctas_per_n;
         auto rows = [=](int64_t ti, int row, int64_t& m) -> bool {
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, split, epi_warps, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty,
                            err, warp, lane);
     }
 

@@ -46,9 +46,9 @@ __global__ void __launch_bounds__(128, 1) peak_tcgen05_kernel(int64_t iters, int
         const uint64_t ad = smem_desc_sw128(smem_u32(sa)), bd = smem_desc_sw128(smem_u32(sb));
         for (int64_t it = 0; it < iters; it++) {
 #pragma unroll
-            for (int j = 0; j < 4; j++) mma_f8f6f4(d, ad + 2 * j, bd + 2 * j, idesc, (it > 0 || j > 0) ? 1u : 0u);
+            for (int j = 0; j < 4; j++) mma_f8f6f4(d, ad + 2 * j, bd + 2 * j, idesc, (it > 0 || j > 0) ? 1u : 0u, 1u);
         }
-        mma_commit(&bar);
+        mma_commit(&bar, 1u);
         if (!mbar_wait_bounded(&bar, 0u, kPeakWaitNs)) record_status(status, ESB_ERR_TIMEOUT);
     }
     __syncthreads();

@@ -810,6 +810,34 @@ __host__ __device__ inline bool epi_cells_ok(const EpiParams& ep)
            (!ep.residual || ep.res_b == ep.out.b);
 }
 
+// How the 8 epilogue warps share the tiles (two groups of 4 warps, each
+// covering the 128 rows): by columns (the first group takes [0, mid)), or
+// alternate tiles whole (alt), or the first group alone.  Every tile costs a
+// warp a fixed time (two barrier waits, a TMEM round trip, the row's address)
+// beside its columns, about 1000 cycles: alternating halves it per tile, and
+// is the only way to use both groups on a 16-column tile.  It needs
+// enough tiles to even out the one that is drained last.
+struct EpiSplit {
+    int warps;           // epilogue warps in use
+    bool alt;
+    int mid;
+    __device__ __forceinline__ int tempty_count() const { return alt ? 4 : warps; }
+};
+
+template <bool GEN>
+__device__ __forceinline__ EpiSplit epi_split(const EpiParams& ep, int BN, int64_t my_tiles)
+{
+    const bool cells = GEN && epi_cells_ok(ep);
+    const bool swar = !GEN && ep.codes_out && ep.out.b == 4;       // 16-column chunks of whole words
+    const int half = BN / 2;
+    EpiSplit e;
+    e.alt = (cells || swar) && (BN < 32 || (BN <= 64 && my_tiles >= 8));
+    e.mid = swar ? ((BN / 16 + 1) / 2) * 16 : half;
+    const bool split = cells || (swar && BN >= 32) || (half % 16 == 0 && half % ep.out_cpw == 0);
+    e.warps = (e.alt || split) ? 8 : 4;
+    return e;
+}
+
 // Shared memory of epi_cells (static, one per kernel instance).
 struct EpiCellsSmem {
     uint2 cells[kEpiCells];
@@ -826,8 +854,8 @@ struct EpiCellsSmem {
 // 57 us without).
 template <int OB, bool RES, bool CH, bool CELLS, class RowMap>
 __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float* thr, const EpiCellsSmem& sm, int h0,
-                                                int hmax, const RowMap& rows, int64_t my_tiles, int64_t n0, int64_t N,
-                                                int BN, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
+                                                int hmax, const RowMap& rows, int64_t my_tiles, bool alt, int64_t n0,
+                                                int64_t N, int BN, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                                 uint64_t* tempty, volatile int* err, int warp, int lane)
 {
     constexpr int CPW = 32 / OB;
@@ -851,14 +879,15 @@ __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float
     const int live = (int)(N - n0 < (int64_t)BN ? N - n0 : (int64_t)BN);
     const int passes = (live + CC - 1) / CC;
     const int pmid = (passes + 1) >> 1;
-    const int p_lo = (warp >> 2) ? pmid : 0, p_hi = (warp >> 2) ? passes : pmid;
+    const int grp = warp >> 2;
+    const int p_lo = !alt && grp ? pmid : 0, p_hi = alt || grp ? passes : pmid;
     const int64_t w00 = n0 / CPW;
     const bool vec = WPC == 4 ? ep.codes_vec == 4 && (w00 & 3) == 0 : ep.codes_vec >= 2 && (w00 & 1) == 0;
     const bool rvec = RES && (reinterpret_cast<uintptr_t>(ep.residual) & 15u) == 0 && (ep.res_ld & 3) == 0 &&
                       (w00 & (WPC - 1)) == 0;
-    const bool tail_words = n0 + BN >= N && (warp >> 2) == 1;   // zero-code words past the outputs
+    const bool tail_words = n0 + BN >= N && (alt || grp == 1);   // zero-code words past the outputs
     const int row = quarter * 32 + lane;
-    for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
+    for (int64_t ti = alt ? grp : 0; ti < my_tiles && !*err; ti += alt ? 2 : 1) {
         const int a = (int)(ti & 1);
         if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> 1) & 1), err)) { *err = 1; break; }
         tc_fence_after();
@@ -962,7 +991,7 @@ __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float
 
 template <int OB, class RowMap>
 __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr, EpiCellsSmem& sm, const RowMap& rows,
-                                          int64_t my_tiles, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
+                                          int64_t my_tiles, bool alt, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
                                           float acc_scale, uint64_t* tfull, uint64_t* tempty, volatile int* err,
                                           int warp, int lane)
 {
@@ -978,14 +1007,14 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
     asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
     const bool ch = ep.scale || ep.bias, res = ep.residual != nullptr;
     if (!fits || *const_cast<volatile int*>(&sm.bad) != 0) {
-        if (res) epi_cells_tiles<OB, true, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     } else if (ch) {
-        if (res) epi_cells_tiles<OB, true, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     } else {
-        if (res) epi_cells_tiles<OB, true, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     }
 }
 
@@ -1081,12 +1110,11 @@ __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, in
 // Epilogue role (warps 0 .. epi_warps - 1): drains the accumulator tiles of
 // this CTA in order, tile ti from TMEM buffer ti & 1 (columns (ti & 1) * BN
 // ..), and frees the buffer on tempty once its columns are in registers.
-// Warp w reads TMEM lanes 32 (w & 3) .. +31 (= tile rows); with split, warps
-// 0-3 take the columns [0, BN/2) and warps 4-7 [BN/2, BN).  rows(ti, row, m)
+// Warp w reads TMEM lanes 32 (w & 3) .. +31 (= tile rows); sp says which
+// columns and tiles are the warp's (see EpiSplit).  rows(ti, row, m)
 // gives the output row m of a tile row and whether it exists.  LEAN4: the
 // host has established 4-bit codes as the only output with a scalar scale
-// and bias (every column chunk inside N, each warp's columns a multiple of
-// 32); the instance then holds just the
+// and bias (every column chunk inside N); the instance then holds just the
 // FMA-pipe requantisation and, for device values that rule it out, the
 // out-of-line per-word path.  GEN: the output is not 4-bit codes; the
 // instance holds the general-width code path and the out-of-line path for
@@ -1094,8 +1122,8 @@ __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, in
 // small hot loop).
 template <bool LEAN4, bool GEN, class RowMap>
 __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* thr, const RowMap& rows,
-                                            int64_t my_tiles, int64_t n0, int64_t N, int BN, bool split,
-                                            int epi_warps, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
+                                            int64_t my_tiles, int64_t n0, int64_t N, int BN, const EpiSplit& sp,
+                                            uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                             uint64_t* tempty, volatile int* err, int warp, int lane)
 {
     // the tables of epi_cells and of the bisection path below share their storage
@@ -1106,11 +1134,11 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     if constexpr (GEN) {
         if (epi_cells_ok(ep)) {
             if (ep.out.b == 3)
-                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             else if (ep.out.b == 5)
-                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             else
-                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             return;
         }
     }
@@ -1118,9 +1146,10 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     const int row = quarter * 32 + lane;              // TMEM lane = tile row
     __shared__ EpiParams sh_ep;                       // copies for the out-of-line general path
     __shared__ EpiCtx sh_cx;
-    const int half_cols = BN / 2;
-    const int c_lo = split ? (warp >> 2) * half_cols : 0;
-    const int c_hi = split ? c_lo + half_cols : BN;
+    const int epi_warps = sp.warps, grp = warp >> 2;
+    const bool split = epi_warps == 8 && !sp.alt;
+    const int c_lo = split && grp ? sp.mid : 0;
+    const int c_hi = split && !grp ? sp.mid : BN;
     const EpiCtx cx = make_epi_ctx(ep, thr);
     const bool swar = ep.codes_out && ep.out.b == 4;
     const float sc_fixed = ep.scale ? 0.0f : (cx.dq ? __fmul_rn(ep.scale0, cx.dqs) : ep.scale0);
@@ -1194,10 +1223,10 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     }
     // the warp holding the tile's last columns of the last N-tile writes the padding words
     const bool pad_words = ep.codes_out && (n0 + BN >= N) && ((n0 + BN) / cpw < ep.ldo) &&
-                           (split ? (warp >> 2) == 1 : true);
+                           (split ? grp == 1 : true);
     uint32_t zero_word = 0u;
     for (int j = 0; j < cpw; j++) zero_word |= ep.out.zero_code << (ep.out.b * j);
-    for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
+    for (int64_t ti = sp.alt ? grp : 0; ti < my_tiles && !*err; ti += sp.alt ? 2 : 1) {
         const int a = (int)(ti & 1);
         if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> 1) & 1), err)) { *err = 1; break; }
         tc_fence_after();
@@ -1433,13 +1462,20 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     }
 }
 
-// Bounded wait of the MMA thread for its own last commit before TMEM is
-// freed (also on the abort path).
-__device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err)
+// wait_or_abort by a whole warp, with one answer for all its lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* err)
 {
-    mma_commit(drain);
+    return __all_sync(0xffffffffu, wait_or_abort(bar, parity, err));
+}
+
+// Bounded wait of the MMA warp for its own last commit before TMEM is
+// freed (also on the abort path).
+__device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err, uint32_t leader)
+{
+    __syncwarp();
+    mma_commit(drain, leader);
     volatile int no_abort = 0;
-    if (!wait_or_abort(drain, 0u, &no_abort)) *err = 1;
+    if (!warp_wait(drain, 0u, &no_abort)) *err = 1;
 }
 
 // ------------------------------------------------------------- host side
