@@ -1,0 +1,36 @@
+"""Projection of rows that no 16-byte path takes: a thread per short row, and
+warp segments of longer ones, at every width, odd strides and alignments."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as o
+from paper_2109_03513_gb300 import esb, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("b,k,signed", [(2, 0, True), (3, 1, False), (4, 2, True), (4, 0, False), (5, 2, True), (6, 5, True),
+                                        (7, 3, False), (8, 4, True)])
+@pytest.mark.parametrize("rows,cols,ldc_extra,shift", [(1000, 3, 0, 0), (333, 1, 3, 0), (70, 0, 0, 1), (200, 9, 1, 1), (129, 63, 0, 0),
+                                                       (5, 1000, 0, 1), (3, 1025, 2, 0), (40, 17, 9, 0)])
+def test_project_any_rows(b, k, signed, rows, cols, ldc_extra, shift):
+    cpw = 32 // b
+    cols = {0: 2 * cpw, 9: 2 * cpw + 1}.get(cols, cols)           # the last short row, the first long one
+    x = synth.normal((rows, cols), seed=rows + cols, std=1.5)
+    x[0, 0], x[-1, -1] = float("nan"), -float("inf")
+    buf = torch.zeros(rows * cols + 8, dtype=torch.float32, device="cuda")
+    xd = buf[shift:shift + rows * cols].view(rows, cols)          # 4-byte aligned only
+    xd.copy_(x)
+    ldc = esb.esb_row_words(cols, b) + ldc_extra
+    out = torch.full((rows, ldc), -1, dtype=torch.int32, device="cuda")
+    for alpha in (0.7, 1e-44):                                    # ordinary; thresholds no cell table holds
+        esb.esb_project(xd, esb.Fmt(b, k, signed), alpha=alpha, rounding=rows & 1, codes=out, ldc=ldc)
+        exp = o.project_packed(x.numpy(), np.float32(alpha), b, k, signed=signed, rounding=rows & 1, ld_words=ldc)
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), exp)
