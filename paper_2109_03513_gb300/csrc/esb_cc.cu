@@ -321,6 +321,50 @@ esb_dwconv3_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const uint32
     }
 }
 
+// Buckets (0..7) of the sums of two channels against their 7 ascending
+// integer thresholds, as j0 | j1 << 16: three levels of a packed compare whose
+// result is a mask, and selects by that mask (10 instructions for the pair; the
+// compares on fp32 values took 10 for each).
+__device__ __forceinline__ uint32_t bucket_pair(__half2 acc, const __half2 (&A)[7])
+{
+    auto u = [](__half2 h) -> uint32_t { return *reinterpret_cast<const uint32_t*>(&h); };
+    auto sel = [](uint32_t m, uint32_t a, uint32_t b) -> uint32_t { return (m & a) | (~m & b); };
+    auto h = [](uint32_t v) -> __half2 { return *reinterpret_cast<const __half2*>(&v); };
+    const uint32_t m2 = __hge2_mask(acc, A[3]);
+    const uint32_t m1 = __hge2_mask(acc, h(sel(m2, u(A[5]), u(A[1]))));
+    const uint32_t m0 = __hge2_mask(acc, h(sel(m2, sel(m1, u(A[6]), u(A[4])), sel(m1, u(A[2]), u(A[0])))));
+    return (m2 & 0x00040004u) | (m1 & 0x00020002u) | (m0 & 0x00010001u);
+}
+
+// Eight buckets from four pairs, one per nibble.
+__device__ __forceinline__ uint32_t pack_pairs(const uint32_t (&x)[4])
+{
+    uint32_t b[4];
+#pragma unroll
+    for (int m = 0; m < 4; m++) b[m] = x[m] | (x[m] >> 12);      // byte 0: j0 | j1 << 4
+    return __byte_perm(__byte_perm(b[0], b[1], 0x0040u), __byte_perm(b[2], b[3], 0x0040u), 0x5410u);
+}
+
+constexpr int kDwBound = 1297;     // one past the largest sum of 9 products of 4-bit images
+
+// Smallest integer a in [-kDwBound, kDwBound] with act(fma(sc, a, b)) >= T
+// (kDwBound: none below it), for sc > 0, where that is a step function of a.
+__device__ inline float dw_threshold(float sc, float b, float T, int act)
+{
+    auto reach = [&](float a) { return cc_act(__fmaf_rn(sc, a, b), act) >= T; };
+    const float L = (float)kDwBound;
+    float a = ceilf(__fdividef(T - b, sc));
+    a = fminf(fmaxf(a, -L), L);                       // a NaN guess becomes -L
+    if (reach(a) && (a <= -L || !reach(a - 1.0f))) return a;
+    if (a < L && reach(a + 1.0f) && !reach(a)) return a + 1.0f;
+    int lo = -kDwBound - 1, hi = kDwBound;            // the guess is off: bisection
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (reach((float)mid)) hi = mid; else lo = mid;
+    }
+    return (float)hi;
+}
+
 // Depthwise 3x3 of 4-bit codes on packed fp16 pairs.  Every 4-bit image is
 // an integer of magnitude at most 12, so every partial sum of the 9 taps is
 // an integer of magnitude at most 9 * 12 * 12 = 1296 < 2^11: fp16 holds each
@@ -337,11 +381,12 @@ esb_dwconv3_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const uint32
 template <int STRIDE>
 __global__ void __launch_bounds__(128, 6)
 esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const uint32_t* __restrict__ W, int ldw,
-                       int kw, int H, int Wd, int C, int pad, int P, int Q, int QS, int rows, CcEpi ep)
+                       int kw, int H, int Wd, int C, int pad, int P, int Q, int QS, int rows, CcEpi ep, int tables)
 {
     constexpr int QT = STRIDE == 1 ? 4 : 2;
     constexpr int NIN = (QT - 1) * STRIDE + 3;
-    extern __shared__ __half2 wtab2[];                // [9][words * 4] filter images, channel pairs
+    // [9][words * 4] filter images, channel pairs; with tables, then [words][7][4] thresholds
+    extern __shared__ __align__(16) __half2 wtab2[];
     __shared__ __half2 lut2[256];                     // code byte -> (image of low nibble, image of high nibble)
     __shared__ float T[128];
     __shared__ float Rs[8];
@@ -373,14 +418,39 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
     // codes only, any scale and bias: the word's 8 codes from their buckets at once
     const bool words8 = b4 && !lean && !ep.residual && !ep.acc_out && !ep.y_out;
     const uint32_t sgn_out = ep.out.is_signed ? 1u : 0u;
+    // non-negative outputs: a negative y is in bucket 0 by the compares alone
+    const bool nonneg = !ep.out.is_signed || ep.act != ESB_ACT_NONE;
     __syncthreads();
+    // per-channel thresholds on the integer sum, where every scale is positive
+    __half* const atab = reinterpret_cast<__half*>(wtab2 + 9 * cp2);
+    bool ptab = tables && words8 && nonneg;           // the same in every thread
+    if (ptab) {
+        bool bad = false;
+        for (int i = threadIdx.x; i < cp2 * 2 * 7; i += blockDim.x) {
+            const int w = i / 56, rem = i - w * 56;
+            const int j = rem >> 3, ch = rem & 7;     // threshold j of channel 8 w + ch
+            const int c = w * 8 + ch;
+            float a = (float)kDwBound;
+            if (c < C) {
+                float sc = ep.scale ? __ldg(ep.scale + c) : ep.scale0;
+                if (dq) sc = __fmul_rn(sc, dqs);
+                const float bi = ep.bias ? __ldg(ep.bias + c) : ep.bias0;
+                if (!(sc > 0.0f) || !isfinite(sc) || !isfinite(bi)) bad = true;
+                else a = dw_threshold(sc, bi, T[j], ep.act);
+            }
+            atab[i] = __float2half_rn(a);
+        }
+        ptab = !__syncthreads_or(bad);
+    }
     if (lean && threadIdx.x < 7) Rs[threadIdx.x] = acc_raw_threshold(sc_fixed, ep.bias0, T[threadIdx.x], ep.act, 1.0f);
     __syncthreads();
-    Thr7 t7, r7;
+    Thr7 t7;
+    __half2 A[7];
 #pragma unroll
     for (int i = 0; i < 7; i++) {
         t7.t[i] = b4 ? T[i] : 0.0f;
-        r7.t[i] = lean ? Rs[i] : 0.0f;
+        // integer thresholds, exact in fp16; +-inf (never, always) one past the sums
+        A[i] = __float2half2_rn(lean ? fminf(fmaxf(Rs[i], (float)-kDwBound), (float)kDwBound) : 0.0f);
     }
     const int rcpw = ep.residual ? 32 / ep.res_b : 1;
     const uint32_t rmask = ep.residual ? (1u << ep.res_b) - 1u : 0u;
@@ -454,16 +524,33 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
             for (int c = 0; c < NIN; c++) xw[c] = xn[c];
         }
         const int cvalid = C - w * 8;
-        float scv[8], biv[8];
-        if (!lean) {
+        const uint32_t nib = cvalid >= 8 ? 0xffffffffu : (1u << (4 * cvalid)) - 1u;   // channels of the word
+        if (lean || ptab) {
+            // the word's codes from the integer sums alone, a channel pair of
+            // every output at a time (its 7 thresholds in registers)
+            const __half2* const aw = reinterpret_cast<const __half2*>(atab) + w * 28;
+            uint32_t x[QT][4];
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
-                const int c = w * 8 + j < C ? w * 8 + j : C - 1;
-                float sc = ep.scale ? __ldg(ep.scale + c) : ep.scale0;
-                if (dq) sc = __fmul_rn(sc, dqs);
-                scv[j] = sc;
-                biv[j] = ep.bias ? __ldg(ep.bias + c) : ep.bias0;
+            for (int m = 0; m < 4; m++) {
+                __half2 Am[7];
+#pragma unroll
+                for (int i = 0; i < 7; i++) Am[i] = ptab ? aw[i * 4 + m] : A[i];
+#pragma unroll
+                for (int uu = 0; uu < QT; uu++) x[uu][m] = bucket_pair(acc[uu][m], Am);
             }
+#pragma unroll
+            for (int uu = 0; uu < QT; uu++)
+                if (q0 + uu < Q) ep.codes_out[obase + (int64_t)uu * ldo] = codes8_b4(pack_pairs(x[uu]) & nib, 0u, ep.out.k);
+            continue;
+        }
+        float scv[8], biv[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int c = w * 8 + j < C ? w * 8 + j : C - 1;
+            float sc = ep.scale ? __ldg(ep.scale + c) : ep.scale0;
+            if (dq) sc = __fmul_rn(sc, dqs);
+            scv[j] = sc;
+            biv[j] = ep.bias ? __ldg(ep.bias + c) : ep.bias0;
         }
 #pragma unroll
         for (int uu = 0; uu < QT; uu++) {
@@ -476,35 +563,28 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
                 a[2 * m] = f2.x;
                 a[2 * m + 1] = f2.y;
             }
-            if (lean) {
-                uint32_t J = 0u;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const float v = a[j];
-                    const bool b2 = v >= r7.t[3];
-                    const bool b1 = v >= (b2 ? r7.t[5] : r7.t[1]);
-                    const bool b0 = v >= (b2 ? (b1 ? r7.t[6] : r7.t[4]) : (b1 ? r7.t[2] : r7.t[0]));
-                    const uint32_t jb = (b2 ? 4u : 0u) | (b1 ? 2u : 0u) | (b0 ? 1u : 0u);
-                    J |= (j < cvalid ? jb : 0u) << (4 * j);
-                }
-                ep.codes_out[ow] = codes8_b4(J, 0u, ep.out.k);
-                continue;
-            }
             if (words8) {
                 // per element: y = fma(scale, acc, bias), the activation, then
-                // the bucket of |y| (zero for negatives of an unsigned set);
+                // the bucket of y (of |y| where negatives keep their sign);
                 // codes8_b4 turns buckets and signs into the word (zero
                 // buckets keep sign 0), as project_by_thr7 does per code
                 uint32_t J = 0u, S = 0u;
+                if (nonneg) {
+                    const float hi = ep.act == ESB_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const uint32_t u = __float_as_uint(cc_act(__fmaf_rn(scv[j], a[j], biv[j]), ep.act));
-                    const uint32_t neg = u >> 31;
-                    const uint32_t jb = bucket7(__uint_as_float(u & 0x7fffffffu), t7);
-                    J |= ((j < cvalid && (sgn_out | (neg ^ 1u))) ? jb : 0u) << (4 * j);
-                    S |= (neg & sgn_out) << (4 * j + 3);
+                    for (int j = 0; j < 8; j++) {
+                        const float y = __fmaf_rn(scv[j], a[j], biv[j]);
+                        J |= bucket7(y > hi ? hi : y, t7) << (4 * j);     // NaN: bucket 0
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const uint32_t u = __float_as_uint(__fmaf_rn(scv[j], a[j], biv[j]));
+                        J |= bucket7(__uint_as_float(u & 0x7fffffffu), t7) << (4 * j);
+                        S |= ((u >> 31) & sgn_out) << (4 * j + 3);
+                    }
                 }
-                ep.codes_out[ow] = codes8_b4(J, S, ep.out.k);
+                ep.codes_out[ow] = codes8_b4(J & nib, S & nib, ep.out.k);
                 continue;
             }
             const int64_t pix = (int64_t)row * Q + q0 + uu;
@@ -535,10 +615,10 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
 
 // One resident wave of blocks (each block's set-up -- filter table,
 // thresholds -- is then paid once per block and amortised over many items).
-template <class Kern>
+template <class Kern, class... Extra>
 static cudaError_t launch_dw_wave(Kern kern, size_t smem, int64_t items, const esb_conv_desc& d, int P, int Q, int QS,
                                   const uint32_t* X, int64_t ldx, int kx, const uint32_t* W, int64_t ldw, int kw,
-                                  const CcEpi& ep, cudaStream_t st)
+                                  const CcEpi& ep, cudaStream_t st, Extra... extra)
 {
     int64_t blocks = (items + 127) / 128;
     int per_sm = 0;
@@ -548,8 +628,19 @@ static cudaError_t launch_dw_wave(Kern kern, size_t smem, int64_t items, const e
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     kern<<<(unsigned)blocks, 128, smem, st>>>(X, (int)ldx, kx, W, (int)ldw, kw, d.h, d.w, d.c, d.pad, P, Q, QS,
-                                              d.n * P, ep);
+                                              d.n * P, ep, extra...);
     return cudaGetLastError();
+}
+
+// Per-channel threshold tables (codes-only outputs with a scale or bias per
+// channel): 7 thresholds of about 25 instructions per channel and block
+// against some 300 saved per item, so they pay when a thread has enough items
+// for the channels (56 x 56 x 144, batch 64, 7.7 items a thread: 89 us on
+// the per-element path, 62 us with; 7 x 7 x 960, 0.9 items, stays per element).
+static bool dw_tables_pay(int64_t items, int words)
+{
+    const double per_thread = (double)items / (6.0 * 128.0 * device_sm_count());
+    return words <= 160 && per_thread * 300.0 > 1.5 * words * 56.0 * 25.0 / 128.0;
 }
 
 template <int B, int STRIDE>
@@ -561,9 +652,12 @@ static cudaError_t launch_dw3(const esb_conv_desc& d, int P, int Q, const uint32
     const int64_t items = (int64_t)d.n * P * QS * ep.ldo;
     const int words = (d.c + 32 / B - 1) / (32 / B);
     if constexpr (B == 4) {
-        if (h16)
-            return launch_dw_wave(esb_dwconv3_b4h_kernel<STRIDE>, sizeof(__half2) * 9 * (size_t)words * 4, items, d, P,
-                                  Q, QS, X, ldx, kx, W, ldw, kw, ep, st);
+        if (h16) {
+            const int tables = (ep.scale || ep.bias) && ep.codes_out && dw_tables_pay(items, words);
+            return launch_dw_wave(esb_dwconv3_b4h_kernel<STRIDE>,
+                                  sizeof(__half2) * 4 * (size_t)words * (9 + (tables ? 7 : 0)), items, d, P, Q, QS, X, ldx,
+                                  kx, W, ldw, kw, ep, st, tables);
+        }
     }
     return launch_dw_wave(esb_dwconv3_kernel<B, STRIDE>, sizeof(int32_t) * 9 * (size_t)words * (32 / B), items, d, P,
                           Q, QS, X, ldx, kx, W, ldw, kw, ep, st);
