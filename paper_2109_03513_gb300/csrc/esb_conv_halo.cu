@@ -18,8 +18,10 @@
 // 8-row core matrices, SBO = 128 bytes between them, LBO = one plane between
 // 16-code chunks), every tap is one descriptor, and the MMA warp issues
 // r * s * (chunks / 2) tcgen05.mma (K = 32) per tile from a single decode.
-// B (the filters, K = (tap, channel)) is resident as in the GEMM kernel, and
-// the epilogue is the shared one; rows with q >= Q or past the image's last
+// B (the filters, K = (tap, channel)) is resident, in the same layout: planes
+// of BN rows x 16 bytes, BN * 16 + 16 bytes apart (the decoders' 8-lane stores
+// then hit distinct banks), so that the descriptors of both operands advance
+// by constants from one K step to the next.  The epilogue is the shared one; rows with q >= Q or past the image's last
 // output row are computed from zero slots and not stored.
 //
 // Channel blocks of 128 codes are separate stages, so a tile's halo never
@@ -65,8 +67,7 @@ __device__ __forceinline__ void halo_mma_fixed(uint32_t d, uint64_t a_desc, uint
 #pragma unroll
         for (int j = 0; j < PAIRS; j++) {
             const uint32_t ao = (uint32_t)((((t / S) * WS + (t % S)) * 16 + 2 * j * (int)PB) >> 4);
-            const int kq = t * UT + j;
-            const uint32_t bo = (uint32_t)(((kq >> 2) * BN * 128 + (kq & 3) * 32) >> 4);
+            const uint32_t bo = (uint32_t)((t * UT + j) * 2 * (BN + 1));
             mma_f8f6f4(d, a_desc + ao, b_desc + bo, idesc, acc, leader);
             acc = 1u;
         }
@@ -204,18 +205,19 @@ __device__ __noinline__ void halo_decode(const HaloGeom g, int T, uint8_t* st, i
 template <bool FAST, bool GEN>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, OpFmt fb, int BN, int nkb,
-                     int stages, int n_tiles, int64_t m_tiles, float acc_scale, EpiParams ep)
+                     int stages, int n_tiles, int64_t m_tiles, float acc_scale, const __grid_constant__ EpiParams ep)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sB = smem;                                        // nkb blocks of BN x 128 bytes (SW128)
-    uint8_t* sA = sB + nkb * BN * kBK;                         // stages x stage_bytes (halo planes)
+    const int b_pitch = (BN + 1) * 16;                         // chunk planes of B
+    uint8_t* sB = smem;                                        // 8 nkb planes
+    uint8_t* sA = sB + nkb * 8 * b_pitch;                      // stages x stage_bytes (halo planes), 128-byte aligned
     float* thr = reinterpret_cast<float*>(sA + stages * g.stage_bytes);
     uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
     uint64_t* empty = full + kWsMaxStages;
     uint64_t* tfull = empty + kWsMaxStages;
-    uint64_t* tempty = tfull + 2;
-    uint64_t* drain = tempty + 2;
+    uint64_t* tempty = tfull + kMaxAcc;
+    uint64_t* drain = tempty + kMaxAcc;
     uint64_t* rawb = drain + 1;                                // kWsMaxStages: bulk-copy fills
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rawb + kWsMaxStages);
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -227,8 +229,9 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     const int64_t ctas_per_n = gridDim.x / n_tiles;
     const int64_t n0 = (int64_t)n_tile * BN;
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
+    const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
+    while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
     const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     const int cbs = g.cblocks;
     // the layout above must fit the dynamic allocation (uniform for the CTA)
@@ -252,7 +255,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
             mbar_init(&empty[s], 1);
             mbar_init(&rawb[s], 1);                   // the issuer's arrive.expect_tx, then the copies' bytes
         }
-        for (int a = 0; a < 2; a++) {
+        for (int a = 0; a < (1 << lacc); a++) {
             mbar_init(&tfull[a], 1);
             mbar_init(&tempty[a], sp.tempty_count());
         }
@@ -275,7 +278,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     if (!(bulk && warp == kWsProdWarp0)) {
         const int nbdec = bulk ? kWsThreads - 32 : kWsThreads;
         const int t = (bulk && warp > kWsProdWarp0) ? tid - 32 : tid;
-        ws_decode_b<FAST>(srcB, n0, K, fb, BN, nkb, sB, t, nbdec);
+        ws_decode_b<FAST>(srcB, n0, K, fb, BN, nkb, sB, t, nbdec, nullptr, b_pitch);
         fence_proxy_async_smem();
         if (warp == kWsMmaWarp) asm volatile("bar.sync 1, %0;" ::"r"(nbdec) : "memory");
         else asm volatile("bar.arrive 1, %0;" ::"r"(nbdec) : "memory");
@@ -367,16 +370,16 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
         const int units_tap = (g.ldx * g.spw) >> 5;            // 32-slot K steps per tap
         const bool r3 = g.R == 3 && g.S == 3;
         const uint64_t a_desc = smem_desc_noswz(smem_u32(sA), (uint32_t)g.pb, 128u);
-        const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
+        const uint64_t b_desc = smem_desc_noswz(smem_u32(sB), (uint32_t)b_pitch, 128u);
         // in the descriptors' 16-byte units
         const uint64_t a_step = (uint64_t)(g.stage_bytes >> 4), p_step = (uint64_t)((2 * g.pb) >> 4);
-        const uint32_t b_step = (uint32_t)(BN * kBK) >> 4;
+        const uint64_t b_step = (uint64_t)((2 * b_pitch) >> 4);
         int s = 0;                                             // stage and phase of the next K-block
         uint32_t ph = 0u;
         bool ok = true;
         for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
-            const int a = (int)(ti & 1);
-            ok = warp_wait(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err);
+            const int a = (int)(ti & ((1 << lacc) - 1));
+            ok = warp_wait(&tempty[a], (uint32_t)((ti >> lacc) & 1) ^ 1u, err);
             if (!ok) break;
             tc_fence_after();
             const uint32_t d = tmem_base + (uint32_t)(a * BN);
@@ -386,7 +389,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t a_st = a_desc + (uint64_t)s * a_step;
-                const uint64_t b_blk = b_desc + (uint64_t)cb * b_step;               // block cb: 4 K steps on
+                const uint64_t b_blk = b_desc + (uint64_t)(cb * (g.spw >> 1)) * b_step;   // block cb: 16 words on
                 const int pairs = (min(16, g.ldx - cb * 16) * g.spw) >> 5;   // K steps (plane pairs) of the block
                 if (r3 && ws == 64 && units_tap == 2 && BN == 64) {           // 56 x 56 x 64
                     halo_mma_fixed<64, 3, 3, 2, 2, 64>(d, a_st, b_blk, idesc, acc, leader);
@@ -395,14 +398,13 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
                 } else if (r3 && ws == 16 && units_tap == 8 && pairs == 4 && BN == 64) {   // 14 x 14 x 256
                     halo_mma_fixed<16, 3, 3, 8, 4, 64>(d, a_st, b_blk, idesc, acc, leader);
                 } else {
-                    uint32_t kq0 = (uint32_t)(cb * (g.spw >> 1));
+                    uint64_t bt0 = b_blk;
                     for (int r = 0; r < g.R; r++) {
-                        for (int sx = 0; sx < g.S; sx++, kq0 += (uint32_t)units_tap) {
-                            uint64_t at = a_st + (uint64_t)(r * ws + sx);
+                        for (int sx = 0; sx < g.S; sx++, bt0 += (uint64_t)units_tap * b_step) {
+                            uint64_t at = a_st + (uint64_t)(r * ws + sx), bt = bt0;
 #pragma unroll 4
-                            for (int j = 0; j < pairs; j++, at += p_step) {
-                                const uint32_t kq = kq0 + (uint32_t)j;
-                                mma_f8f6f4(d, at, b_desc + (uint64_t)((kq >> 2) * b_step + (kq & 3u) * 2u), idesc, acc, leader);
+                            for (int j = 0; j < pairs; j++, at += p_step, bt += b_step) {
+                                mma_f8f6f4(d, at, bt, idesc, acc, leader);
                                 acc = 1u;
                             }
                         }
@@ -427,7 +429,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
             m = ((int64_t)nimg * P + p) * Q + q;
             return q < Q && p < P;
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 
@@ -512,7 +514,7 @@ static bool halo_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, const O
     for (int i = -1; i < (int)(sizeof(cands) / sizeof(cands[0])); i++) {
         const int bn = i < 0 ? bn0 : cands[i];
         if (bn <= 0 || (i >= 0 && bn >= bn0) || bn % out_cpw != 0) continue;
-        const int64_t fixed = 1024 + (int64_t)hp->nkb * bn * kBK + 4 * 128 + 512;
+        const int64_t fixed = 1024 + (int64_t)hp->nkb * 8 * (bn + 1) * 16 + 4 * 128 + 512;
         int64_t stg = (maxs - fixed) / g.stage_bytes;
         if (stg > kWsMaxStages) stg = kWsMaxStages;
         if (stg < 2) continue;
@@ -567,12 +569,8 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     const int64_t grid = per_n * n_tiles;
     RowsSrc b{W, (int64_t)d.r * d.s * ldw, N};
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    // The specialised instance: 4-bit B, bulk-copied input rows and 4-bit
-    // codes as the only output, with a scalar scale and bias, in whole N-tiles
-    // and with a monotone requantisation (unsigned codes or an activation).
-    const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias &&
-                      !ep.residual && !ep.acc_out && !ep.y_out && ep.acc_lim > 0.0f && N % hp.BN == 0 &&
-                      (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
+    // The specialised instance: 4-bit B, bulk-copied input rows, LEAN4 epilogue
+    const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && lean4_ok(ep, N, hp.BN);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(fast ? esb_conv_halo_kernel<true, false>
                            : (gen ? esb_conv_halo_kernel<false, true> : esb_conv_halo_kernel<false, false>),

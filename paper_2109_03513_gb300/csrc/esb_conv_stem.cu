@@ -108,7 +108,7 @@ __device__ __forceinline__ void stem_filter(const StemGeom& g, const uint32_t* W
 template <bool FAST, bool GEN>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpFmt fa, OpFmt fb, int BN, int nkb, int n_tiles,
-                     int m_tiles, float acc_scale, EpiParams ep)
+                     int m_tiles, float acc_scale, const __grid_constant__ EpiParams ep)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -118,8 +118,8 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
     uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
     uint64_t* empty = full + kStemMaxRing;
     uint64_t* tfull = empty + kStemMaxRing;
-    uint64_t* tempty = tfull + 2;
-    uint64_t* drain = tempty + 2;
+    uint64_t* tempty = tfull + kMaxAcc;
+    uint64_t* drain = tempty + kMaxAcc;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -130,8 +130,9 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
     const int64_t n0 = (int64_t)n_tile * BN;
     // consecutive tiles: (image, segment, output row), the row fastest
     const int t_lo = (int)((int64_t)m_tiles * cta / ctas), t_hi = (int)((int64_t)m_tiles * (cta + 1) / ctas);
+    const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
+    while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
     const EpiSplit sp = epi_split<GEN>(ep, BN, t_hi - t_lo);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -143,7 +144,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        for (int a = 0; a < 2; a++) {
+        for (int a = 0; a < (1 << lacc); a++) {
             mbar_init(&tfull[a], 1);
             mbar_init(&tempty[a], sp.tempty_count());
         }
@@ -216,8 +217,8 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
         int p = t_lo % g.P;
         bool ok = true;
         for (int T = t_lo; T < t_hi && ok; T++) {
-            const int i = T - t_lo, a = i & 1;
-            ok = warp_wait(&tempty[a], (uint32_t)((i >> 1) & 1) ^ 1u, err);
+            const int i = T - t_lo, a = i & ((1 << lacc) - 1);
+            ok = warp_wait(&tempty[a], (uint32_t)((i >> lacc) & 1) ^ 1u, err);
             if (!ok) break;
             const int add = (i == 0 || p == 0) ? g.R : nnew;
             if (add == g.R) base = s;
@@ -263,7 +264,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
             m = ((int64_t)n * P + p) * Q + q;
             return live && q < Q;
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
                                err, warp, lane);
     }
 
@@ -330,7 +331,7 @@ static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx,
     const int64_t maxs = max_dyn_smem() - st;
     sp->BN = bn0;
     sp->nkb = (d.r * g.G * 16 + kBK - 1) / kBK;
-    const int64_t fixed = 1024 + (int64_t)sp->nkb * bn0 * kBK + 4 * 128 + (2 * kStemMaxRing + 5) * 8 + 64;
+    const int64_t fixed = 1024 + (int64_t)sp->nkb * bn0 * kBK + 4 * 128 + (2 * kStemMaxRing + 2 * kMaxAcc + 1) * 8 + 64;
     int64_t nr = (maxs - fixed) / g.pitch;
     if (nr > kStemMaxRing) nr = kStemMaxRing;
     if (nr < d.r + 2 * d.stride) return false;                     // a tile's rows and two more output rows' worth
@@ -367,9 +368,7 @@ bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     if (per_n < 1) per_n = 1;
     if (per_n > m_tiles) per_n = m_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    // the specialised epilogue, as in the halo convolution
-    const bool fast = ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
-                      ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
+    const bool fast = lean4_ok(ep, N, BN);                   // the specialised epilogue
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(kStemKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
                       (size_t)sp.smem, st, sp.g, W, ldw, N, fa, fb, BN, sp.nkb, n_tiles, m_tiles, acc_scale, ep);

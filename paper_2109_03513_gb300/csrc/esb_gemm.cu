@@ -99,11 +99,12 @@ struct ConvSrc {
         const int word = (int)(w - (int64_t)tap * kw);
         return tap_ptr(x, tap / S, tap - (tap / S) * S, word);
     }
-    __device__ __forceinline__ Cursor cursor(int64_t w) const
+    __device__ __forceinline__ Cursor cursor(int64_t w64) const
     {
         Cursor c;
-        const int tap = (int)(w / kw);
-        c.word = (int)(w - (int64_t)tap * kw);
+        const int w = (int)w64;                       // a row's K words: far below 2^31
+        const int tap = w / kw;
+        c.word = w - tap * kw;
         c.r = tap / S;
         c.s = tap - c.r * S;
         c.off = ((int64_t)c.r * W + c.s) * ldx + c.word;
@@ -474,10 +475,10 @@ __device__ __noinline__ void fill_stage_any(const Src src, int64_t m0, uint8_t* 
     }
 }
 
-template <class SrcA, bool GEN>
+template <class SrcA, bool LEAN4, bool GEN>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpFmt fa, OpFmt fb, int BN, int nkb,
-                   int stages, int n_tiles, int64_t m_tiles, float acc_scale, EpiParams ep, int bstream)
+                   int stages, int n_tiles, int64_t m_tiles, float acc_scale, const __grid_constant__ EpiParams ep, int bstream)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -491,8 +492,8 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
     uint64_t* empty = full + kWsMaxStages;
     uint64_t* tfull = empty + kWsMaxStages;
-    uint64_t* tempty = tfull + 2;
-    uint64_t* drain = tempty + 2;
+    uint64_t* tempty = tfull + kMaxAcc;
+    uint64_t* drain = tempty + kMaxAcc;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -503,8 +504,9 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     const int64_t ctas_per_n = gridDim.x / n_tiles;
     const int64_t n0 = (int64_t)n_tile * BN;
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
+    const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < 2 * BN) tmem_cols <<= 1;
+    while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
     // E4M3 tables of the word-walk decoder (widths other than 4)
     __shared__ uint8_t luta[256], lutb[256];
     __shared__ int4 ptab[kWsProdWarps][32];          // producers' per-stage tap tables (im2col rows)
@@ -522,7 +524,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
             mbar_init(&full[s], 1);                   // the producer warp that filled the stage
             mbar_init(&empty[s], 1);                  // the MMA commit that drained it
         }
-        for (int a = 0; a < 2; a++) {
+        for (int a = 0; a < (1 << lacc); a++) {
             mbar_init(&tfull[a], 1);
             mbar_init(&tempty[a], sp.tempty_count());
         }
@@ -538,7 +540,8 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     // (ws_setup).
     uint32_t tmem_base = 0;
     if (warp < kWsProdWarp0)
-        tmem_base = ws_setup<false>(srcB, n0, K, fb, BN, bstream ? 0 : nkb, sB, thr, ep, tmem_slot, tid, lutb);
+        tmem_base = ws_setup<false>(srcB, n0, K, fb, BN, bstream ? 0 : nkb, sB, tmem_slot, tid, lutb);
+    if (warp < kWsEpiWarps) ws_thresholds(thr, ep, warp, lane);
 
     if (warp >= kWsProdWarp0) {
         // ---------------------------------------------- A producers
@@ -590,7 +593,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                         const typename SrcA::Cursor c = srcA.cursor(w0);
 #pragma unroll 1
                         for (int q = 0; q < 4; q++) {
-                            fill_q<B>(st, q, kBM, left, fa.k, fa.ew, lane, [&](int u) -> const uint32_t* {
+                            fill_q<B>(st, 0, q, kBM, left, fa.k, fa.ew, lane, [&](int u) -> const uint32_t* {
                                 const int sl = u * S::RPI + lane / S::LPR;
                                 const int64_t base = __shfl_sync(0xffffffffu, (long long)rbase[0], sl);
                                 const uint32_t bd = __shfl_sync(0xffffffffu, rbnd[0], sl);
@@ -608,7 +611,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                     } else {
 #pragma unroll 1
                         for (int q = 0; q < 4; q++)
-                            fill_rows_q<B>(srcA, (cta_in_n + ti * ctas_per_n) * kBM, kBM, kb, q, K, fa, st, lane);
+                            fill_rows_q<B>(srcA, (cta_in_n + ti * ctas_per_n) * kBM, kBM, kb, q, K, fa, st, 0, lane);
                     }
                 });
             } else if (fa.planes == 1 && srcA.linear()) {
@@ -642,7 +645,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
                     with_width(fb.b, [&](auto width) {
 #pragma unroll 1
                         for (int q = 0; q < (BN + 31) >> 5; q++)
-                            fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sb, lane);
+                            fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sb, 0, lane);
                     });
                 } else if (fb.planes == 1 && srcB.linear()) {
 #pragma unroll 1
@@ -671,8 +674,8 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
         uint32_t ph = 0u;
         bool ok = true;
         for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
-            const int a = (int)(ti & 1);
-            ok = warp_wait(&tempty[a], (uint32_t)((ti >> 1) & 1) ^ 1u, err);
+            const int a = (int)(ti & ((1 << lacc) - 1));
+            ok = warp_wait(&tempty[a], (uint32_t)((ti >> lacc) & 1) ^ 1u, err);
             if (!ok) break;
             tc_fence_after();
             const uint32_t d = tmem_base + (uint32_t)(a * BN);
@@ -703,7 +706,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<false, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 
@@ -828,19 +831,39 @@ static cudaError_t launch_tc(const SrcA& a, const SrcB& b, int64_t M, int64_t N,
     return cudaGetLastError();
 }
 
+// The instances of the kernel by epilogue: 4-bit codes, 4-bit codes of the
+// specialised epilogue, other outputs.
+template <class SrcA>
+struct WsKernels {
+    typedef void (*Kernel)(SrcA, RowsSrc, int64_t, int64_t, int64_t, OpFmt, OpFmt, int, int, int, int, int64_t, float, EpiParams, int);
+    static constexpr Kernel k[3] = {esb_gemm_ws_kernel<SrcA, false, false>, esb_gemm_ws_kernel<SrcA, true, false>,
+                                    esb_gemm_ws_kernel<SrcA, false, true>};
+};
+
 template <class SrcA>
 static int ws_static_smem(cudaError_t* err)
 {
     static int v = -1;
     if (v < 0) {
-        cudaFuncAttributes a0, a1;
-        *err = cudaFuncGetAttributes(&a0, esb_gemm_ws_kernel<SrcA, false>);
-        if (*err != cudaSuccess) return -1;
-        *err = cudaFuncGetAttributes(&a1, esb_gemm_ws_kernel<SrcA, true>);
-        if (*err != cudaSuccess) return -1;
-        v = (int)(a0.sharedSizeBytes > a1.sharedSizeBytes ? a0.sharedSizeBytes : a1.sharedSizeBytes);
+        size_t m = 0;
+        for (auto k : WsKernels<SrcA>::k) {
+            cudaFuncAttributes a;
+            *err = cudaFuncGetAttributes(&a, k);
+            if (*err != cudaSuccess) return -1;
+            if (a.sharedSizeBytes > m) m = a.sharedSizeBytes;
+        }
+        v = (int)m;
     }
     return v;
+}
+
+// 4-bit codes as the only output, a scalar scale and bias, whole N-tiles and
+// a monotone requantisation (unsigned codes or an activation): what the
+// specialised epilogue (LEAN4) takes.
+bool lean4_ok(const EpiParams& ep, int64_t N, int BN)
+{
+    return ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
+           ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
 }
 
 // Warp-specialised launch: B resident when its N-tile fits in shared
@@ -867,10 +890,10 @@ static bool launch_ws(const SrcA& a, const RowsSrc& b, int64_t M, int64_t N, int
     }
     static bool configured = false;
     if (!configured) {
-        *err = cudaFuncSetAttribute(esb_gemm_ws_kernel<SrcA, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-        if (*err != cudaSuccess) return true;
-        *err = cudaFuncSetAttribute(esb_gemm_ws_kernel<SrcA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-        if (*err != cudaSuccess) return true;
+        for (auto k : WsKernels<SrcA>::k) {
+            *err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
+            if (*err != cudaSuccess) return true;
+        }
         configured = true;
     }
     const int n_tiles = (int)((N + BN - 1) / BN);
@@ -881,8 +904,9 @@ static bool launch_ws(const SrcA& a, const RowsSrc& b, int64_t M, int64_t N, int
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
-    *err = launch_pdl(gen ? esb_gemm_ws_kernel<SrcA, true> : esb_gemm_ws_kernel<SrcA, false>, dim3((unsigned)grid), dim3(kWsThreads), (size_t)L.smem_bytes, st, a, b,
-                      M, N, K, fa, fb, BN, L.nkb, L.stages, n_tiles, m_tiles, acc_scale, ep, bstream);
+    *err = launch_pdl(WsKernels<SrcA>::k[lean4_ok(ep, N, BN) ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kWsThreads),
+                      (size_t)L.smem_bytes, st, a, b, M, N, K, fa, fb, BN, L.nkb, L.stages, n_tiles, m_tiles, acc_scale, ep,
+                      bstream);
     return true;
 }
 

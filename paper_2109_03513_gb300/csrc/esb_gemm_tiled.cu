@@ -19,7 +19,7 @@
 //     tcgen05 kernels (ws_epilogue).  Each CTA keeps one N-tile and walks
 //     the M-tiles.  BN is 256, or 240 for outputs of 3, 5 or 6 bits, whose
 //     10, 6 or 5 codes per word divide 240 (a word never straddles tiles).
-//     Measured at 4096^3 with 6-bit codes: 124 us for the call, against 1458
+//     Measured at 4096^3 with 6-bit codes: 62 us for the call, against 1458
 //     us for the streamed kernel, which decodes every operand row again in
 //     each tile (the only one to take these widths before).
 // The contraction is exact: fp32 TMEM accumulation of integer-valued
@@ -233,10 +233,10 @@ __device__ __forceinline__ void tile_linear(const TileSrc& t, int64_t warp_unit,
             live ? tile_unit_any(p, (int64_t)(kb0 + i) * kBK + g * 16, K, t.f) : make_uint4(0u, 0u, 0u, 0u);
 }
 
-// HBM-bound by its output (one byte per code).  Both operands in one launch:
-// the 256 x 4096 x 9216 classifier layer went from 55.3 to 44.4 us with one
-// launch for two, four K-blocks' loads in flight per warp and no division per
-// chunk. the first blocks take A's units, the rest B's.
+// HBM-bound by its output (one byte per code).  Both operands in one launch
+// (the first blocks take A's units, the rest B's), four K-blocks' loads in
+// flight per warp and no division per chunk: 20.4 us in two launches before,
+// 11.4 us now for 256 x 9216 and 4096 x 9216 4-bit operands.
 __global__ void __launch_bounds__(256) esb_tile_kernel(TileSrc ta, TileSrc tb, int64_t K, int nkb, unsigned blocks_a)
 {
     griddep_wait();                                   // codes and workspace may belong to the previous launch
@@ -326,7 +326,7 @@ template <bool LEAN4, bool GEN>
 __global__ void __launch_bounds__(kTiledThreads, 1)
 esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict__ Bt, int64_t M, int64_t N, int64_t mpad,
                       int64_t npad, int nkb, int kbc, int nch, int BNr, int stages, int n_tiles, int64_t m_tiles,
-                      float acc_scale, EpiParams ep)
+                      float acc_scale, const __grid_constant__ EpiParams ep)
 {
     const int BN = LEAN4 ? kTiledBN : BNr;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -337,8 +337,8 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     uint64_t* full = reinterpret_cast<uint64_t*>(thr + 128);
     uint64_t* empty = full + kWsMaxStages;
     uint64_t* tfull = empty + kWsMaxStages;
-    uint64_t* tempty = tfull + 2;
-    uint64_t* drain = tempty + 2;
+    uint64_t* tempty = tfull + kMaxAcc;
+    uint64_t* drain = tempty + kMaxAcc;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* err = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -351,6 +351,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
     uint32_t tmem_cols = 32;                                     // a power of two >= the regions used
     while (tmem_cols < (uint32_t)(nbuf * nch * BN)) tmem_cols <<= 1;
+    constexpr int lacc = 1;                              // nch == 1: two buffers (BN >= 240)
     const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -450,7 +451,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
                            err, warp, lane);
     }
 
@@ -603,11 +604,7 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     if (per_n > m_tiles) per_n = m_tiles;
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    // the specialised epilogue: 4-bit codes as the only output with a scalar
-    // scale and bias, whole N-tiles, a monotone requantisation, K in one chunk
-    const bool fast = nch == 1 && BN == kTiledBN && ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias &&
-                      !ep.residual && !ep.acc_out && !ep.y_out && ep.acc_lim > 0.0f && N % BN == 0 &&
-                      (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
+    const bool fast = nch == 1 && BN == kTiledBN && lean4_ok(ep, N, BN);   // the specialised epilogue
     // one chunk of other widths' codes only: the general-width epilogue instance
     const bool gen = nch == 1 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
     return launch_pdl(kTiledKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,

@@ -366,10 +366,14 @@ __device__ __forceinline__ uint32_t fmt_zero_word(int b, int k)
     return z;
 }
 
+// Where 16-byte chunk g of a row of an operand block lies: the SW128 layout
+// (pitch 0), or chunk planes of 16 bytes a row, `pitch` bytes apart.
+__device__ __forceinline__ uint32_t chunk_at(int r, int g, int pitch) { return pitch ? (uint32_t)(g * pitch + r * 16) : swz(r, g); }
+
 // Piece pc (4 words, of which the first `left` codes are inside K) of stage
 // row r, decoded and stored.
 template <int B>
-__device__ __forceinline__ void store_piece(uint8_t* stage, int r, int pc, const uint4& v, int64_t left, int k, int ew,
+__device__ __forceinline__ void store_piece(uint8_t* stage, int pitch, int r, int pc, const uint4& v, int64_t left, int k, int ew,
                                             uint32_t zero_word)
 {
     using S = SlotFmt<B>;
@@ -384,7 +388,7 @@ __device__ __forceinline__ void store_piece(uint8_t* stage, int r, int pc, const
         uint32_t o[4];
 #pragma unroll
         for (int i = 0; i < 4 / RW; i++) decode_slots<B>(w[c * (4 / RW) + i], k, ew, o + i * RW);
-        *reinterpret_cast<uint4*>(stage + swz(r, RW * pc + c)) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4*>(stage + chunk_at(r, RW * pc + c, pitch)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
 }
 
@@ -394,7 +398,7 @@ __device__ __forceinline__ void store_piece(uint8_t* stage, int r, int pc, const
 // lane per row read 16 bytes of 32 rows at a time, and the L1 took a pass per
 // row), and all LPR loads are in flight together.
 template <int B, class F>
-__device__ __forceinline__ void fill_q(uint8_t* stage, int q, int nrows, int64_t left, int k, int ew, int lane, const F& ptr)
+__device__ __forceinline__ void fill_q(uint8_t* stage, int pitch, int q, int nrows, int64_t left, int k, int ew, int lane, const F& ptr)
 {
     using S = SlotFmt<B>;
     const uint32_t zw = fmt_zero_word(B, k);
@@ -407,7 +411,7 @@ __device__ __forceinline__ void fill_q(uint8_t* stage, int q, int nrows, int64_t
     }
 #pragma unroll
     for (int u = 0; u < S::LPR; u++)
-        if (r0 + u * S::RPI < nrows) store_piece<B>(stage, r0 + u * S::RPI, pc, v[u], left, k, ew, zw);
+        if (r0 + u * S::RPI < nrows) store_piece<B>(stage, pitch, r0 + u * S::RPI, pc, v[u], left, k, ew, zw);
 }
 
 // CH loaded words of B-bit codes in the word-slot layout (ok: word i
@@ -709,7 +713,7 @@ __device__ __forceinline__ bool by_pieces(const Src& src, const OpFmt& f)
 // warp.  K: the kernel's K (4-bit codes); word slots count codes to korig.
 template <int B>
 __device__ __noinline__ void fill_rows_q(const RowsSrc src, int64_t n0, int nrows, int kb, int q, int64_t K, const OpFmt f,
-                                         uint8_t* stage, int lane)
+                                         uint8_t* stage, int pitch, int lane)
 {
     using S = SlotFmt<B>;
     const int64_t w0 = (int64_t)kb * S::NW + 4 * (lane % S::LPR);
@@ -717,7 +721,7 @@ __device__ __noinline__ void fill_rows_q(const RowsSrc src, int64_t n0, int nrow
     const int64_t r0 = n0 + q * 32 + lane / S::LPR;
     const RowsSrc::Cursor c = src.cursor(w0);
     const uint32_t* p = src.base + r0 * src.ld + c.w;
-    fill_q<B>(stage, q, nrows, left, f.k, f.ew, lane, [&](int u) -> const uint32_t* {
+    fill_q<B>(stage, pitch, q, nrows, left, f.k, f.ew, lane, [&](int u) -> const uint32_t* {
         return r0 + u * S::RPI < src.rows ? p + (int64_t)(u * S::RPI) * src.ld : nullptr;
     });
 }
@@ -756,43 +760,90 @@ static __device__ __noinline__ void epi_chunk_any(const EpiParams* __restrict__ 
 }
 
 
-struct Raw8 { uint32_t r[8]; };
-
-// One packed word of 4-bit output codes (8 columns from n_first) with
-// per-channel scale/bias, residual or extra outputs; out of line so the
-// caller's accumulator registers stay in registers.
-static __device__ __noinline__ uint32_t epi_word_b4(const EpiParams* __restrict__ sep, const EpiCtx* __restrict__ scx,
-                                                    Raw8 v, float acc_scale, float sc_fixed, int64_t m, bool mrow,
-                                                    int64_t n_first, int64_t N)
+// One 16-column chunk with fp32 or int32 outputs, or with per-channel scale
+// and bias and 4-bit codes: every output of the columns inside N, and the two
+// words of 4-bit codes (codes_out with another width takes epi_chunk_any).
+// Four columns at a time in a rolled loop: y and acc go out 16 bytes at a time
+// where N and the pointers allow, and the code stays small (a call with one
+// chunk per warp, such as 64 x 64 x 576 with y, is bound by fetching it and by
+// the parameters' loads: 13.9 us with a column at a time, 16.5 us with 16
+// unrolled, 14.2 us in this form before the parameters were read up front,
+// 11.8 us now).
+// Out of line: reads its own TMEM chunk.
+static __device__ __noinline__ uint2 epi_chunk16(const EpiParams& ep, const EpiCtx* __restrict__ scx, uint32_t taddr,
+                                                 float acc_scale, float sc_fixed, int64_t m, bool mrow, int64_t n0, int64_t N)
 {
-    const EpiParams& ep = *sep;
-    const EpiCtx& cx = *scx;
-    uint32_t J = 0u, S = 0u;
+    // every field once, together: the stores below could alias them
+    const float* const scale = ep.scale;
+    const float* const bias = ep.bias;
+    const uint32_t* const residual = ep.residual;
+    float* const y_out = ep.y_out;
+    int32_t* const acc_out = ep.acc_out;
+    const float bias0 = ep.bias0, res_scale = ep.res_scale, dqs = scx->dqs;
+    const int act = ep.act, res_b = ep.res_b, res_k = ep.res_k, out_signed = ep.out.is_signed, out_k = ep.out.k;
+    const int64_t res_ld = ep.res_ld;
+    const bool codes = ep.codes_out != nullptr;
+    const bool dq = scx->dq;
+    const Thr7 t7 = scx->t7;
+    const bool vec = n0 + 16 <= N && (N & 3) == 0 && mrow;
+    const bool vy = vec && (reinterpret_cast<uintptr_t>(y_out) & 15u) == 0;
+    const bool va = vec && (reinterpret_cast<uintptr_t>(acc_out) & 15u) == 0;
+    const int live = mrow ? (int)(N - n0 < 16 ? N - n0 : 16) : 0;   // columns to store
+    uint32_t J0 = 0u, J1 = 0u, S0 = 0u, S1 = 0u;
 #pragma unroll 1
-    for (int j = 0; j < 8; j++) {
-        const int64_t n = n_first + j;
-        const float af = __uint_as_float(v.r[j]) * acc_scale;
-        if (mrow && n < N) {
-            if (ep.acc_out) ep.acc_out[m * N + n] = __float2int_rn(af);
+    for (int g = 0; g < 4; g++) {
+        uint32_t r[4];
+        tmem_ld4(taddr + 4 * g, r);
+        float a[4], y[4];
+        uint32_t j4 = 0u, s4 = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const bool in = 4 * g + j < live;
+            const int64_t n = in ? n0 + 4 * g + j : 0;
+            a[j] = __uint_as_float(r[j]) * acc_scale;
             float sc = sc_fixed;
-            if (ep.scale) { sc = __ldg(ep.scale + n); if (cx.dq) sc = __fmul_rn(sc, cx.dqs); }
-            const float bi = ep.bias ? __ldg(ep.bias + n) : ep.bias0;
-            float y = __fmaf_rn(sc, af, bi);
-            if (ep.residual) {
-                const int rcpw = 32 / ep.res_b;
-                const int nq = (int)n / rcpw;                 // 32-bit: a column index is below 2^31
-        const uint32_t rc = (__ldg(ep.residual + m * ep.res_ld + nq) >> (ep.res_b * ((int)n - nq * rcpw))) &
-                                    ((1u << ep.res_b) - 1u);
-                y = __fmaf_rn(ep.res_scale, code_image_f(rc, ep.res_b, ep.res_k), y);
+            if (scale) { sc = __ldg(scale + n); if (dq) sc = __fmul_rn(sc, dqs); }
+            const float bi = bias ? __ldg(bias + n) : bias0;
+            y[j] = __fmaf_rn(sc, a[j], bi);
+            if (residual && in) {
+                const int rcpw = 32 / res_b;
+                const int nq = (int)n / rcpw;         // 32-bit: a column index is below 2^31
+                const uint32_t rc = (__ldg(residual + m * res_ld + nq) >> (res_b * ((int)n - nq * rcpw))) &
+                                    ((1u << res_b) - 1u);
+                y[j] = __fmaf_rn(res_scale, code_image_f(rc, res_b, res_k), y[j]);
             }
-            y = apply_act(y, ep.act);
-            if (ep.y_out) ep.y_out[m * N + n] = y;
-            const uint32_t u = __float_as_uint(y);
-            J |= bucket7(ep.out.is_signed ? fabsf(y) : y, cx.t7) << (4 * j);
-            S |= ((u >> 31) & (uint32_t)ep.out.is_signed) << (4 * j + 3);
+            y[j] = apply_act(y[j], act);
+            if (in && codes) {
+                j4 |= bucket7(out_signed ? fabsf(y[j]) : y[j], t7) << (4 * j);
+                s4 |= ((__float_as_uint(y[j]) >> 31) & (uint32_t)out_signed) << (4 * j + 3);
+            }
         }
+        if (acc_out) {
+            int32_t* p = acc_out + m * N + n0 + 4 * g;
+            if (va) {
+                *reinterpret_cast<int4*>(p) = make_int4(__float2int_rn(a[0]), __float2int_rn(a[1]), __float2int_rn(a[2]),
+                                                        __float2int_rn(a[3]));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    if (4 * g + j < live) p[j] = __float2int_rn(a[j]);
+            }
+        }
+        if (y_out) {
+            float* p = y_out + m * N + n0 + 4 * g;
+            if (vy) {
+                *reinterpret_cast<float4*>(p) = make_float4(y[0], y[1], y[2], y[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    if (4 * g + j < live) p[j] = y[j];
+            }
+        }
+        const int sh = 16 * (g & 1);
+        if (g < 2) { J0 |= j4 << sh; S0 |= s4 << sh; }
+        else { J1 |= j4 << sh; S1 |= s4 << sh; }
     }
-    return codes8_b4(J, S, ep.out.k);
+    return make_uint2(codes8_b4(J0, S0, out_k), codes8_b4(J1, S1, out_k));
 }
 
 // Output codes of 3, 5 or 6 bits as the only output: the projection of y by
@@ -838,6 +889,12 @@ __device__ __forceinline__ EpiSplit epi_split(const EpiParams& ep, int BN, int64
     return e;
 }
 
+// Accumulator buffers in TMEM: four where the columns allow, so that the MMA
+// warp runs ahead of the epilogue (with two, each tile of a narrow layer
+// waited for the hand-off of the last but one, both ways).
+__host__ __device__ inline int acc_buffers_log2(int BN) { return BN <= 128 ? 2 : 1; }
+constexpr int kMaxAcc = 4;
+
 // Shared memory of epi_cells (static, one per kernel instance).
 struct EpiCellsSmem {
     uint2 cells[kEpiCells];
@@ -850,11 +907,12 @@ struct EpiCellsSmem {
 // bisection over thr).  All three are fixed outside the loop, so a pass has no
 // branch and its columns' chains of loads and compares interleave: the
 // epilogue warps are two to a scheduler and bound by latency, not by issue
+// (out of line: each has its own register allocation, and none spills)
 // (4096^3, 6-bit: 111 us for the GEMM kernel with these tests per column,
-// 57 us without).
+// 48 us without).
 template <int OB, bool RES, bool CH, bool CELLS, class RowMap>
-__device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float* thr, const EpiCellsSmem& sm, int h0,
-                                                int hmax, const RowMap& rows, int64_t my_tiles, bool alt, int64_t n0,
+__device__ __noinline__ void epi_cells_tiles(const EpiParams& ep, const float* thr, const EpiCellsSmem& sm, int h0,
+                                                int hmax, const RowMap& rows, int64_t my_tiles, bool alt, int lacc, int64_t n0,
                                                 int64_t N, int BN, uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                                 uint64_t* tempty, volatile int* err, int warp, int lane)
 {
@@ -888,8 +946,8 @@ __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float
     const bool tail_words = n0 + BN >= N && (alt || grp == 1);   // zero-code words past the outputs
     const int row = quarter * 32 + lane;
     for (int64_t ti = alt ? grp : 0; ti < my_tiles && !*err; ti += alt ? 2 : 1) {
-        const int a = (int)(ti & 1);
-        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> 1) & 1), err)) { *err = 1; break; }
+        const int a = (int)(ti & ((1 << lacc) - 1));
+        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> lacc) & 1), err)) { *err = 1; break; }
         tc_fence_after();
         int64_t m = 0;
         const bool mrow = rows(ti, row, m);
@@ -960,6 +1018,9 @@ __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float
                                              : project_by_table(y, thr, ep.out);
                     word[w] |= c << (OB * j);
                 }
+                // two words' chains interleave (with channel loads, one):
+                // enough to cover the table's latency without spilling
+                if (CH || (w & 1)) asm volatile("" ::: "memory");
             }
             if ((ps + 1) * CC > live) {               // columns past N: the zero code
 #pragma unroll
@@ -991,7 +1052,7 @@ __device__ __forceinline__ void epi_cells_tiles(const EpiParams& ep, const float
 
 template <int OB, class RowMap>
 __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr, EpiCellsSmem& sm, const RowMap& rows,
-                                          int64_t my_tiles, bool alt, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
+                                          int64_t my_tiles, bool alt, int lacc, int64_t n0, int64_t N, int BN, uint32_t tmem_base,
                                           float acc_scale, uint64_t* tfull, uint64_t* tempty, volatile int* err,
                                           int warp, int lane)
 {
@@ -1007,14 +1068,14 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
     asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
     const bool ch = ep.scale || ep.bias, res = ep.residual != nullptr;
     if (!fits || *const_cast<volatile int*>(&sm.bad) != 0) {
-        if (res) epi_cells_tiles<OB, true, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, false>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     } else if (ch) {
-        if (res) epi_cells_tiles<OB, true, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, true, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     } else {
-        if (res) epi_cells_tiles<OB, true, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-        else epi_cells_tiles<OB, false, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        if (res) epi_cells_tiles<OB, true, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else epi_cells_tiles<OB, false, false, true>(ep, thr, sm, h0, hmax, rows, my_tiles, alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
     }
 }
 
@@ -1033,11 +1094,12 @@ __device__ __forceinline__ void ws_alloc(int warp, uint32_t* tmem_slot, uint32_t
 
 // Decode of the CTA's N-tile of B (rows n0 .. n0 + BN, every K-block) once
 // into sB in the SW128 K-major layout, by threads t = 0 .. nthreads - 1 of
-// the calling warps.  B4: B is known to be 4-bit.  The caller fences
+// the calling warps (by pieces: with a pitch, in chunk planes instead).  B4:
+// B is known to be 4-bit.  The caller fences
 // (fence_proxy_async_smem) and synchronises before the MMA reads sB.
 template <bool B4>
 __device__ __forceinline__ void ws_decode_b(const RowsSrc& srcB, int64_t n0, int64_t K, const OpFmt& fb, int BN,
-                                            int nkb, uint8_t* sB, int t, int nthreads, const uint8_t* lutb = nullptr)
+                                            int nkb, uint8_t* sB, int t, int nthreads, const uint8_t* lutb = nullptr, int pitch = 0)
 {
     if (B4 || by_pieces(srcB, fb)) {
         // 32 rows of one K-block per warp and step
@@ -1047,7 +1109,7 @@ __device__ __forceinline__ void ws_decode_b(const RowsSrc& srcB, int64_t n0, int
 #pragma unroll 1
             for (int u = t >> 5; u < nkb * qn; u += nwarp) {
                 const int kb = u / qn, q = u - kb * qn;
-                fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sB + kb * BN * kBK, lane);
+                fill_rows_q<decltype(width)::value>(srcB, n0, BN, kb, q, K, fb, sB + kb * (pitch ? 8 * pitch : BN * kBK), pitch, lane);
             }
         };
         if (B4) go(IntC<4>());
@@ -1083,32 +1145,26 @@ __device__ __forceinline__ void ws_thresholds(float* thr, const EpiParams& ep, i
 
 // Setup role (warps 0 .. kWsProdWarp0 - 1, while the producers already load
 // A): all setup warps decode B (ws_decode_b); the MMA warp waits for that on
-// named barrier 1 and leaves, while warps 0-7 build the thresholds
-// (ws_thresholds: the MMA does not wait for them).  B4: B is known to be
-// 4-bit.  Returns the TMEM base address (allocated by ws_alloc before the
-// CTA barrier).
+// named barrier 1, the others only arrive.  B4: B is known to be 4-bit.
+// Returns the TMEM base address (allocated by ws_alloc before the CTA
+// barrier).
 template <bool B4>
 __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, int64_t K, const OpFmt& fb, int BN,
-                                             int nkb, uint8_t* sB, float* thr, const EpiParams& ep,
-                                             uint32_t* tmem_slot, int tid, const uint8_t* lutb = nullptr)
+                                             int nkb, uint8_t* sB, uint32_t* tmem_slot, int tid, const uint8_t* lutb = nullptr)
 {
     constexpr int kSetupThreads = kWsProdWarp0 * 32;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = tid >> 5;
     griddep_wait();                                   // B and the alphas may come from the previous launch
     ws_decode_b<B4>(srcB, n0, K, fb, BN, nkb, sB, tid, kSetupThreads, lutb);
     fence_proxy_async_smem();
-    if (warp == kWsMmaWarp) {
-        asm volatile("bar.sync 1, %0;" ::"n"(kSetupThreads) : "memory");
-    } else {
-        asm volatile("bar.arrive 1, %0;" ::"n"(kSetupThreads) : "memory");
-        ws_thresholds(thr, ep, warp, lane);
-    }
+    if (warp == kWsMmaWarp) asm volatile("bar.sync 1, %0;" ::"n"(kSetupThreads) : "memory");
+    else asm volatile("bar.arrive 1, %0;" ::"n"(kSetupThreads) : "memory");
     tc_fence_after();
     return *tmem_slot;
 }
 
 // Epilogue role (warps 0 .. epi_warps - 1): drains the accumulator tiles of
-// this CTA in order, tile ti from TMEM buffer ti & 1 (columns (ti & 1) * BN
+// this CTA in order, tile ti from TMEM buffer a = ti mod 2^lacc (columns a * BN
 // ..), and frees the buffer on tempty once its columns are in registers.
 // Warp w reads TMEM lanes 32 (w & 3) .. +31 (= tile rows); sp says which
 // columns and tiles are the warp's (see EpiSplit).  rows(ti, row, m)
@@ -1122,7 +1178,7 @@ __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, in
 // small hot loop).
 template <bool LEAN4, bool GEN, class RowMap>
 __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* thr, const RowMap& rows,
-                                            int64_t my_tiles, int64_t n0, int64_t N, int BN, const EpiSplit& sp,
+                                            int64_t my_tiles, int64_t n0, int64_t N, int BN, const EpiSplit& sp, int lacc,
                                             uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                             uint64_t* tempty, volatile int* err, int warp, int lane)
 {
@@ -1134,11 +1190,11 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     if constexpr (GEN) {
         if (epi_cells_ok(ep)) {
             if (ep.out.b == 3)
-                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             else if (ep.out.b == 5)
-                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             else
-                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
             return;
         }
     }
@@ -1227,8 +1283,8 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     uint32_t zero_word = 0u;
     for (int j = 0; j < cpw; j++) zero_word |= ep.out.zero_code << (ep.out.b * j);
     for (int64_t ti = sp.alt ? grp : 0; ti < my_tiles && !*err; ti += sp.alt ? 2 : 1) {
-        const int a = (int)(ti & 1);
-        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> 1) & 1), err)) { *err = 1; break; }
+        const int a = (int)(ti & ((1 << lacc) - 1));
+        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> lacc) & 1), err)) { *err = 1; break; }
         tc_fence_after();
         int64_t m = 0;
         const bool mrow = rows(ti, row, m);
@@ -1340,7 +1396,10 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
         }
         for (int c = c_lo; c < (gen ? c_lo : c_hi); c += 16) {
             if (GEN || (!LEAN4 && !swar)) {
-                epi_chunk_any(&sh_ep, &sh_cx, taddr + (uint32_t)c, acc_scale, m, mrow, n0 + c, N, wsw);
+                if (!ep.codes_out)
+                    epi_chunk16(ep, &sh_cx, taddr + (uint32_t)c, acc_scale, sc_fixed, m, mrow, n0 + c, N);
+                else
+                    epi_chunk_any(&sh_ep, &sh_cx, taddr + (uint32_t)c, acc_scale, m, mrow, n0 + c, N, wsw);
                 if (c + 16 >= c_hi) {
                     tc_fence_before();
                     __syncwarp();
@@ -1352,20 +1411,29 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
             // 4-bit output codes: 16 columns (two code words) per TMEM load
             // (compact code: measured faster than 32-column loads)
             constexpr int nc = 16;
-            uint32_t r[16];
-            tmem_ld16(taddr + (uint32_t)c, r);
-            if (c + nc >= c_hi) {                     // every column of this warp is in registers
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
-            }
             // columns of the chunk inside N (codes past N are masked to the zero code)
             const int64_t ncl64 = N - (n0 + c);
             const int ncl = ncl64 < nc ? (int)ncl64 : nc;
             const bool lean = lean_ok && ncl > 0;
             uint32_t wds[2];
+            // other outputs, per-channel scale or bias; LEAN4: device values that rule the FMA search out
+            const bool full = LEAN4 ? !(lean && fma_ok) : (!lean && !(lres && ncl > 0));
+            uint32_t r[16];
+            if (full) {
+                const uint2 q = epi_chunk16(ep, &sh_cx, taddr + (uint32_t)c, acc_scale, sc_fixed, m, mrow, n0 + c, N);
+                wds[0] = q.x;
+                wds[1] = q.y;
+            } else {
+                tmem_ld16(taddr + (uint32_t)c, r);
+            }
+            if (c + nc >= c_hi) {                     // every column of this warp is in registers
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
+            }
 #pragma unroll
             for (int h = 0; h < 2; h++) {
+                if (full) break;
                 uint32_t J = 0u, S = 0u;
                 const int live_h = ncl - 8 * h;       // nibbles of this word inside N
                 const uint32_t nib = live_h >= 8 ? 0xffffffffu : (live_h <= 0 ? 0u : (1u << (4 * live_h)) - 1u);
@@ -1432,11 +1500,6 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                         if (out_signed) S |= (__float_as_uint(y) >> 31) << (4 * j + 3);
                     }
                     wds[h] = codes8_b4(J & nib, S & nib, ep.out.k);
-                } else {
-                    Raw8 v;
-#pragma unroll
-                    for (int j = 0; j < 8; j++) v.r[j] = r[8 * h + j];
-                    wds[h] = epi_word_b4(&sh_ep, &sh_cx, v, acc_scale, sc_fixed, m, mrow, n0 + c + 8 * h, N);
                 }
             }
             if (mrow) {
@@ -1482,6 +1545,7 @@ __device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err, uin
 
 int pick_bn(int64_t N, int out_cpw);          // N-tile width (esb_gemm.cu)
 int max_dyn_smem();                           // opt-in shared memory per block
+bool lean4_ok(const EpiParams& ep, int64_t N, int BN);   // the LEAN4 epilogue takes the call (esb_gemm.cu)
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
 float acc_fma_limit(int64_t K, int ba, int ka, int bb, int kb);   // FMA-pipe requantisation bound (esb_gemm.cu)
 
