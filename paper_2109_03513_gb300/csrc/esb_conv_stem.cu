@@ -21,7 +21,8 @@
 //
 // 224 x 224 x 3, 7x7/2 -> 64, batch 64, 4-bit: 372 us on the im2col kernel
 // (49 single words gathered and decoded per output pixel, 5 of the 8 K slots
-// of each word padding), 89 us here.
+// of each word padding), 86 us here; 3x3/2 -> 32: 53 us (69 while the decoders
+// stepped through every row and divided for every tile).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -52,38 +53,41 @@ __device__ __forceinline__ uint32_t stem_pixel(uint32_t w, int k)
     return e4m3_4<B>(spread4<B>(rot_word<B>(w, k)), k);
 }
 
-// One input row into a ring slot, by one warp: lane l takes pixel positions
-// l, l + 32, ... (every load in flight before the first store), each stored
-// to its place in every copy.
-template <int B>
-__device__ __forceinline__ void stem_row(const StemGeom& g, int n, int h, int x0, uint8_t* slot, int lane, int k,
-                                         uint32_t cmask)
+// One input row by one warp: lane l takes pixel positions l, l + 32, ... of a
+// batch of 32 * kStemUn.  Loaded ahead of its slot, then each pixel is decoded
+// and stored to its place in every copy (position j is pixel j - stride f of
+// copy f).
+constexpr int kStemUn = 8;
+
+struct StemRow {                     // row h (of image n), pixel x0 at position 0
+    const uint32_t* x;               // first pixel of the row; nullptr: outside the image
+    int x0;
+};
+
+__device__ __forceinline__ void stem_load(const StemGeom& g, const StemRow& row, int j0, int lane, uint32_t zw,
+                                          uint32_t (&w)[kStemUn])
 {
-    constexpr int UN = 8;
-    const int npos = 4 * g.U + g.stride * (g.phi - 1);
-    const bool hin = (unsigned)h < (unsigned)g.H;
-    const uint32_t* xr = g.X + ((int64_t)n * g.H + (hin ? h : 0)) * g.W * g.ldx;
-#pragma unroll 1
-    for (int j0 = 0; j0 < npos; j0 += 32 * UN) {
-        uint32_t w[UN];
-        uint32_t ok = 0u;
 #pragma unroll
-        for (int u = 0; u < UN; u++) {
-            const int x = x0 + j0 + 32 * u + lane;
-            const bool in = hin && (unsigned)x < (unsigned)g.W;
-            w[u] = in ? __ldg(xr + (int64_t)x * g.ldx) : 0u;
-            ok |= (in ? 1u : 0u) << u;
-        }
+    for (int u = 0; u < kStemUn; u++) {
+        const int x = row.x0 + j0 + 32 * u + lane;
+        w[u] = zw;
+        if (row.x && (unsigned)x < (unsigned)g.W) w[u] = __ldg(row.x + (int64_t)x * g.ldx);
+    }
+}
+
+template <int B>
+__device__ __forceinline__ void stem_store(const StemGeom& g, int j0, uint8_t* slot, int lane, int k, uint32_t cmask,
+                                           const uint32_t (&w)[kStemUn])
+{
+    const int n4 = 4 * g.U;                           // positions of a copy
+    uint8_t* const p0 = slot + (j0 + lane) * 4;
+    const int f1 = g.U * 16 - 4 * g.stride;           // from copy 0 to copy 1
 #pragma unroll
-        for (int u = 0; u < UN; u++) {
-            const int j = j0 + 32 * u + lane;
-            const uint32_t v = ((ok >> u) & 1u) ? stem_pixel<B>(w[u], k) & cmask : 0u;
-            for (int f = 0; f < g.phi; f++) {
-                const int jf = j - g.stride * f;
-                if ((unsigned)jf < (unsigned)(4 * g.U))
-                    *reinterpret_cast<uint32_t*>(slot + f * g.U * 16 + jf * 4) = v;
-            }
-        }
+    for (int u = 0; u < kStemUn; u++) {
+        const int j = j0 + 32 * u + lane;
+        const uint32_t v = stem_pixel<B>(w[u], k) & cmask;
+        if (j < n4) *reinterpret_cast<uint32_t*>(p0 + 128 * u) = v;
+        if (g.phi > 1 && (unsigned)(j - g.stride) < (unsigned)n4) *reinterpret_cast<uint32_t*>(p0 + 128 * u + f1) = v;
     }
 }
 
@@ -185,24 +189,58 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
         // ---------------------------------------------- row decoders: row rho by warp rho % 7
         const int pw = warp - kWsProdWarp0;
         with_width(fa.b, [&](auto width) {
-            int turn = 0, s = 0;                      // rho % kWsProdWarps, rho % NR
+            constexpr int B = decltype(width)::value;
+            const uint32_t zw = fmt_zero_word(B, fa.k);
+            const int npos = 4 * g.U + g.stride * (g.phi - 1);
+            // cursor of this warp's next row: tile T (output row p of strip
+            // `strip`), filter row r, ring slot s and its phase
+            int T = t_lo, strip = t_lo / g.P, p = t_lo - strip * g.P, r = 0, s = 0;
             uint32_t ph = 0u;
-            for (int T = t_lo; T < t_hi && !*err; T++) {
-                const int strip = T / g.P, p = T - strip * g.P;
-                const int n = strip / g.nseg, seg = strip - n * g.nseg;
-                const int x0 = g.stride * g.phi * seg * g.Ui - g.pad;
-                const int r0 = (T == t_lo || p == 0) ? 0 : g.R - nnew;
-                for (int r = r0; r < g.R; r++) {
-                    if (turn == pw) {
-                        if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
-                        stem_row<decltype(width)::value>(g, n, p * g.stride - g.pad + r, x0, sA + s * g.pitch, lane, fa.k, cmask);
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&full[s]);
-                    }
-                    if (++turn == kWsProdWarps) turn = 0;
-                    if (++s == g.NR) { s = 0; ph ^= 1u; }
+            auto skip = [&](int rows) {               // `rows` rows on in the sequence
+                s += rows;
+                if (s >= g.NR) { s -= g.NR; ph ^= 1u; }
+                while (rows > 0) {
+                    const int left = g.R - r;
+                    if (rows < left) { r += rows; break; }
+                    rows -= left;
+                    T++;
+                    r = g.R - nnew;
+                    if (++p == g.P) { p = 0; strip++; r = 0; }
                 }
+            };
+            auto row_at = [&]() -> StemRow {
+                const int n = g.nseg == 1 ? strip : strip / g.nseg, seg = g.nseg == 1 ? 0 : strip - n * g.nseg;
+                const int h = p * g.stride - g.pad + r;
+                StemRow q;
+                q.x = (unsigned)h < (unsigned)g.H ? g.X + ((int64_t)n * g.H + h) * g.W * g.ldx : nullptr;
+                q.x0 = g.stride * g.phi * seg * g.Ui - g.pad;
+                return q;
+            };
+            skip(pw);
+            uint32_t w[kStemUn];
+            StemRow row;
+            if (T < t_hi) { row = row_at(); stem_load(g, row, 0, lane, zw, w); }
+            while (T < t_hi) {
+                if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
+                uint8_t* const slot = sA + s * g.pitch;
+                uint64_t* const done = &full[s];
+                // the batches of this row, then the next row's first one
+#pragma unroll 1
+                for (int j0 = 0; j0 < npos; j0 += 32 * kStemUn) {
+                    uint32_t wn[kStemUn];
+                    const bool more = j0 + 32 * kStemUn < npos;
+                    if (!more) {
+                        skip(kWsProdWarps);
+                        if (T < t_hi) row = row_at(); else row.x = nullptr;
+                    }
+                    stem_load(g, row, more ? j0 + 32 * kStemUn : 0, lane, zw, wn);
+                    stem_store<B>(g, j0, slot, lane, fa.k, cmask, w);
+#pragma unroll
+                    for (int u = 0; u < kStemUn; u++) w[u] = wn[u];
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(done);
             }
         });
     } else if (warp == kWsMmaWarp) {
@@ -334,7 +372,8 @@ static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx,
     const int64_t fixed = 1024 + (int64_t)sp->nkb * bn0 * kBK + 4 * 128 + (2 * kStemMaxRing + 2 * kMaxAcc + 1) * 8 + 64;
     int64_t nr = (maxs - fixed) / g.pitch;
     if (nr > kStemMaxRing) nr = kStemMaxRing;
-    if (nr < d.r + 2 * d.stride) return false;                     // a tile's rows and two more output rows' worth
+    // a tile's rows and two more output rows' worth; a decoder's next row is within one turn of the ring
+    if (nr < d.r + 2 * d.stride || nr < kWsProdWarps + 1) return false;
     g.NR = (int)nr;
     sp->smem = fixed + nr * g.pitch;
     return true;
