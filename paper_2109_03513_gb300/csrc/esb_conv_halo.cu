@@ -45,11 +45,29 @@ struct HaloGeom {
     int hr;              // halo rows (rows_out + R - 1)
     int ns;              // slots per plane (128 + (R-1) * Ws + S - 1)
     int pb;              // bytes per plane (ns * 16)
+    int tail;            // pixels of the last input row: W, or fewer where a 1x1's pixels are taken 128 at a time
     int cblocks;         // channel blocks of 16 words
     int spw;             // K slots per input word: 8 (4-bit codes, 5/6-bit word slots) or 16 (2/3-bit word slots)
     int stage_bytes;     // planes of one channel block (<= 8 planes), then raw rows
     int planes_bytes;    // the planes part of a stage
     int raw_bytes;       // raw code rows of a tile (one channel block only), or 0: register path
+};
+
+// A CTA's tiles first, first + step, ... as (image, tile within it) without a
+// division per tile (each role's scalar work per tile counts: its instructions
+// come one per 5 to 10 cycles).
+struct TileCursor {
+    int img, t;
+    int dimg, dt, tpi;
+    __device__ __forceinline__ TileCursor(int first, int step, int tiles_per_image)
+        : img(first / tiles_per_image), t(first - (first / tiles_per_image) * tiles_per_image), dimg(step / tiles_per_image),
+          dt(step - (step / tiles_per_image) * tiles_per_image), tpi(tiles_per_image) {}
+    __device__ __forceinline__ void next()
+    {
+        img += dimg;
+        t += dt;
+        if (t >= tpi) { t -= tpi; img++; }
+    }
 };
 
 // The MMAs of one stage (channel block) with every offset a compile-time
@@ -132,7 +150,7 @@ __device__ __forceinline__ void halo_load(const HaloGeom& g, int T, int cb, int 
         const int hi = rel >> g.lws;                               // halo row (-1: left guard)
         const int j = rel & wsm;
         const int h = p0 - g.pad + hi;
-        const bool ok = slot < g.ns && rel >= 0 && hi < g.hr && j < g.W && (unsigned)h < (unsigned)g.H;
+        const bool ok = slot < g.ns && rel >= 0 && hi < g.hr && (unsigned)h < (unsigned)g.H && j < (h + 1 < g.H ? g.W : g.tail);
         v[u] = make_uint4(zw, zw, zw, zw);
         if (ok) v[u] = __ldg(reinterpret_cast<const uint4*>(xi + ((int64_t)h * g.W + j) * g.ldx) + pc);
     }
@@ -156,38 +174,33 @@ __device__ __forceinline__ void halo_store(const HaloGeom& g, int cb, int i0, in
 // (one thread) copies the input rows of tile T that lie inside the image,
 // whole (w pixels of ldx words, contiguous in NHWC), into the stage's raw
 // area with one cp.async.bulk each, completing on mbarrier `raw_bar`.
-__device__ __forceinline__ void halo_issue_rows(const HaloGeom& g, int64_t T, uint8_t* st, uint64_t* raw_bar)
+__device__ __forceinline__ void halo_issue_rows(const HaloGeom& g, int nimg, int p0, uint8_t* st, uint64_t* raw_bar)
 {
-    const int nimg = (int)(T / g.tpi);
-    const int p0 = (int)(T - (int64_t)nimg * g.tpi) * g.rows_out;
     uint8_t* raw = st + g.planes_bytes;
-    const int row_words = g.W * g.ldx;
-    int valid = 0;
-    for (int i = 0; i < g.hr; i++) {
-        const int h = p0 - g.pad + i;
-        valid += (h >= 0 && h < g.H) ? 1 : 0;
-    }
-    mbar_arrive_expect_tx(raw_bar, (uint32_t)(valid * row_words * 4));
-    for (int i = 0; i < g.hr; i++) {
-        const int h = p0 - g.pad + i;
-        if (h >= 0 && h < g.H)
-            bulk_copy_g2s(raw + (size_t)i * row_words * 4, g.X + ((int64_t)nimg * g.H + h) * row_words,
-                          (uint32_t)(row_words * 4), raw_bar);
-    }
+    const uint32_t row_bytes = (uint32_t)(g.W * g.ldx) * 4u;
+    const int h0 = p0 - g.pad;
+    const int lo = h0 < 0 ? -h0 : 0;                               // rows lo .. hi - 1 lie in the image
+    const int hi = g.H - h0 < g.hr ? g.H - h0 : g.hr;
+    const uint32_t last = (uint32_t)(g.tail * g.ldx) * 4u;
+    const bool cut = h0 + hi == g.H;                               // the image's last row is among them
+    uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) * row_bytes : 0u;
+    if (cut && hi > lo) bytes -= row_bytes - last;
+    mbar_arrive_expect_tx(raw_bar, bytes);
+    const uint32_t* src = g.X + ((int64_t)nimg * g.H + h0 + lo) * (int64_t)(g.W * g.ldx);
+    for (int i = lo; i < hi; i++, src += g.W * g.ldx)
+        bulk_copy_g2s(raw + (size_t)i * row_bytes, src, cut && i + 1 == hi ? last : row_bytes, raw_bar);
 }
 
 // The decoders' share of one bulk-filled tile: items first, first + stride,
 // ... (zero codes for padding slots and rows outside the image).
 template <int B>
-__device__ __noinline__ void halo_decode(const HaloGeom g, int T, uint8_t* st, int first, int stride, int k, int ew)
+__device__ __forceinline__ void halo_decode(const HaloGeom& g, int p0, uint8_t* st, int first, int stride, int k, int ew,
+                                            uint32_t zw)
 {
-    const int nimg = T / g.tpi;
-    const int p0 = (T - nimg * g.tpi) * g.rows_out;
     const uint8_t* raw = st + g.planes_bytes;
     const int wsm = (1 << g.lws) - 1;
     const int npc = g.ldx >> 2;
     const uint32_t recip = 65536u / (uint32_t)npc + 1u;
-    const uint32_t zw = fmt_zero_word(B, k);
     const int items = g.ns * npc;
 #pragma unroll 1                                      // compact: it shares the SM's instruction cache
     for (int i = first; i < items; i += stride) {
@@ -196,10 +209,18 @@ __device__ __noinline__ void halo_decode(const HaloGeom g, int T, uint8_t* st, i
         const int hi = rel >> g.lws;
         const int j = rel & wsm;
         const int h = p0 - g.pad + hi;
-        const bool ok = rel >= 0 && hi < g.hr && j < g.W && (unsigned)h < (unsigned)g.H;
+        const bool ok = rel >= 0 && hi < g.hr && (unsigned)h < (unsigned)g.H && j < (h + 1 < g.H ? g.W : g.tail);
         const uint4* src = reinterpret_cast<const uint4*>(raw + ((size_t)hi * g.W + j) * g.ldx * 4);
         halo_store_piece<B>(st, g.pb, slot, pc, ok ? src[pc] : make_uint4(zw, zw, zw, zw), k, ew);
     }
+}
+
+// The same out of line, for the instances that hold every width.
+template <int B>
+__device__ __noinline__ void halo_decode_call(const HaloGeom g, int T, uint8_t* st, int first, int stride, int k, int ew)
+{
+    const int nimg = T / g.tpi;
+    halo_decode<B>(g, (T - nimg * g.tpi) * g.rows_out, st, first, stride, k, ew, fmt_zero_word(B, k));
 }
 
 template <bool FAST, bool GEN>
@@ -299,19 +320,29 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
             uint32_t ph = 0u;
             if (p == 0) {
                 if (lane == 0) {
-                    for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
+                    TileCursor tc((int)cta_in_n, (int)ctas_per_n, g.tpi);
+                    for (int64_t ti = 0; ti < my_tiles && !*err; ti++, tc.next()) {
                         if (!wait_or_abort(&empty[s], ph ^ 1u, err)) { *err = 1; break; }
-                        halo_issue_rows(g, cta_in_n + ti * ctas_per_n, sA + s * g.stage_bytes, &rawb[s]);
+                        halo_issue_rows(g, tc.img, tc.t * g.rows_out, sA + s * g.stage_bytes, &rawb[s]);
                         if (++s == stages) { s = 0; ph ^= 1u; }
                     }
                 }
             } else {
                 const int d = p - 1;                  // decoder index 0 .. kHaloDecoders - 1
                 auto decode_tiles = [&](auto width) {
+                    constexpr int B = decltype(width)::value;
+                    TileCursor tc((int)cta_in_n, (int)ctas_per_n, g.tpi);
+                    const uint32_t zw = fmt_zero_word(B, fa.k);
                     for (int64_t ti = 0; ti < my_tiles && !*err; ti++) {
                         if (!wait_or_abort(&rawb[s], ph, err)) { *err = 1; break; }
-                        halo_decode<decltype(width)::value>(g, (int)(cta_in_n + ti * ctas_per_n), sA + s * g.stage_bytes,
-                                                            d * 32 + lane, kHaloDecoders * 32, fa.k, fa.ew);
+                        uint8_t* const st = sA + s * g.stage_bytes;
+                        if (FAST) {
+                            halo_decode<B>(g, tc.t * g.rows_out, st, d * 32 + lane, kHaloDecoders * 32, fa.k, fa.ew, zw);
+                            tc.next();
+                        } else {
+                            halo_decode_call<B>(g, (int)(cta_in_n + ti * ctas_per_n), st, d * 32 + lane, kHaloDecoders * 32, fa.k,
+                                                fa.ew);
+                        }
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&full[s]);
@@ -419,15 +450,17 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
         ws_drain(drain, err, leader);
     } else if (warp < sp.warps) {
         // ---------------------------------------------- epilogue
-        const int ctas = (int)ctas_per_n, first = (int)cta_in_n;   // tile counts fit in 32 bits (host check)
-        const int tpi = g.tpi, rows_out = g.rows_out, lws = g.lws, P = g.P, Q = g.Q;
+        // tile counts fit in 32 bits (host check)
+        const int rows_out = g.rows_out, lws = g.lws, P = g.P, Q = g.Q, tpi = g.tpi;
+        const int qlast = g.tail < g.W ? g.tail : Q;              // outputs of the last row
+        const int ctas = (int)ctas_per_n, first = (int)cta_in_n;
         auto rows = [=](int64_t ti, int row, int64_t& m) -> bool {
             const int T = first + (int)ti * ctas;
             const int nimg = T / tpi;
             const int p = (T - nimg * tpi) * rows_out + (row >> lws);
             const int q = row & ((1 << lws) - 1);
             m = ((int64_t)nimg * P + p) * Q + q;
-            return q < Q && p < P;
+            return p < P && q < (p + 1 < P ? Q : qlast);
         };
         ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
@@ -448,7 +481,7 @@ constexpr double kHaloMinUse = 0.7;
 struct HaloPlan {
     HaloGeom g;
     int BN, nkb, stages;
-    int64_t K, smem;
+    int64_t K, smem, tiles;
 };
 
 // Static shared memory of the kernel (the larger of its two instances).
@@ -473,10 +506,28 @@ static int halo_static_smem(cudaError_t* err)
 // Geometry, N-tile width and shared-memory budget of the halo path, or
 // false when the shape does not suit it.  BN starts at bn0 and shrinks
 // (keeping whole output words) until the resident B and two halo stages fit.
-static bool halo_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, const OpFmt& fa, int bn0, int out_cpw,
+static bool halo_plan(const esb_conv_desc& d0, int P, int Q, int64_t ldx, const OpFmt& fa, int bn0, int out_cpw,
                       HaloPlan* hp, cudaError_t* err)
 {
     *err = cudaSuccess;
+    // A 1x1 filter sees no rows: its pixels are one image of rows of 128, so
+    // that every tile is full whatever the width.  With one channel block only:
+    // over several, image rows measured faster (28x28x144 -> 32: 12.0 against
+    // 13.6 us; 7x7x960 -> 160 on the im2col kernel 16 against 23 us), while
+    // 112x112x32 -> 16 gains 58 -> 51 us and 56x56x24 -> 144 33 -> 31.
+    esb_conv_desc d = d0;
+    hp->g.tail = d.w;
+    if (d.r == 1 && d.s == 1 && d.stride == 1 && d.pad == 0 && ldx <= 16) {
+        const int64_t pixels = (int64_t)d.n * d.h * d.w;
+        if (pixels >= (1ll << 30)) return false;
+        d.n = 1;
+        d.w = kBM;
+        d.h = (int)((pixels + kBM - 1) / kBM);
+        P = d.h;
+        Q = kBM;
+        hp->g.tail = (int)(pixels - (int64_t)(d.h - 1) * kBM);
+    }
+    hp->tiles = 0;
     // 4-bit codes, or 5/6-bit codes in the word-slot layout (8 K slots per
     // word, the same K per pixel word as 4-bit codes)
     const bool slot8 = fa.spw == 8 && (fa.b == 5 || fa.b == 6);
@@ -505,6 +556,7 @@ static bool halo_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, const O
     g.raw_bytes = (g.cblocks == 1) ? ((g.hr * d.w * (int)ldx * 4 + 127) / 128) * 128 : 0;
     g.stage_bytes = g.planes_bytes + g.raw_bytes;
     if ((int64_t)d.n * g.tpi >= (1ll << 30)) return false;
+    hp->tiles = (int64_t)d.n * g.tpi;
     const int st_smem = halo_static_smem(err);
     if (st_smem < 0) return false;
     const int maxs = max_dyn_smem() - st_smem;
@@ -562,7 +614,7 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     }
     const int64_t N = d.cout;
     const int n_tiles = (int)((N + hp.BN - 1) / hp.BN);
-    const int64_t m_tiles = (int64_t)d.n * hp.g.tpi;
+    const int64_t m_tiles = hp.tiles;
     int64_t per_n = device_sm_count() / n_tiles;
     if (per_n < 1) per_n = 1;
     if (per_n > m_tiles) per_n = m_tiles;

@@ -103,3 +103,22 @@ def test_tiled_gemm_packed_widths(M, N, K, f, monkeypatch):
     _, _, codes = esb.esb_gemm(Ad, esb.Fmt(f[0], f[1], False), Bd, esb.Fmt(*f), K, ep=ep, want_acc=False, want_codes=True,
                                workspace=ws[:16])
     assert np.array_equal(u32(codes), o.pack(want[1], fo[0], fo[1], ld_words=codes.shape[1]))
+
+
+@pytest.mark.parametrize("n,h,w,c,cout", [(1, 7, 9, 64, 40), (3, 17, 5, 24, 16), (2, 16, 8, 160, 96), (1, 1, 1, 32, 8)])
+@pytest.mark.parametrize("f", [(4, 2), (5, 2), (3, 1)])
+def test_pointwise_convolution_tiles_cross_rows_and_images(n, h, w, c, cout, f):
+    """1x1 filters on tiles of 128 consecutive pixels: ragged last tile, one
+    and several channel blocks, residual added."""
+    X, W = packed(n * h * w, c, f, 5, signed=False), packed(cout, c, f, 6)
+    res = packed(n * h * w, cout, f, 7)
+    fo = (f[0], f[1], True)
+    ep = esb.Epilogue(scale0=0.003, bias0=0.1, residual=dev_i32(res), res_fmt=esb.Fmt(*f), res_scale=0.05, alpha_out=0.5,
+                      fmt_out=esb.Fmt(*fo))
+    _, _, codes = esb.esb_conv2d_nhwc(dev_i32(X), esb.Fmt(f[0], f[1], False), dev_i32(W), esb.Fmt(*f), n, h, w, c, cout, 1, 1,
+                                      1, 0, ep=ep, want_acc=False, want_codes=True)
+    acc = o.gemm_i64(X, f, W, f, n * h * w, cout, c)
+    img = np.vectorize(lambda v: o.image(int(v), *f))(o.unpack(res, cout, f[0]))
+    _, co = o.epilogue(acc, np.full(cout, 0.003, np.float32), np.full(cout, 0.1, np.float32), esb.ESB_ACT_NONE, 0.5, fo,
+                       res_images=img, res_scale=0.05)
+    assert np.array_equal(u32(codes), o.pack(co, fo[0], fo[1], ld_words=codes.shape[1]))
