@@ -325,10 +325,9 @@ __device__ void tiled_chunked_epilogue(const EpiParams& ep, const float* thr, in
 template <bool LEAN4, bool GEN>
 __global__ void __launch_bounds__(kTiledThreads, 1)
 esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict__ Bt, int64_t M, int64_t N, int64_t mpad,
-                      int64_t npad, int nkb, int kbc, int nch, int BNr, int stages, int n_tiles, int64_t m_tiles,
+                      int64_t npad, int nkb, int kbc, int nch, int BN, int stages, int n_tiles, int64_t m_tiles,
                       float acc_scale, const __grid_constant__ EpiParams ep)
 {
-    const int BN = LEAN4 ? kTiledBN : BNr;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int kStage = kTileA + BN * kBK;                        // A tile then B tile (both 1024-aligned)
@@ -351,7 +350,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     const int64_t my_tiles = (m_tiles > cta_in_n) ? (m_tiles - cta_in_n + ctas_per_n - 1) / ctas_per_n : 0;
     uint32_t tmem_cols = 32;                                     // a power of two >= the regions used
     while (tmem_cols < (uint32_t)(nbuf * nch * BN)) tmem_cols <<= 1;
-    constexpr int lacc = 1;                              // nch == 1: two buffers (BN >= 240)
+    constexpr int lacc = 1;                              // nch == 1: two buffers
     const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -489,6 +488,26 @@ static bool tiled_plan(int64_t K, int ba, int ka, int bb, int kb, int out_cpw, i
     return *BN % out_cpw == 0;
 }
 
+// Narrower N-tiles when the widest would leave SMs idle (few row tiles: a
+// classifier at a small batch).  A CTA streams 128 + BN rows of each K-block,
+// so the width that minimises waves x (128 + BN); whole words per tile, at
+// least 64 columns, the wider on a tie.  The whole call at 256 x 4096 x 9216:
+// 37 us with 32 CTAs of 256 columns, 29 us with 128 CTAs of 64; 100 x 1000 x
+// 4096 of 6-bit codes with y: 153 and 62 us.
+static int tiled_bn(int64_t M, int64_t N, int bn0, int out_cpw)
+{
+    const int64_t sms = device_sm_count(), mt = cdiv(M, kBM);
+    if (mt * cdiv(N, bn0) >= sms) return bn0;
+    int best = bn0;
+    int64_t cbest = cdiv(mt * cdiv(N, bn0), sms) * (kBM + bn0);
+    for (int bn = bn0 - 16; bn >= 64; bn -= 16) {
+        if (bn % out_cpw) continue;
+        const int64_t c = cdiv(mt * cdiv(N, bn), sms) * (kBM + bn);
+        if (c < cbest) { cbest = c; best = bn; }
+    }
+    return best;
+}
+
 size_t gemm_tiled_workspace_bytes(int64_t M, int64_t N, int64_t K)
 {
     const int64_t nkb = cdiv(K, kBK);
@@ -565,6 +584,7 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     int kbc = 0, nch = 0, BN = 0;
     const int out_cpw = o.codes_out ? 32 / o.ep->fmt_out.b : 8;
     if (!tiled_plan(K, ba, ka, bb, kb, out_cpw, &kbc, &nch, &BN)) return cudaErrorInvalidValue;
+    if (nch == 1) BN = tiled_bn(M, N, BN, out_cpw);
     EpiParams ep = make_epi(o);
     ep.dq_pow2 = ldexpf(1.0f, -(ka + kb));
     ep.acc_lim = nch == 1 ? acc_fma_limit(K, ba, ka, bb, kb) : 0.0f;
@@ -604,7 +624,7 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     if (per_n > m_tiles) per_n = m_tiles;
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool fast = nch == 1 && BN == kTiledBN && lean4_ok(ep, N, BN);   // the specialised epilogue
+    const bool fast = nch == 1 && lean4_ok(ep, N, BN);   // the specialised epilogue
     // one chunk of other widths' codes only: the general-width epilogue instance
     const bool gen = nch == 1 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
     return launch_pdl(kTiledKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,
