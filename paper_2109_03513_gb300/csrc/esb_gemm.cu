@@ -989,9 +989,13 @@ static bool conv_force_im2col()
 // Words of each pixel that enter the implicit GEMM's K: all ldx of them
 // (the halo kernel and the 16-byte decode read whole 4-word pieces) unless
 // at least half are padding (a first layer's 3 channels in a 4-word row),
-// then only the words that hold channels.
+// then only the words that hold channels.  Four-word rows at stride 1 enter
+// whole all the same: that is one MMA step per tap on the halo kernel, which
+// decodes each pixel once (112 x 112 x 16 -> 96, 1x1: 91 us by single words on
+// the im2col kernel, 71 us there; -> 32, 3x3: 169 and 80 us).
 static int conv_k_words(const esb_conv_desc& d, int64_t ldx, int bx)
 {
+    if (d.stride == 1 && ldx == 4) return (int)ldx;
     const int cpw = 32 / bx;
     const int used = (d.c + cpw - 1) / cpw;
     return (2 * used <= ldx) ? used : (int)ldx;
