@@ -30,8 +30,8 @@ __device__ __forceinline__ void warp_granules(int64_t gran, int64_t& g_lo, int64
 // Codes of one granule (warp-collective): lane l turns its values 4l .. 4l
 // + 3 into 16 bits of codes, lane pairs (l, l + 1) join their halves into
 // code word 16 g + l / 2 with a shuffle.
-template <bool SIGNED>
-__device__ __forceinline__ void project_granule_b4(const float4 q, int64_t g, int64_t nw, const Thr7& t7, int k,
+template <bool SIGNED, class Tab>
+__device__ __forceinline__ void project_granule_b4(const float4 q, int64_t g, int64_t nw, const Tab& t7, int k,
                                                    uint32_t* __restrict__ codes)
 {
     const int lane = threadIdx.x & 31;
@@ -49,8 +49,8 @@ __device__ __forceinline__ void project_granule_b4(const float4 q, int64_t g, in
 }
 
 // One code word (8 values, 2 x float4) of a flat tensor.
-template <bool SIGNED>
-__device__ __forceinline__ uint32_t word_b4(const float4 qa, const float4 qb, const Thr7& t7, int k)
+template <bool SIGNED, class Tab>
+__device__ __forceinline__ uint32_t word_b4(const float4 qa, const float4 qb, const Tab& t7, int k)
 {
     const float v[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
     uint32_t J = 0u, S = 0u;
@@ -68,8 +68,8 @@ __device__ __forceinline__ uint32_t word_b4(const float4 qa, const float4 qb, co
 // each warp reads its first `stash_g` granules from its shared-memory stash
 // (written by that pass) and the rest in batches of 8 coalesced 16-byte
 // loads per lane; the last warp also takes the partial granule at the end.
-template <bool SIGNED, bool STREAM>
-__device__ __forceinline__ void project_flat_b4(const float* __restrict__ x, int64_t n, const Thr7& t7, int k,
+template <bool SIGNED, bool STREAM, class Tab>
+__device__ __forceinline__ void project_flat_b4(const float* __restrict__ x, int64_t n, const Tab& t7, int k,
                                                 uint32_t* __restrict__ codes, const float4* stash = nullptr,
                                                 int stash_g = 0)
 {
@@ -182,8 +182,15 @@ project_vec_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
     const uint32_t amask = p.is_signed ? 0x7fffffffu : 0xffffffffu;
 
     if (B == 4 && flat) {                                 // flat codes: coalesced warp tiles
-        if (p.is_signed) project_flat_b4<true, true>(x, rows * cols, t7, p.k, codes);
-        else project_flat_b4<false, true>(x, rows * cols, t7, p.k, codes);
+        __shared__ uint2 lin_tab[B == 4 ? kLinCells : 1];
+        Lin7 lin;
+        if (build_lin7(lin_tab, lin, T)) {
+            if (p.is_signed) project_flat_b4<true, true>(x, rows * cols, lin, p.k, codes);
+            else project_flat_b4<false, true>(x, rows * cols, lin, p.k, codes);
+        } else {
+            if (p.is_signed) project_flat_b4<true, true>(x, rows * cols, t7, p.k, codes);
+            else project_flat_b4<false, true>(x, rows * cols, t7, p.k, codes);
+        }
         return;
     }
 
@@ -953,8 +960,15 @@ calibrate_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols
 #pragma unroll
         for (int i = 0; i < 7; i++) t7.t[i] = T[i];
         if (flat) {                                     // flat codes: the statistics pass's granules
-            if (p.is_signed) project_flat_b4<true, true>(x, n, t7, p.k, codes, stash, stash_g);
-            else project_flat_b4<false, true>(x, n, t7, p.k, codes, stash, stash_g);
+            __shared__ uint2 lin_tab[B == 4 ? kLinCells : 1];
+            Lin7 lin;
+            if (build_lin7(lin_tab, lin, T)) {
+                if (p.is_signed) project_flat_b4<true, true>(x, n, lin, p.k, codes, stash, stash_g);
+                else project_flat_b4<false, true>(x, n, lin, p.k, codes, stash, stash_g);
+            } else {
+                if (p.is_signed) project_flat_b4<true, true>(x, n, t7, p.k, codes, stash, stash_g);
+                else project_flat_b4<false, true>(x, n, t7, p.k, codes, stash, stash_g);
+            }
             cal_depart(sync);
             return;
         }

@@ -34,3 +34,24 @@ def test_project_any_rows(b, k, signed, rows, cols, ldc_extra, shift):
         esb.esb_project(xd, esb.Fmt(b, k, signed), alpha=alpha, rounding=rows & 1, codes=out, ldc=ldc)
         exp = o.project_packed(x.numpy(), np.float32(alpha), b, k, signed=signed, rounding=rows & 1, ld_words=ldc)
         assert np.array_equal(out.cpu().numpy().view(np.uint32), exp)
+
+
+@pytest.mark.parametrize("k", [0, 1, 2, 3])
+@pytest.mark.parametrize("signed", [True, False])
+@pytest.mark.parametrize("alpha", [0.37, 1.0, 3e31, 1e-31, 1e-40])
+def test_project_flat_4bit_cell_table(k, signed, alpha):
+    """Flat 4-bit projection: every threshold, its neighbours one ulp away,
+    zeros, infinities and NaN; alphas whose thresholds leave the table's range
+    keep the register search."""
+    a = np.float32(alpha)
+    q = o.set_nonneg(4, k).astype(np.float64)
+    t = (0.5 * (q[1:] + q[:-1]) * float(a)).astype(np.float32)
+    bits = t.view(np.uint32).astype(np.int64)
+    near = np.concatenate([bits + d for d in range(-3, 4)]).clip(0, 0x7F7FFFFF).astype(np.uint32).view(np.float32)
+    x = np.concatenate([near, -near, np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-45, 3e38], np.float32),
+                        (synth.normal((3000,), seed=k).numpy() * 4 * a).astype(np.float32)])
+    x = np.concatenate([x, np.zeros(-x.size % 128 + 64, np.float32)])[: (x.size + 63) // 8 * 8]
+    for rounding in (0, 1):
+        codes = esb.esb_project(torch.from_numpy(x).cuda(), esb.Fmt(4, k, signed), alpha=float(a), rounding=rounding, ldc=x.size // 8)
+        exp = o.project_packed(x, a, 4, k, signed=signed, rounding=rounding, ld_words=x.size // 8)
+        assert np.array_equal(codes.cpu().numpy().view(np.uint32), exp)
