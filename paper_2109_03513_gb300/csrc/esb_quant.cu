@@ -249,20 +249,17 @@ project_vec_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
         });
 }
 
-// General path: any alignment and strides.  The projection of one value: the
-// register bucket search for b = 4, the cell table for the other widths
-// (their bisection when the table does not hold).
-//
-// Rows of at most two code words (ROWS; an image's 3 channels in 4-word
-// rows): a thread per row, every word of it written by that thread, 16 bytes
-// at a time where the rows allow.  Longer rows: a warp takes 32 words of one
-// row, codes its values with coalesced loads and packs them through shared
-// memory.  Both HBM-bound in principle; 3.2 M rows of 3 values: 106 us with a
-// thread per word (three of four words all padding, and a 64-bit division and
-// eight predicated bisections for each), 24 us with a thread per row.
-template <int B, bool ROWS>
+// Rows of at most two code words, any alignment and strides (an image's 3
+// channels in 4-word rows): a thread per row, every word of it written by that
+// thread, 16 bytes at a time where the rows allow.  3.2 M rows of 3 values: 106
+// us with a thread per word (three of four words all padding, and a 64-bit
+// division and eight predicated bisections for each), 24 us this way; rows of
+// 9 values 50 and 15 us.  Longer rows stay with a thread per word, whose
+// neighbours share cache lines: warp segments packed through shared memory
+// took 20 us there against 16 at 1001 columns, 81 against 27 at 17.
+template <int B>
 __global__ void __launch_bounds__(256)
-project_any_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ldx,
+project_rows_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ldx,
                    float alpha, const float* __restrict__ alpha_dev, ProjParams p,
                    uint32_t* __restrict__ codes, int64_t ldc, int vec)
 {
@@ -271,7 +268,6 @@ project_any_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
     constexpr int CAP = B <= 6 ? 1024 : 2048;
     __shared__ float T[L];
     __shared__ uint2 cells[B == 4 ? 1 : CAP];
-    __shared__ uint8_t seg[ROWS ? 1 : 8][ROWS ? 1 : 32 * CPW];
     const float a = alpha_dev ? __ldg(alpha_dev) : alpha;
     build_thresholds(T, p, a, threadIdx.x >> 5, threadIdx.x & 31, 0, blockDim.x >> 5);
     __syncthreads();
@@ -289,62 +285,66 @@ project_any_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
     uint32_t zw = 0u;
 #pragma unroll
     for (int j = 0; j < CPW; j++) zw |= p.zero_code << (B * j);
-    if (ROWS) {
-        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-        const int used = cols > CPW ? 2 : 1;
-        for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += stride) {
-            const float* xr = x + r * ldx;
-            uint32_t* cr = codes + r * ldc;
-            uint32_t w[2] = {zw, zw};
-            for (int i = 0; i < used; i++) {
-                const int left = (int)cols - i * CPW; // values of this word
-                float v[CPW];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int used = cols > CPW ? 2 : 1;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += stride) {
+        const float* xr = x + r * ldx;
+        uint32_t* cr = codes + r * ldc;
+        uint32_t w[2] = {zw, zw};
+        for (int i = 0; i < used; i++) {
+            const int left = (int)cols - i * CPW; // values of this word
+            float v[CPW];
 #pragma unroll
-                for (int j = 0; j < CPW; j++) v[j] = j < left ? __ldg(xr + i * CPW + j) : 0.0f;
-                uint32_t word = 0u;
-#pragma unroll
-                for (int j = 0; j < CPW; j++) {
-                    if (j >= left) break;
-                    word |= code_of(v[j]) << (B * j);
-                }
-                if (left < CPW) {
-                    const uint32_t keep = left > 0 ? (1u << (B * left)) - 1u : 0u;
-                    word = (word & keep) | (zw & ~keep);
-                }
-                w[i] = word;
-            }
-            if (vec) {                                // 16-byte rows
-                *reinterpret_cast<uint4*>(cr) = make_uint4(w[0], w[1], zw, zw);
-                for (int64_t q = 4; q < ldc; q += 4) *reinterpret_cast<uint4*>(cr + q) = make_uint4(zw, zw, zw, zw);
-            } else {
-                cr[0] = w[0];
-                if (ldc > 1) cr[1] = w[1];
-                for (int64_t q = 2; q < ldc; q++) cr[q] = zw;
-            }
-        }
-        return;
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t* sg = seg[ROWS ? 0 : warp];
-    const int64_t tpr = (ldc + 31) / 32;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; t < rows * tpr; t += nwarps) {
-        const int64_t r = tpr == 1 ? t : t / tpr;
-        const int64_t w0 = (t - r * tpr) * 32;
-        const int64_t c0 = w0 * CPW;
-        const int left = (int)(cols - c0 < 32 * CPW ? (cols > c0 ? cols - c0 : 0) : 32 * CPW);
-        const float* xr = x + r * ldx + c0;
-        const int top = (int)(ldc - w0 < 32 ? (ldc - w0) * CPW : 32 * CPW);   // codes of the segment's words
-#pragma unroll 4
-        for (int i = lane; i < top; i += 32) sg[i] = (uint8_t)(i < left ? code_of(__ldg(xr + i)) : p.zero_code);
-        __syncwarp();
-        if (w0 + lane < ldc) {
+            for (int j = 0; j < CPW; j++) v[j] = j < left ? __ldg(xr + i * CPW + j) : 0.0f;
             uint32_t word = 0u;
 #pragma unroll
-            for (int j = 0; j < CPW; j++) word |= (uint32_t)sg[lane * CPW + j] << (B * j);
-            codes[r * ldc + w0 + lane] = word;
+            for (int j = 0; j < CPW; j++) {
+                if (j >= left) break;
+                word |= code_of(v[j]) << (B * j);
+            }
+            if (left < CPW) {
+                const uint32_t keep = left > 0 ? (1u << (B * left)) - 1u : 0u;
+                word = (word & keep) | (zw & ~keep);
+            }
+            w[i] = word;
         }
-        __syncwarp();
+        if (vec) {                                // 16-byte rows
+            *reinterpret_cast<uint4*>(cr) = make_uint4(w[0], w[1], zw, zw);
+            for (int64_t q = 4; q < ldc; q += 4) *reinterpret_cast<uint4*>(cr + q) = make_uint4(zw, zw, zw, zw);
+        } else {
+            cr[0] = w[0];
+            if (ldc > 1) cr[1] = w[1];
+            for (int64_t q = 2; q < ldc; q++) cr[q] = zw;
+        }
+    }
+}
+
+// General path: any alignment and strides; one thread per code word.
+template <int B>
+__global__ void __launch_bounds__(256)
+project_any_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ldx,
+                   float alpha, const float* __restrict__ alpha_dev, ProjParams p,
+                   uint32_t* __restrict__ codes, int64_t ldc)
+{
+    constexpr int CPW = 32 / B;
+    constexpr int L = 1 << (B - 1);
+    __shared__ float T[L];
+    const float a = alpha_dev ? __ldg(alpha_dev) : alpha;
+    build_thresholds(T, p, a, threadIdx.x >> 5, threadIdx.x & 31, 0, blockDim.x >> 5);
+    __syncthreads();
+    const int64_t total = rows * ldc;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += stride) {
+        const int64_t r = u / ldc;
+        const int64_t w = u - r * ldc;
+        uint32_t word = 0;
+#pragma unroll
+        for (int j = 0; j < CPW; j++) {
+            const int64_t c = w * CPW + j;
+            const uint32_t code = (c < cols) ? project_by_table_t<B>(x[r * ldx + c], T, p) : p.zero_code;
+            word |= code << (B * j);
+        }
+        codes[u] = word;  // row-major: r * ldc + w == u
     }
 }
 
@@ -368,14 +368,17 @@ static cudaError_t launch_project_b(const float* x, int64_t rows, int64_t cols, 
         project_vec_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc);
     } else {
         const bool by_rows = cols <= 2 * (32 / B);
-        const int64_t units = by_rows ? rows : rows * ((ldc + 31) / 32) * 32;
+        const int64_t units = by_rows ? rows : rows * ldc;
         int64_t blocks = (units + threads - 1) / threads;
         const int64_t cap = (int64_t)sms * 8;
         if (blocks > cap) blocks = cap;
         if (blocks < 1) blocks = 1;
-        const int v16 = ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
-        auto kernel = by_rows ? project_any_kernel<B, true> : project_any_kernel<B, false>;
-        kernel<<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc, v16);
+        if (by_rows) {
+            const int v16 = ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
+            project_rows_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc, v16);
+        } else {
+            project_any_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc);
+        }
     }
     return cudaGetLastError();
 }

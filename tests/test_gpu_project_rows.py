@@ -1,5 +1,6 @@
-"""Projection of rows that no 16-byte path takes: a thread per short row, and
-warp segments of longer ones, at every width, odd strides and alignments."""
+"""Projection of rows that no 16-byte path takes, a thread per short row and a
+thread per word of longer ones, at every width, odd strides and alignments;
+and the cell table of flat 4-bit rows."""
 import numpy as np
 import pytest
 import torch
