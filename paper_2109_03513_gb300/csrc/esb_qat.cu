@@ -50,6 +50,7 @@ struct DnTable {
     float xq[1 << B];
 };
 
+enum { kDnSegments = 0, kDnFlat = 1, kDnWords = 2 };
 constexpr int kDnUnroll = 6;       // granules in flight per warp (flat 4-bit path)
 
 // One value by division, for a sigma that is not finite (or +-0 with eps lost).
@@ -61,7 +62,7 @@ __device__ __noinline__ uint32_t dn_code_div(float x, float m, float s, float al
 template <int B>
 __global__ void __launch_bounds__(kQatThreads)
 dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const double* __restrict__ stats,
-                  float alpha, ProjParams p, uint32_t* __restrict__ codes, int64_t ldc, float* __restrict__ xq, int flat)
+                  float alpha, ProjParams p, uint32_t* __restrict__ codes, int64_t ldc, float* __restrict__ xq, int mode)
 {
     constexpr int CPW = 32 / B;
     constexpr int L = 1 << (B - 1);
@@ -101,7 +102,7 @@ dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const
     };
     const int64_t gwarp = (int64_t)blockIdx.x * (kQatThreads / 32) + warp;
     const int64_t nwarps = (int64_t)gridDim.x * (kQatThreads / 32);
-    if (B == 4 && flat) {
+    if (B == 4 && mode == kDnFlat) {
         // granules of 128 values: lane l takes values 4l .. 4l + 3, lane
         // pairs join their halves of a code word
         const int64_t n = rows * cols;                // a multiple of 8
@@ -142,7 +143,28 @@ dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const
         }
         return;
     }
-    // general path: a warp takes 32 words of one row, codes its values with
+    if (mode == kDnWords) {
+        // rows of fewer words than a warp has lanes: a thread per word
+        const int64_t total = rows * ldc, stride = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += stride) {
+            const int64_t r = u < (1ll << 32) && ldc < (1ll << 31) ? (int64_t)((uint32_t)u / (uint32_t)ldc) : u / ldc;
+            const int64_t c0 = (u - r * ldc) * CPW;
+            const float* xr = x + r * cols + c0;
+            uint32_t word = 0u;
+#pragma unroll
+            for (int j = 0; j < CPW; j++) {
+                uint32_t code = p.zero_code;
+                if (c0 + j < cols) {
+                    code = code_of(__ldg(xr + j));
+                    if (xq) xq[r * cols + c0 + j] = sm.xq[code];
+                }
+                word |= code << (B * j);
+            }
+            codes[u] = word;
+        }
+        return;
+    }
+    // longer rows: a warp takes 32 words of one row, codes its values with
     // coalesced loads, then packs them through shared memory
     const int64_t tpr = (ldc + 31) / 32;
     uint8_t* sg = seg[warp];
@@ -403,12 +425,14 @@ cudaError_t launch_dn_project(const float* x, int64_t rows, int64_t cols, const 
     const ProjParams p = make_proj_params(b, k, is_signed, rounding);
     auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     const int flat = b == 4 && ldc * 8 == cols && al16(x) && (!xq || al16(xq));
-    int64_t blocks = qat_blocks(flat ? rows * cols / 4 : rows * ((ldc + 31) / 32) * 32) * 2;
+    const int mode = flat ? kDnFlat : (ldc < 32 ? kDnWords : kDnSegments);
+    const int64_t units = mode == kDnFlat ? rows * cols / 4 : mode == kDnWords ? rows * ldc : rows * ((ldc + 31) / 32) * 32;
+    const int64_t blocks = (int64_t)qat_blocks(units) * 2;
     using Kernel = void (*)(const float*, int64_t, int64_t, const double*, float, ProjParams, uint32_t*, int64_t, float*, int);
     static const Kernel kernels[] = {dn_project_kernel<2>, dn_project_kernel<3>, dn_project_kernel<4>, dn_project_kernel<5>,
                                      dn_project_kernel<6>, dn_project_kernel<7>, dn_project_kernel<8>};
     return launch_pdl(kernels[b - 2], dim3((unsigned)blocks), dim3(kQatThreads), 0, st, x, rows, cols, stats, alpha, p,
-                      codes, ldc, xq, flat);
+                      codes, ldc, xq, mode);
 }
 
 cudaError_t launch_dn_grad(const float* g, const float* x, int64_t n, const double* stats, void* workspace, float* gx,
