@@ -247,12 +247,13 @@ dn_grad_partials_kernel(const float* __restrict__ g, const float* __restrict__ x
         }
     }
     for (int64_t i = nv * 4 + t0; i < n; i += stride) add(g[i], x[i]);
-    const bool ok = fabsf(s1h + s1l) < __int_as_float(0x7f800000) && fabsf(s2h + s2l) < __int_as_float(0x7f800000) &&
-                    (mx == 0.0f || mx > 0x1p-40f) && stats_ok;
+    auto finite = [&]() { return fabsf(s1h + s1l) < __int_as_float(0x7f800000) && fabsf(s2h + s2l) < __int_as_float(0x7f800000); };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (__all_sync(0xffffffffu, ok)) {
+    bool pairs = __all_sync(0xffffffffu, finite() && (mx == 0.0f || mx > 0x1p-40f) && stats_ok);
+    if (pairs) {
         // the warp's sums in pairs; fp64 only once per warp (its pipe takes
-        // a block's worth of conversions and adds longer than the loads)
+        // a block's worth of conversions and adds longer than the loads).
+        // Lanes whose own sums are finite can still overflow together.
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float a = __shfl_xor_sync(0xffffffffu, s1h, o), b = __shfl_xor_sync(0xffffffffu, s1l, o);
@@ -260,6 +261,9 @@ dn_grad_partials_kernel(const float* __restrict__ g, const float* __restrict__ x
             df_add(s1h, s1l, a); s1l += b;
             df_add(s2h, s2l, c); s2l += d;
         }
+        pairs = __all_sync(0xffffffffu, finite());
+    }
+    if (pairs) {
         if (lane == 0) sh[warp] = make_double2((double)s1h + (double)s1l, (double)s2h + (double)s2l);
     } else {                                          // this warp's elements again in fp64
         const double mu = __ldg(stats);

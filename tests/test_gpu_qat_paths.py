@@ -69,3 +69,26 @@ def test_dn_backward_ranges(n, shift, kind):
     mean_err = 2.0 ** -40 * float(gc.abs().mean()) / s
     tol = 2.0 ** -24 * exp.abs() + 2.0 ** -40 * (t1.abs() + t2.abs()) + mean_err + 2.0 ** -149
     assert bool(((got - exp).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("n", [5, 4097, 70001])
+@pytest.mark.parametrize("kind", ["g", "gx"])
+def test_dn_backward_sums_that_overflow_between_lanes(n, kind):
+    """Every lane's own sum is finite in fp32 but a warp's is not: the sum of
+    g (constant 2e37), or only that of g (x - mu) (g = 1e37 (x - mu) alternating
+    in sign, so that g itself sums to about zero)."""
+    x = synth.normal((n,), seed=n, mean=0.4, std=1.3)
+    if kind == "g":
+        g = torch.full((n,), 2e37)
+    else:
+        x = 0.4 + 1.3 * (1.0 - 2.0 * (torch.arange(n) % 2)).float()
+        g = 1e37 * (x - 0.4)
+    xc, gc = x.double(), g.double()
+    mu, sg = float(xc.mean()), float((xc - xc.mean()).square().mean().sqrt())
+    got = esb.esb_dn_backward(g.cuda(), x.cuda(), torch.tensor([mu, sg], dtype=torch.float64, device="cuda")).cpu().double()
+    s, c = sg + 1e-7, xc - mu
+    t1, t2 = (gc - gc.mean()) / s, c * ((gc * c).sum() / (n * sg * s * s))
+    # recomputed in fp64: the sums are trees of some 30 levels (2^-48 of the magnitudes summed), and
+    # |x - mu| is at most about 4 sigma
+    tol = 2.0 ** -24 * (t1 - t2).abs() + 2.0 ** -44 * (t1.abs() + t2.abs() + float(gc.abs().mean()) / s)
+    assert bool(((got - (t1 - t2)).abs() <= tol).all())
