@@ -986,19 +986,21 @@ static bool conv_force_im2col()
     return v != 0;
 }
 
-// Words of each pixel that enter the implicit GEMM's K: all ldx of them
-// (the halo kernel and the 16-byte decode read whole 4-word pieces) unless
-// at least half are padding (a first layer's 3 channels in a 4-word row),
-// then only the words that hold channels.  Four-word rows at stride 1 enter
-// whole all the same: that is one MMA step per tap on the halo kernel, which
-// decodes each pixel once (112 x 112 x 16 -> 96, 1x1: 91 us by single words on
-// the im2col kernel, 71 us there; -> 32, 3x3: 169 and 80 us).
-static int conv_k_words(const esb_conv_desc& d, int64_t ldx, int bx)
+// Words of each pixel that enter the implicit GEMM's K: all ldx of them, or
+// the filter's ldw where its rows are shorter (the halo kernel and the 16-byte
+// decode read whole 4-word pieces), unless at least half are padding (a first
+// layer's 3 channels in a 4-word row), then only the words that hold channels.
+// Four-word rows at stride 1 enter whole all the same: that is one MMA step
+// per tap on the halo kernel, which decodes each pixel once (112 x 112 x 16 ->
+// 96, 1x1: 91 us by single words on the im2col kernel, 71 us there; -> 32,
+// 3x3: 169 and 80 us).
+static int conv_k_words(const esb_conv_desc& d, int64_t ldx, int bx, int64_t ldw, int bw)
 {
     if (d.stride == 1 && ldx == 4) return (int)ldx;
     const int cpw = 32 / bx;
     const int used = (d.c + cpw - 1) / cpw;
-    return (2 * used <= ldx) ? used : (int)ldx;
+    const int whole = (int)((bw == bx && ldw < ldx) ? ldw : ldx);   // no tap may run past its filter words
+    return (2 * used <= ldx) ? used : whole;
 }
 
 // Filter rows of the im2col K: plain rows when every tap's ldx input words
@@ -1025,7 +1027,7 @@ cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t*
     ep.acc_lim = acc_fma_limit((int64_t)d.r * d.s * d.c, bx, kx, bw, kw);   // padding slots add exact zeros
     const int64_t M = (int64_t)d.n * P * Q;
     const int64_t N = d.cout;
-    const int kwx = conv_k_words(d, ldx, bx);
+    const int kwx = conv_k_words(d, ldx, bx, ldw, bw);
     const int64_t K = (int64_t)d.r * d.s * kwx * (32 / bx);
     const int BN = pick_bn(N, ep.out_cpw);
     ConvSrc a;
@@ -1052,7 +1054,7 @@ int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx
                        int kw, int out_b)
 {
     const int cpw = 32 / out_b;
-    const int kwd = conv_k_words(d, ldx, bx);
+    const int kwd = conv_k_words(d, ldx, bx, ldw, bw);
     const int64_t K = (int64_t)d.r * d.s * kwd * (32 / bx);
     OpFmt fa = make_opfmt(bx, kx), fb = make_opfmt(bw, kw);
     int64_t Kx = plan_planes(fa, fb, K);
