@@ -986,17 +986,12 @@ static bool conv_force_im2col()
     return v != 0;
 }
 
-// Words of each pixel that enter the implicit GEMM's K: all ldx of them, or
-// the filter's ldw where its rows are shorter (the halo kernel and the 16-byte
-// decode read whole 4-word pieces), unless at least half are padding (a first
+// Words of each pixel that enter the implicit GEMM's K on the im2col kernels:
+// all ldx of them, or the filter's ldw where its rows are shorter (the 16-byte
+// decode reads whole 4-word pieces), unless at least half are padding (a first
 // layer's 3 channels in a 4-word row), then only the words that hold channels.
-// Four-word rows at stride 1 enter whole all the same: that is one MMA step
-// per tap on the halo kernel, which decodes each pixel once (112 x 112 x 16 ->
-// 96, 1x1: 91 us by single words on the im2col kernel, 71 us there; -> 32,
-// 3x3: 169 and 80 us).
 static int conv_k_words(const esb_conv_desc& d, int64_t ldx, int bx, int64_t ldw, int bw)
 {
-    if (d.stride == 1 && ldx == 4) return (int)ldx;
     const int cpw = 32 / bx;
     const int used = (d.c + cpw - 1) / cpw;
     const int whole = (int)((bw == bx && ldw < ldx) ? ldw : ldx);   // no tap may run past its filter words
@@ -1019,6 +1014,74 @@ static RowsSrc conv_filter_rows(const esb_conv_desc& d, const uint32_t* W, int64
     return b;
 }
 
+// The contraction of a convolution whose taps take kwx words of each pixel:
+// the filter rows, the operands' formats and the kernels' K.
+struct ConvK {
+    RowsSrc b;
+    OpFmt fa, fb;
+    int64_t K;
+};
+
+static ConvK conv_k(const esb_conv_desc& d, const uint32_t* W, int64_t ldx, int bx, int kx, int64_t ldw, int bw, int kw, int kwx)
+{
+    ConvK c{conv_filter_rows(d, W, ldx, bx, ldw, bw, kwx), make_opfmt(bx, kx), make_opfmt(bw, kw), 0};
+    const int64_t words = (int64_t)d.r * d.s * kwx;
+    c.K = plan_planes(c.fa, c.fb, words * (32 / bx));             // significand planes
+    if (c.b.linear()) {
+        if (const int64_t Ks = plan_slots(c.fa, c.fb, words * c.fa.cpw, words)) c.K = Ks;
+    }
+    return c;
+}
+
+// The halo kernel takes whole pixel rows.  Four-word rows are that to it
+// whatever they hold: one MMA step per tap, and each pixel decoded once (112 x
+// 112 x 16 -> 96, 1x1: 91 us by single words on the im2col kernel, 71 us there;
+// -> 32, 3x3: 169 and 80 us).
+static bool conv_halo_rows(const ConvK& c) { return c.K > 0 && c.fa.planes == 1 && c.b.kp == 0; }
+static int conv_halo_words(const esb_conv_desc& d, int64_t ldx, int kwx) { return d.stride == 1 && ldx == 4 ? 4 : kwx; }
+
+// Stride-1 layers of four-word rows that the halo kernel refuses (wide images,
+// odd sizes) on the im2col kernel: the whole row in K by 16-byte pieces, or the
+// kwx words that hold channels one by one.  Whole rows take up to four times
+// the K-blocks, each several times cheaper and with a prologue some 7 us
+// shorter, so they lose only where a pixel has one word of channels and a CTA
+// many K-blocks, and where the filters then no longer stay resident.  Measured,
+// whole and by words, 4-bit (K-blocks of a CTA's tiles by whole rows in front):
+//   12: 3x3, 33 x 33 x 3 -> 64, batch 64      16.7 and 20.9 us
+//   26: 7x7, 20 x 20 x 3 -> 32, batch 64      21.7 and 26.9
+//   62: 11x11, 20 x 20 x 3 -> 32, batch 64    52.5 and 47.5
+//   63: 3x3, 224 x 224 x 3 -> 64, batch 8     59.2 and 54.1
+//   70: 5x5, 150 x 150 x 3 -> 16, batch 8     51.9 and 49.7
+//   63, two words of channels: 3x3, 224 x 224 x 16 -> 64    59.2 and 99.3
+//   not resident: 11x11, 200 x 200 x 3 -> 64, batch 4       254 and 191
+// Significand planes and filters of another width do not decode by pieces
+// (3x3, 56 x 56 x 3 -> 32, (8,5): 706 us whole, 301 by words).
+static bool conv_whole_pays(const esb_conv_desc& d, int64_t M, const ConvK& whole, int kwx, int out_cpw)
+{
+    cudaError_t e = cudaSuccess;
+    const int st = ws_static_smem<ConvSrc>(&e);
+    const int bn = resident_bn(M, d.cout, out_cpw, pick_bn(d.cout, out_cpw));   // as launch_ws
+    if (!conv_halo_rows(whole) || st < 0 || ws_layout(whole.K, bn, max_dyn_smem() - st).stages < 3) return false;
+    const int64_t sms = device_sm_count(), tiles = ((M + kBM - 1) / kBM) * ((d.cout + bn - 1) / bn);
+    return kwx > 1 || (tiles + sms - 1) / sms * ((whole.K + kBK - 1) / kBK) <= 48;
+}
+
+// The im2col kernels' contraction; *kwx: words of each pixel in K.
+static ConvK conv_im2col(const esb_conv_desc& d, int64_t M, const uint32_t* W, int64_t ldx, int bx, int kx, int64_t ldw, int bw,
+                         int kw, int out_cpw, int* kwx)
+{
+    *kwx = conv_k_words(d, ldx, bx, ldw, bw);
+    const int whole = conv_halo_words(d, ldx, *kwx);
+    if (whole != *kwx) {
+        const ConvK c = conv_k(d, W, ldx, bx, kx, ldw, bw, kw, whole);
+        if (conv_whole_pays(d, M, c, *kwx, out_cpw)) {
+            *kwx = whole;
+            return c;
+        }
+    }
+    return conv_k(d, W, ldx, bx, kx, ldw, bw, kw, *kwx);
+}
+
 cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, int bx, int kx,
                            const uint32_t* W, int64_t ldw, int bw, int kw, const GemmOutputs& o, cudaStream_t st)
 {
@@ -1027,51 +1090,39 @@ cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t*
     ep.acc_lim = acc_fma_limit((int64_t)d.r * d.s * d.c, bx, kx, bw, kw);   // padding slots add exact zeros
     const int64_t M = (int64_t)d.n * P * Q;
     const int64_t N = d.cout;
-    const int kwx = conv_k_words(d, ldx, bx, ldw, bw);
-    const int64_t K = (int64_t)d.r * d.s * kwx * (32 / bx);
     const int BN = pick_bn(N, ep.out_cpw);
+    cudaError_t e = cudaSuccess;
+    if (!conv_force_im2col()) {
+        if (launch_conv_stem(d, P, Q, X, ldx, make_opfmt(bx, kx), W, ldw, make_opfmt(bw, kw), BN, ep, st, &e)) return e;
+        const ConvK h = conv_k(d, W, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
+        if (conv_halo_rows(h) && launch_conv_halo(d, P, Q, X, ldx, h.fa, W, ldw, h.fb, BN, ep, st, &e)) return e;
+    }
+    int kwx;
+    const ConvK c = conv_im2col(d, M, W, ldx, bx, kx, ldw, bw, kw, ep.out_cpw, &kwx);
     ConvSrc a;
     a.X = X; a.ldx = (int)ldx; a.rows = (int)M; a.H = d.h; a.W = d.w; a.P = P; a.Q = Q; a.R = d.r; a.S = d.s;
     a.stride = d.stride; a.pad = d.pad; a.kw = kwx;
-    RowsSrc b = conv_filter_rows(d, W, ldx, bx, ldw, bw, kwx);
-    OpFmt fa = make_opfmt(bx, kx), fb = make_opfmt(bw, kw);
-    int64_t Kx = plan_planes(fa, fb, K);              // the kernels' K (significand planes)
-    if (b.linear()) {
-        const int64_t words = (int64_t)d.r * d.s * kwx;
-        if (const int64_t Ks = plan_slots(fa, fb, words * fa.cpw, words)) Kx = Ks;
-    }
-    cudaError_t e = cudaSuccess;
-    if (!conv_force_im2col() && launch_conv_stem(d, P, Q, X, ldx, make_opfmt(bx, kx), W, ldw, make_opfmt(bw, kw), BN, ep, st, &e))
-        return e;
-    if (Kx > 0 && !conv_force_im2col() && fa.planes == 1 && b.kp == 0 &&
-        launch_conv_halo(d, P, Q, X, ldx, fa, W, ldw, fb, BN, ep, st, &e))
-        return e;
-    if (Kx > 0 && launch_ws(a, b, M, N, Kx, fa, fb, BN, ep, st, &e)) return e;
-    return launch_tc(a, b, M, N, Kx, fa, fb, BN, ep, st);
+    if (c.K > 0 && launch_ws(a, c.b, M, N, c.K, c.fa, c.fb, BN, ep, st, &e)) return e;
+    return launch_tc(a, c.b, M, N, c.K, c.fa, c.fb, BN, ep, st);
 }
 
 int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int64_t ldw, int bw,
                        int kw, int out_b)
 {
-    const int cpw = 32 / out_b;
-    const int kwd = conv_k_words(d, ldx, bx, ldw, bw);
-    const int64_t K = (int64_t)d.r * d.s * kwd * (32 / bx);
-    OpFmt fa = make_opfmt(bx, kx), fb = make_opfmt(bw, kw);
-    int64_t Kx = plan_planes(fa, fb, K);
-    const RowsSrc b = conv_filter_rows(d, nullptr, ldx, bx, ldw, bw, kwd);
-    const bool same_layout = b.kp == 0 && fa.planes == 1;
-    if (b.linear()) {                                 // as launch_conv_tc
-        const int64_t words = (int64_t)d.r * d.s * kwd;
-        if (const int64_t Ks = plan_slots(fa, fb, words * fa.cpw, words)) Kx = Ks;
+    const int cpw = 32 / out_b;                                   // as launch_conv_tc
+    if (!conv_force_im2col()) {
+        if (conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, cpw)) return ESB_CONV_KERNEL_STEM;
+        const ConvK h = conv_k(d, nullptr, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
+        if (conv_halo_rows(h) && conv_halo_ok(d, P, Q, ldx, bx, kx, cpw)) return ESB_CONV_KERNEL_HALO;
     }
-    if (!conv_force_im2col() && conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, cpw)) return ESB_CONV_KERNEL_STEM;
-    if (Kx > 0 && !conv_force_im2col() && same_layout && conv_halo_ok(d, P, Q, ldx, bx, kx, cpw))
-        return ESB_CONV_KERNEL_HALO;
+    const int64_t M = (int64_t)d.n * P * Q;
+    int kwx;
+    const ConvK c = conv_im2col(d, M, nullptr, ldx, bx, kx, ldw, bw, kw, cpw, &kwx);
     cudaError_t e = cudaSuccess;
     const int st = ws_static_smem<ConvSrc>(&e);
     if (st < 0) return -1;
-    const int bn = resident_bn((int64_t)d.n * P * Q, d.cout, cpw, pick_bn(d.cout, cpw));   // as launch_ws
-    if (Kx > 0 && ws_layout(Kx, bn, max_dyn_smem() - st).stages >= 3) return ESB_CONV_KERNEL_IM2COL;
+    const int bn = resident_bn(M, d.cout, cpw, pick_bn(d.cout, cpw));   // as launch_ws
+    if (c.K > 0 && ws_layout(c.K, bn, max_dyn_smem() - st).stages >= 3) return ESB_CONV_KERNEL_IM2COL;
     return ESB_CONV_KERNEL_STREAMED;
 }
 

@@ -1,5 +1,7 @@
 """GPU parity of convolutions whose pixel rows, filter rows and code widths do
-not line up, against the CPU oracle: input rows padded beyond the filter's."""
+not line up, against the CPU oracle: input rows padded beyond the filter's, and
+four-word rows at stride 1 off the halo kernel (whole rows or single words in
+the im2col K)."""
 import numpy as np
 import pytest
 import torch
@@ -59,3 +61,26 @@ def test_input_rows_longer_than_filter_rows(f, c, ldx, r, stride):
     guarded = torch.full((cout * r * r + 2, ldw), 0x15151515, dtype=torch.int32, device="cuda")
     guarded[:-2] = dev_i32(W)
     check(X, f, guarded[:-2], W, f, (n, h, w, c, cout, r, r, stride, pad))
+
+
+@pytest.mark.parametrize("n,h,w,c,cout,r,fx,fw", [
+    (1, 6, 140, 3, 24, 3, (4, 2), (4, 2)),           # wider than the halo kernel's tile, few tiles: whole rows
+    (3, 200, 210, 3, 16, 3, (4, 2), (4, 2)),         # many tiles: single words
+    (3, 200, 210, 3, 16, 3, (6, 3), (6, 3)),
+    (3, 200, 210, 10, 16, 3, (4, 2), (4, 2)),        # two words of channels
+    (2, 20, 20, 16, 40, 3, (4, 1), (4, 1)),          # too little of the halo tile used
+    (2, 20, 20, 3, 40, 5, (5, 2), (5, 2)),
+    (2, 7, 7, 6, 16, 5, (3, 1), (3, 1)),
+    (1, 24, 200, 3, 96, 11, (4, 2), (4, 2)),         # whole rows would not stay resident
+    (1, 24, 200, 9, 96, 11, (4, 2), (4, 2)),
+    (2, 19, 21, 3, 24, 3, (8, 5), (8, 5)),           # significand planes
+    (2, 19, 21, 5, 24, 3, (6, 4), (5, 2)),
+    (2, 19, 21, 3, 24, 3, (4, 2), (6, 3)),           # filters of another width
+    (2, 56, 56, 16, 24, 3, (4, 2), (3, 1)),
+])
+def test_four_word_rows_off_the_halo_kernel(n, h, w, c, cout, r, fx, fw):
+    geo = (n, h, w, c, cout, r, r, 1, r // 2)
+    assert esb.esb_conv2d_kernel(*geo, esb.Fmt(*fx, False), esb.Fmt(*fw)) in (esb.ESB_CONV_KERNEL_IM2COL, esb.ESB_CONV_KERNEL_STREAMED)
+    X = packed(n * h * w, c, fx, 5, esb.esb_row_words(c, fx[0]), signed=False)
+    W = packed(cout * r * r, c, fw, 6, esb.esb_row_words(c, fw[0]))
+    check(X, fx, dev_i32(W), W, fw, geo)
