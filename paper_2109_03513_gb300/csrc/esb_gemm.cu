@@ -85,7 +85,7 @@ struct ConvSrc {
         x.sn = sn > 0 ? sn : 0;
         return x;
     }
-    __device__ __forceinline__ bool inside(const Row& x, int r, int s) const
+    static __device__ __forceinline__ bool inside(const Row& x, int r, int s)
     {
         return (unsigned)(r - x.rlo) < (unsigned)x.rn && (unsigned)(s - x.slo) < (unsigned)x.sn;
     }
@@ -168,9 +168,15 @@ __device__ __forceinline__ void conv_tap_table(const ConvSrc& src, int64_t w0, i
 
 // 4-bit codes: the K-block's 16 words of row `row` (rows past M and taps
 // outside the image give the E4M3 zero), decoded and stored to stage row r.
-__device__ __forceinline__ void walk_b4_tab(const ConvSrc& src, const ConvSrc::Row& row, const int4* tab, int64_t k0,
-                                            int64_t K, const OpFmt& f, uint8_t* stage, int r)
+// Out of line, like the word-slot walks: inlined beside the decode by pieces
+// they cost the producers more instructions per word (7x7, 224 x 224 x 3 -> 64,
+// batch 2: 63.1 us inlined, 55.0 us this way; 5x5, 150 x 150 x 3 -> 16: 49.6
+// and 42.7).
+static __device__ __noinline__ void walk_b4_tab(const uint32_t* X, ConvSrc::Row row, const int4* tab, int64_t k0, int64_t K, int k,
+                                                int ew, uint8_t* stage, int r)
 {
+    OpFmt f;
+    f.k = k; f.ew = ew;
 #pragma unroll 1
     for (int hf = 0; hf < 2; hf++) {                  // two halves of 8 words: a small loop body
         uint32_t wv[8];
@@ -179,8 +185,8 @@ __device__ __forceinline__ void walk_b4_tab(const ConvSrc& src, const ConvSrc::R
 #pragma unroll
         for (int i = 0; i < 8; i++) {
             const int4 e = tab[8 * hf + i];
-            const bool in = (kh + i * 8 < K) && src.inside(row, e.x, e.y);
-            wv[i] = in ? __ldg(src.X + (row.base + e.z)) : 0u;
+            const bool in = (kh + i * 8 < K) && ConvSrc::inside(row, e.x, e.y);
+            wv[i] = in ? __ldg(X + (row.base + e.z)) : 0u;
             ok |= (in ? 1u : 0u) << i;
         }
         store_b4_words<8>(wv, ok, kh, K, f, stage, r, 4 * hf);
@@ -189,25 +195,27 @@ __device__ __forceinline__ void walk_b4_tab(const ConvSrc& src, const ConvSrc::R
 
 // Word-slot codes (see plan_slots): the K-block's NW words, CH at a time.
 template <int B>
-__device__ __forceinline__ void walk_slots_tab(const ConvSrc& src, const ConvSrc::Row& row, const int4* tab,
-                                               int64_t k0, const OpFmt& f, uint8_t* stage, int r)
+static __device__ __noinline__ void walk_slots_tab(const uint32_t* X, ConvSrc::Row row, const int4* tab, int64_t k0, int64_t korig,
+                                                   int k, int ew, uint8_t* stage, int r)
 {
     constexpr int CPW = 32 / B;
     constexpr int SPW = CPW > 8 ? 16 : (CPW > 4 ? 8 : 4);
     constexpr int NW = kBK / SPW;
     constexpr int CH = 8;                             // words per chunk (a small loop body)
+    OpFmt f;
+    f.k = k; f.ew = ew;
     const int64_t w0 = k0 / SPW;
 #pragma unroll 1
     for (int c0 = 0; c0 < NW; c0 += CH) {
-        const int64_t left = f.korig - (w0 + c0) * CPW;
+        const int64_t left = korig - (w0 + c0) * CPW;
         const int lim = left < 0 ? 0 : (left > CH * CPW ? CH * CPW : (int)left);
         uint32_t wv[CH];
         uint32_t ok = 0u;
 #pragma unroll
         for (int i = 0; i < CH; i++) {
             const int4 e = tab[c0 + i];
-            const bool in = (i * CPW < lim) && src.inside(row, e.x, e.y);
-            wv[i] = in ? __ldg(src.X + (row.base + e.z)) : 0u;
+            const bool in = (i * CPW < lim) && ConvSrc::inside(row, e.x, e.y);
+            wv[i] = in ? __ldg(X + (row.base + e.z)) : 0u;
             ok |= (in ? 1u : 0u) << i;
         }
         store_slot_words<B, CH>(wv, ok, lim, f, stage, r, c0 * SPW / 16);
@@ -217,14 +225,14 @@ __device__ __forceinline__ void walk_slots_tab(const ConvSrc& src, const ConvSrc
 __device__ __forceinline__ void walk_row_tab(const ConvSrc& src, const ConvSrc::Row& row, const int4* tab,
                                              int64_t k0, int64_t K, const OpFmt& f, uint8_t* stage, int r)
 {
-    if (f.b == 4) { walk_b4_tab(src, row, tab, k0, K, f, stage, r); return; }
     switch (f.b) {
-    case 2: walk_slots_tab<2>(src, row, tab, k0, f, stage, r); return;
-    case 3: walk_slots_tab<3>(src, row, tab, k0, f, stage, r); return;
-    case 5: walk_slots_tab<5>(src, row, tab, k0, f, stage, r); return;
-    case 6: walk_slots_tab<6>(src, row, tab, k0, f, stage, r); return;
-    case 7: walk_slots_tab<7>(src, row, tab, k0, f, stage, r); return;
-    default: walk_slots_tab<8>(src, row, tab, k0, f, stage, r); return;
+    case 2: walk_slots_tab<2>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
+    case 3: walk_slots_tab<3>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
+    case 4: walk_b4_tab(src.X, row, tab, k0, K, f.k, f.ew, stage, r); return;
+    case 5: walk_slots_tab<5>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
+    case 6: walk_slots_tab<6>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
+    case 7: walk_slots_tab<7>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
+    default: walk_slots_tab<8>(src.X, row, tab, k0, f.korig, f.k, f.ew, stage, r); return;
     }
 }
 
@@ -1047,13 +1055,13 @@ static int conv_halo_words(const esb_conv_desc& d, int64_t ldx, int kwx) { retur
 // shorter, so they lose only where a pixel has one word of channels and a CTA
 // many K-blocks, and where the filters then no longer stay resident.  Measured,
 // whole and by words, 4-bit (K-blocks of a CTA's tiles by whole rows in front):
-//   12: 3x3, 33 x 33 x 3 -> 64, batch 64      16.7 and 20.9 us
-//   26: 7x7, 20 x 20 x 3 -> 32, batch 64      21.7 and 26.9
-//   62: 11x11, 20 x 20 x 3 -> 32, batch 64    52.5 and 47.5
-//   63: 3x3, 224 x 224 x 3 -> 64, batch 8     59.2 and 54.1
-//   70: 5x5, 150 x 150 x 3 -> 16, batch 8     51.9 and 49.7
-//   63, two words of channels: 3x3, 224 x 224 x 16 -> 64    59.2 and 99.3
-//   not resident: 11x11, 200 x 200 x 3 -> 64, batch 4       254 and 191
+//   12: 3x3, 33 x 33 x 3 -> 64, batch 64      16.6 and 19.6 us
+//   26: 7x7, 20 x 20 x 3 -> 32, batch 64      21.4 and 24.4
+//   62: 11x11, 20 x 20 x 3 -> 32, batch 64    52.5 and 42.0
+//   63: 3x3, 224 x 224 x 3 -> 64, batch 8     59.2 and 48.4
+//   70: 5x5, 150 x 150 x 3 -> 16, batch 8     51.9 and 42.7
+//   63, two words of channels: 3x3, 224 x 224 x 16 -> 64    59.2 and 85.4
+//   not resident: 11x11, 200 x 200 x 3 -> 64, batch 4       254 and 151
 // Significand planes and filters of another width do not decode by pieces
 // (3x3, 56 x 56 x 3 -> 32, (8,5): 706 us whole, 301 by words).
 static bool conv_whole_pays(const esb_conv_desc& d, int64_t M, const ConvK& whole, int kwx, int out_cpw)
