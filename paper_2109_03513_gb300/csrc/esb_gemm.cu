@@ -874,6 +874,24 @@ bool lean4_ok(const EpiParams& ep, int64_t N, int BN)
            ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
 }
 
+// The epilogue's paths in microseconds per 128 x 16 outputs, from tiles whose
+// time it sets (2x2/2 convolutions of 700000 rows).
+double epi_cost16_codes(int out_b, bool whole)
+{
+    if (out_b == 4) return whole ? 0.3 : 0.7;                     // LEAN4, else the lean path
+    return out_b == 3 || out_b == 5 || out_b == 6 ? 0.47 : 2.0;   // cell table, else a bisection
+}
+
+double epi_cost16(const EpiParams& ep, int64_t N, int BN)
+{
+    const bool ch = ep.scale || ep.bias;
+    if (!ep.codes_out) return 1.5;                                // fp32 or int32 alone
+    if (ep.acc_out || ep.y_out) return ep.out.b == 4 ? 2.1 : 5.0;
+    if (ep.out.b != 4) return ch && epi_cells_ok(ep) ? 0.8 : (epi_cells_ok(ep) ? 0.47 : 2.0);
+    if (ch || (ep.residual && ep.res_b != 4)) return 2.1;
+    return ep.residual ? 0.8 : epi_cost16_codes(4, lean4_ok(ep, N, BN));
+}
+
 // Warp-specialised launch: B resident when its N-tile fits in shared
 // memory with at least three A stages, else streamed with A through the
 // stages; returns false (nothing launched) when neither fits.
@@ -1119,7 +1137,7 @@ int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx
 {
     const int cpw = 32 / out_b;                                   // as launch_conv_tc
     if (!conv_force_im2col()) {
-        if (conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, cpw)) return ESB_CONV_KERNEL_STEM;
+        if (conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, out_b)) return ESB_CONV_KERNEL_STEM;
         const ConvK h = conv_k(d, nullptr, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
         if (conv_halo_rows(h) && conv_halo_ok(d, P, Q, ldx, bx, kx, cpw)) return ESB_CONV_KERNEL_HALO;
     }

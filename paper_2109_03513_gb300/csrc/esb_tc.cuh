@@ -1549,9 +1549,16 @@ bool lean4_ok(const EpiParams& ep, int64_t N, int BN);   // the LEAN4 epilogue t
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
 float acc_fma_limit(int64_t K, int ba, int ka, int bb, int kb);   // FMA-pipe requantisation bound (esb_gemm.cu)
 
-// Strided convolution of up to 4 channels (esb_conv_stem.cu); the same
-// contract: false when the shape does not suit it.
-bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int out_cpw);
+// Cost of the epilogue of a 128-row tile in microseconds per 16 columns
+// (esb_gemm.cu); _codes: codes alone, a scalar scale and bias, whole N-tiles or not.
+double epi_cost16(const EpiParams& ep, int64_t N, int BN);
+double epi_cost16_codes(int out_b, bool whole);
+
+// Strided convolution of up to 4 channels (esb_conv_stem.cu): false,
+// launching nothing, when the shape does not suit it or im2col is faster;
+// otherwise launches and stores the launch status in *err.  conv_stem_ok: the
+// choice for codes of out_b bits alone with a scalar scale and bias.
+bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int out_b);
 bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa, const uint32_t* W,
                       int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st, cudaError_t* err);
 

@@ -38,14 +38,28 @@ CASES = [
     (1, 12, 70, 3, 16, 2, 2, 2, 0, (7, 3), (4, 2)),           # mixed widths, even filter
     (2, 15, 257, 3, 48, 4, 1, 4, 0, (4, 3), (5, 1)),
     (1, 8, 52, 3, 8, 8, 8, 2, 7, (4, 0), (6, 2)),             # padding of seven
+    (40, 9, 252, 3, 64, 7, 7, 2, 3, (4, 2), (4, 2)),          # full tile rows, two tiles a block
 ]
 
 
 @pytest.mark.parametrize("n,h,w,c,cout,r,s,stride,pad,fx,fw", CASES)
 def test_stem_convolution_matches_oracle(n, h, w, c, cout, r, s, stride, pad, fx, fw):
+    check(n, h, w, c, cout, r, s, stride, pad, fx, fw, esb.ESB_CONV_KERNEL_STEM)
+
+
+@pytest.mark.parametrize("n,h,w,c,cout,r,s,stride,pad,fx,fw", [
+    (40, 51, 51, 3, 287, 2, 2, 2, 1, (3, 0), (3, 0)),         # a fifth of the tile rows used, a costly epilogue
+    (60, 40, 40, 3, 64, 3, 3, 2, 1, (2, 1), (2, 1)),
+    (60, 31, 31, 2, 40, 3, 3, 2, 1, (6, 3), (6, 3)),
+    (200, 40, 20, 4, 64, 3, 3, 4, 1, (4, 2), (4, 2)),
+])
+def test_strided_layers_left_to_im2col_match_oracle(n, h, w, c, cout, r, s, stride, pad, fx, fw):
+    check(n, h, w, c, cout, r, s, stride, pad, fx, fw, esb.ESB_CONV_KERNEL_IM2COL)
+
+
+def check(n, h, w, c, cout, r, s, stride, pad, fx, fw, kernel):
     signed_x = (n + h) % 2 == 0
-    assert esb.esb_conv2d_kernel(n, h, w, c, cout, r, s, stride, pad, esb.Fmt(*fx, signed_x), esb.Fmt(*fw),
-                                 out_b=fx[0]) == esb.ESB_CONV_KERNEL_STEM
+    assert esb.esb_conv2d_kernel(n, h, w, c, cout, r, s, stride, pad, esb.Fmt(*fx, signed_x), esb.Fmt(*fw), out_b=fx[0]) == kernel
     x = (synth.normal if signed_x else synth.half_normal)((n * h * w, c), seed=h + c).numpy()
     wt = synth.he_normal((cout * r * s, c), fan_in=r * s * c, seed=cout + r).numpy()
     ax, _ = o.calibrate(x, *fx, signed_x)
