@@ -622,7 +622,7 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     RowsSrc b{W, (int64_t)d.r * d.s * ldw, N};
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
     // The specialised instance: 4-bit B, bulk-copied input rows, LEAN4 epilogue
-    const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && lean4_ok(ep, N, hp.BN);
+    const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && lean4_ok(ep);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(fast ? esb_conv_halo_kernel<true, false>
                            : (gen ? esb_conv_halo_kernel<false, true> : esb_conv_halo_kernel<false, false>),

@@ -405,14 +405,14 @@ bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int
     StemPlan sp;
     cudaError_t e;
     const int bn = pick_bn(d.cout, 32 / out_b);
-    return bn > 0 && stem_plan(d, P, Q, ldx, bx, kx, bw, kw, bn, epi_cost16_codes(out_b, d.cout % bn == 0), &sp, &e);
+    return bn > 0 && stem_plan(d, P, Q, ldx, bx, kx, bw, kw, bn, epi_cost16_codes(out_b), &sp, &e);
 }
 
 bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa, const uint32_t* W,
                       int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st, cudaError_t* err)
 {
     StemPlan sp;
-    if (!stem_plan(d, P, Q, ldx, fa.b, fa.k, fb.b, fb.k, BN, epi_cost16(ep, d.cout, BN), &sp, err)) return *err != cudaSuccess;
+    if (!stem_plan(d, P, Q, ldx, fa.b, fa.k, fb.b, fb.k, BN, epi_cost16(ep), &sp, err)) return *err != cudaSuccess;
     sp.g.X = X;
     static bool configured = false;
     if (!configured) {
@@ -429,7 +429,7 @@ bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     if (per_n < 1) per_n = 1;
     if (per_n > m_tiles) per_n = m_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool fast = lean4_ok(ep, N, BN);                   // the specialised epilogue
+    const bool fast = lean4_ok(ep);                   // the specialised epilogue
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
     *err = launch_pdl(kStemKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
                       (size_t)sp.smem, st, sp.g, W, ldw, N, fa, fb, BN, sp.nkb, n_tiles, m_tiles, acc_scale, ep);

@@ -865,31 +865,31 @@ static int ws_static_smem(cudaError_t* err)
     return v;
 }
 
-// 4-bit codes as the only output, a scalar scale and bias, whole N-tiles and
+// 4-bit codes as the only output, a scalar scale and bias, sums below 2^20 and
 // a monotone requantisation (unsigned codes or an activation): what the
 // specialised epilogue (LEAN4) takes.
-bool lean4_ok(const EpiParams& ep, int64_t N, int BN)
+bool lean4_ok(const EpiParams& ep)
 {
     return ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
-           ep.acc_lim > 0.0f && N % BN == 0 && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
+           ep.acc_lim > 0.0f && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
 }
 
 // The epilogue's paths in microseconds per 128 x 16 outputs, from tiles whose
 // time it sets (2x2/2 convolutions of 700000 rows).
-double epi_cost16_codes(int out_b, bool whole)
+double epi_cost16_codes(int out_b)
 {
-    if (out_b == 4) return whole ? 0.3 : 0.7;                     // LEAN4, else the lean path
+    if (out_b == 4) return 0.3;
     return out_b == 3 || out_b == 5 || out_b == 6 ? 0.47 : 2.0;   // cell table, else a bisection
 }
 
-double epi_cost16(const EpiParams& ep, int64_t N, int BN)
+double epi_cost16(const EpiParams& ep)
 {
     const bool ch = ep.scale || ep.bias;
     if (!ep.codes_out) return 1.5;                                // fp32 or int32 alone
     if (ep.acc_out || ep.y_out) return ep.out.b == 4 ? 2.1 : 5.0;
     if (ep.out.b != 4) return ch && epi_cells_ok(ep) ? 0.8 : (epi_cells_ok(ep) ? 0.47 : 2.0);
     if (ch || (ep.residual && ep.res_b != 4)) return 2.1;
-    return ep.residual ? 0.8 : epi_cost16_codes(4, lean4_ok(ep, N, BN));
+    return ep.residual ? 0.8 : (lean4_ok(ep) ? 0.3 : 0.5);
 }
 
 // Warp-specialised launch: B resident when its N-tile fits in shared
@@ -930,7 +930,7 @@ static bool launch_ws(const SrcA& a, const RowsSrc& b, int64_t M, int64_t N, int
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
     const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
-    *err = launch_pdl(WsKernels<SrcA>::k[lean4_ok(ep, N, BN) ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kWsThreads),
+    *err = launch_pdl(WsKernels<SrcA>::k[lean4_ok(ep) ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kWsThreads),
                       (size_t)L.smem_bytes, st, a, b, M, N, K, fa, fb, BN, L.nkb, L.stages, n_tiles, m_tiles, acc_scale, ep,
                       bstream);
     return true;

@@ -624,7 +624,7 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     if (per_n > m_tiles) per_n = m_tiles;
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool fast = nch == 1 && lean4_ok(ep, N, BN);   // the specialised epilogue
+    const bool fast = nch == 1 && lean4_ok(ep);   // the specialised epilogue
     // one chunk of other widths' codes only: the general-width epilogue instance
     const bool gen = nch == 1 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
     return launch_pdl(kTiledKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,

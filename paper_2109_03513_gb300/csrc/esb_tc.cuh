@@ -734,23 +734,26 @@ static __device__ __noinline__ void epi_chunk_any(const EpiParams* __restrict__ 
 {
     const EpiParams& ep = *sep;
     const EpiCtx cx = *scx;
-    uint32_t r[16];
-    tmem_ld16(taddr, r);
     const int cpw = ep.out_cpw;
     uint32_t word = word_slot_w[0];
     int slot = (int)word_slot_w[1];
     int64_t wcol = (int64_t)word_slot_w[2] | ((int64_t)word_slot_w[3] << 32);
+#pragma unroll 1
+    for (int g = 0; g < 4; g++) {                     // four columns at a time: a small loop body, as in epi_chunk16
+        uint32_t r[4];
+        tmem_ld4(taddr + 4 * g, r);
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-        const int64_t n = n_first + j;
-        uint32_t code = ep.out.zero_code;
-        if (mrow && n < N) code = epi_element(ep, cx, __uint_as_float(r[j]) * acc_scale, m, n, N);
-        word |= code << (ep.out.b * slot);
-        if (++slot == cpw) {
-            if (ep.codes_out && mrow && wcol < ep.ldo) ep.codes_out[m * ep.ldo + wcol] = word;
-            word = 0;
-            slot = 0;
-            wcol++;
+        for (int j = 0; j < 4; j++) {
+            const int64_t n = n_first + 4 * g + j;
+            uint32_t code = ep.out.zero_code;
+            if (mrow && n < N) code = epi_element(ep, cx, __uint_as_float(r[j]) * acc_scale, m, n, N);
+            word |= code << (ep.out.b * slot);
+            if (++slot == cpw) {
+                if (ep.codes_out && mrow && wcol < ep.ldo) ep.codes_out[m * ep.ldo + wcol] = word;
+                word = 0;
+                slot = 0;
+                wcol++;
+            }
         }
     }
     word_slot_w[0] = word;
@@ -1163,6 +1166,56 @@ __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, in
     return *tmem_slot;
 }
 
+// The tiles of outputs that have no path of their own in ws_epilogue (fp32 or
+// int32 outputs, per-channel scale or bias), 16 columns at a time through
+// epi_chunk16 or, for codes of another width than 4, epi_chunk_any.  A loop of
+// its own: called from the loop of the fast paths, these functions made it keep
+// their constants in local memory (200000 x 300 x 128, 4-bit codes alone: signed
+// 207 us, 115 without the calls; 200000 x 64, 8-bit codes: 98 and 82).
+template <class RowMap>
+__device__ __noinline__ void epi_chunk_tiles(const EpiParams& ep, const EpiParams* sep, const EpiCtx* scx, const RowMap& rows,
+                                             int64_t my_tiles, bool alt, int grp, int lacc, int64_t n0, int64_t N, int BN, int c_lo,
+                                             int c_hi, bool pad_words, uint32_t tmem_base, float acc_scale, float sc_fixed,
+                                             uint64_t* tfull, uint64_t* tempty, volatile int* err, int quarter, int lane)
+{
+    const int cpw = ep.out_cpw, row = quarter * 32 + lane;
+    const bool any = ep.codes_out && ep.out.b != 4;
+    uint32_t zero_word = 0u;
+    for (int j = 0; j < cpw; j++) zero_word |= ep.out.zero_code << (ep.out.b * j);
+    for (int64_t ti = alt ? grp : 0; ti < my_tiles && !*err; ti += alt ? 2 : 1) {
+        const int a = (int)(ti & ((1 << lacc) - 1));
+        if (!wait_or_abort(&tfull[a], (uint32_t)((ti >> lacc) & 1), err)) { *err = 1; break; }
+        tc_fence_after();
+        int64_t m = 0;
+        const bool mrow = rows(ti, row, m);
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN);
+        uint32_t wsw[4] = {0u, 0u, (uint32_t)(((n0 + c_lo) / cpw) & 0xffffffff),
+                           (uint32_t)(((n0 + c_lo) / cpw) >> 32)};   // epi_chunk_any: word, slot, column
+        for (int c = c_lo; c < c_hi; c += 16) {
+            uint2 q = make_uint2(zero_word, zero_word);
+            if (any) epi_chunk_any(sep, scx, taddr + (uint32_t)c, acc_scale, m, mrow, n0 + c, N, wsw);
+            else if (n0 + c < N) q = epi_chunk16(ep, scx, taddr + (uint32_t)c, acc_scale, sc_fixed, m, mrow, n0 + c, N);
+            if (c + 16 >= c_hi) {                     // every column of this warp has been read
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
+            }
+            if (ep.codes_out && !any && mrow) {
+                const int64_t w0 = (n0 + c) >> 3;
+                uint32_t* dst = ep.codes_out + m * ep.ldo + w0;
+                if (ep.codes_vec >= 2 && (w0 & 1) == 0 && w0 + 2 <= ep.ldo) {
+                    *reinterpret_cast<uint2*>(dst) = q;
+                } else {
+                    if (w0 < ep.ldo) dst[0] = q.x;
+                    if (w0 + 1 < ep.ldo) dst[1] = q.y;
+                }
+            }
+        }
+        if (pad_words && mrow)
+            for (int64_t wq = (n0 + BN) / cpw; wq < ep.ldo; wq++) ep.codes_out[m * ep.ldo + wq] = zero_word;
+    }
+}
+
 // Epilogue role (warps 0 .. epi_warps - 1): drains the accumulator tiles of
 // this CTA in order, tile ti from TMEM buffer a = ti mod 2^lacc (columns a * BN
 // ..), and frees the buffer on tempty once its columns are in registers.
@@ -1170,12 +1223,11 @@ __device__ __forceinline__ uint32_t ws_setup(const RowsSrc& srcB, int64_t n0, in
 // columns and tiles are the warp's (see EpiSplit).  rows(ti, row, m)
 // gives the output row m of a tile row and whether it exists.  LEAN4: the
 // host has established 4-bit codes as the only output with a scalar scale
-// and bias (every column chunk inside N); the instance then holds just the
-// FMA-pipe requantisation and, for device values that rule it out, the
-// out-of-line per-word path.  GEN: the output is not 4-bit codes; the
-// instance holds the general-width code path and the out-of-line path for
-// fp32/int32 outputs, and none of the 4-bit code (each instance keeps a
-// small hot loop).
+// and bias and sums below 2^20 (lean4_ok); the instance then holds just the
+// FMA-pipe requantisation.  GEN: the output is not 4-bit codes; the instance
+// holds the general-width code path and none of the 4-bit code.  Calls that
+// an instance has no path for take epi_chunk_tiles (each instance keeps a
+// small hot loop, without calls).
 template <bool LEAN4, bool GEN, class RowMap>
 __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* thr, const RowMap& rows,
                                             int64_t my_tiles, int64_t n0, int64_t N, int BN, const EpiSplit& sp, int lacc,
@@ -1254,22 +1306,30 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     }
     asm volatile("bar.sync 2, %0;" ::"r"(epi_warps * 32) : "memory");   // exactly the epilogue warps in use
     const int cpw = ep.out_cpw;
+    // the warp holding the tile's last columns of the last N-tile writes the padding words
+    const bool pad_words = ep.codes_out && (n0 + BN >= N) && ((n0 + BN) / cpw < ep.ldo) &&
+                           (split ? grp == 1 : true);
+    // the paths of this instance; LEAN4's only one, the FMA-pipe search, can be ruled out by device values
+    if (GEN ? !gen : (LEAN4 ? !raw_ok : !(lean_ok || lres))) {
+        epi_chunk_tiles(ep, &sh_ep, &sh_cx, rows, my_tiles, sp.alt, grp, lacc, n0, N, BN, c_lo, c_hi, pad_words, tmem_base, acc_scale,
+                        sc_fixed, tfull, tempty, err, quarter, lane);
+        return;
+    }
     const float T0 = cx.t7.t[0], T1 = cx.t7.t[1], T2 = cx.t7.t[2], T3 = cx.t7.t[3], T4 = cx.t7.t[4],
                 T5 = cx.t7.t[5], T6 = cx.t7.t[6];
     float R0 = 0.0f, R1 = 0.0f, R2 = 0.0f, R3 = 0.0f, R4 = 0.0f, R5 = 0.0f, R6 = 0.0f;
     if (raw_ok) {
         R0 = sh_raw[0]; R1 = sh_raw[1]; R2 = sh_raw[2]; R3 = sh_raw[3]; R4 = sh_raw[4]; R5 = sh_raw[5]; R6 = sh_raw[6];
     }
-    // The same search on the FMA pipe when |acc| <= L - 2 < 2^20 (the ALU
+    // LEAN4: the same search on the FMA pipe when |acc| <= L - 2 < 2^20 (the ALU
     // pipe is the epilogue's bottleneck): with A_j = R_j / rs clamped to
     // [-L, L] and k_j = 1 - 2 A_j, sat(fma(raw, 2/rs, k_j)) = sat(2 acc -
     // 2 A_j + 1) is exactly [acc >= A_j] (an odd integer below 2^24 before
     // the clamp to [0, 1]); the next threshold is chosen by fmas with those
     // 0/1 factors, and the bucket bits are packed by fmas with powers of 16
     // (every intermediate an integer below 2^24: exact).
-    const bool fma_ok = raw_ok && ep.acc_lim > 0.0f;
     float cK = 0.0f, K0 = 0.0f, K1 = 0.0f, K3 = 0.0f, D51 = 0.0f, D20 = 0.0f, D40 = 0.0f, E3 = 0.0f;
-    if (fma_ok) {
+    if (LEAN4) {
         const float L = ep.acc_lim;
         auto kf = [&](float R) { return 1.0f - 2.0f * fminf(fmaxf(R * acc_scale, -L), L); };
         const float k0 = kf(R0), k1 = kf(R1), k2 = kf(R2), k3 = kf(R3), k4 = kf(R4), k5 = kf(R5), k6 = kf(R6);
@@ -1277,9 +1337,6 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
         K0 = k0; K1 = k1; K3 = k3;
         D51 = k5 - k1; D20 = k2 - k0; D40 = k4 - k0; E3 = (k6 - k4) - (k2 - k0);
     }
-    // the warp holding the tile's last columns of the last N-tile writes the padding words
-    const bool pad_words = ep.codes_out && (n0 + BN >= N) && ((n0 + BN) / cpw < ep.ldo) &&
-                           (split ? grp == 1 : true);
     uint32_t zero_word = 0u;
     for (int j = 0; j < cpw; j++) zero_word |= ep.out.zero_code << (ep.out.b * j);
     for (int64_t ti = sp.alt ? grp : 0; ti < my_tiles && !*err; ti += sp.alt ? 2 : 1) {
@@ -1289,12 +1346,10 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
         int64_t m = 0;
         const bool mrow = rows(ti, row, m);
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN);
-        uint32_t wsw[4] = {0u, 0u, (uint32_t)(((n0 + c_lo) / cpw) & 0xffffffff),
-                           (uint32_t)(((n0 + c_lo) / cpw) >> 32)};   // general path: word, slot, column
         uint32_t gword = 0u;                          // gen path: word being packed, its next slot, its column
         int gslot = 0;
         int64_t gcol = (n0 + c_lo) / cpw;
-        if (gen) {
+        if constexpr (GEN) {
             // columns [c_lo, c_end) are the warp's chunks holding outputs
             // inside N, 16 columns a chunk in four groups of four (a small
             // loop body with four independent threshold searches); the rest
@@ -1394,38 +1449,17 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
             if (mrow)
                 for (; gcol < wend && gcol < ep.ldo; gcol++) ep.codes_out[m * ep.ldo + gcol] = zero_word;
         }
-        for (int c = c_lo; c < (gen ? c_lo : c_hi); c += 16) {
-            if (GEN || (!LEAN4 && !swar)) {
-                if (!ep.codes_out)
-                    epi_chunk16(ep, &sh_cx, taddr + (uint32_t)c, acc_scale, sc_fixed, m, mrow, n0 + c, N);
-                else
-                    epi_chunk_any(&sh_ep, &sh_cx, taddr + (uint32_t)c, acc_scale, m, mrow, n0 + c, N, wsw);
-                if (c + 16 >= c_hi) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_tmem_free(&tempty[a]);
-                }
-                continue;
-            }
-            if constexpr (!GEN) {
+        if constexpr (!GEN)
+        for (int c = c_lo; c < c_hi; c += 16) {
             // 4-bit output codes: 16 columns (two code words) per TMEM load
             // (compact code: measured faster than 32-column loads)
             constexpr int nc = 16;
             // columns of the chunk inside N (codes past N are masked to the zero code)
             const int64_t ncl64 = N - (n0 + c);
             const int ncl = ncl64 < nc ? (int)ncl64 : nc;
-            const bool lean = lean_ok && ncl > 0;
             uint32_t wds[2];
-            // other outputs, per-channel scale or bias; LEAN4: device values that rule the FMA search out
-            const bool full = LEAN4 ? !(lean && fma_ok) : (!lean && !(lres && ncl > 0));
             uint32_t r[16];
-            if (full) {
-                const uint2 q = epi_chunk16(ep, &sh_cx, taddr + (uint32_t)c, acc_scale, sc_fixed, m, mrow, n0 + c, N);
-                wds[0] = q.x;
-                wds[1] = q.y;
-            } else {
-                tmem_ld16(taddr + (uint32_t)c, r);
-            }
+            if (ncl > 0) tmem_ld16(taddr + (uint32_t)c, r);
             if (c + nc >= c_hi) {                     // every column of this warp is in registers
                 tc_fence_before();
                 __syncwarp();
@@ -1433,11 +1467,12 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
             }
 #pragma unroll
             for (int h = 0; h < 2; h++) {
-                if (full) break;
+                wds[h] = zero_word;
+                if (ncl <= 0) continue;               // a chunk past N
                 uint32_t J = 0u, S = 0u;
                 const int live_h = ncl - 8 * h;       // nibbles of this word inside N
                 const uint32_t nib = live_h >= 8 ? 0xffffffffu : (live_h <= 0 ? 0u : (1u << (4 * live_h)) - 1u);
-                if (lean && fma_ok) {
+                if (LEAN4) {
                     float jh[2];
 #pragma unroll
                     for (int q = 0; q < 2; q++) {
@@ -1456,7 +1491,7 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                     }
                     J = (__float_as_uint(jh[0]) & 0xffffu) | (__float_as_uint(jh[1]) << 16);
                     wds[h] = codes8_b4(J & nib, 0u, ep.out.k);
-                } else if (!LEAN4 && lean && raw_ok) {
+                } else if (lean_ok && raw_ok) {
                     // bucket = number of raw thresholds <= raw accumulator
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
@@ -1467,7 +1502,7 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                         J |= ((b2 ? 4u : 0u) | (b1 ? 2u : 0u) | (b0 ? 1u : 0u)) << (4 * j);
                     }
                     wds[h] = codes8_b4(J & nib, 0u, ep.out.k);
-                } else if (!LEAN4 && lean) {
+                } else if (lean_ok) {
                     // 4-bit output codes only, scalar scale/bias, no residual:
                     // y = fma(scale * 2^(kA+kB+12), raw, bias) equals
                     // fma(scale, acc, bias) exactly (power-of-two scaling),
@@ -1485,7 +1520,7 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                         if (out_signed) S |= (__float_as_uint(y) >> 31) << (4 * j + 3);
                     }
                     wds[h] = codes8_b4(J & nib, S & nib, ep.out.k);
-                } else if (!LEAN4 && lres && ncl > 0) {
+                } else {
                     const uint32_t rw = mrow ? __ldg(ep.residual + m * ep.res_ld + ((n0 + c) >> 3) + h) : 0u;
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
@@ -1513,7 +1548,6 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                     for (int q = 0; q < 2; q++)
                         if (w0 + q < ep.ldo) dst[q] = wds[q];
                 }
-            }
             }
         }
         // the last N-tile also fills the row's words past its columns (the
@@ -1545,14 +1579,14 @@ __device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err, uin
 
 int pick_bn(int64_t N, int out_cpw);          // N-tile width (esb_gemm.cu)
 int max_dyn_smem();                           // opt-in shared memory per block
-bool lean4_ok(const EpiParams& ep, int64_t N, int BN);   // the LEAN4 epilogue takes the call (esb_gemm.cu)
+bool lean4_ok(const EpiParams& ep);           // the LEAN4 epilogue takes the call (esb_gemm.cu)
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
 float acc_fma_limit(int64_t K, int ba, int ka, int bb, int kb);   // FMA-pipe requantisation bound (esb_gemm.cu)
 
 // Cost of the epilogue of a 128-row tile in microseconds per 16 columns
-// (esb_gemm.cu); _codes: codes alone, a scalar scale and bias, whole N-tiles or not.
-double epi_cost16(const EpiParams& ep, int64_t N, int BN);
-double epi_cost16_codes(int out_b, bool whole);
+// (esb_gemm.cu); _codes: codes alone, a scalar scale and bias.
+double epi_cost16(const EpiParams& ep);
+double epi_cost16_codes(int out_b);
 
 // Strided convolution of up to 4 channels (esb_conv_stem.cu): false,
 // launching nothing, when the shape does not suit it or im2col is faster;
