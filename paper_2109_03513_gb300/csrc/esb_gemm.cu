@@ -303,8 +303,8 @@ esb_gemm_tc_kernel(SrcA srcA, SrcB srcB, int64_t M, int64_t N, int64_t K, OpFmt 
     __shared__ uint8_t luta[256], lutb[256];
     const bool walk_a = fa.planes == 1 && srcA.linear() && !(fa.b == 4 && srcA.vec4());
     const bool walk_b = fb.planes == 1 && srcB.linear() && !(fb.b == 4 && srcB.vec4());
-    if (walk_a) build_e4m3_lut(luta, fa, tid, kGemmThreads);
-    if (walk_b) build_e4m3_lut(lutb, fb, tid, kGemmThreads);
+    if (walk_a && reads_e4m3_lut(fa)) build_e4m3_lut(luta, fa, tid, kGemmThreads);
+    if (walk_b && reads_e4m3_lut(fb)) build_e4m3_lut(lutb, fb, tid, kGemmThreads);
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = *tmem_slot;
@@ -515,11 +515,11 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
-    // E4M3 tables of the word-walk decoder (widths other than 4)
+    // E4M3 tables of the code-linear word walk
     __shared__ uint8_t luta[256], lutb[256];
     __shared__ int4 ptab[kWsProdWarps][32];          // producers' per-stage tap tables (im2col rows)
-    if (fa.planes == 1) build_e4m3_lut(luta, fa, tid, kWsThreads);
-    if (fb.planes == 1 && fb.b != 4) build_e4m3_lut(lutb, fb, tid, kWsThreads);
+    if (reads_e4m3_lut(fa)) build_e4m3_lut(luta, fa, tid, kWsThreads);
+    if (reads_e4m3_lut(fb)) build_e4m3_lut(lutb, fb, tid, kWsThreads);
     const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {

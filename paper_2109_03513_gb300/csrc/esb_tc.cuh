@@ -313,7 +313,10 @@ __device__ __forceinline__ void tail_masks(int v, uint32_t& mlo, uint32_t& mhi)
 }
 
 // The E4M3 byte of each of the 2^b codes of a whole-byte format (planes ==
-// 1), built by threads t = 0 .. nt-1: the table of the word-walk decoder.
+// 1), built by threads t = 0 .. nt-1: the table of the code-linear word walk
+// (walk_row_kblock), which only an operand whose partner has other codes per
+// word still takes.
+__device__ __forceinline__ bool reads_e4m3_lut(const OpFmt& f) { return f.planes == 1 && f.b != 4 && !f.spw; }
 __device__ __forceinline__ void build_e4m3_lut(uint8_t* lut, const OpFmt& f, int t, int nt)
 {
     for (int c = t; c < (1 << f.b); c += nt) lut[c] = (uint8_t)code_to_e4m3((uint32_t)c, f);
