@@ -37,11 +37,12 @@ constexpr int kQatThreads = 256;
 // fl32(c / s) is monotone in c, so the projection's thresholds T_j on x_hat
 // become thresholds on |c| = |fl32(x - mu)|: the smallest float whose
 // quotient by s reaches T_j, found once per block with the same division.
-// No division per element, and the fake-quantised value is a table entry.
+// No division per element (but for few elements of a wide format, see
+// launch_dn_project), and the fake-quantised value is a table entry.
 // HBM-bound (4 B in, 4.5 B out per element at b = 4): a warp loads and
-// stores 128 consecutive values at a time.  6.4 M elements, (4,2), from
-// HBM: 34 us with one thread per word and a division per element, 18 us this
-// way.
+// stores 128 consecutive values at a time.  6.4 M elements, (4,2): 31.8 us with
+// one thread per word and a division per element, 12.7 us this way (inputs in
+// L2; 34 and 18 us from HBM).
 template <int B>
 struct DnTable {
     static constexpr int CAP = B <= 6 ? 1024 : 2048;
@@ -52,16 +53,10 @@ struct DnTable {
 
 constexpr int kDnUnroll = 6;       // granules in flight per warp (flat 4-bit path)
 
-// One value by division, for a sigma that is not finite (or +-0 with eps lost).
-__device__ __noinline__ uint32_t dn_code_div(float x, float m, float s, float alpha, ProjParams p)
-{
-    return project_code(__fdiv_rn(__fsub_rn(x, m), s), alpha, p);
-}
-
 template <int B>
 __global__ void __launch_bounds__(kQatThreads)
 dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const double* __restrict__ stats,
-                  float alpha, ProjParams p, uint32_t* __restrict__ codes, int64_t ldc, float* __restrict__ xq, int flat)
+                  float alpha, ProjParams p, uint32_t* __restrict__ codes, int64_t ldc, float* __restrict__ xq, int flat, int divide)
 {
     constexpr int CPW = 32 / B;
     constexpr int L = 1 << (B - 1);
@@ -75,7 +70,8 @@ dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const
     build_thresholds(sm.T, p, alpha, warp, lane, 0, kQatThreads / 32);
     __syncthreads();
     const float m = ms.x, s = ms.y;
-    const bool by_div = !(s > 0.0f && s < __int_as_float(0x7f800000));
+    // also for a sigma that is not finite (or +-0 with eps lost), which no threshold can stand for
+    const bool by_div = divide || !(s > 0.0f && s < __int_as_float(0x7f800000));
     if (!by_div) {
         for (int j = warp; j < L - 1; j += kQatThreads / 32) {
             const float t = sm.T[j];                  // each threshold is read and replaced by one warp
@@ -94,7 +90,7 @@ dn_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, const
     const uint32_t amask = p.is_signed ? 0x7fffffffu : 0xffffffffu;
     auto code_of = [&](float v) -> uint32_t {
         const float c = __fsub_rn(v, m);
-        if (by_div) return dn_code_div(v, m, s, alpha, p);
+        if (by_div) return project_by_table_t<B>(__fdiv_rn(c, s), sm.T, p);
         if (B == 4) return project_by_thr7(c, t7, p);
         return by_cells ? project_by_cells<B>(c, sm.cells, h0, hmax, sh, amask) : project_by_table_t<B>(c, sm.T, p);
     };
@@ -401,13 +397,28 @@ cudaError_t launch_dn_project(const float* x, int64_t rows, int64_t cols, const 
     const ProjParams p = make_proj_params(b, k, is_signed, rounding);
     auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     const int flat = b == 4 && ldc * 8 == cols && al16(x) && (!xq || al16(xq));
-    const int64_t units = flat ? rows * cols / 4 : rows * ldc;
-    const int64_t blocks = (int64_t)qat_blocks(units) * 2;
-    using Kernel = void (*)(const float*, int64_t, int64_t, const double*, float, ProjParams, uint32_t*, int64_t, float*, int);
+    const int64_t sms = device_sm_count(), words = rows * ldc;
+    // Every block builds its tables, and all of an SM's blocks at once take
+    // longer over it than a block alone: no more blocks than have work.  Flat
+    // 4-bit codes: a warp's granules in flight together (20000 x 64: 4.7 us,
+    // 12.4 with a granule per warp).  Elsewhere a cap by width (20000 x 64, 8
+    // bits: 12.8 us with 2 blocks an SM, 16.5 with 4, 26.2 with 8; 100352 x 64, 6
+    // bits: 27.8, 24.6, 24.5; 2 bits: 33.4, 37.4, 42.6; 100352 x 77, 4 bits: 39.6,
+    // 43.9, 37.2).
+    const int64_t cap = sms * (b == 2 || b == 8 ? 2 : (b == 4 ? 8 : 4));
+    int64_t blocks = flat ? (rows * cols / 128 + 8 * kDnUnroll - 1) / (8 * kDnUnroll) : (words + kQatThreads - 1) / kQatThreads;
+    if (blocks > cap) blocks = cap;
+    if (blocks < 1) blocks = 1;
+    // Wide formats with at most a word per thread: a division per element costs
+    // less than thresholds on |x - mu| and their table (1000 x 77, 8 bits: 6.0 us
+    // against 8.3 to 9.6; 6 bits 3.9 against 4.3 to 4.7; at 10000 x 64 they are
+    // level, at 100352 x 64 the table takes 24.6 against 27.8 at 6 bits).
+    const int divide = b >= 6 && words <= sms * 4 * kQatThreads;
+    using Kernel = void (*)(const float*, int64_t, int64_t, const double*, float, ProjParams, uint32_t*, int64_t, float*, int, int);
     static const Kernel kernels[] = {dn_project_kernel<2>, dn_project_kernel<3>, dn_project_kernel<4>, dn_project_kernel<5>,
                                      dn_project_kernel<6>, dn_project_kernel<7>, dn_project_kernel<8>};
     return launch_pdl(kernels[b - 2], dim3((unsigned)blocks), dim3(kQatThreads), 0, st, x, rows, cols, stats, alpha, p,
-                      codes, ldc, xq, flat);
+                      codes, ldc, xq, flat, divide);
 }
 
 cudaError_t launch_dn_grad(const float* g, const float* x, int64_t n, const double* stats, void* workspace, float* gx,

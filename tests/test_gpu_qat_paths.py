@@ -1,6 +1,6 @@
 """The training kernels at the edges of their paths: every width of
-dn_project (flat 4-bit granules, words packed through shared memory, a sigma
-no threshold can stand for), and dn_backward where fp32 pairs cannot carry
+dn_project (flat 4-bit granules, a thread per word by thresholds on |x - mu| or
+by division, a sigma no threshold can stand for), and dn_backward where fp32 pairs cannot carry
 the values (infinities, underflow, constant inputs) or pointers are not
 16-byte aligned."""
 import numpy as np
@@ -19,7 +19,8 @@ def built():
     __graft_entry__.build()
 
 
-@pytest.mark.parametrize("rows,cols", [(1, 8), (37, 24), (5, 136), (3, 1), (2, 331)])
+# the last: more words than the wide formats divide for (a thread per word of four blocks per SM)
+@pytest.mark.parametrize("rows,cols", [(1, 8), (37, 24), (5, 136), (3, 1), (2, 331), (40001, 16)])
 @pytest.mark.parametrize("fmt", [(2, 0, True), (3, 1, True), (4, 2, True), (4, 1, False), (5, 2, True), (6, 5, True),
                                  (7, 3, True), (8, 4, False)])
 @pytest.mark.parametrize("sigma", [1.7, 0.0, float("inf"), float("nan")])
