@@ -256,12 +256,16 @@ project_vec_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
 // division and eight predicated bisections for each), 24 us this way; rows of
 // 9 values 50 and 15 us.  Longer rows stay with a thread per word, whose
 // neighbours share cache lines: warp segments packed through shared memory
-// took 20 us there against 16 at 1001 columns, 81 against 27 at 17.
+// took 20 us there against 16 at 1001 columns, 81 against 27 at 17.  So do few
+// rows with much padding (launch_project_b).
+// cells: the cell table (b != 4), worth its set-up only when a thread has
+// several rows (6 bits: 1000 rows 2.97 us without, 3.18 with; 300000 rows 7.5 and
+// 8.1; 3 M rows 28.1 and 22.3; 7 bits, k = 6: 1000 rows 3.9 and 5.2).
 template <int B>
 __global__ void __launch_bounds__(256)
 project_rows_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ldx,
                    float alpha, const float* __restrict__ alpha_dev, ProjParams p,
-                   uint32_t* __restrict__ codes, int64_t ldc, int vec)
+                   uint32_t* __restrict__ codes, int64_t ldc, int vec, int use_cells)
 {
     constexpr int CPW = 32 / B;
     constexpr int L = 1 << (B - 1);
@@ -275,7 +279,7 @@ project_rows_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int
 #pragma unroll
     for (int i = 0; i < 7; i++) t7.t[i] = B == 4 ? T[i] : 0.0f;
     int h0 = 0, hmax = 0;
-    const bool by_cells = B != 4 && build_cells<B, CAP>(cells, h0, hmax, T, p);
+    const bool by_cells = B != 4 && use_cells && build_cells<B, CAP>(cells, h0, hmax, T, p);
     const int sh = cell_shift(p.k);
     const uint32_t amask = p.is_signed ? 0x7fffffffu : 0xffffffffu;
     auto code_of = [&](float v) -> uint32_t {
@@ -367,7 +371,10 @@ static cudaError_t launch_project_b(const float* x, int64_t rows, int64_t cols, 
         if (blocks < 1) blocks = 1;
         project_vec_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc);
     } else {
-        const bool by_rows = cols <= 2 * (32 / B);
+        // a thread writes its whole row: with long rows there must be enough of
+        // them (512 words: 2000 rows 18.9 us, 8.8 with a thread per word; 8000 rows
+        // 19.0 and 27.0; 64 rows of 1024 words 10.4 and 2.6)
+        const bool by_rows = cols <= 2 * (32 / B) && (ldc <= 16 || rows >= 6000);
         const int64_t units = by_rows ? rows : rows * ldc;
         int64_t blocks = (units + threads - 1) / threads;
         const int64_t cap = (int64_t)sms * 8;
@@ -375,7 +382,8 @@ static cudaError_t launch_project_b(const float* x, int64_t rows, int64_t cols, 
         if (blocks < 1) blocks = 1;
         if (by_rows) {
             const int v16 = ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
-            project_rows_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc, v16);
+            project_rows_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc, v16,
+                                                                     rows > cap * threads);
         } else {
             project_any_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc);
         }

@@ -20,7 +20,9 @@ def built():
 @pytest.mark.parametrize("b,k,signed", [(2, 0, True), (3, 1, False), (4, 2, True), (4, 0, False), (5, 2, True), (6, 5, True),
                                         (7, 3, False), (8, 4, True)])
 @pytest.mark.parametrize("rows,cols,ldc_extra,shift", [(1000, 3, 0, 0), (333, 1, 3, 0), (70, 0, 0, 1), (200, 9, 1, 1), (129, 63, 0, 0),
-                                                       (5, 1000, 0, 1), (3, 1025, 2, 0), (40, 17, 9, 0)])
+                                                       (5, 1000, 0, 1), (3, 1025, 2, 0), (40, 17, 9, 0),
+                                                       (320001, 3, 0, 0),             # several rows a thread: the cell table
+                                                       (70, 3, 40, 0), (6001, 3, 40, 0)])  # long padding: a thread per word, per row
 def test_project_any_rows(b, k, signed, rows, cols, ldc_extra, shift):
     cpw = 32 // b
     cols = {0: 2 * cpw, 9: 2 * cpw + 1}.get(cols, cols)           # the last short row, the first long one
