@@ -188,8 +188,9 @@ __device__ __forceinline__ F2 f2_mul(const F2& a, const F2& b)
     r.l = fmaf(a.h, b.h, -r.h) + fmaf(a.h, b.l, a.l * b.h);
     return r;
 }
-// Scalars whose products with ordinary values stay well inside fp32's range.
-__device__ __forceinline__ bool f2_safe(double d) { return d == 0.0 || (fabs(d) > 0x1p-60 && fabs(d) < 0x1p60); }
+// Scalars that a pair holds to 2^-48 and whose products with ordinary values
+// stay well inside fp32's range.
+__device__ __forceinline__ bool f2_safe(double d) { return d == 0.0 || (fabs(d) > 0x1p-100 && fabs(d) < 0x1p60); }
 
 constexpr int kGradUnroll = 4;
 
@@ -204,16 +205,19 @@ dn_grad_partials_kernel(const float* __restrict__ g, const float* __restrict__ x
 {
     __shared__ double2 sh[kQatThreads / 32];
     __shared__ F2 sh_mu;
-    __shared__ int sh_ok;
+    __shared__ float sh_gmin;
     griddep_wait();
     if (threadIdx.x == 0) {                           // fp64 in one thread (see dn_project_kernel)
         const double mu = __ldg(stats), sigma = __ldg(stats + 1);
         sh_mu = f2_of(mu);
-        sh_ok = sigma > 0x1p-40 && sigma < 0x1p40 && fabs(mu) < 0x1p60;
+        // a thread's largest |g| for which the error terms of its products
+        // g (x - mu), about 2^-24 |g| sigma, stay above the subnormals
+        const bool ok = sigma > 0x1p-40 && sigma < 0x1p40 && fabs(mu) < 0x1p60;
+        sh_gmin = ok ? (float)fmax(0x1p-100, 0x1p-100 / sigma) : __int_as_float(0x7f800000);
     }
     __syncthreads();
     const F2 mu2 = sh_mu;
-    const bool stats_ok = sh_ok != 0;
+    const float gmin = sh_gmin;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float s1h = 0.0f, s1l = 0.0f, s2h = 0.0f, s2l = 0.0f, mx = 0.0f;
@@ -245,7 +249,7 @@ dn_grad_partials_kernel(const float* __restrict__ g, const float* __restrict__ x
     for (int64_t i = nv * 4 + t0; i < n; i += stride) add(g[i], x[i]);
     auto finite = [&]() { return fabsf(s1h + s1l) < __int_as_float(0x7f800000) && fabsf(s2h + s2l) < __int_as_float(0x7f800000); };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    bool pairs = __all_sync(0xffffffffu, finite() && (mx == 0.0f || mx > 0x1p-40f) && stats_ok);
+    bool pairs = __all_sync(0xffffffffu, finite() && gmin < 1.0f && (mx == 0.0f || mx > gmin));
     if (pairs) {
         // the warp's sums in pairs; fp64 only once per warp (its pipe takes
         // a block's worth of conversions and adds longer than the loads).
@@ -292,7 +296,7 @@ dn_grad_partials_kernel(const float* __restrict__ g, const float* __restrict__ x
 struct GradScalars {
     double mu, s, gm, k2;                             // for the elements fp64 recomputes
     F2 mu2, gm2, k22, inv2;
-    int safe;
+    int safe, none;                                   // none: mean and k2 are zero (no gradient at all)
 };
 __global__ void __launch_bounds__(kQatThreads)
 dn_grad_total_kernel(double2* part, int nparts, int64_t n, const double* __restrict__ stats)
@@ -330,6 +334,7 @@ dn_grad_kernel(const float* __restrict__ g, const float* __restrict__ x, int64_t
         sc.mu = mu; sc.s = s; sc.gm = t.x; sc.k2 = t.y;
         sc.mu2 = f2_of(mu); sc.gm2 = f2_of(t.x); sc.k22 = f2_of(t.y); sc.inv2 = f2_of(inv);
         sc.safe = f2_safe(mu) && f2_safe(t.x) && f2_safe(t.y) && f2_safe(inv) && inv != 0.0;
+        sc.none = sc.safe && t.x == 0.0 && t.y == 0.0;
     }
     __syncthreads();
     const bool safe = sc.safe != 0;
@@ -340,8 +345,10 @@ dn_grad_kernel(const float* __restrict__ g, const float* __restrict__ x, int64_t
         const F2 r = f2_sub(a.h, b);                  // a.h - (b.h + b.l)
         const float y = r.h + (r.l + a.l);
         // not finite, or small enough that an error term may have underflowed
-        if (!safe || !(fabsf(y) > 0x1p-80f) || !(fabsf(y) < __int_as_float(0x7f800000)))
+        if (!safe || !(fabsf(y) > 0x1p-100f) || !(fabsf(y) < __int_as_float(0x7f800000))) {
+            if (sc.none && __float_as_uint(gi) == 0u && fabsf(xi) < __int_as_float(0x7f800000)) return 0.0f;
             return (float)(((double)gi - sc.gm) / sc.s - ((double)xi - sc.mu) * sc.k2);
+        }
         return y;
     };
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;

@@ -39,13 +39,15 @@ def test_dn_project_widths(rows, cols, fmt, sigma):
 
 
 @pytest.mark.parametrize("n,shift", [(1, 0), (3, 0), (4097, 0), (70001, 1)])
-@pytest.mark.parametrize("kind", ["ordinary", "tiny", "huge", "inf", "zero", "mean"])
+@pytest.mark.parametrize("kind", ["ordinary", "small", "tiny", "huge", "inf", "zero", "mean"])
 def test_dn_backward_ranges(n, shift, kind):
     """Against fp64: one rounding to fp32 (2^-24 relative), plus the pairs'
     2^-44 of the larger of the two terms that are subtracted."""
     x = synth.normal((n + shift,), seed=n, mean=0.4, std=1.3)
     g = synth.normal((n + shift,), seed=n + 1)
-    if kind == "tiny":
+    if kind == "small":
+        g = g * 1e-22
+    elif kind == "tiny":
         g = g * 1e-36
     elif kind == "huge":
         g, x = g * 1e30, x * 1e25
@@ -93,3 +95,15 @@ def test_dn_backward_sums_that_overflow_between_lanes(n, kind):
     # |x - mu| is at most about 4 sigma
     tol = 2.0 ** -24 * (t1 - t2).abs() + 2.0 ** -44 * (t1.abs() + t2.abs() + float(gc.abs().mean()) / s)
     assert bool(((got - (t1 - t2)).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("mu,sigma", [(0.0, float("nan")), (float("nan"), 1.0), (float("nan"), 0.0), (0.5, float("inf")), (0.5, 0.0)])
+def test_dn_backward_of_no_gradient(mu, sigma):
+    """A gradient of zeros is zero, but NaN where the statistics or x make the fp64 expression so."""
+    x = torch.tensor([0.5, -1.0, float("inf"), float("nan"), 3.0])
+    g = torch.zeros(5)
+    st = torch.tensor([mu, sigma], dtype=torch.float64)
+    got = esb.esb_dn_backward(g.cuda(), x.cuda(), st.cuda()).cpu().double()
+    c, s = x.double() - mu, sigma + 1e-7
+    k2 = float((g.double() * c).sum()) / (5 * sigma * s * s) if sigma > 0 else 0.0
+    assert torch.equal(got.isnan(), ((g.double() - 0.0) / s - c * k2).isnan()) and bool((got[~got.isnan()] == 0).all())
