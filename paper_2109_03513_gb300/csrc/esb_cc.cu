@@ -378,7 +378,13 @@ __device__ inline float dw_threshold(float sc, float b, float T, int act)
 // are those of the integer kernel above, plus a word-at-a-time one for
 // codes-only outputs with per-channel scale and bias; the next filter row's
 // input words are loaded while the current row is multiplied.
-template <int STRIDE>
+// CODES: 4-bit codes alone, without a residual (lean, per-channel tables or
+// per element); the other outputs have an instance of their own: in one body
+// the registers of the threshold pairs were spilled, and calls with y or a
+// residual paid for code that they never ran (11 x 11 x 8, batch 8, y and
+// codes: 15.7 us in one body, 11.2 us apart; 56 x 56 x 144, batch 64, scale per
+// channel: 63.6 and 58.2).
+template <int STRIDE, bool CODES>
 __global__ void __launch_bounds__(128, 6)
 esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const uint32_t* __restrict__ W, int ldw,
                        int kw, int H, int Wd, int C, int pad, int P, int Q, int QS, int rows, CcEpi ep, int tables)
@@ -413,17 +419,15 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
     const float dqs = dq ? __fmul_rn(__ldg(ep.alpha_a_dev), __ldg(ep.alpha_b_dev)) * ep.dq_pow2 : 1.0f;
     const float sc_fixed = ep.scale ? 0.0f : (dq ? __fmul_rn(ep.scale0, dqs) : ep.scale0);
     const bool b4 = ep.out.b == 4 && ep.codes_out;
-    const bool lean = b4 && ep.acc24 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
-                      sc_fixed > 0.0f && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
-    // codes only, any scale and bias: the word's 8 codes from their buckets at once
-    const bool words8 = b4 && !lean && !ep.residual && !ep.acc_out && !ep.y_out;
+    const bool lean = CODES && ep.acc24 && !ep.scale && !ep.bias && sc_fixed > 0.0f &&
+                      (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
     const uint32_t sgn_out = ep.out.is_signed ? 1u : 0u;
     // non-negative outputs: a negative y is in bucket 0 by the compares alone
     const bool nonneg = !ep.out.is_signed || ep.act != ESB_ACT_NONE;
     __syncthreads();
     // per-channel thresholds on the integer sum, where every scale is positive
     __half* const atab = reinterpret_cast<__half*>(wtab2 + 9 * cp2);
-    bool ptab = tables && words8 && nonneg;           // the same in every thread
+    bool ptab = CODES && tables && !lean && nonneg;   // the same in every thread
     if (ptab) {
         bool bad = false;
         for (int i = threadIdx.x; i < cp2 * 2 * 7; i += blockDim.x) {
@@ -563,8 +567,9 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
                 a[2 * m] = f2.x;
                 a[2 * m + 1] = f2.y;
             }
-            if (words8) {
-                // per element: y = fma(scale, acc, bias), the activation, then
+            if constexpr (CODES) {
+                // any scale and bias: the word's 8 codes from their buckets at
+                // once; per element y = fma(scale, acc, bias), the activation, then
                 // the bucket of y (of |y| where negatives keep their sign);
                 // codes8_b4 turns buckets and signs into the word (zero
                 // buckets keep sign 0), as project_by_thr7 does per code
@@ -585,30 +590,30 @@ esb_dwconv3_b4h_kernel(const uint32_t* __restrict__ X, int ldx, int kx, const ui
                     }
                 }
                 ep.codes_out[ow] = codes8_b4(J & nib, S & nib, ep.out.k);
-                continue;
-            }
-            const int64_t pix = (int64_t)row * Q + q0 + uu;
-            uint32_t word = 0;
+            } else {
+                const int64_t pix = (int64_t)row * Q + q0 + uu;
+                uint32_t word = 0;
 #pragma unroll
-            for (int j = 0; j < 8; j++) {
-                const int c = w * 8 + j;
-                uint32_t code = ep.out.zero_code;
-                if (c < C) {
-                    const int64_t o = pix * C + c;
-                    if (ep.acc_out) ep.acc_out[o] = (int32_t)a[j];
-                    float y = __fmaf_rn(scv[j], a[j], biv[j]);
-                    if (ep.residual) {
-                        const uint32_t rc =
-                            (__ldg(ep.residual + pix * ep.res_ld + c / rcpw) >> (ep.res_b * (c % rcpw))) & rmask;
-                        y = __fmaf_rn(ep.res_scale, code_image_f(rc, ep.res_b, ep.res_k), y);
+                for (int j = 0; j < 8; j++) {
+                    const int c = w * 8 + j;
+                    uint32_t code = ep.out.zero_code;
+                    if (c < C) {
+                        const int64_t o = pix * C + c;
+                        if (ep.acc_out) ep.acc_out[o] = (int32_t)a[j];
+                        float y = __fmaf_rn(scv[j], a[j], biv[j]);
+                        if (ep.residual) {
+                            const uint32_t rc =
+                                (__ldg(ep.residual + pix * ep.res_ld + c / rcpw) >> (ep.res_b * (c % rcpw))) & rmask;
+                            y = __fmaf_rn(ep.res_scale, code_image_f(rc, ep.res_b, ep.res_k), y);
+                        }
+                        y = cc_act(y, ep.act);
+                        if (ep.y_out) ep.y_out[o] = y;
+                        if (ep.codes_out) code = b4 ? project_by_thr7(y, t7, ep.out) : project_by_table(y, T, ep.out);
                     }
-                    y = cc_act(y, ep.act);
-                    if (ep.y_out) ep.y_out[o] = y;
-                    if (ep.codes_out) code = b4 ? project_by_thr7(y, t7, ep.out) : project_by_table(y, T, ep.out);
+                    word |= code << (ep.out.b * j);
                 }
-                word |= code << (ep.out.b * j);
+                if (ep.codes_out) ep.codes_out[ow] = word;
             }
-            if (ep.codes_out) ep.codes_out[ow] = word;
         }
     }
 }
@@ -653,8 +658,9 @@ static cudaError_t launch_dw3(const esb_conv_desc& d, int P, int Q, const uint32
     const int words = (d.c + 32 / B - 1) / (32 / B);
     if constexpr (B == 4) {
         if (h16) {
-            const int tables = (ep.scale || ep.bias) && ep.codes_out && dw_tables_pay(items, words);
-            return launch_dw_wave(esb_dwconv3_b4h_kernel<STRIDE>,
+            const bool codes = ep.codes_out && ep.out.b == 4 && !ep.residual && !ep.acc_out && !ep.y_out;
+            const int tables = codes && (ep.scale || ep.bias) && dw_tables_pay(items, words);
+            return launch_dw_wave(codes ? esb_dwconv3_b4h_kernel<STRIDE, true> : esb_dwconv3_b4h_kernel<STRIDE, false>,
                                   sizeof(__half2) * 4 * (size_t)words * (9 + (tables ? 7 : 0)), items, d, P, Q, QS, X, ldx,
                                   kx, W, ldw, kw, ep, st, tables);
         }
