@@ -343,17 +343,18 @@ __device__ __forceinline__ uint32_t bucket7(float a, const Thr7& T)
     return j;
 }
 
-// The same bucket by a table over cells of |x| / T_6 for the HBM-bound
-// projections.  The 7-threshold search costs some 12 ALU instructions a value,
-// and the ALU pipe (80% busy, the FMA pipe 5%) bound them.  Here the cell index
-// is FMA-pipe work -- a saturating multiply by about 1 / T_6 (NaN -> 0), a
-// multiply-add that leaves round(126 t) in the low mantissa bits -- then one
-// 8-byte shared load {threshold, bucket below it} and one compare.  The index
-// is a non-decreasing function of |x| whatever its roundings, so a threshold
-// in a lower cell is at or below the value, one in a higher cell above it, and
-// the value's own cell holds at most one, which is compared exactly (checked
-// by the build; else the register search stays).  2^28 values of N(0,1): 257
-// us by the register search, 221 us (5.5 TB/s) by the table.
+// The same bucket by a table over cells of |x| / T_6 for the HBM-bound flat
+// projection (project_vec_kernel).  The 7-threshold search costs some 12 ALU
+// instructions a value, and the ALU pipe (80% busy, the FMA pipe 5%) bound it.
+// Here the cell index is FMA-pipe work -- a saturating multiply by about 1 /
+// T_6 (NaN -> 0), a multiply-add that leaves round(126 t) in the low mantissa
+// bits -- then one 8-byte shared load {threshold, bucket below it} and one
+// compare.  The index is a non-decreasing function of |x| whatever its
+// roundings, so a threshold in a lower cell is at or below the value, one in a
+// higher cell above it, and the value's own cell holds at most one, which is
+// compared exactly (checked by the build; else the register search stays).
+// 2^28 values of N(0,1): 257 us by the register search, 221 us (5.5 TB/s) by
+// the table.
 constexpr int kLinCells = 127;
 struct Lin7 {
     const uint2* tab;

@@ -971,15 +971,12 @@ calibrate_project_kernel(const float* __restrict__ x, int64_t rows, int64_t cols
 #pragma unroll
         for (int i = 0; i < 7; i++) t7.t[i] = T[i];
         if (flat) {                                     // flat codes: the statistics pass's granules
-            __shared__ uint2 lin_tab[B == 4 ? kLinCells : 1];
-            Lin7 lin;
-            if (build_lin7(lin_tab, lin, T)) {
-                if (p.is_signed) project_flat_b4<true, true>(x, n, lin, p.k, codes, stash, stash_g);
-                else project_flat_b4<false, true>(x, n, lin, p.k, codes, stash, stash_g);
-            } else {
-                if (p.is_signed) project_flat_b4<true, true>(x, n, t7, p.k, codes, stash, stash_g);
-                else project_flat_b4<false, true>(x, n, t7, p.k, codes, stash, stash_g);
-            }
+            // by the register search: the cell table that project_vec_kernel
+            // takes costs its set-up after the grid barrier, and its code is
+            // fetched cold (32 x 56 x 56 x 64 values: 14.3 us, 15.4 with the
+            // table; from HBM 16.3 and 17.4; 2^18 values 7.2 and 7.4)
+            if (p.is_signed) project_flat_b4<true, true>(x, n, t7, p.k, codes, stash, stash_g);
+            else project_flat_b4<false, true>(x, n, t7, p.k, codes, stash, stash_g);
             cal_depart(sync);
             return;
         }
