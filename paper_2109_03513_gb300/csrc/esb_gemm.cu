@@ -1085,13 +1085,14 @@ static int conv_halo_words(const esb_conv_desc& d, int64_t ldx, int kwx) { retur
 //   63, two words of channels: 3x3, 224 x 224 x 16 -> 64    59.2 and 85.4
 //   not resident: 11x11, 200 x 200 x 3 -> 64, batch 4       254 and 151
 // Significand planes and filters of another width do not decode by pieces
-// (3x3, 56 x 56 x 3 -> 32, (8,5): 706 us whole, 301 by words).
+// (3x3, 56 x 56 x 3 -> 32, (8,5): 706 us whole, 301 by words), and 2- and 3-bit
+// words take twice the slots (7x7, 13 x 13 x 16 -> 5, 2-bit: 26.3 and 20.7).
 static bool conv_whole_pays(const esb_conv_desc& d, int64_t M, const ConvK& whole, int kwx, int out_cpw)
 {
     cudaError_t e = cudaSuccess;
     const int st = ws_static_smem<ConvSrc>(&e);
     const int bn = resident_bn(M, d.cout, out_cpw, pick_bn(d.cout, out_cpw));   // as launch_ws
-    if (!conv_halo_rows(whole) || st < 0 || ws_layout(whole.K, bn, max_dyn_smem() - st).stages < 3) return false;
+    if (!conv_halo_rows(whole) || whole.fa.spw == 16 || st < 0 || ws_layout(whole.K, bn, max_dyn_smem() - st).stages < 3) return false;
     const int64_t sms = device_sm_count(), tiles = ((M + kBM - 1) / kBM) * ((d.cout + bn - 1) / bn);
     return kwx > 1 || (tiles + sms - 1) / sms * ((whole.K + kBK - 1) / kBK) <= 48;
 }

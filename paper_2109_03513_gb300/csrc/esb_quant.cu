@@ -352,6 +352,25 @@ project_any_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
     }
 }
 
+// Whether project_rows_kernel takes the call.  It pays where a row has padding
+// words or idle slots to skip; full words of many codes are as fast, or faster,
+// with a thread each (us by rows and by words, 6-bit rows in words of 5):
+//   one word: 3 of 5 columns, 3 M rows, 4 words      22.3 and 101
+//   16 2-bit columns, 64000 rows, one word           4.8 and 4.2; 3 8-bit ones, 512000 rows 20.6 and 18.4
+//   two words: 9 4-bit columns, 1000 rows            2.5 and 2.8; 16 of them 3.5 and 2.6
+//   10 6-bit columns, two words: 8000 rows 4.1 and 3.3, 64000 4.6 and 5.0, 2 M 28 and 48
+//   32 2-bit columns, two words, 64000 rows          10.7 and 6.3; 17 of them 3.7 and 5.2
+// A thread writes its whole row, so long rows must be many (512 words: 2000 rows
+// 18.9 and 8.8 us, 8000 rows 19.0 and 27.0; 64 rows of 1024 words 10.4 and 2.6).
+template <int B>
+static bool project_by_rows(int64_t rows, int64_t cols, int64_t ldc)
+{
+    constexpr int CPW = 32 / B;
+    if (cols > 2 * CPW || (ldc > 16 && rows < 6000)) return false;
+    if (cols <= CPW) return B == 2 ? cols <= 12 : (B != 8 || ldc > 1);
+    return B == 2 ? cols <= CPW + 4 : (B == 4 ? cols <= CPW + 4 : rows >= 65536);
+}
+
 template <int B>
 static cudaError_t launch_project_b(const float* x, int64_t rows, int64_t cols, int64_t ldx, float alpha,
                                     const float* alpha_dev, const ProjParams& p, uint32_t* codes,
@@ -371,10 +390,7 @@ static cudaError_t launch_project_b(const float* x, int64_t rows, int64_t cols, 
         if (blocks < 1) blocks = 1;
         project_vec_kernel<B><<<(unsigned)blocks, threads, 0, st>>>(x, rows, cols, ldx, alpha, alpha_dev, p, codes, ldc);
     } else {
-        // a thread writes its whole row: with long rows there must be enough of
-        // them (512 words: 2000 rows 18.9 us, 8.8 with a thread per word; 8000 rows
-        // 19.0 and 27.0; 64 rows of 1024 words 10.4 and 2.6)
-        const bool by_rows = cols <= 2 * (32 / B) && (ldc <= 16 || rows >= 6000);
+        const bool by_rows = project_by_rows<B>(rows, cols, ldc);
         const int64_t units = by_rows ? rows : rows * ldc;
         int64_t blocks = (units + threads - 1) / threads;
         const int64_t cap = (int64_t)sms * 8;

@@ -22,10 +22,12 @@ def built():
 @pytest.mark.parametrize("rows,cols,ldc_extra,shift", [(1000, 3, 0, 0), (333, 1, 3, 0), (70, 0, 0, 1), (200, 9, 1, 1), (129, 63, 0, 0),
                                                        (5, 1000, 0, 1), (3, 1025, 2, 0), (40, 17, 9, 0),
                                                        (320001, 3, 0, 0),             # several rows a thread: the cell table
-                                                       (70, 3, 40, 0), (6001, 3, 40, 0)])  # long padding: a thread per word, per row
+                                                       (70, 3, 40, 0), (6001, 3, 40, 0),   # long padding: a thread per word, per row
+                                                       (65537, -1, 0, 0), (65535, -1, 1, 0), (300, -1, 1, 1), (300, -2, 1, 0)])
 def test_project_any_rows(b, k, signed, rows, cols, ldc_extra, shift):
     cpw = 32 // b
-    cols = {0: 2 * cpw, 9: 2 * cpw + 1}.get(cols, cols)           # the last short row, the first long one
+    # the longest short row, the first long one; a word and one code (by rows from 65536 rows on, or at once)
+    cols = {0: 2 * cpw, 9: 2 * cpw + 1, -1: cpw + 1, -2: cpw + 5}.get(cols, cols)
     x = synth.normal((rows, cols), seed=rows + cols, std=1.5)
     x[0, 0], x[-1, -1] = float("nan"), -float("inf")
     buf = torch.zeros(rows * cols + 8, dtype=torch.float32, device="cuda")
