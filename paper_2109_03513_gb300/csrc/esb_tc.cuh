@@ -886,12 +886,13 @@ __device__ __forceinline__ EpiSplit epi_split(const EpiParams& ep, int BN, int64
 {
     const bool cells = GEN && epi_cells_ok(ep);
     const bool swar = !GEN && ep.codes_out && ep.out.b == 4;       // 16-column chunks of whole words
-    const int half = BN / 2;
+    // whole 16-column chunks and whole words on both sides (epi_cells splits by passes of its own)
+    const int cpw = ep.codes_out ? ep.out_cpw : 16;
+    const int unit = cpw == 6 ? 48 : (cpw == 5 || cpw == 10 ? 80 : 16);
     EpiSplit e;
     e.alt = (cells || swar) && (BN < 32 || (BN <= 64 && my_tiles >= 8));
-    e.mid = swar ? ((BN / 16 + 1) / 2) * 16 : half;
-    const bool split = cells || (swar && BN >= 32) || (half % 16 == 0 && half % ep.out_cpw == 0);
-    e.warps = (e.alt || split) ? 8 : 4;
+    e.mid = ((BN / unit + 1) / 2) * unit;
+    e.warps = (e.alt || cells || e.mid < BN) ? 8 : 4;
     return e;
 }
 
