@@ -512,9 +512,9 @@ enum {
  * out_b bits (0: no code output).  The filter stride is taken to be ldx
  * when fw.b == fx.b and esb_row_words(c, fw.b) otherwise, and the call to
  * have codes alone as its output (4-bit codes for out_b = 0), with a scalar
- * scale and bias: other calls of a strided layer of up to 4 channels may take
- * the im2col kernel where this answers the stem kernel, or the other way
- * round.  The choice depends only on these and on the device's shared memory
+ * scale and bias: other calls of a strided layer of up to 4 channels or of a
+ * 1x1 layer may take the im2col kernel where this answers the stem or halo
+ * kernel, or the other way round.  The choice depends only on these and on the device's shared memory
  * and SM count (queried on the current device); results are identical
  * whichever kernel runs.  Setting ESB_CONV_IM2COL=1 in the
  * environment before the first call disables the halo and stem kernels.

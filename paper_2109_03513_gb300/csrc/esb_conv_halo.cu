@@ -484,7 +484,7 @@ struct HaloPlan {
     int64_t K, smem, tiles;
 };
 
-// Static shared memory of the kernel (the larger of its two instances).
+// Static shared memory of the kernel (the largest of its three instances).
 static int halo_static_smem(cudaError_t* err)
 {
     static int v = -1;
@@ -506,7 +506,8 @@ static int halo_static_smem(cudaError_t* err)
 // Geometry, N-tile width and shared-memory budget of the halo path, or
 // false when the shape does not suit it.  BN starts at bn0 and shrinks
 // (keeping whole output words) until the resident B and two halo stages fit.
-static bool halo_plan(const esb_conv_desc& d0, int P, int Q, int64_t ldx, const OpFmt& fa, int bn0, int out_cpw,
+// e16: the epilogue's cost (epi_cost16).
+static bool halo_plan(const esb_conv_desc& d0, int P, int Q, int64_t ldx, const OpFmt& fa, int bn0, int out_cpw, double e16,
                       HaloPlan* hp, cudaError_t* err)
 {
     *err = cudaSuccess;
@@ -514,11 +515,15 @@ static bool halo_plan(const esb_conv_desc& d0, int P, int Q, int64_t ldx, const 
     // that every tile is full whatever the width.  With one channel block only:
     // over several, image rows measured faster (28x28x144 -> 32: 12.0 against
     // 13.6 us; 7x7x960 -> 160 on the im2col kernel 16 against 23 us), while
-    // 112x112x32 -> 16 gains 58 -> 51 us and 56x56x24 -> 144 33 -> 31.
+    // 112x112x32 -> 16 gains 58 -> 48 us and 56x56x24 -> 144 33 -> 30.  Not where
+    // a costly epilogue meets fewer tiles than SMs: the im2col kernel then takes
+    // narrower N-tiles (66x68x64 -> 97, batch 2, 8-bit codes with a residual: 53.4
+    // us here, 24.0 there).
     esb_conv_desc d = d0;
     hp->g.tail = d.w;
-    if (d.r == 1 && d.s == 1 && d.stride == 1 && d.pad == 0 && ldx <= 16) {
-        const int64_t pixels = (int64_t)d.n * d.h * d.w;
+    const int64_t pixels = (int64_t)d.n * d.h * d.w;
+    const bool idle = bn0 > 0 && (pixels + kBM - 1) / kBM * ((d.cout + bn0 - 1) / bn0) < device_sm_count();
+    if (d.r == 1 && d.s == 1 && d.stride == 1 && d.pad == 0 && ldx <= 16 && !(idle && e16 >= 1.0)) {
         if (pixels >= (1ll << 30)) return false;
         d.n = 1;
         d.w = kBM;
@@ -578,14 +583,15 @@ static bool halo_plan(const esb_conv_desc& d0, int P, int Q, int64_t ldx, const 
     return false;
 }
 
-bool conv_halo_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int out_cpw)
+bool conv_halo_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int out_b)
 {
+    const int out_cpw = 32 / out_b;
     HaloPlan hp;
     cudaError_t e;
     OpFmt fa = make_opfmt(bx, kx);
     if (bx == 5 || bx == 6) fa.spw = 8;               // as plan_slots for same-width input and filters
     if (bx == 2 || bx == 3) fa.spw = 16;
-    return halo_plan(d, P, Q, ldx, fa, pick_bn(d.cout, out_cpw), out_cpw, &hp, &e);
+    return halo_plan(d, P, Q, ldx, fa, pick_bn(d.cout, out_cpw), out_cpw, epi_cost16_codes(out_b), &hp, &e);
 }
 
 bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa,
@@ -593,7 +599,7 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
                       cudaError_t* err)
 {
     HaloPlan hp;
-    if (!halo_plan(d, P, Q, ldx, fa, BN, ep.out_cpw, &hp, err)) return *err != cudaSuccess;
+    if (!halo_plan(d, P, Q, ldx, fa, BN, ep.out_cpw, epi_cost16(ep), &hp, err)) return *err != cudaSuccess;
     if (hp.smem <= 0 || hp.smem > max_dyn_smem() - halo_static_smem(err)) {
         *err = cudaErrorInvalidConfiguration;
         return true;

@@ -344,30 +344,36 @@ struct StemPlan {
 };
 
 // Whether this kernel finishes before the im2col kernel, by a model of both in
-// microseconds: waves of tiles (one CTA per SM) times a tile's cost.  Both
-// tiles are 128 rows, but here only `use` = Q / (128 nseg) of them are outputs,
-// so a costly epilogue counts 1 / use times; the im2col kernel pays for each
-// filter tap's word (another filter width: code by code) and a longer prologue.
-// A tile's two roles overlap but for about a quarter of the shorter one.
+// microseconds: a fixed part (launch, prologue), and waves of tiles (one CTA per
+// SM) times a tile's cost.  Both tiles are 128 rows, but here only `use` = Q /
+// (128 nseg) of them are outputs, so a costly epilogue counts 1 / use times; the
+// im2col kernel pays for each filter tap's word (another filter width: code by
+// code) and a longer prologue, and takes narrower N-tiles where few row tiles
+// leave SMs idle (resident_bn).  A tile's two roles overlap but for about a
+// quarter of the shorter one.
 // Measured, this kernel and im2col, 7x7/2 -> 64, 4-bit codes alone: 295 and 291
 // us at 26 columns (use 0.2), 125 and 282 at 64, 85 and 286 at 100; with a
 // scale per channel 592 and 381 at 64, 392 and 382 at 100; with y 847 and 327
 // at 32; 2x2/2 -> 287, 3-bit, at 26: 283 and 69; 6-bit 3x3/2 -> 64: 134 and 101
-// at 64, 91 and 101 at 100.
-static bool stem_pays(const StemGeom& g, int64_t n, int64_t N, int BN, bool mixed, double e16)
+// at 64, 91 and 101 at 100; one image of 224 x 224: 10.5 and 19.2; 10 x 10 -> 164
+// sums alone, batch 3: 26.0 and 14.2.
+static bool stem_pays(const StemGeom& g, int64_t n, int64_t N, int BN, int out_cpw, bool mixed, double e16)
 {
     const double sms = device_sm_count();
-    const int64_t n_tiles = (N + BN - 1) / BN, m_tiles = (n * g.P * g.Q + kBM - 1) / kBM;
-    const double epi = e16 * BN / 16;
+    const int64_t m = n * g.P * g.Q;
+    const int bni = resident_bn(m, N, out_cpw, BN);
+    const double epi = e16 * BN / 16, epi_i = e16 * bni / 16;
     const double gather = fmax(2.0, 0.5 + 0.15 * g.R * g.S) * (mixed ? 3 : 1);
-    const double im2col = 7.0 + ceil((double)(m_tiles * n_tiles) / sms) * (fmax(epi, gather) + 0.25 * fmin(epi, gather));
-    return ceil((double)(n * g.P * g.nseg * n_tiles) / sms) * fmax(epi, 0.8 + 0.06 * g.R * g.G) < im2col;
+    const double im2col = 14.0 + ceil((double)(((m + kBM - 1) / kBM) * ((N + bni - 1) / bni)) / sms) *
+                                    (fmax(epi_i, gather) + 0.25 * fmin(epi_i, gather));
+    const double stem = 9.0 + ceil((double)(n * g.P * g.nseg * ((N + BN - 1) / BN)) / sms) * fmax(epi, 0.8 + 0.06 * g.R * g.G);
+    return stem < im2col;
 }
 
 // Up to 4 channels, stride 2 or 4 (stride 1 has the halo kernel), whole-byte
 // formats, where it pays (stem_pays).  e16: the epilogue's cost (epi_cost16).
-static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int bn0, double e16,
-                      StemPlan* sp, cudaError_t* err)
+static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int bw, int kw, int bn0, int out_cpw,
+                      double e16, StemPlan* sp, cudaError_t* err)
 {
     *err = cudaSuccess;
     if (d.c > 4 || (d.stride != 2 && d.stride != 4) || fmt_needs_split(bx, kx) || fmt_needs_split(bw, kw) || d.r > 16 || d.s > 16 ||
@@ -383,7 +389,7 @@ static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx,
     g.nseg = (per + umax - g.G) / (umax - g.G + 1);
     g.Ui = (per + g.nseg - 1) / g.nseg;
     g.U = g.Ui + g.G - 1;
-    if ((int64_t)d.n * P * g.nseg >= (1ll << 30) || !stem_pays(g, d.n, d.cout, bn0, bx != bw, e16)) return false;
+    if ((int64_t)d.n * P * g.nseg >= (1ll << 30) || !stem_pays(g, d.n, d.cout, bn0, out_cpw, bx != bw, e16)) return false;
     g.pitch = (kBM + g.G - 1) * 16;
     const int st = stem_static_smem(err);
     if (st < 0) return false;
@@ -405,14 +411,14 @@ bool conv_stem_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int
     StemPlan sp;
     cudaError_t e;
     const int bn = pick_bn(d.cout, 32 / out_b);
-    return bn > 0 && stem_plan(d, P, Q, ldx, bx, kx, bw, kw, bn, epi_cost16_codes(out_b), &sp, &e);
+    return bn > 0 && stem_plan(d, P, Q, ldx, bx, kx, bw, kw, bn, 32 / out_b, epi_cost16_codes(out_b), &sp, &e);
 }
 
 bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa, const uint32_t* W,
                       int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st, cudaError_t* err)
 {
     StemPlan sp;
-    if (!stem_plan(d, P, Q, ldx, fa.b, fa.k, fb.b, fb.k, BN, epi_cost16(ep), &sp, err)) return *err != cudaSuccess;
+    if (!stem_plan(d, P, Q, ldx, fa.b, fa.k, fb.b, fb.k, BN, ep.out_cpw, epi_cost16(ep), &sp, err)) return *err != cudaSuccess;
     sp.g.X = X;
     static bool configured = false;
     if (!configured) {

@@ -783,7 +783,7 @@ static int streamed_bn(int64_t M, int64_t N, int out_cpw, int bn0)
 // (128 rows each, again for every N-tile) and its BN rows of B once; the
 // width (a multiple of 16 and of the output codes per word, at most bn0)
 // that minimises waves x tiles per CTA x (128 + BN), the wider on a tie.
-static int resident_bn(int64_t M, int64_t N, int out_cpw, int bn0)
+int resident_bn(int64_t M, int64_t N, int out_cpw, int bn0)
 {
     const int64_t sms = device_sm_count();
     const int64_t mt = (M + kBM - 1) / kBM;
@@ -883,7 +883,8 @@ bool lean4_ok(const EpiParams& ep)
 double epi_cost16_codes(int out_b)
 {
     if (out_b == 4) return 0.3;
-    return out_b == 3 || out_b == 5 || out_b == 6 ? 0.47 : 2.0;   // cell table, else a bisection
+    if (out_b == 3 || out_b == 5 || out_b == 6) return 0.47;      // cell table
+    return out_b == 2 ? 1.25 : 2.0;                               // bisection
 }
 
 double epi_cost16(const EpiParams& ep)
@@ -891,7 +892,7 @@ double epi_cost16(const EpiParams& ep)
     const bool ch = ep.scale || ep.bias;
     if (!ep.codes_out) return 1.5;                                // fp32 or int32 alone
     if (ep.acc_out || ep.y_out) return ep.out.b == 4 ? 2.1 : 5.0;
-    if (ep.out.b != 4) return ch && epi_cells_ok(ep) ? 0.8 : (epi_cells_ok(ep) ? 0.47 : 2.0);
+    if (ep.out.b != 4) return !epi_cells_ok(ep) ? (ep.out.b == 2 ? 1.25 : 2.0) : (ch ? 0.8 : 0.47);
     if (ch || (ep.residual && ep.res_b != 4)) return 2.1;
     return ep.residual ? 0.8 : (lean4_ok(ep) ? 0.3 : 0.5);
 }
@@ -1144,7 +1145,7 @@ int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx
     if (!conv_force_im2col()) {
         if (conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, out_b)) return ESB_CONV_KERNEL_STEM;
         const ConvK h = conv_k(d, nullptr, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
-        if (conv_halo_rows(h) && conv_halo_ok(d, P, Q, ldx, bx, kx, cpw)) return ESB_CONV_KERNEL_HALO;
+        if (conv_halo_rows(h) && conv_halo_ok(d, P, Q, ldx, bx, kx, out_b)) return ESB_CONV_KERNEL_HALO;
     }
     const int64_t M = (int64_t)d.n * P * Q;
     int kwx;

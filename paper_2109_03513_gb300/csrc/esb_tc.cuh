@@ -1582,6 +1582,7 @@ __device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err, uin
 // ------------------------------------------------------------- host side
 
 int pick_bn(int64_t N, int out_cpw);          // N-tile width (esb_gemm.cu)
+int resident_bn(int64_t M, int64_t N, int out_cpw, int bn0);   // the same where few row tiles leave SMs idle
 int max_dyn_smem();                           // opt-in shared memory per block
 bool lean4_ok(const EpiParams& ep);           // the LEAN4 epilogue takes the call (esb_gemm.cu)
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
@@ -1602,11 +1603,12 @@ bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
 
 // Stride-1 convolution from a decoded input halo (esb_conv_halo.cu).  Returns
 // false, launching nothing, when the shape does not suit it (stride != 1,
-// A not 4-bit, rows wider than 128 - pad, too little of the tile used, or
-// too little shared memory); otherwise launches and stores the launch
-// status in *err.  BN is the preferred N-tile width; a smaller one is used
-// when the resident filters would not fit.
-bool conv_halo_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int out_cpw);
+// neither 4-bit codes nor 2-, 3-, 5- or 6-bit word slots, rows wider than 128 -
+// pad, too little of the tile used, or too little shared memory); otherwise
+// launches and stores the launch status in *err.  BN is the preferred N-tile
+// width; a smaller one is used when the resident filters would not fit.
+// conv_halo_ok: as conv_stem_ok.
+bool conv_halo_ok(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx, int kx, int out_b);
 bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, int64_t ldx, const OpFmt& fa,
                       const uint32_t* W, int64_t ldw, const OpFmt& fb, int BN, const EpiParams& ep, cudaStream_t st,
                       cudaError_t* err);
