@@ -41,8 +41,10 @@ def test_dn_project_widths(rows, cols, fmt, sigma):
 @pytest.mark.parametrize("n,shift", [(1, 0), (3, 0), (4097, 0), (70001, 1)])
 @pytest.mark.parametrize("kind", ["ordinary", "small", "tiny", "huge", "inf", "zero", "mean"])
 def test_dn_backward_ranges(n, shift, kind):
-    """Against fp64: one rounding to fp32 (2^-24 relative), plus the pairs'
-    2^-44 of the larger of the two terms that are subtracted."""
+    """Against fp64: one rounding to fp32 (2^-24 relative), plus 2^-40 of the two
+    terms that are subtracted and of the mean's term.  The pairs carry some 46
+    bits (their low parts are plain fp32 sums), fewer than fp64's 53, and x - mu
+    loses those of mu / sigma (13 at a mean of 1e4, where c is small against g)."""
     x = synth.normal((n + shift,), seed=n, mean=0.4, std=1.3)
     g = synth.normal((n + shift,), seed=n + 1)
     if kind == "small":

@@ -1,8 +1,7 @@
 """GPU parity of the 3-, 5- and 6-bit paths against the CPU oracle at the
 sizes where they can go wrong: the cell-table epilogue (passes of 20 or 24
 columns, ragged N, residuals, per-channel scales, thresholds no table can
-hold) and the tiled GEMM's packed operand runs (48 or 80 codes, N-tiles of
-240 columns)."""
+hold) and the tiled GEMM's packed operand runs (48 or 80 codes)."""
 import numpy as np
 import pytest
 import torch
@@ -74,9 +73,10 @@ def test_cell_table_epilogue(N, fo, act, per_channel, residual, alpha_out, ldo_e
 
 
 @pytest.mark.parametrize("M,N,K,f", [
-    (130, 256, 80, (6, 3)),         # one run, no tail; a 16-column second N-tile
+    # few row tiles: N-tiles of 80 columns (96 for 5-bit codes); the full width is in test_gpu_many_tiles.py
+    (130, 256, 80, (6, 3)),         # one run, no tail; four N-tiles, the last of 16 columns
     (1, 300, 81, (6, 2)),           # one code past a run
-    (200, 481, 47, (5, 2)),         # tail only; three N-tiles, the last of one column
+    (200, 481, 47, (5, 2)),         # tail only; six N-tiles, the last of one column
     (129, 260, 1000, (5, 2)),
     (64, 512, 560, (3, 1)),         # whole runs
     (150, 270, 159, (3, 0)),
