@@ -365,8 +365,12 @@ esb_status esb_dn_project(const float* x, int64_t rows, int64_t cols, const doub
  * through DN with the batch's mean and sigma, which depend on every
  * element: with c = x - mu, s = sigma + 1e-7 and d = n,
  *   grad_x[j] = (grad[j] - mean(grad)) / s - c[j] sum_i(grad[i] c[i]) / (d sigma s^2)
- * (the second term is 0 when sigma = 0).  Sums in fp64 in a fixed order;
- * grad_x rounded to fp32.
+ * (the second term is 0 when sigma = 0).  Each thread's sums and each
+ * element's terms are unevaluated pairs of fp32 numbers, about 46 significant
+ * bits (mu and mean(grad) as pairs too, so x - mu loses those of mu / sigma);
+ * values outside the pairs' range (not finite, or near the subnormals) are
+ * recomputed in fp64, and fp64 joins the warps' sums and computes the
+ * scalars.  The order of every sum is fixed; grad_x is rounded to fp32.
  *   grad, x [device] n floats; stats [device] {mu, sigma} of the forward
  *   workspace [device] >= esb_dn_backward_workspace_bytes(n), 16-byte aligned
  *   grad_x [device] n floats
@@ -431,8 +435,7 @@ esb_status esb_gemm(int64_t M, int64_t N, int64_t K,
  *              call overwrites it)
  * Shapes the tiled kernel does not take (N < 256, fewer than 2^32
  * multiply-adds of 4-bit operands, or fewer than 2^28 with output codes of
- * 3, 5 or 6 bits, where the other kernels finish first) run esb_gemm's
- * kernels; the workspace is then unused.  With output codes of 3, 5 or 6
+ * 3, 5 or 6 bits) run esb_gemm's kernels; the workspace is then unused.  With output codes of 3, 5 or 6
  * bits a workspace that is NULL, too small or misaligned also selects
  * esb_gemm's kernels.  Errors: as esb_gemm, and otherwise ALIGN (workspace)
  * or INVALID_ARG (workspace too small). */
@@ -498,7 +501,7 @@ esb_status esb_conv2d_nhwc(const esb_conv_desc* d,
 
 /* Kernels behind esb_conv2d_nhwc. */
 enum {
-    ESB_CONV_KERNEL_HALO = 1,      /* stride 1, 4-bit X: input rows decoded once,
+    ESB_CONV_KERNEL_HALO = 1,      /* stride 1, 2- to 6-bit X: input rows decoded once,
                                       each filter tap a shifted view (tcgen05) */
     ESB_CONV_KERNEL_IM2COL = 2,    /* implicit im2col, filters resident in shared memory */
     ESB_CONV_KERNEL_STREAMED = 3,  /* implicit im2col, filters streamed per K-block */

@@ -617,8 +617,9 @@ __device__ __forceinline__ uint32_t elect_one()
 // it with the same operands and the lane with `leader` issues it: operands
 // computed by warp-uniform code are in uniform registers, where the
 // instruction takes them (from a branch that only one lane enters each one
-// is moved there first, which made the issuing thread, at about 500 cycles
-// per MMA and commit, the slowest role of the small tiles).
+// is moved there first, which made the issuing thread, at about 500 cycles per
+// MMA and commit by clock reads in the kernel, the slowest role of the small
+// tiles).
 __device__ __forceinline__ void mma_f8f6f4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                            uint32_t idesc, uint32_t accumulate, uint32_t leader)
 {

@@ -223,7 +223,7 @@ __device__ __noinline__ void halo_decode_call(const HaloGeom g, int T, uint8_t* 
     halo_decode<B>(g, (T - nimg * g.tpi) * g.rows_out, st, first, stride, k, ew, fmt_zero_word(B, k));
 }
 
-template <bool FAST, bool GEN>
+template <bool FAST, int EPI>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, OpFmt fb, int BN, int nkb,
                      int stages, int n_tiles, int64_t m_tiles, float acc_scale, const __grid_constant__ EpiParams ep)
@@ -253,7 +253,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
     const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
-    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
+    const EpiSplit sp = epi_split<EPI>(ep, BN, my_tiles);
     const int cbs = g.cblocks;
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
@@ -462,7 +462,7 @@ esb_conv_halo_kernel(HaloGeom g, RowsSrc srcB, int64_t N, int64_t K, OpFmt fa, O
             m = ((int64_t)nimg * P + p) * Q + q;
             return p < P && q < (p + 1 < P ? Q : qlast);
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<EPI>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 
@@ -484,20 +484,24 @@ struct HaloPlan {
     int64_t K, smem, tiles;
 };
 
-// Static shared memory of the kernel (the largest of its three instances).
+// The instances by epilogue (epi_kind); [kEpiLean4] is the specialised one: 4-bit
+// B, bulk-copied input rows.
+typedef void (*HaloKernel)(HaloGeom, RowsSrc, int64_t, int64_t, OpFmt, OpFmt, int, int, int, int, int64_t, float, EpiParams);
+static const HaloKernel kHaloKernels[4] = {esb_conv_halo_kernel<false, kEpiB4>, esb_conv_halo_kernel<true, kEpiLean4>,
+                                           esb_conv_halo_kernel<false, kEpiGen>, esb_conv_halo_kernel<false, kEpiTable>};
+
+// Static shared memory of the kernel (the largest of its instances).
 static int halo_static_smem(cudaError_t* err)
 {
     static int v = -1;
     if (v < 0) {
-        cudaFuncAttributes a0, a1, a2;
-        *err = cudaFuncGetAttributes(&a0, esb_conv_halo_kernel<false, false>);
-        if (*err != cudaSuccess) return -1;
-        *err = cudaFuncGetAttributes(&a1, esb_conv_halo_kernel<true, false>);
-        if (*err != cudaSuccess) return -1;
-        *err = cudaFuncGetAttributes(&a2, esb_conv_halo_kernel<false, true>);
-        if (*err != cudaSuccess) return -1;
-        size_t m = a0.sharedSizeBytes > a1.sharedSizeBytes ? a0.sharedSizeBytes : a1.sharedSizeBytes;
-        if (a2.sharedSizeBytes > m) m = a2.sharedSizeBytes;
+        size_t m = 0;
+        for (HaloKernel k : kHaloKernels) {
+            cudaFuncAttributes a;
+            *err = cudaFuncGetAttributes(&a, k);
+            if (*err != cudaSuccess) return -1;
+            if (a.sharedSizeBytes > m) m = a.sharedSizeBytes;
+        }
         v = (int)m;
     }
     return v;
@@ -607,15 +611,10 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     hp.g.X = X;
     static bool configured = false;
     if (!configured) {
-        *err = cudaFuncSetAttribute(esb_conv_halo_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    max_dyn_smem() - halo_static_smem(err));
-        if (*err != cudaSuccess) return true;
-        *err = cudaFuncSetAttribute(esb_conv_halo_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    max_dyn_smem() - halo_static_smem(err));
-        if (*err != cudaSuccess) return true;
-        *err = cudaFuncSetAttribute(esb_conv_halo_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    max_dyn_smem() - halo_static_smem(err));
-        if (*err != cudaSuccess) return true;
+        for (HaloKernel k : kHaloKernels) {
+            *err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_smem() - halo_static_smem(err));
+            if (*err != cudaSuccess) return true;
+        }
         configured = true;
     }
     const int64_t N = d.cout;
@@ -627,11 +626,9 @@ bool launch_conv_halo(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     const int64_t grid = per_n * n_tiles;
     RowsSrc b{W, (int64_t)d.r * d.s * ldw, N};
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    // The specialised instance: 4-bit B, bulk-copied input rows, LEAN4 epilogue
-    const bool fast = fb.b == 4 && hp.g.raw_bytes > 0 && lean4_ok(ep);
-    const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
-    *err = launch_pdl(fast ? esb_conv_halo_kernel<true, false>
-                           : (gen ? esb_conv_halo_kernel<false, true> : esb_conv_halo_kernel<false, false>),
+    const int kind = epi_kind(ep);
+    const bool fast = kind == kEpiLean4 && fb.b == 4 && hp.g.raw_bytes > 0;   // what the specialised instance takes
+    *err = launch_pdl(kHaloKernels[kind == kEpiLean4 && !fast ? kEpiB4 : kind],
                       dim3((unsigned)grid), dim3(kWsThreads), (size_t)hp.smem, st, hp.g, b, N,
                       hp.K, fa, fb, hp.BN, hp.nkb, hp.stages, n_tiles, m_tiles, acc_scale, ep);
     return true;

@@ -110,7 +110,7 @@ __device__ __forceinline__ void stem_filter(const StemGeom& g, const uint32_t* W
 
 }  // namespace
 
-template <bool FAST, bool GEN>
+template <int EPI>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpFmt fa, OpFmt fb, int BN, int nkb, int n_tiles,
                      int m_tiles, float acc_scale, const __grid_constant__ EpiParams ep)
@@ -138,7 +138,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
     const int lacc = acc_buffers_log2(BN);
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < (BN << lacc)) tmem_cols <<= 1;
-    const EpiSplit sp = epi_split<GEN>(ep, BN, t_hi - t_lo);
+    const EpiSplit sp = epi_split<EPI>(ep, BN, t_hi - t_lo);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -303,7 +303,7 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
             m = ((int64_t)n * P + p) * Q + q;
             return live && q < Q;
         };
-        ws_epilogue<FAST, GEN>(ep, thr, rows, t_hi - t_lo, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<EPI>(ep, thr, rows, t_hi - t_lo, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
                                err, warp, lane);
     }
 
@@ -318,8 +318,8 @@ esb_conv_stem_kernel(StemGeom g, const uint32_t* Wt, int64_t ldw, int64_t N, OpF
 // ------------------------------------------------------------- host side
 
 typedef void (*StemKernel)(StemGeom, const uint32_t*, int64_t, int64_t, OpFmt, OpFmt, int, int, int, int, float, EpiParams);
-static const StemKernel kStemKernels[3] = {esb_conv_stem_kernel<false, false>, esb_conv_stem_kernel<true, false>,
-                                           esb_conv_stem_kernel<false, true>};
+static const StemKernel kStemKernels[4] = {esb_conv_stem_kernel<kEpiB4>, esb_conv_stem_kernel<kEpiLean4>,
+                                           esb_conv_stem_kernel<kEpiGen>, esb_conv_stem_kernel<kEpiTable>};
 
 static int stem_static_smem(cudaError_t* err)
 {
@@ -435,9 +435,7 @@ bool launch_conv_stem(const esb_conv_desc& d, int P, int Q, const uint32_t* X, i
     if (per_n < 1) per_n = 1;
     if (per_n > m_tiles) per_n = m_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool fast = lean4_ok(ep);                   // the specialised epilogue
-    const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
-    *err = launch_pdl(kStemKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
+    *err = launch_pdl(kStemKernels[epi_kind(ep)], dim3((unsigned)(per_n * n_tiles)), dim3(kWsThreads),
                       (size_t)sp.smem, st, sp.g, W, ldw, N, fa, fb, BN, sp.nkb, n_tiles, m_tiles, acc_scale, ep);
     return true;
 }

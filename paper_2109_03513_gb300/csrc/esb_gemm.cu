@@ -23,8 +23,8 @@
 //    stages (B resident), else each stage carries the B block of its
 //    K-block too (B streamed); 7 producer warps decode the stages of a ring
 //    of up to 8; one MMA warp issues tcgen05.mma (M = 128, N = BN, K = 32)
-//    into one of two TMEM accumulators and commits each stage to the
-//    mbarrier that frees it; 8 epilogue warps drain the other accumulator
+//    into one of two or four TMEM accumulators and commits each stage to the
+//    mbarrier that frees it; 8 epilogue warps drain the finished ones
 //    with tcgen05.ld, so the post-processing of tile i overlaps the MMAs of
 //    tile i+1 and the decode of later tiles (the paper's ping-pong buffers
 //    and overlapped timing graph, Sec. IV-C/IV-D).
@@ -483,7 +483,7 @@ __device__ __noinline__ void fill_stage_any(const Src src, int64_t m0, uint8_t* 
     }
 }
 
-template <class SrcA, bool LEAN4, bool GEN>
+template <class SrcA, int EPI>
 __global__ void __launch_bounds__(kWsThreads, 1)
 esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpFmt fa, OpFmt fb, int BN, int nkb,
                    int stages, int n_tiles, int64_t m_tiles, float acc_scale, const __grid_constant__ EpiParams ep, int bstream)
@@ -520,7 +520,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
     __shared__ int4 ptab[kWsProdWarps][32];          // producers' per-stage tap tables (im2col rows)
     if (reads_e4m3_lut(fa)) build_e4m3_lut(luta, fa, tid, kWsThreads);
     if (reads_e4m3_lut(fb)) build_e4m3_lut(lutb, fb, tid, kWsThreads);
-    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
+    const EpiSplit sp = epi_split<EPI>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -718,7 +718,7 @@ esb_gemm_ws_kernel(SrcA srcA, RowsSrc srcB, int64_t M, int64_t N, int64_t K, OpF
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
+        ws_epilogue<EPI>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty, err,
                     warp, lane);
     }
 
@@ -843,13 +843,12 @@ static cudaError_t launch_tc(const SrcA& a, const SrcB& b, int64_t M, int64_t N,
     return cudaGetLastError();
 }
 
-// The instances of the kernel by epilogue: 4-bit codes, 4-bit codes of the
-// specialised epilogue, other outputs.
+// The instances of the kernel by epilogue (epi_kind).
 template <class SrcA>
 struct WsKernels {
     typedef void (*Kernel)(SrcA, RowsSrc, int64_t, int64_t, int64_t, OpFmt, OpFmt, int, int, int, int, int64_t, float, EpiParams, int);
-    static constexpr Kernel k[3] = {esb_gemm_ws_kernel<SrcA, false, false>, esb_gemm_ws_kernel<SrcA, true, false>,
-                                    esb_gemm_ws_kernel<SrcA, false, true>};
+    static constexpr Kernel k[4] = {esb_gemm_ws_kernel<SrcA, kEpiB4>, esb_gemm_ws_kernel<SrcA, kEpiLean4>,
+                                    esb_gemm_ws_kernel<SrcA, kEpiGen>, esb_gemm_ws_kernel<SrcA, kEpiTable>};
 };
 
 template <class SrcA>
@@ -871,11 +870,18 @@ static int ws_static_smem(cudaError_t* err)
 
 // 4-bit codes as the only output, a scalar scale and bias, sums below 2^20 and
 // a monotone requantisation (unsigned codes or an activation): what the
-// specialised epilogue (LEAN4) takes.
+// specialised epilogue (kEpiLean4) takes.
 bool lean4_ok(const EpiParams& ep)
 {
     return ep.codes_out && ep.out.b == 4 && !ep.scale && !ep.bias && !ep.residual && !ep.acc_out && !ep.y_out &&
            ep.acc_lim > 0.0f && (!ep.out.is_signed || ep.act != ESB_ACT_NONE);
+}
+
+int epi_kind(const EpiParams& ep)
+{
+    if (lean4_ok(ep)) return kEpiLean4;
+    if (ep.codes_out && ep.out.b == 4) return kEpiB4;
+    return epi_cells_ok(ep) ? kEpiTable : kEpiGen;
 }
 
 // The epilogue's paths in microseconds per 128 x 16 outputs, from tiles whose
@@ -934,8 +940,7 @@ static bool launch_ws(const SrcA& a, const RowsSrc& b, int64_t M, int64_t N, int
     if (per_n > m_tiles) per_n = m_tiles;
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool gen = !(ep.codes_out && ep.out.b == 4);       // the general-width epilogue instance
-    *err = launch_pdl(WsKernels<SrcA>::k[lean4_ok(ep) ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kWsThreads),
+    *err = launch_pdl(WsKernels<SrcA>::k[epi_kind(ep)], dim3((unsigned)grid), dim3(kWsThreads),
                       (size_t)L.smem_bytes, st, a, b, M, N, K, fa, fb, BN, L.nkb, L.stages, n_tiles, m_tiles, acc_scale, ep,
                       bstream);
     return true;

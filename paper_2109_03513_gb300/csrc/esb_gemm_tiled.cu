@@ -12,13 +12,14 @@
 //     per code out.
 //  2. esb_gemm_tiled_kernel, persistent and warp-specialised: one producer
 //     thread bulk-copies whole tiles (A: 128 rows, 16 KiB; B: BN rows,
-//     30 or 32 KiB) into a ring of shared-memory stages (cp.async.bulk
+//     up to 32 KiB) into a ring of shared-memory stages (cp.async.bulk
 //     completing on mbarriers), the MMA thread issues four 128 x BN x 32
 //     tcgen05.mma per K-block into one of two BN-column TMEM accumulators,
 //     and eight epilogue warps drain them through the epilogue of the other
 //     tcgen05 kernels (ws_epilogue).  Each CTA keeps one N-tile and walks
-//     the M-tiles.  BN is 256, or 240 for outputs of 3, 5 or 6 bits, whose
-//     10, 6 or 5 codes per word divide 240 (a word never straddles tiles).
+//     the M-tiles.  BN is at most 256, or 240 for outputs of 3, 5 or 6 bits,
+//     whose 10, 6 or 5 codes per word divide 240 (a word never straddles
+//     tiles), and down to 64 where few row tiles leave SMs idle (tiled_bn).
 //     Measured at 4096^3 with 6-bit codes: 62 us for the call, against 1458
 //     us for the streamed kernel, which decodes every operand row again in
 //     each tile (the only one to take these widths before).
@@ -40,7 +41,7 @@ namespace esb {
 namespace {
 
 constexpr int kTiledBN = 256;                  // N-tile width (rows of a B tile); 128 with > 2 K-chunks
-constexpr int kTiledBNOdd = 240;               // for 3, 5, 6 or 10 output codes per word
+constexpr int kTiledBNOdd = 240;               // for 10, 6 or 5 output codes per word (3, 5, 6 bits)
 constexpr int kTiledThreads = 320;             // warps 0-7 epilogue, 8 MMA, 9 producer
 constexpr int kTiledProdWarp = 9;
 constexpr int kTileA = kBM * kBK;              // 16 KiB
@@ -322,7 +323,7 @@ __device__ void tiled_chunked_epilogue(const EpiParams& ep, const float* thr, in
     }
 }
 
-template <bool LEAN4, bool GEN>
+template <int EPI>
 __global__ void __launch_bounds__(kTiledThreads, 1)
 esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict__ Bt, int64_t M, int64_t N, int64_t mpad,
                       int64_t npad, int nkb, int kbc, int nch, int BN, int stages, int n_tiles, int64_t m_tiles,
@@ -351,7 +352,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
     uint32_t tmem_cols = 32;                                     // a power of two >= the regions used
     while (tmem_cols < (uint32_t)(nbuf * nch * BN)) tmem_cols <<= 1;
     constexpr int lacc = 1;                              // nch == 1: two buffers
-    const EpiSplit sp = epi_split<GEN>(ep, BN, my_tiles);
+    const EpiSplit sp = epi_split<EPI>(ep, BN, my_tiles);
     // the layout above must fit the dynamic allocation (uniform for the CTA)
     if ((uintptr_t)(reinterpret_cast<const volatile uint8_t*>(err) + 4 - smem_raw) > dynamic_smem_bytes()) {
         if (tid == 0) record_status(ep.status, ESB_ERR_INTERNAL);
@@ -450,7 +451,7 @@ esb_gemm_tiled_kernel(const uint8_t* __restrict__ At, const uint8_t* __restrict_
             m = (first + ti * ctas) * kBM + row;
             return m < M;
         };
-        ws_epilogue<LEAN4, GEN>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
+        ws_epilogue<EPI>(ep, thr, rows, my_tiles, n0, N, BN, sp, lacc, tmem_base, acc_scale, tfull, tempty,
                            err, warp, lane);
     }
 
@@ -515,11 +516,15 @@ size_t gemm_tiled_workspace_bytes(int64_t M, int64_t N, int64_t K)
     return (size_t)(cdiv(M, kBM) * nkb * kTileA + cdiv(N, kTiledBN) * nkb * (int64_t)kTiledBN * kBK);
 }
 
-// The tiled path pays an extra launch and a pass over both operands:
-// below about 2^32 multiply-adds the other kernels finish first (when they
-// can: their decode is fast for 4-bit operands only).  ESB_GEMM_TILED_MIN_MACS
-// in the environment (read per call) moves that threshold (0: every shape
-// the kernel takes).
+// The tiled path pays an extra launch and a pass over both operands.  The
+// lines, 2^32 multiply-adds for 4-bit operands and 2^28 for the outputs that
+// esb_gemm's kernels also take, were drawn when the pass was two launches and
+// the GEMM had 256-column tiles only.  Measured since (esb_gemm's kernels and
+// this one, us): 4 bits, 2^28 (512 x 512 x 1024) 12.4 and 7.8, 2^30 (1024^3) 13.4
+// and 8.1, 2^32 (2048 x 2048 x 1024) 27.3 and 11.3, 2^26 (256 x 512 x 512) 8.1 and
+// 7.2; 6 bits 23.7 and 14.5, 23.9 and 14.8, 64.2 and 20.1, 13.4 and 11.9: they
+// could lie lower.  ESB_GEMM_TILED_MIN_MACS in the environment (read per call)
+// moves them (0: every shape the kernel takes).
 bool gemm_tiled_ok(int64_t M, int64_t N, int64_t K, int ba, int ka, int bb, int kb, int out_cpw)
 {
     int kbc, nch, BN;
@@ -532,14 +537,14 @@ bool gemm_tiled_ok(int64_t M, int64_t N, int64_t K, int ba, int ka, int bb, int 
     return (double)M * N * K >= min_macs;
 }
 
-// 3, 5, 6 or 10 output codes per word: esb_gemm's kernels take every shape
-// of these too, so a call without (enough) workspace runs there.
+// 5, 6 or 10 output codes per word: esb_gemm's kernels take every shape of
+// these too, so a call without (enough) workspace runs there.
 bool gemm_tiled_optional(int out_cpw) { return kTiledBN % out_cpw != 0; }
 
 typedef void (*TiledKernel)(const uint8_t*, const uint8_t*, int64_t, int64_t, int64_t, int64_t, int, int, int, int, int,
                             int, int64_t, float, EpiParams);
-static const TiledKernel kTiledKernels[3] = {esb_gemm_tiled_kernel<false, false>, esb_gemm_tiled_kernel<true, false>,
-                                             esb_gemm_tiled_kernel<false, true>};
+static const TiledKernel kTiledKernels[4] = {esb_gemm_tiled_kernel<kEpiB4>, esb_gemm_tiled_kernel<kEpiLean4>,
+                                             esb_gemm_tiled_kernel<kEpiGen>, esb_gemm_tiled_kernel<kEpiTable>};
 
 static int tiled_static_smem(cudaError_t* err)
 {
@@ -624,10 +629,9 @@ cudaError_t launch_gemm_tiled(int64_t M, int64_t N, int64_t K, const uint32_t* A
     if (per_n > m_tiles) per_n = m_tiles;
     const int64_t grid = per_n * n_tiles;
     const float acc_scale = ldexpf(1.0f, fa.csc + fb.csc);
-    const bool fast = nch == 1 && lean4_ok(ep);   // the specialised epilogue
-    // one chunk of other widths' codes only: the general-width epilogue instance
-    const bool gen = nch == 1 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
-    return launch_pdl(kTiledKernels[fast ? 1 : (gen ? 2 : 0)], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,
+    // K in chunks has an epilogue of its own, in every instance; fp32 and int32 outputs run in the 4-bit one
+    const bool codes = nch == 1 && ep.codes_out && !ep.acc_out && !ep.y_out;
+    return launch_pdl(kTiledKernels[codes ? epi_kind(ep) : kEpiB4], dim3((unsigned)grid), dim3(kTiledThreads), smem, st,
                       (const uint8_t*)At, (const uint8_t*)Bt, M, N, mpad, npad, nkb, kbc, nch, BN, stages, (int)n_tiles,
                       m_tiles, acc_scale, ep);
 }

@@ -859,21 +859,30 @@ static __device__ __noinline__ uint2 epi_chunk16(const EpiParams& ep, const EpiC
 // one 16-byte store where the row allows it.
 constexpr int kEpiCells = 256;     // entries of the table; larger tables keep the bisection
 
-// Whether ws_epilogue takes epi_cells for these outputs (host and device
-// agree: it sets the number of epilogue warps).
+// Whether the kEpiTable instance takes these outputs.
 __host__ __device__ inline bool epi_cells_ok(const EpiParams& ep)
 {
     return ep.codes_out && !ep.acc_out && !ep.y_out && (ep.out.b == 3 || ep.out.b == 5 || ep.out.b == 6) &&
            (!ep.residual || ep.res_b == ep.out.b);
 }
 
+// The kernel instances by epilogue (each keeps a small hot loop): 4-bit codes,
+// the specialised path for them (lean4_ok), other outputs, and codes of 3, 5 or
+// 6 bits by the cell table.
+enum { kEpiB4 = 0, kEpiLean4 = 1, kEpiGen = 2, kEpiTable = 3 };
+
 // How the 8 epilogue warps share the tiles (two groups of 4 warps, each
 // covering the 128 rows): by columns (the first group takes [0, mid)), or
 // alternate tiles whole (alt), or the first group alone.  Every tile costs a
 // warp a fixed time (two barrier waits, a TMEM round trip, the row's address)
 // beside its columns, about 1000 cycles: alternating halves it per tile, and
-// is the only way to use both groups on a 16-column tile.  It needs
-// enough tiles to even out the one that is drained last.
+// is the only way to use both groups on a 16-column tile.  It needs enough
+// tiles to even out the one that is drained last: 48 columns of signed 4-bit
+// codes, by columns and alternately, 51.8 and 45.6 us at 20 tiles a CTA, 25.2 and
+// 22.8 at 8, 15.9 and 14.6 at 4, 12.1 and 11.6 at 2; 64 columns 54.0 and 52.8 at
+// 20, 12.4 and 12.2 at 2; other outputs and 32 columns within 4 % throughout.
+// By columns below 8, where half of an odd number of tiles is one in three or
+// more.
 struct EpiSplit {
     int warps;           // epilogue warps in use
     bool alt;
@@ -881,11 +890,11 @@ struct EpiSplit {
     __device__ __forceinline__ int tempty_count() const { return alt ? 4 : warps; }
 };
 
-template <bool GEN>
+template <int EPI>
 __device__ __forceinline__ EpiSplit epi_split(const EpiParams& ep, int BN, int64_t my_tiles)
 {
-    const bool cells = GEN && epi_cells_ok(ep);
-    const bool swar = !GEN && ep.codes_out && ep.out.b == 4;       // 16-column chunks of whole words
+    const bool cells = EPI == kEpiTable;
+    const bool swar = EPI <= kEpiLean4 && ep.codes_out && ep.out.b == 4;       // 16-column chunks of whole words
     // whole 16-column chunks and whole words on both sides (epi_cells splits by passes of its own)
     const int cpw = ep.codes_out ? ep.out_cpw : 16;
     const int unit = cpw == 6 ? 48 : (cpw == 5 || cpw == 10 ? 80 : 16);
@@ -1088,7 +1097,7 @@ __device__ __forceinline__ void epi_cells(const EpiParams& ep, const float* thr,
 
 // ------------------------------------ roles of the warp-specialised kernels
 
-// TMEM for the two accumulator buffers, allocated by the MMA warp before the
+// TMEM for the accumulator buffers, allocated by the MMA warp before the
 // CTA's first barrier (the caller then runs __syncthreads, and ws_setup reads
 // the base address after it).
 __device__ __forceinline__ void ws_alloc(int warp, uint32_t* tmem_slot, uint32_t tmem_cols)
@@ -1228,31 +1237,26 @@ __device__ __noinline__ void epi_chunk_tiles(const EpiParams& ep, const EpiParam
 // gives the output row m of a tile row and whether it exists.  LEAN4: the
 // host has established 4-bit codes as the only output with a scalar scale
 // and bias and sums below 2^20 (lean4_ok); the instance then holds just the
-// FMA-pipe requantisation.  GEN: the output is not 4-bit codes; the instance
-// holds the general-width code path and none of the 4-bit code.  Calls that
-// an instance has no path for take epi_chunk_tiles (each instance keeps a
-// small hot loop, without calls).
-template <bool LEAN4, bool GEN, class RowMap>
+// FMA-pipe requantisation.  kEpiGen: the output is not 4-bit codes; the instance
+// holds the general-width code path and none of the 4-bit code.  kEpiTable: 3-,
+// 5- or 6-bit codes alone (epi_cells_ok).  Calls that an instance has no path
+// for take epi_chunk_tiles (each instance keeps a small hot loop, without calls).
+template <int EPI, class RowMap>
 __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* thr, const RowMap& rows,
                                             int64_t my_tiles, int64_t n0, int64_t N, int BN, const EpiSplit& sp, int lacc,
                                             uint32_t tmem_base, float acc_scale, uint64_t* tfull,
                                             uint64_t* tempty, volatile int* err, int warp, int lane)
 {
-    // the tables of epi_cells and of the bisection path below share their storage
-    __shared__ union GenSmem {
-        EpiCellsSmem cells;
-        struct { float rawT[128], gres[256]; } gen;
-    } sh_gen;
-    if constexpr (GEN) {
-        if (epi_cells_ok(ep)) {
-            if (ep.out.b == 3)
-                epi_cells<3>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-            else if (ep.out.b == 5)
-                epi_cells<5>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-            else
-                epi_cells<6>(ep, thr, sh_gen.cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
-            return;
-        }
+    constexpr bool LEAN4 = EPI == kEpiLean4, GEN = EPI == kEpiGen;
+    if constexpr (EPI == kEpiTable) {
+        __shared__ EpiCellsSmem sh_cells;
+        if (ep.out.b == 3)
+            epi_cells<3>(ep, thr, sh_cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else if (ep.out.b == 5)
+            epi_cells<5>(ep, thr, sh_cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        else
+            epi_cells<6>(ep, thr, sh_cells, rows, my_tiles, sp.alt, lacc, n0, N, BN, tmem_base, acc_scale, tfull, tempty, err, warp, lane);
+        return;
     }
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;              // TMEM lane = tile row
@@ -1285,7 +1289,7 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
     // over the 2^(b-1) - 1 thresholds; with a positive scalar scale (and an
     // unsigned output or an activation) over the same thresholds moved onto
     // the raw accumulator (gen_raw, as raw_ok above), one compare per level.
-    const bool gen = GEN && !LEAN4 && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
+    const bool gen = GEN && ep.codes_out && ep.out.b != 4 && !ep.acc_out && !ep.y_out;
     const bool gen_raw = gen && !ep.scale && !ep.bias && !ep.residual && isfinite(sc_lean) && sc_fixed > 0.0f &&
                          (!out_signed || ep.act != ESB_ACT_NONE);
     // 4-bit codes out with a 4-bit residual and a scalar scale and bias
@@ -1297,8 +1301,8 @@ __device__ __forceinline__ void ws_epilogue(const EpiParams& ep, const float* th
                       ep.res_b == 4 && isfinite(sc_lean) && (sc_lean != 0.0f || sc_fixed == 0.0f);
     __shared__ float sh_resimg[16];
     if (lres && warp == 0 && lane < 16) sh_resimg[lane] = code_image_f((uint32_t)lane, 4, ep.res_k);
-    float* const sh_rawT = sh_gen.gen.rawT;           // gen: the thresholds searched (raw or on y)
-    float* const sh_gres = sh_gen.gen.gres;           // gen: images of the residual's codes
+    __shared__ float sh_rawT[GEN ? 128 : 1];          // gen: the thresholds searched (raw or on y)
+    __shared__ float sh_gres[GEN ? 256 : 1];          // gen: images of the residual's codes
     const bool gres = gen && !gen_raw && ep.residual;
     if (gres)
         for (int i = warp * 32 + lane; i < (1 << ep.res_b); i += epi_warps * 32)
@@ -1584,7 +1588,8 @@ __device__ __forceinline__ void ws_drain(uint64_t* drain, volatile int* err, uin
 int pick_bn(int64_t N, int out_cpw);          // N-tile width (esb_gemm.cu)
 int resident_bn(int64_t M, int64_t N, int out_cpw, int bn0);   // the same where few row tiles leave SMs idle
 int max_dyn_smem();                           // opt-in shared memory per block
-bool lean4_ok(const EpiParams& ep);           // the LEAN4 epilogue takes the call (esb_gemm.cu)
+bool lean4_ok(const EpiParams& ep);           // the kEpiLean4 epilogue takes the call (esb_gemm.cu)
+int epi_kind(const EpiParams& ep);            // the instance for a call (esb_gemm.cu)
 EpiParams make_epi(const GemmOutputs& o);     // epilogue parameters of a call
 float acc_fma_limit(int64_t K, int ba, int ka, int bb, int kb);   // FMA-pipe requantisation bound (esb_gemm.cu)
 
