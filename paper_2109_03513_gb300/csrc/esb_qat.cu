@@ -416,11 +416,12 @@ cudaError_t launch_dn_project(const float* x, int64_t rows, int64_t cols, const 
     int64_t blocks = flat ? (rows * cols / 128 + 8 * kDnUnroll - 1) / (8 * kDnUnroll) : (words + kQatThreads - 1) / kQatThreads;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    // Wide formats with at most a word per thread: a division per element costs
-    // less than thresholds on |x - mu| and their table (1000 x 77, 8 bits: 6.0 us
-    // against 8.3 to 9.6; 6 bits 3.9 against 4.3 to 4.7; at 10000 x 64 they are
-    // level, at 100352 x 64 the table takes 24.6 against 27.8 at 6 bits).
-    const int divide = b >= 6 && words <= sms * 4 * kQatThreads;
+    // Wide formats with few words per thread: a division per element costs less
+    // than thresholds on |x - mu| and their table (1000 x 77, 8 bits: 6.0 us against
+    // 8.3 to 9.6; 6 bits 3.9 against 4.3 to 4.7; 10000 x 64, 8 bits 9.7 against 10.8
+    // to 12.3; at 20000 x 64, 320000 words, they are level; at 100352 x 64 the table
+    // takes 24.6 against 27.8 at 6 bits).
+    const int divide = b >= 6 && words <= sms * 8 * kQatThreads;
     using Kernel = void (*)(const float*, int64_t, int64_t, const double*, float, ProjParams, uint32_t*, int64_t, float*, int, int);
     static const Kernel kernels[] = {dn_project_kernel<2>, dn_project_kernel<3>, dn_project_kernel<4>, dn_project_kernel<5>,
                                      dn_project_kernel<6>, dn_project_kernel<7>, dn_project_kernel<8>};

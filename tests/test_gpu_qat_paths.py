@@ -19,8 +19,8 @@ def built():
     __graft_entry__.build()
 
 
-# the last: more words than the wide formats divide for (a thread per word of four blocks per SM)
-@pytest.mark.parametrize("rows,cols", [(1, 8), (37, 24), (5, 136), (3, 1), (2, 331), (40001, 16)])
+# the last: more words than the wide formats divide for
+@pytest.mark.parametrize("rows,cols", [(1, 8), (37, 24), (5, 136), (3, 1), (2, 331), (80001, 16)])
 @pytest.mark.parametrize("fmt", [(2, 0, True), (3, 1, True), (4, 2, True), (4, 1, False), (5, 2, True), (6, 5, True),
                                  (7, 3, True), (8, 4, False)])
 @pytest.mark.parametrize("sigma", [1.7, 0.0, float("inf"), float("nan")])
