@@ -344,8 +344,9 @@ struct StemPlan {
 };
 
 // Whether this kernel finishes before the im2col kernel, by a model of both in
-// microseconds: a fixed part (launch, prologue), and waves of tiles (one CTA per
-// SM) times a tile's cost.  Both tiles are 128 rows, but here only `use` = Q /
+// microseconds: a fixed part (launch, prologue; here also the filters' decode,
+// 0.9 us a pass of 288 chunks), and waves of tiles (one CTA per SM) times a
+// tile's cost.  Both tiles are 128 rows, but here only `use` = Q /
 // (128 nseg) of them are outputs, so a costly epilogue counts 1 / use times; the
 // im2col kernel pays for each filter tap's word (another filter width: code by
 // code) and a longer prologue, and takes narrower N-tiles where few row tiles
@@ -356,8 +357,9 @@ struct StemPlan {
 // scale per channel 592 and 381 at 64, 392 and 382 at 100; with y 847 and 327
 // at 32; 2x2/2 -> 287, 3-bit, at 26: 283 and 69; 6-bit 3x3/2 -> 64: 134 and 101
 // at 64, 91 and 101 at 100; one image of 224 x 224: 10.5 and 19.2; 10 x 10 -> 164
-// sums alone, batch 3: 26.0 and 14.2.
-static bool stem_pays(const StemGeom& g, int64_t n, int64_t N, int BN, int out_cpw, bool mixed, double e16)
+// sums alone, batch 3: 26.0 and 14.2; 11x11/2 -> 238, 6-bit, 11 x 13, batch 20: 52.2
+// and 29.3.
+static bool stem_pays(const StemGeom& g, int64_t n, int64_t N, int BN, int nkb, int out_cpw, bool mixed, double e16)
 {
     const double sms = device_sm_count();
     const int64_t m = n * g.P * g.Q;
@@ -366,7 +368,8 @@ static bool stem_pays(const StemGeom& g, int64_t n, int64_t N, int BN, int out_c
     const double gather = fmax(2.0, 0.5 + 0.15 * g.R * g.S) * (mixed ? 3 : 1);
     const double im2col = 14.0 + ceil((double)(((m + kBM - 1) / kBM) * ((N + bni - 1) / bni)) / sms) *
                                     (fmax(epi_i, gather) + 0.25 * fmin(epi_i, gather));
-    const double stem = 9.0 + ceil((double)(n * g.P * g.nseg * ((N + BN - 1) / BN)) / sms) * fmax(epi, 0.8 + 0.06 * g.R * g.G);
+    const double filters = fmax(0.0, nkb * 8.0 * BN / (kWsProdWarp0 * 32) - 9.0);   // passes past the fixed part's
+    const double stem = 9.0 + 0.9 * filters + ceil((double)(n * g.P * g.nseg * ((N + BN - 1) / BN)) / sms) * fmax(epi, 0.8 + 0.06 * g.R * g.G);
     return stem < im2col;
 }
 
@@ -389,13 +392,13 @@ static bool stem_plan(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx,
     g.nseg = (per + umax - g.G) / (umax - g.G + 1);
     g.Ui = (per + g.nseg - 1) / g.nseg;
     g.U = g.Ui + g.G - 1;
-    if ((int64_t)d.n * P * g.nseg >= (1ll << 30) || !stem_pays(g, d.n, d.cout, bn0, out_cpw, bx != bw, e16)) return false;
+    sp->BN = bn0;
+    sp->nkb = (d.r * g.G * 16 + kBK - 1) / kBK;
+    if ((int64_t)d.n * P * g.nseg >= (1ll << 30) || !stem_pays(g, d.n, d.cout, bn0, sp->nkb, out_cpw, bx != bw, e16)) return false;
     g.pitch = (kBM + g.G - 1) * 16;
     const int st = stem_static_smem(err);
     if (st < 0) return false;
     const int64_t maxs = max_dyn_smem() - st;
-    sp->BN = bn0;
-    sp->nkb = (d.r * g.G * 16 + kBK - 1) / kBK;
     const int64_t fixed = 1024 + (int64_t)sp->nkb * bn0 * kBK + 4 * 128 + (2 * kStemMaxRing + 2 * kMaxAcc + 1) * 8 + 64;
     int64_t nr = (maxs - fixed) / g.pitch;
     if (nr > kStemMaxRing) nr = kStemMaxRing;

@@ -1073,8 +1073,15 @@ static ConvK conv_k(const esb_conv_desc& d, const uint32_t* W, int64_t ldx, int 
 // whatever they hold: one MMA step per tap, and each pixel decoded once (112 x
 // 112 x 16 -> 96, 1x1: 91 us by single words on the im2col kernel, 71 us there;
 // -> 32, 3x3: 169 and 80 us).
+// Not with fewer tiles than SMs under a costly epilogue, where the im2col kernel
+// takes narrower N-tiles (24 x 24 x 3 -> 114, 1x1, 2-bit, batch 8: 22.0 and 16.6).
 static bool conv_halo_rows(const ConvK& c) { return c.K > 0 && c.fa.planes == 1 && c.b.kp == 0; }
 static int conv_halo_words(const esb_conv_desc& d, int64_t ldx, int kwx) { return d.stride == 1 && ldx == 4 ? 4 : kwx; }
+static bool conv_halo_wanted(const esb_conv_desc& d, int64_t M, const ConvK& c, int words, int kwx, int bn, double e16)
+{
+    const int64_t tiles = (M + kBM - 1) / kBM * ((d.cout + bn - 1) / bn);
+    return conv_halo_rows(c) && (words == kwx || e16 < 1.0 || tiles >= device_sm_count());
+}
 
 // Stride-1 layers of four-word rows that the halo kernel refuses (wide images,
 // odd sizes) on the im2col kernel: the whole row in K by 16-byte pieces, or the
@@ -1131,8 +1138,11 @@ cudaError_t launch_conv_tc(const esb_conv_desc& d, int P, int Q, const uint32_t*
     cudaError_t e = cudaSuccess;
     if (!conv_force_im2col()) {
         if (launch_conv_stem(d, P, Q, X, ldx, make_opfmt(bx, kx), W, ldw, make_opfmt(bw, kw), BN, ep, st, &e)) return e;
-        const ConvK h = conv_k(d, W, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
-        if (conv_halo_rows(h) && launch_conv_halo(d, P, Q, X, ldx, h.fa, W, ldw, h.fb, BN, ep, st, &e)) return e;
+        const int kwm = conv_k_words(d, ldx, bx, ldw, bw), kwh = conv_halo_words(d, ldx, kwm);
+        const ConvK h = conv_k(d, W, ldx, bx, kx, ldw, bw, kw, kwh);
+        if (conv_halo_wanted(d, M, h, kwh, kwm, BN, epi_cost16(ep)) &&
+            launch_conv_halo(d, P, Q, X, ldx, h.fa, W, ldw, h.fb, BN, ep, st, &e))
+            return e;
     }
     int kwx;
     const ConvK c = conv_im2col(d, M, W, ldx, bx, kx, ldw, bw, kw, ep.out_cpw, &kwx);
@@ -1147,12 +1157,15 @@ int conv_kernel_choice(const esb_conv_desc& d, int P, int Q, int64_t ldx, int bx
                        int kw, int out_b)
 {
     const int cpw = 32 / out_b;                                   // as launch_conv_tc
+    const int64_t M = (int64_t)d.n * P * Q;
     if (!conv_force_im2col()) {
         if (conv_stem_ok(d, P, Q, ldx, bx, kx, bw, kw, out_b)) return ESB_CONV_KERNEL_STEM;
-        const ConvK h = conv_k(d, nullptr, ldx, bx, kx, ldw, bw, kw, conv_halo_words(d, ldx, conv_k_words(d, ldx, bx, ldw, bw)));
-        if (conv_halo_rows(h) && conv_halo_ok(d, P, Q, ldx, bx, kx, out_b)) return ESB_CONV_KERNEL_HALO;
+        const int kwm = conv_k_words(d, ldx, bx, ldw, bw), kwh = conv_halo_words(d, ldx, kwm);
+        const ConvK h = conv_k(d, nullptr, ldx, bx, kx, ldw, bw, kw, kwh);
+        if (conv_halo_wanted(d, M, h, kwh, kwm, pick_bn(d.cout, cpw), epi_cost16_codes(out_b)) &&
+            conv_halo_ok(d, P, Q, ldx, bx, kx, out_b))
+            return ESB_CONV_KERNEL_HALO;
     }
-    const int64_t M = (int64_t)d.n * P * Q;
     int kwx;
     const ConvK c = conv_im2col(d, M, nullptr, ldx, bx, kx, ldw, bw, kw, cpw, &kwx);
     cudaError_t e = cudaSuccess;
